@@ -639,7 +639,7 @@ def main() -> None:
     total_kernel_ms = sum(kms)
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": traffic,
-                "kernel": "flux_closed_kernel<3,d> + flux_pending_kernel<3,d> (interface fluxes, "
+                "kernel": "flux_closed_kernel<3,d> + flux_correct_kernel<3,d> (interface fluxes, "
                           "one direction of one RK stage per evaluation)",
                 "kernel_share": flux_ms / total_kernel_ms if total_kernel_ms else None,
                 "peak_source": f"derived: {SM_COUNT} SMs x {FP64_FLOP_PER_CLK_PER_SM} FP64 flop/clk x "

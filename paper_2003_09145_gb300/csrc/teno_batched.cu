@@ -64,8 +64,9 @@ __global__ void __launch_bounds__(BLOCK) batched_stage_kernel(BatchArgs A, Schem
   __shared__ double s_alpha[3];
   __shared__ double s_dt, s_idx;
   __shared__ double s_F[BLOCK][3];
-  __shared__ int s_pend[BLOCK];   // tile faces the certified test leaves pending
+  __shared__ int s_pend[BLOCK];   // tile faces with open reconstructions: face | mask << 16
   __shared__ int s_npend;
+  __shared__ teno::CorrectScratch<1> s_cor[NW];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
   for (;;) {
@@ -161,29 +162,38 @@ __global__ void __launch_bounds__(BLOCK) batched_stage_kernel(BatchArgs A, Schem
 #pragma unroll
         for (int j = 0; j < 6; ++j) cells[j] = off + teno::ghost(face - 3 + j, n, A.bc);
         double out[3];
-        if (teno::interface_flux_closed<1, 0>(A.Uin, A.aux, A.fh, A.ncell, cells, 0u, alpha, nal, S, out,
-                                              A.status)) {
+        const unsigned open = teno::interface_flux_closed<1, 0>(A.Uin, A.aux, A.fh, A.ncell, cells, 0u, alpha, nal,
+                                                                S, out, A.status);
+        if (!(open & teno::kRough)) {
           s_F[tid][0] = out[0];
           s_F[tid][1] = out[1];
           s_F[tid][2] = out[2];
-        } else {
-          s_pend[atomicAdd(&s_npend, 1)] = tid;
         }
+        if (open) s_pend[atomicAdd(&s_npend, 1)] = int(unsigned(tid) | open << 16);
       }
       __syncthreads();
-      if (tid < s_npend) {
-        const int t = s_pend[tid];
-        const int64_t f2 = i0 + t;
-        int64_t cells[6];
+      // the open faces, shared out evenly (a warp's time is its FP64
+      // instruction count: few faces per warp while they last, up to 32)
+      const int npend = s_npend;
+      int per = 2;
+      while (per < 32 && npend > per * NW) per *= 2;
+      auto cells_of = [&](uint32_t f, int64_t (&cells)[6], unsigned& flips) {
+        flips = 0u;
 #pragma unroll
-        for (int j = 0; j < 6; ++j) cells[j] = off + teno::ghost(f2 - 3 + j, n, A.bc);
-        double out[3];
-        unsigned fl[3][2];
-        teno::interface_flux<1, 0, false, teno::kFluxChar>(A.Uin, A.aux, A.ncell, cells, 0u, alpha, nal, S, out, fl,
-                                                           A.status);
-        s_F[t][0] = out[0];
-        s_F[t][1] = out[1];
-        s_F[t][2] = out[2];
+        for (int j = 0; j < 6; ++j) cells[j] = off + teno::ghost(i0 + f - 3 + j, n, A.bc);
+      };
+      for (int k0 = warp * per; k0 < npend; k0 += NW * per) {
+        const bool mine = lane < per && k0 + lane < npend;
+        const unsigned e = mine ? unsigned(s_pend[k0 + lane]) : 0u;
+        const int t = int(e & 0xffffu);
+        double out[3] = {s_F[t][0], s_F[t][1], s_F[t][2]};
+        teno::warp_correct<1, 0, false>(A.Uin, A.aux, A.ncell, cells_of, unsigned(t), alpha, S, e >> 16, out,
+                                        A.status, s_cor[warp]);
+        if (mine) {
+          s_F[t][0] = out[0];
+          s_F[t][1] = out[1];
+          s_F[t][2] = out[2];
+        }
       }
       __syncthreads();
       const int64_t cell = i0 + tid;

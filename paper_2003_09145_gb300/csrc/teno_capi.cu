@@ -96,7 +96,7 @@ Layout layout_of(const teno_grid* g, int op) {
   L.fhat = off;
   off += round_up(sizeof(double) * nvar * size_t(maxifc));
   L.list = off;
-  off += round_up(sizeof(uint32_t) * size_t(maxifc));
+  off += round_up(sizeof(uint2) * size_t(maxifc));
   L.ghost = off;   // fixed-state ghost cells (state, primitives, half fluxes of 6 face slots)
   off += round_up(sizeof(double) * size_t(teno::ghost_block_doubles(g->ndim)));
   if (op == TENO_OP_RK3) {
@@ -257,7 +257,7 @@ teno_status stage_finish(const teno_grid* g, const Layout& L, char* ws, const do
   auto* alpha = reinterpret_cast<unsigned long long*>(ws + L.alpha);
   double* aux = reinterpret_cast<double*>(ws + L.aux);
   double* Fhat = reinterpret_cast<double*>(ws + L.fhat);
-  uint32_t* list = reinterpret_cast<uint32_t*>(ws + L.list);
+  uint2* list = reinterpret_cast<uint2*>(ws + L.list);
   double* fh = flags ? nullptr : reinterpret_cast<double*>(ws + L.fh);   // the flag path is one-pass
   unsigned* count = reinterpret_cast<unsigned*>(ws + L.alpha + teno::kPendingCountOffset);
   if (with_dt) {

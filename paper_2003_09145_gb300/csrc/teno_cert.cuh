@@ -153,6 +153,113 @@ TENO_CERT_HD bool certify_keep_values(double v0, double v1, double v2, double v3
 }
 
 // ---------------------------------------------------------------------------
+// The selections of one reconstruction (LAD, eq. 3.1-3.4, or a fixed C_T) in
+// single precision, from the binary64 first differences e_k = v_{k+1} - v_k:
+// returns true with the three delta bits in `sel` if the binary64 evaluation
+// of the same differences takes them, false if a decision lies within its
+// error bound (the caller then decides in binary64).
+//
+// The differences are truncated to FP32 (error below 2^-20 |e_k| + 2^-126),
+// so the bounds scale with the local variation, not with the values.  With
+// E_k the larger magnitude of stencil k's two differences, |a_k| <= 2 E_k
+// and |c_k| <= 4 E_k are within 2 (2^-20 E_k) + 2u E_k and 4 (2^-20 E_k) + 4u
+// E_k of their exact values (c_0, c_2: one rounding each; c_1, a_k too):
+// da = 2.2 2^-20 E_k + 2^-123, dc = 2 da cover them.  Then, as in
+// certify_keep, db_k bounds |b_k - beta_k| (4u b_k for b_k's own
+// evaluation; the slack of da covers the bound's own roundings), dtau bounds
+// |tau - tau(e)|, and with D_k = b_k + eps:
+//  * D_k is within db_k + 4u D_k of its exact value;
+//  * threshold j of m (eq. 3.1) is certainly met when tau + dtau <=
+//    thr_j dmin_lo (1 - 1e-6), certainly not when tau - dtau > thr_j dmin_hi
+//    (1 + 1e-6), dmin_lo and dmin_hi the least lower and upper bound of the
+//    D_k; m is certain when both counts agree; below the keep-all threshold
+//    thr_keep every stencil is kept whatever m is;
+//  * gamma_k ~ x_k^6 with x_k = 1 + tau / D_k: x_k is within
+//    e_k = dtau / (D_k + tau) + db_k / D_k + 12u of its exact value, relative
+//    (e the largest of the three); q_k = x_k / max x lies in (0, 1], q_k^6 and
+//    its share of the sum of the three are within (1 + e)^24 - 1 <= 26 e
+//    (e <= 2^-9) and some 40 roundings (2e-5 >= 335 u) of theirs;
+//  * the margins are 2^28 times the binary64 evaluation's rounding.
+// m_fixed: the magnitude of C_T; -1: LAD's m; -2: not known here (keep-all only).
+// ---------------------------------------------------------------------------
+TENO_CERT_HD float fdiv(float a, float b) {
+#ifdef __CUDA_ARCH__
+  return __fdiv_rn(a, b);
+#else
+  return a / b;
+#endif
+}
+
+TENO_CERT_HD bool select_diffs(double f0, double f1, double f2, double f3, float eps4_f, float thr_keep_f,
+                               const float* thr_f, int nthr, int b_l, int m_fixed, unsigned keep_all,
+                               const float* ct_f, unsigned& sel) {
+  const float u = 0x1p-24f;
+  const float e0 = hi_float(f0), e1 = hi_float(f1), e2 = hi_float(f2), e3 = hi_float(f3);
+  const float a0 = fsub(e1, e0), a1 = fsub(e2, e1), a2 = fsub(e3, e2);
+  const float c0 = ffma(3.0f, e1, -e0), c1 = fadd(e1, e2), c2 = ffma(-3.0f, e2, e3);
+  const float k = 13.0f / 3.0f;
+  const float b0 = ffma(fmul(k, a0), a0, fmul(c0, c0));
+  const float b1 = ffma(fmul(k, a1), a1, fmul(c1, c1));
+  const float b2 = ffma(fmul(k, a2), a2, fmul(c2, c2));
+  const float q = 2.2f * 0x1p-20f, q0 = 0x1p-123f;
+  const float da0 = ffma(q, fmaxf(fabsf(e0), fabsf(e1)), q0), da1 = ffma(q, fmaxf(fabsf(e1), fabsf(e2)), q0),
+              da2 = ffma(q, fmaxf(fabsf(e2), fabsf(e3)), q0);
+  const float dc0 = 2.0f * da0, dc1 = 2.0f * da1, dc2 = 2.0f * da2;
+  const float db0 = ffma(4.0f * u, b0, ffma(fmul(k, ffma(2.0f, fabsf(a0), da0)), da0, fmul(ffma(2.0f, fabsf(c0), dc0), dc0)));
+  const float db1 = ffma(4.0f * u, b1, ffma(fmul(k, ffma(2.0f, fabsf(a1), da1)), da1, fmul(ffma(2.0f, fabsf(c1), dc1), dc1)));
+  const float db2 = ffma(4.0f * u, b2, ffma(fmul(k, ffma(2.0f, fabsf(a2), da2)), da2, fmul(ffma(2.0f, fabsf(c2), dc2), dc2)));
+  const float tau = fabsf(fsub(b2, b0));
+  const float dtau = ffma(u, tau, fadd(db0, db2));
+  if (!(dtau <= 1.0e30f)) return false;
+  const float D0 = fadd(b0, eps4_f), D1 = fadd(b1, eps4_f), D2 = fadd(b2, eps4_f);
+  const float N0 = fadd(D0, tau), N1 = fadd(D1, tau), N2 = fadd(D2, tau);
+  const float i0 = fdiv(1.0f, D0), i1 = fdiv(1.0f, D1), i2 = fdiv(1.0f, D2);
+  // dtau / N_k <= dtau / (least N_k)
+  const float et = fdiv(dtau, fminf(N0, fminf(N1, N2)));
+  const float e = ffma(1.0f + 8.0f * u, fadd(et, fmaxf(fmul(db0, i0), fmaxf(fmul(db1, i1), fmul(db2, i2)))), 12.0f * u);
+  if (!(e <= 0x1p-9f)) return false;
+  const float lo = fmul(fminf(ffma(-4.0f * u, D0, fsub(D0, db0)),
+                              fminf(ffma(-4.0f * u, D1, fsub(D1, db1)), ffma(-4.0f * u, D2, fsub(D2, db2)))),
+                        1.0f - 1e-6f);
+  const float tp = fadd(tau, dtau);
+  if (tp <= fmul(thr_keep_f, lo)) {
+    sel = 7u;
+    return true;
+  }
+  if (m_fixed < -1) return false;
+  int m = m_fixed;
+  if (m_fixed < 0) {
+    const float hi = fmul(fminf(ffma(4.0f * u, D0, fadd(D0, db0)),
+                                fminf(ffma(4.0f * u, D1, fadd(D1, db1)), ffma(4.0f * u, D2, fadd(D2, db2)))),
+                          1.0f + 1e-6f);
+    const float tm = fsub(tau, dtau);
+    int sure = 0, may = 0;   // the thresholds decrease, so the counts are prefixes
+    for (int j = 0; j < nthr; ++j) {
+      sure += tp <= fmul(thr_f[j], lo) ? 1 : 0;
+      may += tm <= fmul(thr_f[j], hi) ? 1 : 0;
+    }
+    if (sure != may) return false;
+    m = b_l + sure;
+  }
+  if ((keep_all >> m) & 1u) {
+    sel = 7u;
+    return true;
+  }
+  const float x0 = fmul(N0, i0), x1 = fmul(N1, i1), x2 = fmul(N2, i2);
+  const float xm = fdiv(1.0f, fmaxf(x0, fmaxf(x1, x2)));
+  const float y0 = fmul(x0, xm), y1 = fmul(x1, xm), y2 = fmul(x2, xm);
+  const float r0 = fmul(y0, y0), r1 = fmul(y1, y1), r2 = fmul(y2, y2);
+  const float h0 = fmul(fmul(r0, r0), r0), h1 = fmul(fmul(r1, r1), r1), h2 = fmul(fmul(r2, r2), r2);
+  const float lim = fmul(ct_f[m], fadd(fadd(h0, h1), h2));
+  const float M = ffma(26.0f, e, 2e-5f);
+  const float up = fmul(lim, fadd(1.0f, M)), dn = fmul(lim, fsub(1.0f, M));
+  const bool k0 = h0 >= up, k1 = h1 >= up, k2 = h2 >= up;
+  if (!(k0 || h0 <= dn) || !(k1 || h1 <= dn) || !(k2 || h2 <= dn)) return false;
+  sel = (k0 ? 1u : 0u) | (k1 ? 2u : 0u) | (k2 ? 4u : 0u);
+  return true;
+}
+
+// ---------------------------------------------------------------------------
 // The test for all 2 nvar reconstructions of one Euler interface.
 // cert_begin takes the interface's Roe state (u~, b1/2, b2/2, 1/(2c)) and the
 // halved Lax-Friedrichs speeds; cert_point takes one stencil point (its state
@@ -255,20 +362,29 @@ TENO_CERT_HD void cert_point(int j, const double (&Uj)[NDIM + 2], double unj, do
   }
 }
 
+// cert_open: bit 2 f (side v+) and 2 f + 1 (side v-) set where the test does
+// not prove that field f keeps every stencil; cert_keep: none is set.
 template <int NDIM>
-TENO_CERT_HD bool cert_keep(const CertIfc<NDIM>& C, float thr_f, float eps4_f) {
+TENO_CERT_HD unsigned cert_open(const CertIfc<NDIM>& C, float thr_f, float eps4_f) {
   constexpr int NVAR = NDIM + 2;
   const float kd = 8.0f * 0x1p-20f;
   const float ku = ffma(8.0f * 0x1p-24f, C.vmax, 0x1p-100f);
-  bool keep = true;
+  unsigned open = 0u;
 #pragma unroll
   for (int f = 0; f < NVAR; ++f) {
-    keep = keep && certify_keep(C.vp32[0][f], C.vp32[1][f], C.vp32[2][f], C.vp32[3][f], C.vp32[4][f],
-                                ffma(kd, C.mp[f], ku), thr_f, eps4_f);
-    keep = keep && certify_keep(C.vm32[5][f], C.vm32[4][f], C.vm32[3][f], C.vm32[2][f], C.vm32[1][f],
-                                ffma(kd, C.mm[f], ku), thr_f, eps4_f);
+    if (!certify_keep(C.vp32[0][f], C.vp32[1][f], C.vp32[2][f], C.vp32[3][f], C.vp32[4][f],
+                      ffma(kd, C.mp[f], ku), thr_f, eps4_f))
+      open |= 1u << (2 * f);
+    if (!certify_keep(C.vm32[5][f], C.vm32[4][f], C.vm32[3][f], C.vm32[2][f], C.vm32[1][f],
+                      ffma(kd, C.mm[f], ku), thr_f, eps4_f))
+      open |= 2u << (2 * f);
   }
-  return keep;
+  return open;
+}
+
+template <int NDIM>
+TENO_CERT_HD bool cert_keep(const CertIfc<NDIM>& C, float thr_f, float eps4_f) {
+  return cert_open<NDIM>(C, thr_f, eps4_f) == 0u;
 }
 
 }  // namespace teno_cert

@@ -17,6 +17,9 @@ static __constant__ double c_lad[16] = {
     1e-0, 1e-1, 1e-2, 1e-3, 1e-4,  1e-5,  1e-6,  1e-7,
     1e-8, 1e-9, 1e-10, 1e-11, 1e-12, 1e-13, 1e-14, 1e-15};
 
+static __constant__ float c_lad_f[16] = {1e-0f, 1e-1f, 1e-2f,  1e-3f,  1e-4f,  1e-5f,  1e-6f,  1e-7f,
+                                         1e-8f, 1e-9f, 1e-10f, 1e-11f, 1e-12f, 1e-13f, 1e-14f, 1e-15f};
+
 // TENO weights of eq. 2.15 for each selection pattern sel = delta_0 |
 // delta_1 << 1 | delta_2 << 2, with the linear weights c = (0.1, 0.6, 0.3):
 // omega_k = delta_k c_k / sum_j delta_j c_j.  Pattern 0 cannot occur (the
@@ -35,19 +38,21 @@ static __constant__ double c_omega[8][3] = {
 // f^ = v2 + sum_k w_k e_k with, for weights omega = c_omega[sel],
 // w = (-omega_0/3, 5 omega_0/6 + omega_1/6, omega_1/3 + 2 omega_2/3, -omega_2/6)
 // (candidates of eq. 2.4-2.6 relative to v2: (5 e1/6 - e0/3), (e1/6 + e2/3),
-// (2 e2/3 - e3/6)).  With every stencil kept this is eq. 2.3.
-#define TENO_COEF_ROW(o0, o1, o2) \
-  {-(o0) / 3.0, 5.0 * (o0) / 6.0 + (o1) / 6.0, (o1) / 3.0 + 2.0 * (o2) / 3.0, -(o2) / 6.0}
-static __constant__ double c_coef[8][4] = {
-    TENO_COEF_ROW(0.0, 0.0, 0.0),
-    TENO_COEF_ROW(0.1 / 0.1, 0.0, 0.0),
-    TENO_COEF_ROW(0.0, 0.6 / 0.6, 0.0),
-    TENO_COEF_ROW(0.1 / (0.1 + 0.6), 0.6 / (0.1 + 0.6), 0.0),
-    TENO_COEF_ROW(0.0, 0.0, 0.3 / 0.3),
-    TENO_COEF_ROW(0.1 / (0.1 + 0.3), 0.0, 0.3 / (0.1 + 0.3)),
-    TENO_COEF_ROW(0.0, 0.6 / (0.6 + 0.3), 0.3 / (0.6 + 0.3)),
-    TENO_COEF_ROW(0.1 / (0.1 + 0.6 + 0.3), 0.6 / (0.1 + 0.6 + 0.3), 0.3 / (0.1 + 0.6 + 0.3))};
-#undef TENO_COEF_ROW
+// (2 e2/3 - e3/6)); with every stencil kept this is eq. 2.3.  The table holds
+// w[sel] - w[7]: what the selection changes against keeping every stencil.
+#define TENO_CUT_ROW(o0, o1, o2)                                                                       \
+  {-((o0) - 0.1) / 3.0, 5.0 * ((o0) - 0.1) / 6.0 + ((o1) - 0.6) / 6.0,                                 \
+   ((o1) - 0.6) / 3.0 + 2.0 * ((o2) - 0.3) / 3.0, -((o2) - 0.3) / 6.0}
+static __constant__ double c_cut[8][4] = {
+    TENO_CUT_ROW(0.0, 0.0, 0.0),
+    TENO_CUT_ROW(1.0, 0.0, 0.0),
+    TENO_CUT_ROW(0.0, 1.0, 0.0),
+    TENO_CUT_ROW(0.1 / (0.1 + 0.6), 0.6 / (0.1 + 0.6), 0.0),
+    TENO_CUT_ROW(0.0, 0.0, 1.0),
+    TENO_CUT_ROW(0.1 / (0.1 + 0.3), 0.0, 0.3 / (0.1 + 0.3)),
+    TENO_CUT_ROW(0.0, 0.6 / (0.6 + 0.3), 0.3 / (0.6 + 0.3)),
+    TENO_CUT_ROW(0.1, 0.6, 0.3)};
+#undef TENO_CUT_ROW
 
 // The same flux on the point values: f^ = sum_j c_lin[sel][j] v_j with
 // (omega_0/3, -7 omega_0/6 - omega_1/6, 11 omega_0/6 + 5 omega_1/6 + omega_2/3,
@@ -109,6 +114,7 @@ struct Scheme {
   // binary64 condition 1 + max chi~ / H == 1, i.e. max chi~ <= H 2^-53.
   // Entries past B_u - B_l are 0 (the count is clamped to B_u - B_l).
   double thr[kMaxLadder];
+  float thr_f[kMaxLadder];   // thr rounded to binary32 (the certified selection's margin covers it)
 };
 
 // entries per field of the fixed-state ghost block: one per face (2 d + side)
@@ -275,17 +281,20 @@ __device__ __forceinline__ int teno5a_magnitude(double e0, double e1, double e2,
 //  * when max chi~ is small enough that chi_k >= 1/(3 (1 + max chi~)^6) > C_T
 //    holds for every k (Scheme::keep_all), all stencils are kept without
 //    evaluating gamma.
+// With `cut` (not for WENO-Z) it returns acc + (f^ - the value with every
+// stencil kept) instead.
 // ---------------------------------------------------------------------------
 template <bool WITH_M>
 __device__ __forceinline__ double teno5_lad(double v0, double v1, double v2,
                                             double v3, double v4, double acc,
-                                            const Scheme& S, unsigned& flag) {
+                                            const Scheme& S, unsigned& flag, bool cut = false) {
   if (!WITH_M && S.keep_idx >= 0 &&
       teno_cert::certify_keep_values(v0, v1, v2, v3, v4, S.thr_keep_f, S.eps4_f)) {
     // Certified single-precision pre-test (teno_cert.cuh): the exact values
     // satisfy tau <= thr[keep_idx] * dmin with margin, so the binary64 test
     // below and the bound of Scheme::keep_all would both keep every stencil.
     flag = 7u;
+    if (cut) return acc;
     return fma(c_lin[7][0], v0, fma(c_lin[7][1], v1, fma(c_lin[7][2], v2, fma(c_lin[7][3], v3, fma(c_lin[7][4], v4, acc)))));
   }
   const double e0 = v1 - v0, e1 = v2 - v1, e2 = v3 - v2, e3 = v4 - v3;
@@ -326,7 +335,7 @@ __device__ __forceinline__ double teno5_lad(double v0, double v1, double v2,
     const double r = 1.0 / As;
     const double o0 = A0 * r, o1 = A1 * r, o2 = A2 * r;
     flag = 7u;
-    // f^ = v2 + sum_k w_k e_k (see c_coef)
+    // f^ = v2 + sum_k w_k e_k (see c_cut)
     const double w0 = o0 * (-1.0 / 3.0), w1 = fma(o0, 5.0 / 6.0, o1 * (1.0 / 6.0));
     const double w2 = fma(o1, 1.0 / 3.0, o2 * (2.0 / 3.0)), w3 = o2 * (-1.0 / 6.0);
     return fma(w0, e0, fma(w1, e1, fma(w2, e2, fma(w3, e3, v2 + acc))));
@@ -384,8 +393,29 @@ __device__ __forceinline__ double teno5_lad(double v0, double v1, double v2,
     }
     flag = sel | (static_cast<unsigned>(m) << 3);
   }
+  if (cut) {
+    if (sel == 7u) return acc;
+    return fma(c_cut[sel][0], e0, fma(c_cut[sel][1], e1, fma(c_cut[sel][2], e2, fma(c_cut[sel][3], e3, acc))));
+  }
   // eq. 2.4-2.7 with the weights of eq. 2.15 (c_lin)
   return fma(c_lin[sel][0], v0, fma(c_lin[sel][1], v1, fma(c_lin[sel][2], v2, fma(c_lin[sel][3], v3, fma(c_lin[sel][4], v4, acc)))));
+}
+
+// ---------------------------------------------------------------------------
+// The selections alone (delta_0..2 as bits 0..2) of five values with first
+// differences e: teno5_lad's, decided in single precision where teno_cert can
+// prove the binary64 outcome, else in binary64.  (Not for WENO-Z, which has
+// no selections.)
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ unsigned teno_select(const double (&v)[5], const double (&e)[4], const Scheme& S) {
+  unsigned sel = 7u;
+  const int m = S.variant == kSchemeLad ? -1 : (S.variant == kSchemeTeno5 ? S.m_fixed : -2);
+  if (teno_cert::select_diffs(e[0], e[1], e[2], e[3], S.eps4_f, S.thr_keep_f, S.thr_f, S.nthr, S.b_l, m, S.keep_all,
+                              c_lad_f, sel))
+    return sel;
+  unsigned flag;
+  teno5_lad<false>(v[0], v[1], v[2], v[3], v[4], 0.0, S, flag);
+  return flag & 7u;
 }
 
 }  // namespace teno

@@ -119,6 +119,10 @@ template <int NDIM>
 __device__ __forceinline__ bool cert_keep(const CertIfc<NDIM>& C, const Scheme& S) {
   return teno_cert::cert_keep<NDIM>(C, S.thr_keep_f, S.eps4_f);
 }
+template <int NDIM>
+__device__ __forceinline__ unsigned cert_open(const CertIfc<NDIM>& C, const Scheme& S) {
+  return teno_cert::cert_open<NDIM>(C, S.thr_keep_f, S.eps4_f);
+}
 
 // ---------------------------------------------------------------------------
 // Every stencil kept at every field and side: closed form.  With fixed linear
@@ -321,21 +325,27 @@ __device__ __forceinline__ void closed_out(const double (&Ft)[NDIM + 2], const d
 }
 
 // ---------------------------------------------------------------------------
-// The certified closed form alone, with the per-cell F_DIR/2 of the cell
+// The closed form alone, with the per-cell F_DIR/2 of the cell
 // pass (`fh`, momentum and energy components only: [nvar - 1][ncell]), in
 // two passes over the six stencil points: the FP32 test (and the exponents
 // of the sums), then the fixed-point sums, so that the test's state is dead
-// before the sums' state is live.  Returns false, with `out` unwritten, when
-// the test does not keep every stencil or the fixed point does not cover a
-// sum; otherwise `out` equals interface_flux's up to the rounding of the
-// sums (which that one-pass form evaluates as binary64 chains).
+// before the sums' state is live.  Returns the open reconstructions (bit
+// 2 s + side of field s, cert_open's mask): 0 -- the test keeps every stencil
+// and `out` is the flux (interface_flux's up to the rounding of the sums,
+// which that one-pass form evaluates as binary64 chains); else `out` holds
+// the flux with every stencil kept, to which warp_correct adds the
+// open reconstructions' differences.  kRough: the fixed point does not cover
+// a sum and `out` is unwritten (warp_correct then sums every field).
 // ---------------------------------------------------------------------------
+constexpr unsigned kRough = 1u << 15;
+template <int NDIM>
+constexpr unsigned kAllOpen = (1u << (2 * (NDIM + 2))) - 1u;
 // (GH: the sweep direction has fixed-state ghost cells, read from gc; the
 // half fluxes of the ghost block are taken at direction DIR's block.  With
 // `rout` the interface's Roe state is also returned, whatever the test
 // decides.)
 template <int NDIM, int DIR, bool GH = false>
-__device__ __forceinline__ bool interface_flux_closed(const double* __restrict__ U,
+__device__ __forceinline__ unsigned interface_flux_closed(const double* __restrict__ U,
                                                       const double* __restrict__ aux,
                                                       const double* __restrict__ fh, int64_t ncell,
                                                       const int64_t (&cells)[6], unsigned flips,
@@ -345,7 +355,7 @@ __device__ __forceinline__ bool interface_flux_closed(const double* __restrict__
                                                       const GhostCells& gc = GhostCells(),
                                                       RoeIfc<NDIM>* rout = nullptr) {
   constexpr int NVAR = NDIM + 2;
-  if (S.keep_idx < 0) return false;
+  if (S.keep_idx < 0) return kRough | kAllOpen<NDIM>;
   const double* gfh = GH ? gc.fh + DIR * (NVAR - 1) * kGhostSlots : nullptr;
   RoeIfc<NDIM> R;
   {
@@ -380,6 +390,7 @@ __device__ __forceinline__ bool interface_flux_closed(const double* __restrict__
   uint32_t KU[NVAR], KF[NVAR];
 #pragma unroll
   for (int v = 0; v < NVAR; ++v) KF[v] = 0u;
+  unsigned open;
   {
     CertIfc<NDIM> C;
     cert_begin<NDIM, DIR>(R, alpha, C);
@@ -405,17 +416,16 @@ __device__ __forceinline__ bool interface_flux_closed(const double* __restrict__
       const double pnj = ldc<GH>(aux, gc.aux, ncell, NDIM, c);
       cert_point<NDIM, DIR>(j, Uj, unj, pnj, C);
     }
-    if (!cert_keep<NDIM>(C, S)) return false;
+    open = cert_open<NDIM>(C, S);
   }
   // second pass: the two sums per component in fixed point.  Where its
   // exponent range does not cover a component (values below 2^-959 or above
-  // 2^1007, infinities, NaN) the interface goes to the pending list, whose
-  // characteristic path evaluates it in binary64.  The points are taken in
+  // 2^1007, infinities, NaN) warp_correct evaluates the interface in binary64.  The points are taken in
   // two rounds of three (fully unrolled, the sums' temporaries of all six
   // points would not fit in the registers beside the Roe state; the cell
   // indices, read with a loop index, then sit in the stack frame).
   ClosedFix<NDIM> X;
-  if (!closed_fix_begin<NDIM, DIR>(KU, KF, X)) return false;
+  if (!closed_fix_begin<NDIM, DIR>(KU, KF, X)) return kRough | kAllOpen<NDIM>;
 #pragma unroll 3
   for (int j = 0; j < 6; ++j) {
     double Uj[NVAR], Fhj[NVAR];
@@ -425,7 +435,219 @@ __device__ __forceinline__ bool interface_flux_closed(const double* __restrict__
   double Ft[NVAR], Ut[NVAR];
   closed_fix_out<NDIM>(X, Ft, Ut);
   closed_out<NDIM, DIR>(Ft, Ut, R, nal, out);
-  return true;
+  return open;
+}
+
+// ---------------------------------------------------------------------------
+// The fluxes of interfaces whose certified test left the reconstructions
+// `open` undecided.  The reconstruction is linear for given selections, so
+//   F^ = (F^ with every stencil kept) + sum over the open reconstructions
+//        (f^(selected) - f^(all kept)) r_s,
+// and only the open ones are evaluated (two to four of ten on shocks, one or
+// two in under-resolved smooth flow), by the characteristic path's formulas.
+// A warp works on up to 32 interfaces, one per owning lane: the owners put
+// the Roe states into shared memory, the open (interface, reconstruction)
+// pairs are laid out in a list ordered by field, every lane takes one pair
+// at a time, and the owners add the differences up in field order  So no
+// lane waits for the interface with the most open fields, neighbouring lanes
+// run the same field's formulas, and a short list still fills its warps.
+//
+// What bounds it: FP64 issue.  An FP64 warp instruction holds its SM
+// partition for 64 cycles whatever lanes are active (measured: 64.4 cycles
+// for 1 to 32 lanes, dependent or not), so the layout's aim is few FP64
+// instructions per warp, all lanes on.  Against the characteristic path at
+// every listed interface (one thread each, ten reconstructions): 97 against
+// 163 us for a third of the interfaces of a 64^3 box, 29 against 40 us for
+// 2 % of a 512^2 grid, 15 against 39 us for a handful at 200 cells (then 6 to
+// 16 % off each with the selections decided on first differences in FP32).
+//
+// Where the all-kept flux is much larger than the flux scale (alpha rho,
+// alpha^2 rho, alpha E of the stencil -- a strong pressure jump seen from its
+// cold side), subtracting it back would cancel digits: such an interface,
+// and one with kRough, opens every reconstruction and sums the whole values.
+// ---------------------------------------------------------------------------
+// Whether a flux (stored as 30 F^) exceeds the flux scale twice, in single
+// precision: the halved speeds, and the stencil's largest density and energy.
+template <int NDIM>
+__device__ __forceinline__ bool beyond_flux_scale(const double (&out)[NDIM + 2], const double (&alpha)[NDIM + 2],
+                                                  float rho_max, float e_max) {
+  constexpr int NVAR = NDIM + 2;
+  const float am = 2.0f * fmaxf(hi_float(alpha[0]), hi_float(alpha[NVAR - 1]));
+  const float s0 = 2.0f * float(kFluxScale) * am * rho_max, sE = 2.0f * float(kFluxScale) * am * e_max;
+  bool big = !(fabsf(hi_float(out[0])) <= s0) || !(fabsf(hi_float(out[NVAR - 1])) <= sE);
+#pragma unroll
+  for (int k = 0; k < NDIM; ++k) big = big || !(fabsf(hi_float(out[1 + k])) <= s0 * am);
+  return big;
+}
+
+template <int NDIM>
+struct CorrectScratch {   // one per warp
+  double u[NDIM][32], H[32], cs[32], b1[32], hb1[32], hb2[32], hic[32], hud[32];
+  double d[2 * (NDIM + 2)][32];
+  uint32_t q[32];
+  uint16_t item[2 * (NDIM + 2) * 32];   // owner | reconstruction << 5 | whole << 9
+};
+
+// cells_of(q, cells, flips) gives the stencil of interface q.  Every lane of
+// the warp calls; `open` is 0 in lanes without an interface.  On entry `out`
+// is interface_flux_closed's (unset with kRough), on return the flux.
+template <int NDIM, int DIR, bool GH, class Cells>
+__device__ __forceinline__ void warp_correct(const double* __restrict__ U, const double* __restrict__ aux,
+                                             int64_t ncell, const Cells& cells_of, uint32_t q,
+                                             const double (&alpha)[NDIM + 2], const Scheme& S, unsigned open,
+                                             double (&out)[NDIM + 2], int* __restrict__ status,
+                                             CorrectScratch<NDIM>& W,
+                                             const GhostCells& gc = GhostCells()) {
+  constexpr int NVAR = NDIM + 2, NREC = 2 * NVAR;
+  const unsigned lane = threadIdx.x & 31u;
+  bool whole = false;
+  double q2 = 0.0;
+  __syncwarp();
+  if (open) {
+    int64_t cells[6];
+    unsigned flips;
+    cells_of(q, cells, flips);
+    RoeIfc<NDIM> R;
+    double su2[NDIM], su3[NDIM];
+#pragma unroll
+    for (int k = 0; k < NDIM; ++k) {
+      su2[k] = ldc<GH>(aux, gc.aux, ncell, NDIM + 3 + k, cells[2]);
+      su3[k] = ldc<GH>(aux, gc.aux, ncell, NDIM + 3 + k, cells[3]);
+    }
+    su2[DIR] = flip_sign(su2[DIR], (flips >> 2) & 1u);
+    su3[DIR] = flip_sign(su3[DIR], (flips >> 3) & 1u);
+    roe_interface<NDIM, DIR>(ldc<GH>(aux, gc.aux, ncell, NDIM + 1, cells[2]),
+                             ldc<GH>(aux, gc.aux, ncell, NDIM + 1, cells[3]),
+                             ldc<GH>(aux, gc.aux, ncell, NDIM + 2, cells[2]),
+                             ldc<GH>(aux, gc.aux, ncell, NDIM + 2, cells[3]), su2, su3, S, R, status);
+    float rm = 0.0f, em = 0.0f;
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+      rm = fmaxf(rm, fabsf(hi_float(ldc<GH>(U, gc.U, ncell, 0, cells[j]))));
+      em = fmaxf(em, fabsf(hi_float(ldc<GH>(U, gc.U, ncell, NVAR - 1, cells[j]))));
+    }
+    whole = (open & kRough) || beyond_flux_scale<NDIM>(out, alpha, rm, em);
+#pragma unroll
+    for (int k = 0; k < NDIM; ++k) W.u[k][lane] = R.u[k];
+    W.H[lane] = R.H;
+    W.cs[lane] = R.cs;
+    W.b1[lane] = R.b1;
+    W.hb1[lane] = R.hb1;
+    W.hb2[lane] = R.hb2;
+    W.hic[lane] = R.hic;
+    W.hud[lane] = R.hud;
+    W.q[lane] = q;
+    q2 = R.q2;
+  }
+  const unsigned mask = whole ? kAllOpen<NDIM> : open & kAllOpen<NDIM>;
+  unsigned n = 0;
+#pragma unroll
+  for (int b = 0; b < NREC; ++b) {
+    const unsigned m = __ballot_sync(0xffffffffu, (mask >> b) & 1u);
+    if ((mask >> b) & 1u) {
+      W.item[n + __popc(m & ((1u << lane) - 1u))] =
+          static_cast<uint16_t>(lane | unsigned(b) << 5 | (whole ? 1u << 9 : 0u));
+    } else {
+      W.d[b][lane] = 0.0;
+    }
+    n += __popc(m);
+  }
+  __syncwarp();
+  for (unsigned i = lane; i < n; i += 32u) {
+    const unsigned it = W.item[i];
+    const unsigned o = it & 31u, b = (it >> 5) & 15u, s = b >> 1;
+    const bool minus = b & 1u;
+    int64_t cells[6];
+    unsigned flips;
+    cells_of(W.q[o], cells, flips);
+    double v[5];
+    auto point = [&](int j, double (&Uj)[NVAR], double& un) {
+      const int p = minus ? 5 - j : j;
+      const bool fj = (flips >> p) & 1u;
+      const int64_t c = minus ? cells[5 - j] : cells[j];
+#pragma unroll
+      for (int k = 0; k < NVAR; ++k) Uj[k] = ldc<GH>(U, gc.U, ncell, k, c);
+      Uj[1 + DIR] = flip_sign(Uj[1 + DIR], fj);
+      un = flip_sign(ldc<GH>(aux, gc.aux, ncell, DIR, c), fj);
+      return ldc<GH>(aux, gc.aux, ncell, NDIM, c);
+    };
+    // the split values of the characteristic path (interface_flux)
+    if (s >= 2 && s < NVAR - 1) {   // shear field of the direction t
+      const int t = (int(s) - 2 < DIR) ? int(s) - 2 : int(s) - 1;
+      const double ut = W.u[t][o];
+#pragma unroll
+      for (int j = 0; j < 5; ++j) {
+        const int p = minus ? 5 - j : j;
+        const bool fj = (flips >> p) & 1u;
+        const int64_t c = minus ? cells[5 - j] : cells[j];
+        const double w = fma(-ut, ldc<GH>(U, gc.U, ncell, 0, c), ldc<GH>(U, gc.U, ncell, 1 + t, c));
+        v[j] = (flip_sign(ldc<GH>(aux, gc.aux, ncell, DIR, c), fj) + (minus ? -alpha[1] : alpha[1])) * w;
+      }
+    } else {
+      // acoustic (+-) and entropy fields: the row l_s = wA (hb2, -hb1 u, hb1) +
+      // (u_d, -e_d, 0) (+-hic) (+ e_0 for the entropy field) of project's
+      // combinations, z_s = wA b1 (u_d - u~_d)/2 -+ hic
+      const double hic = s == 0 ? W.hic[o] : (s == 1 ? 0.0 : -W.hic[o]);
+      const double wA = s == 1 ? -2.0 : 1.0;
+      const double mh = wA * W.hb1[o], ud = W.u[DIR][o];
+      double l[NVAR];
+      l[0] = fma(ud, hic, fma(wA, W.hb2[o], s == 1 ? 1.0 : 0.0));
+#pragma unroll
+      for (int k = 0; k < NDIM; ++k) l[1 + k] = k == DIR ? fma(-ud, mh, -hic) : -W.u[k][o] * mh;
+      l[NVAR - 1] = mh;
+      const double za = wA * W.b1[o], z0 = fma(-za, W.hud[o], -hic);
+      const double al = s == 0 ? alpha[0] : (s == 1 ? alpha[1] : alpha[NVAR - 1]);
+      const double as = minus ? -al : al;
+#pragma unroll
+      for (int j = 0; j < 5; ++j) {
+        double Uj[NVAR], un;
+        const double pn = point(j, Uj, un);
+        double w = l[0] * Uj[0];
+#pragma unroll
+        for (int k = 1; k < NVAR; ++k) w = fma(l[k], Uj[k], w);
+        v[j] = fma(un + as, w, pn * fma(za, un, z0));
+      }
+    }
+    const double e[4] = {v[1] - v[0], v[2] - v[1], v[3] - v[2], v[4] - v[3]};
+    const unsigned sel = teno_select(v, e, S);
+    double dl = 0.0;
+    if (it >> 9) {
+      dl = fma(c_lin[sel][0], v[0], fma(c_lin[sel][1], v[1], fma(c_lin[sel][2], v[2], fma(c_lin[sel][3], v[3], c_lin[sel][4] * v[4]))));
+    } else if (sel != 7u) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) dl = fma(c_cut[sel][j], e[j], dl);
+    }
+    W.d[b][o] = dl;
+  }
+  __syncwarp();
+  if (open) {
+    // back-projection of the differences (the whole values), as interface_flux's
+    double f[NVAR];
+#pragma unroll
+    for (int s = 0; s < NVAR; ++s) f[s] = (W.d[2 * s][lane] + W.d[2 * s + 1][lane]) * kFluxScale;
+    double u[NDIM];
+#pragma unroll
+    for (int k = 0; k < NDIM; ++k) u[k] = W.u[k][lane];
+    if (whole)
+#pragma unroll
+      for (int k = 0; k < NVAR; ++k) out[k] = 0.0;
+    const double sa = f[0] + f[NVAR - 1], da = (f[NVAR - 1] - f[0]) * W.cs[lane];
+    const double rho_f = sa + f[1];
+    out[0] += rho_f;
+    double eng = fma(W.H[lane], sa, fma(u[DIR], da, 0.5 * q2 * f[1]));
+    int g = 2;
+#pragma unroll
+    for (int k = 0; k < NDIM; ++k) {
+      if (k == DIR) {
+        out[1 + k] += fma(u[k], rho_f, da);
+      } else {
+        out[1 + k] += fma(u[k], rho_f, f[g]);
+        eng = fma(u[k], f[g], eng);
+        ++g;
+      }
+    }
+    out[NVAR - 1] += eng;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -528,6 +750,28 @@ __device__ __forceinline__ void interface_flux(const double* __restrict__ U,
       return;
     }
 
+    // As in warp_correct: the flux with every stencil kept plus the fields'
+    // differences against it, unless that flux is far beyond the flux scale
+    // (WENO-Z keeps no stencil exactly linear: always the whole values).
+    bool cut = S.variant != kSchemeWenoZ;
+    if (cut) {
+      double Ft[NVAR], Ut[NVAR];
+      float rm = 0.0f, em = 0.0f;
+#pragma unroll
+      for (int j = 0; j < 6; ++j) {
+        double Fhj[NVAR];
+        cell_flux_half<NDIM, DIR>(Ux[j], un[j], pn[j], Fhj);
+        closed_point<NDIM, DIR>(j, Ux[j], Fhj, Ft, Ut);
+        rm = fmaxf(rm, fabsf(hi_float(Ux[j][0])));
+        em = fmaxf(em, fabsf(hi_float(Ux[j][NVAR - 1])));
+      }
+      closed_out<NDIM, DIR>(Ft, Ut, R, nal, out);
+      cut = !beyond_flux_scale<NDIM>(out, alpha, rm, em);
+    }
+    if (!cut)
+#pragma unroll
+      for (int v = 0; v < NVAR; ++v) out[v] = 0.0;
+
     // Characteristic values w = L U and the split fluxes v+- = (g +- alpha w)/2
     // with g = L F.  Since F(U) = u_d U + p (0, e_d, u_d) (eq. 4.7),
     // g = u_d w + p z with z = (hb1 du - hic, -2 hb1 du, 0.., hb1 du + hic),
@@ -561,8 +805,8 @@ __device__ __forceinline__ void interface_flux(const double* __restrict__ U,
     }
 #pragma unroll
     for (int s = 0; s < NVAR; ++s) {
-      const double hp = teno5_lad<WITH_FLAGS>(vp[0][s], vp[1][s], vp[2][s], vp[3][s], vp[4][s], 0.0, S, fl[s][0]);
-      fchar[s] = teno5_lad<WITH_FLAGS>(vm[5][s], vm[4][s], vm[3][s], vm[2][s], vm[1][s], hp, S, fl[s][1]);
+      const double hp = teno5_lad<WITH_FLAGS>(vp[0][s], vp[1][s], vp[2][s], vp[3][s], vp[4][s], 0.0, S, fl[s][0], cut);
+      fchar[s] = teno5_lad<WITH_FLAGS>(vm[5][s], vm[4][s], vm[3][s], vm[2][s], vm[1][s], hp, S, fl[s][1], cut);
     }
     // back-projection F^ = R f^char, columns r_0 = (1, u - c e_n, H - u_n c),
     // r_1 = (1, u, q2/2), r_t = (0, e_t, u_t), r_{nvar-1} = (1, u + c e_n, H + u_n c),
@@ -572,22 +816,22 @@ __device__ __forceinline__ void interface_flux(const double* __restrict__ U,
     const double sa = fchar[0] + fchar[NVAR - 1];
     const double da = fchar[NVAR - 1] - fchar[0];
     const double rho_f = sa + fchar[1];
-    out[0] = rho_f;
+    out[0] += rho_f;
     double eng = fma(H, sa, fma(u[DIR] * cs, da, 0.5 * q2 * fchar[1]));
     {
       int f = 2;
 #pragma unroll
       for (int k = 0; k < NDIM; ++k) {
         if (k == DIR) {
-          out[1 + k] = fma(u[k], rho_f, cs * da);
+          out[1 + k] += fma(u[k], rho_f, cs * da);
         } else {
-          out[1 + k] = fma(u[k], rho_f, fchar[f]);
+          out[1 + k] += fma(u[k], rho_f, fchar[f]);
           eng = fma(u[k], fchar[f], eng);
           ++f;
         }
       }
     }
-    out[NVAR - 1] = eng;
+    out[NVAR - 1] += eng;
   }
 }
 #pragma nv_diag_default 128

@@ -265,15 +265,17 @@ __global__ void __launch_bounds__(128, TENO_FLUX_MINBLOCKS) flux_kernel(
 
 // ---------------------------------------------------------------------------
 // The same fluxes in two passes (no flags).  flux_closed_kernel evaluates the
-// certified closed form -- every interface whose FP32 test keeps all ten
-// stencils -- and appends the others to `list` (one atomic per warp);
-// flux_pending_kernel then takes the listed interfaces through the
-// characteristic path.  Each interface gets the arithmetic of the one-pass
-// kernel, except that the closed form's six-point sums are fixed-point sums
+// closed form with every stencil kept, and its certified FP32 test; the
+// interfaces with reconstructions that the test does not prove to be kept go
+// to `list` with the mask of those (one atomic per warp), and
+// flux_correct_kernel adds their differences (warp_correct).  Against
+// the one-pass kernel the closed form's six-point sums are fixed-point sums
 // rounded once (teno_fixsum.cuh: terms on a grid of an eighth of the largest
-// value's ulp, added exactly) where the one-pass kernel chains binary64
-// operations; the closed-form pass stays small (registers,
-// instruction cache) and its warps do not diverge into the rare slow path.
+// value's ulp, added exactly) where that one chains binary64 operations; the
+// closed-form pass stays small (registers, instruction cache) and its warps
+// do not diverge into the rare slow path.
+// WENO-Z, which keeps no stencil exactly linear, takes flux_wenoz_kernel: the
+// characteristic path at every interface, no list.
 // ---------------------------------------------------------------------------
 #ifndef TENO_CLOSED_MINBLOCKS
 #define TENO_CLOSED_MINBLOCKS 4
@@ -338,7 +340,7 @@ template <int NDIM, int DIR, int WALL, bool ROE = false>
 __global__ void __launch_bounds__(128, TENO_CLOSED_MINBLOCKS) flux_closed_kernel(
     const double* __restrict__ U, const double* __restrict__ aux, const double* __restrict__ fh,
     const unsigned long long* __restrict__ alpha_bits, double* __restrict__ Fhat,
-    uint32_t* __restrict__ list, unsigned* __restrict__ count, int* __restrict__ status, Grid G,
+    uint2* __restrict__ list, unsigned* __restrict__ count, int* __restrict__ status, Grid G,
     Scheme S, double* __restrict__ roe_out = nullptr) {
   constexpr int NVAR = NDIM + 2;
   const int64_t nifc = (G.n[0] + (DIR == 0)) * (G.n[1] + (DIR == 1)) * (G.n[2] + (DIR == 2));
@@ -372,7 +374,7 @@ __global__ void __launch_bounds__(128, TENO_CLOSED_MINBLOCKS) flux_closed_kernel
     interface_cells<NDIM, DIR, WALL == 2>(q, G, cells, flips);
     double out[NVAR];
     RoeIfc<NDIM> R;
-    const bool done = interface_flux_closed<NDIM, DIR, WALL == 2>(
+    const unsigned open = interface_flux_closed<NDIM, DIR, WALL == 2>(
         U, aux, fh + (int64_t)DIR * (NVAR - 1) * G.ncell, G.ncell, cells, WALL == 1 ? flips : 0u, alpha, nal, S,
         out, status, GhostCells{G.gU, G.gaux, G.gfh}, ROE ? &R : nullptr);
     if constexpr (ROE) {
@@ -386,40 +388,78 @@ __global__ void __launch_bounds__(128, TENO_CLOSED_MINBLOCKS) flux_closed_kernel
         roe_out[(int64_t)(NDIM + 4) * nifc + q] = R.hb1;
         roe_out[(int64_t)(NDIM + 5) * nifc + q] = R.hb2;
         roe_out[(int64_t)(NDIM + 6) * nifc + q] = R.hic;
-        roe_out[(int64_t)(NDIM + 7) * nifc + q] = done ? 1.0 : 0.0;
+        roe_out[(int64_t)(NDIM + 7) * nifc + q] = open ? 0.0 : 1.0;
       }
     }
-    if (done) {
+    if (!(open & kRough)) {
 #pragma unroll
       for (int v = 0; v < NVAR; ++v) Fhat[(int64_t)v * nifc + q] = out[v];
     }
-    // append the undecided interfaces of the lanes converged here
+    // append the open interfaces of the lanes converged here
     const unsigned act = __activemask();
-    const unsigned m = __ballot_sync(act, !done);
+    const unsigned m = __ballot_sync(act, open != 0u);
     if (m) {
       const unsigned leader = __ffs(act) - 1;
       unsigned at = 0;
       if (lane == leader) at = atomicAdd(count, __popc(m));
       at = __shfl_sync(act, at, leader);
-      if (!done) list[at + __popc(m & ((1u << lane) - 1u))] = static_cast<uint32_t>(q);
+      if (open) list[at + __popc(m & ((1u << lane) - 1u))] = make_uint2(static_cast<uint32_t>(q), open);
     }
   }
 }
 
+// An FP64 instruction holds its SM partition's pipe for 64 cycles whatever
+// lanes are active, so a warp's time is its FP64 instruction count.  A warp
+// takes 32 listed interfaces when there are enough for every partition of
+// the chip, and fewer (2, 4, 8, 16) when the list is short: a short list is
+// bound by one warp's chain, and few interfaces finish in a single round.
 template <int NDIM, int DIR, bool GH>
-__global__ void __launch_bounds__(128) flux_pending_kernel(
+__global__ void __launch_bounds__(128) flux_correct_kernel(
     const double* __restrict__ U, const double* __restrict__ aux,
     const unsigned long long* __restrict__ alpha_bits, double* __restrict__ Fhat,
-    const uint32_t* __restrict__ list, const unsigned* __restrict__ count, int* __restrict__ status,
-    Grid G, Scheme S) {
+    const uint2* __restrict__ list, const unsigned* __restrict__ count, int* __restrict__ status,
+    Grid G, Scheme S, int nsm) {
   constexpr int NVAR = NDIM + 2;
+  __shared__ CorrectScratch<NDIM> scratch[4];
   const int64_t nifc = (G.n[0] + (DIR == 0)) * (G.n[1] + (DIR == 1)) * (G.n[2] + (DIR == 2));
   const int64_t n = *count;
-  if (blockIdx.x * (int64_t)blockDim.x >= n) return;
+  const int64_t nw = (int64_t)gridDim.x * 4;
+  int per = 2;
+  while (per < 32 && n > (int64_t)per * 4 * nsm) per *= 2;
+  const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  if (blockIdx.x * (int64_t)(4 * per) >= n) return;
   double alpha[NVAR], nal[NVAR];
   half_speeds<NDIM, DIR>(alpha_bits, alpha, nal);
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t q = list[i];
+  auto cells_of = [&](uint32_t q, int64_t (&cells)[6], unsigned& flips) {
+    interface_cells<NDIM, DIR, GH>(q, G, cells, flips);
+  };
+  for (int64_t i0 = ((int64_t)blockIdx.x * 4 + warp) * per; i0 < n; i0 += nw * per) {
+    const int64_t i = i0 + lane;
+    const uint2 e = lane < per && i < n ? list[i] : make_uint2(0u, 0u);
+    double out[NVAR];
+#pragma unroll
+    for (int v = 0; v < NVAR; ++v) out[v] = e.y && !(e.y & kRough) ? Fhat[(int64_t)v * nifc + e.x] : 0.0;
+    warp_correct<NDIM, DIR, GH>(U, aux, G.ncell, cells_of, e.x, alpha, S, e.y, out, status, scratch[warp],
+                                GhostCells{G.gU, G.gaux, G.gfh});
+    if (e.y)
+#pragma unroll
+      for (int v = 0; v < NVAR; ++v) Fhat[(int64_t)v * nifc + e.x] = out[v];
+  }
+}
+
+template <int NDIM, int DIR, bool GH>
+__global__ void __launch_bounds__(128) flux_wenoz_kernel(
+    const double* __restrict__ U, const double* __restrict__ aux,
+    const unsigned long long* __restrict__ alpha_bits, double* __restrict__ Fhat, int* __restrict__ status,
+    Grid G, Scheme Sx) {
+  constexpr int NVAR = NDIM + 2;
+  Scheme S = Sx;
+  S.variant = kSchemeWenoZ;   // known to the compiler: the cutoffs' code folds away
+  S.keep_idx = -1;
+  const int64_t nifc = (G.n[0] + (DIR == 0)) * (G.n[1] + (DIR == 1)) * (G.n[2] + (DIR == 2));
+  double alpha[NVAR], nal[NVAR];
+  half_speeds<NDIM, DIR>(alpha_bits, alpha, nal);
+  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nifc; q += (int64_t)gridDim.x * blockDim.x) {
     int64_t cells[6];
     unsigned flips;
     interface_cells<NDIM, DIR, GH>(q, G, cells, flips);
@@ -639,6 +679,7 @@ Scheme make_scheme(double gamma, double H, double eps, int b_l, int b_u, int var
     }
   }
   // (WENO-Z has no cutoff and no keep-all shortcut: keep_idx stays -1)
+  for (int j = 0; j < kMaxLadder; ++j) S.thr_f[j] = static_cast<float>(S.thr[j]);
   // binary32 constants of the pre-test, rounded towards zero (conservative)
   auto down = [](double x) {
     float f = static_cast<float>(x);
@@ -725,9 +766,9 @@ cudaError_t launch_argmax_finish(int ndim, const unsigned long long* cand, int64
 }
 
 template <int NDIM, int DIR>
-static int flux_launch(int blocks, int threads, int pblocks, cudaStream_t st, const double* U,
+static int flux_launch(int blocks, int threads, int pblocks, int nsm, cudaStream_t st, const double* U,
                        const double* aux, const double* fh, const unsigned long long* alpha, double* Fhat,
-                       uint8_t* flags, uint32_t* list, unsigned* count, int* status, const Grid& G,
+                       uint8_t* flags, uint2* list, unsigned* count, int* status, const Grid& G,
                        const Scheme& S, double* roe_out) {
   const bool gh = G.bc[DIR] == TENO_BC_DIRICHLET;
   if (flags || !list) {
@@ -735,6 +776,11 @@ static int flux_launch(int blocks, int threads, int pblocks, cudaStream_t st, co
     else if (flags) flux_kernel<NDIM, DIR, true, false><<<blocks, threads, 0, st>>>(U, aux, alpha, Fhat, flags, status, G, S);
     else if (gh) flux_kernel<NDIM, DIR, false, true><<<blocks, threads, 0, st>>>(U, aux, alpha, Fhat, flags, status, G, S);
     else flux_kernel<NDIM, DIR, false, false><<<blocks, threads, 0, st>>>(U, aux, alpha, Fhat, flags, status, G, S);
+    return 1;
+  }
+  if (S.variant == kSchemeWenoZ) {
+    if (gh) flux_wenoz_kernel<NDIM, DIR, true><<<pblocks, threads, 0, st>>>(U, aux, alpha, Fhat, status, G, S);
+    else flux_wenoz_kernel<NDIM, DIR, false><<<pblocks, threads, 0, st>>>(U, aux, alpha, Fhat, status, G, S);
     return 1;
   }
   if (G.bc[DIR] == TENO_BC_REFLECTIVE)
@@ -747,15 +793,15 @@ static int flux_launch(int blocks, int threads, int pblocks, cudaStream_t st, co
   else
     flux_closed_kernel<NDIM, DIR, 0><<<blocks, threads, 0, st>>>(U, aux, fh, alpha, Fhat, list, count, status, G, S);
   if (gh)
-    flux_pending_kernel<NDIM, DIR, true><<<pblocks, threads, 0, st>>>(U, aux, alpha, Fhat, list, count, status, G, S);
+    flux_correct_kernel<NDIM, DIR, true><<<pblocks, threads, 0, st>>>(U, aux, alpha, Fhat, list, count, status, G, S, nsm);
   else
-    flux_pending_kernel<NDIM, DIR, false><<<pblocks, threads, 0, st>>>(U, aux, alpha, Fhat, list, count, status, G, S);
+    flux_correct_kernel<NDIM, DIR, false><<<pblocks, threads, 0, st>>>(U, aux, alpha, Fhat, list, count, status, G, S, nsm);
   return 2;
 }
 
 cudaError_t launch_flux(int ndim, int dir, const double* U, const double* aux, const double* fh,
                         const unsigned long long* alpha, double* Fhat,
-                        uint8_t* flags, uint32_t* list, unsigned* count, int* status,
+                        uint8_t* flags, uint2* list, unsigned* count, int* status,
                         const Grid& G, const Scheme& S, int nsm, cudaStream_t st,
                         int* launches, double* roe_out) {
   int64_t nifc = 1;
@@ -766,14 +812,14 @@ cudaError_t launch_flux(int ndim, int dir, const double* U, const double* aux, c
   const int blocks = blocks_for(nifc, threads, nsm * 64);
   const int pblocks = blocks_for(nifc, threads, nsm * 16);
   int n = 0;
-  if (ndim == 1) n = flux_launch<1, 0>(blocks, threads, pblocks, st, U, aux, fh, alpha, Fhat, flags, list, count, status, G, S, roe_out);
+  if (ndim == 1) n = flux_launch<1, 0>(blocks, threads, pblocks, nsm, st, U, aux, fh, alpha, Fhat, flags, list, count, status, G, S, roe_out);
   else if (ndim == 2) {
-    if (dir == 0) n = flux_launch<2, 0>(blocks, threads, pblocks, st, U, aux, fh, alpha, Fhat, flags, list, count, status, G, S, roe_out);
-    else n = flux_launch<2, 1>(blocks, threads, pblocks, st, U, aux, fh, alpha, Fhat, flags, list, count, status, G, S, roe_out);
+    if (dir == 0) n = flux_launch<2, 0>(blocks, threads, pblocks, nsm, st, U, aux, fh, alpha, Fhat, flags, list, count, status, G, S, roe_out);
+    else n = flux_launch<2, 1>(blocks, threads, pblocks, nsm, st, U, aux, fh, alpha, Fhat, flags, list, count, status, G, S, roe_out);
   } else {
-    if (dir == 0) n = flux_launch<3, 0>(blocks, threads, pblocks, st, U, aux, fh, alpha, Fhat, flags, list, count, status, G, S, roe_out);
-    else if (dir == 1) n = flux_launch<3, 1>(blocks, threads, pblocks, st, U, aux, fh, alpha, Fhat, flags, list, count, status, G, S, roe_out);
-    else n = flux_launch<3, 2>(blocks, threads, pblocks, st, U, aux, fh, alpha, Fhat, flags, list, count, status, G, S, roe_out);
+    if (dir == 0) n = flux_launch<3, 0>(blocks, threads, pblocks, nsm, st, U, aux, fh, alpha, Fhat, flags, list, count, status, G, S, roe_out);
+    else if (dir == 1) n = flux_launch<3, 1>(blocks, threads, pblocks, nsm, st, U, aux, fh, alpha, Fhat, flags, list, count, status, G, S, roe_out);
+    else n = flux_launch<3, 2>(blocks, threads, pblocks, nsm, st, U, aux, fh, alpha, Fhat, flags, list, count, status, G, S, roe_out);
   }
   if (launches) *launches = n;
   return cudaGetLastError();
@@ -859,7 +905,7 @@ teno_status forward_stage(const teno_grid* g, char* ws, size_t status_off, size_
   auto* alpha = reinterpret_cast<unsigned long long*>(ws + alpha_off);
   double* aux = reinterpret_cast<double*>(ws + aux_off);
   double* Fhat = reinterpret_cast<double*>(ws + fhat_off);
-  uint32_t* list = list_off ? reinterpret_cast<uint32_t*>(ws + list_off) : nullptr;
+  uint2* list = list_off ? reinterpret_cast<uint2*>(ws + list_off) : nullptr;
   double* fh = fh_off ? reinterpret_cast<double*>(ws + fh_off) : nullptr;
   unsigned* count = reinterpret_cast<unsigned*>(ws + alpha_off + kPendingCountOffset);
   if (cudaMemsetAsync(alpha, 0, kAlphaAndCountBytes, st) != cudaSuccess) return TENO_ERR_CUDA;

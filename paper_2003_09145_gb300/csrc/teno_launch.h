@@ -42,16 +42,16 @@ cudaError_t launch_argmax_finish(int ndim, const unsigned long long* cand, int64
 
 // The interface fluxes of direction `dir` into Fhat.  With `flags`, or
 // without a pending list or the cell pass's half fluxes `fh`, one pass; with
-// `list` (room for one 32-bit entry per interface), its counter `count`
-// (zero on entry) and `fh`, the closed-form pass and the pass over the
-// interfaces it leaves pending.  `launches` (optional) receives the number
+// `list` (room for one entry per interface: its index and the mask of its
+// open reconstructions), its counter `count` (zero on entry) and `fh`, the
+// closed-form pass and the pass that corrects the listed interfaces.  `launches` (optional) receives the number
 // of kernels launched.  With `roe_out` (two-pass fluxes without reflecting or
 // fixed-state faces only) the closed-form pass also writes every
 // interface's Roe state and its certificate's decision, [ndim + 8][#interfaces]
 // (flux_closed_kernel).
 cudaError_t launch_flux(int ndim, int dir, const double* U, const double* aux, const double* fh,
                         const unsigned long long* alpha, double* Fhat,
-                        uint8_t* flags, uint32_t* list, unsigned* count, int* status,
+                        uint8_t* flags, uint2* list, unsigned* count, int* status,
                         const Grid& G, const Scheme& S, int nsm, cudaStream_t st,
                         int* launches, double* roe_out = nullptr);
 
