@@ -45,6 +45,7 @@
 
 #include "teno.h"
 #include "teno_adjoint_core.cuh"
+#include "teno_closed.cuh"
 #include "teno_device.cuh"
 #include "teno_flux.cuh"
 #include "teno_launch.h"
@@ -212,17 +213,31 @@ __global__ void __launch_bounds__(kAdjThreads, TENO_ADJ_KEPT_MINBLOCKS) adj_kept
         su3[k] = aux[(NDIM + 3 + k) * I.ncell + cells[3]];
       }
       teno::roe_interface<NDIM, DIR>(sr2, sr3, sh2, sh3, su2, su3, S, Rf, status);
+      // the forward's certificate: on the Roe state in two binary32 values,
+      // or on the binary64 one outside their range (interface_flux_closed)
+      const double a3[3] = {ha[0], ha[1], ha[NVAR - 1]};
+      const teno::FaceSpeeds F = teno::face_speeds(a3);
+      teno::RoeDf<NDIM> Rd;
+      teno::roe_df<NDIM>(sr2, sr3, sh2, sh3, su2, su3, S, Rd);
       teno::CertIfc<NDIM> C;
-      teno::cert_begin<NDIM, DIR>(Rf, ha, C);
+      for (bool df = F.in_range && teno::roe_df_ok<NDIM>(Rd, S);;) {
+        if (df) teno::cert_begin_df<NDIM, DIR>(Rd, F.ha, S, C);
+        else teno::cert_begin<NDIM, DIR>(Rf, ha, C);
+        uint32_t tr = 0u, te = 0u;
 #pragma unroll
-      for (int j = 0; j < 6; ++j) {
-        double Uj[NVAR];
+        for (int j = 0; j < 6; ++j) {
+          double Uj[NVAR];
 #pragma unroll
-        for (int v = 0; v < NVAR; ++v) {
-          Uj[v] = U[v * I.ncell + cells[j]];
-          Ut[v] = j == 0 ? Uj[v] : (j == 5 ? Ut[v] - Uj[v] : fma(Mi[j], Uj[v], Ut[v]));
+          for (int v = 0; v < NVAR; ++v) {
+            Uj[v] = U[v * I.ncell + cells[j]];
+            Ut[v] = j == 0 ? Uj[v] : (j == 5 ? Ut[v] - Uj[v] : fma(Mi[j], Uj[v], Ut[v]));
+          }
+          tr = max(tr, teno_fix::hi_word(Uj[0]) << 1);
+          te = max(te, teno_fix::hi_word(Uj[NVAR - 1]) << 1);
+          teno::cert_point<NDIM, DIR>(j, Uj, aux[DIR * I.ncell + cells[j]], aux[NDIM * I.ncell + cells[j]], C);
         }
-        teno::cert_point<NDIM, DIR>(j, Uj, aux[DIR * I.ncell + cells[j]], aux[NDIM * I.ncell + cells[j]], C);
+        if (!df || teno::df_range(tr, te)) break;
+        df = false;
       }
       kept = S.keep_idx >= 0 && teno::cert_keep<NDIM>(C, S);
     }

@@ -27,6 +27,7 @@
 #include <cuda_runtime.h>
 
 #include "teno.h"
+#include "teno_closed.cuh"
 #include "teno_device.cuh"
 #include "teno_flux.cuh"
 #include "teno_launch.h"
@@ -145,7 +146,7 @@ __global__ void __launch_bounds__(BLOCK) batched_stage_kernel(BatchArgs A, Schem
     const double dt = s_dt;
     if (!(dt > 0.0)) continue;
     const double alpha[3] = {s_alpha[0], s_alpha[1], s_alpha[2]};
-    const double nal[3] = {-2.0 * s_alpha[0], -2.0 * s_alpha[1], -2.0 * s_alpha[2]};
+    const teno::FaceSpeeds F = teno::face_speeds(alpha);
     const double cdt = dt * s_idx;   // dt / (30 dx), as the grid path's stage coefficient
 
     // (B) fluxes tile by tile, difference fused with the stage update
@@ -162,8 +163,8 @@ __global__ void __launch_bounds__(BLOCK) batched_stage_kernel(BatchArgs A, Schem
 #pragma unroll
         for (int j = 0; j < 6; ++j) cells[j] = off + teno::ghost(face - 3 + j, n, A.bc);
         double out[3];
-        const unsigned open = teno::interface_flux_closed<1, 0>(A.Uin, A.aux, A.fh, A.ncell, cells, 0u, alpha, nal,
-                                                                S, out, A.status);
+        const unsigned open = teno::interface_flux_closed<1, 0, false>(A.Uin, A.aux, A.fh, A.ncell, cells, 0u, alpha,
+                                                                       F, S, out, A.status, teno::GhostCells());
         if (!(open & teno::kRough)) {
           s_F[tid][0] = out[0];
           s_F[tid][1] = out[1];
@@ -187,7 +188,7 @@ __global__ void __launch_bounds__(BLOCK) batched_stage_kernel(BatchArgs A, Schem
         const unsigned e = mine ? unsigned(s_pend[k0 + lane]) : 0u;
         const int t = int(e & 0xffffu);
         double out[3] = {s_F[t][0], s_F[t][1], s_F[t][2]};
-        teno::warp_correct<1, 0, false>(A.Uin, A.aux, A.ncell, cells_of, unsigned(t), alpha, S, e >> 16, out,
+        teno::warp_correct<1, 0, false, int64_t>(A.Uin, A.aux, A.ncell, cells_of, unsigned(t), alpha, S, e >> 16, out,
                                         A.status, s_cor[warp]);
         if (mine) {
           s_F[t][0] = out[0];

@@ -130,13 +130,16 @@ TENO_CERT_HD bool certify_keep(float v0, float v1, float v2, float v3, float v4,
   const float b1 = ffma(fmul(k, a1), a1, fmul(c1, c1));
   const float b2 = ffma(fmul(k, a2), a2, fmul(c2, c2));
   const float da = 4.0f * d, dc = 8.0f * d;   // exact scalings
-  const float db0 = ffma(4.0f * u, b0, ffma(fmul(k, ffma(2.0f, fabsf(a0), da)), da, fmul(ffma(2.0f, fabsf(c0), dc), dc)));
-  const float db1 = ffma(4.0f * u, b1, ffma(fmul(k, ffma(2.0f, fabsf(a1), da)), da, fmul(ffma(2.0f, fabsf(c1), dc), dc)));
-  const float db2 = ffma(4.0f * u, b2, ffma(fmul(k, ffma(2.0f, fabsf(a2), da)), da, fmul(ffma(2.0f, fabsf(c2), dc), dc)));
+  // one bound for the three indicators, from the largest |a|, |c| and b (the
+  // bound is monotone in them)
+  const float am = fmaxf(fabsf(a0), fmaxf(fabsf(a1), fabsf(a2)));
+  const float cm = fmaxf(fabsf(c0), fmaxf(fabsf(c1), fabsf(c2)));
+  const float db = ffma(4.0f * u, fmaxf(b0, fmaxf(b1, b2)),
+                        ffma(fmul(k, ffma(2.0f, am, da)), da, fmul(ffma(2.0f, cm, dc), dc)));
   const float tau = fabsf(fsub(b2, b0));
-  const float dtau = ffma(u, tau, fadd(db0, db2));
+  const float dtau = ffma(u, tau, fadd(db, db));
   const float dmin = fadd(fminf(b0, fminf(b1, b2)), eps4_f);
-  const float ddmin = ffma(4.0f * u, dmin, fmaxf(db0, fmaxf(db1, db2)));
+  const float ddmin = ffma(4.0f * u, dmin, db);
   return (dtau <= 1.0e38f) && (fadd(tau, dtau) <= fmul(thr_f, fmul(fsub(dmin, ddmin), 1.0f - 1e-5f)));
 }
 
@@ -272,94 +275,103 @@ TENO_CERT_HD bool select_diffs(double f0, double f1, double f2, double f3, float
 // (e.g. (u_d/2 + alpha) b1/2 u~_k U_j) through at most nine FP32 roundings,
 // so |v32 - v| <= (4 2^-20 + 9 u)(1 + 2^-18) |.|_abs < 4.6 2^-20 |.|_abs,
 // |.|_abs being the absolute evaluation (which the FP32 one approximates
-// from below by at most the same relative amount).  Inputs below 2^-126 add
-// an absolute error below 2^-100 for any physical scale.  cert_keep passes
-// d = 8 2^-20 |.|_abs + 8 u max|v| + 2^-100, more than 1.7 times the
-// r + 2 u W that certify_keep needs, and at least 2^-21 W.
+// from below by at most the same relative amount).  The absolute evaluation
+// is monotone in every input, so cert_open forms it once per interface, from
+// the largest magnitudes over the six points, instead of at every point; it
+// also bounds max|v| (FP32 rounding is monotone).  Inputs below 2^-126 add
+// an absolute error below 2^-100 for any physical scale.  cert_open passes
+// d = (8 2^-20 + 8 u) |.|_abs + 2^-100, more than 1.7 times the r + 2 u W that
+// certify_keep needs, and at least 2^-21 W.
 // ---------------------------------------------------------------------------
 template <int NDIM>
 struct CertIfc {
   float uf[NDIM], hb1f, hb2f, hicf, b1f, hudf, haf[NDIM + 2];
-  float vp32[6][NDIM + 2], vm32[6][NDIM + 2], mp[NDIM + 2], mm[NDIM + 2], vmax;
+  float vp32[6][NDIM + 2], vm32[6][NDIM + 2];
+  float xm[NDIM + 2], hum, hpm;   // largest |U_v|, |u_d/2|, |p/2| over the points
+  int dir;                        // sweep direction (a constant once inlined)
 };
 
+// From binary32 values of the Roe state (u~, b1/2, b2/2, 1/(2c), each within
+// 2^-20 relative of the exact one) and of the halved speeds.
 template <int NDIM, int DIR>
-TENO_CERT_HD void cert_begin(const double (&u)[NDIM], double hb1, double hb2, double hic,
-                             const double (&alpha)[NDIM + 2], CertIfc<NDIM>& C) {
+TENO_CERT_HD void cert_begin_f(const float (&u)[NDIM], float hb1, float hb2, float hic, const float (&ha)[NDIM + 2],
+                               CertIfc<NDIM>& C) {
   constexpr int NVAR = NDIM + 2;
 #pragma unroll
-  for (int k = 0; k < NDIM; ++k) C.uf[k] = hi_float(u[k]);
-  C.hb1f = hi_float(hb1);
-  C.hb2f = hi_float(hb2);
-  C.hicf = hi_float(hic);
-  // b1 = 2 (b1/2) and u_d/2 from the truncated values (exact scalings: the
-  // same 2^-20 relative bound)
+  for (int k = 0; k < NDIM; ++k) C.uf[k] = u[k];
+  C.hb1f = hb1;
+  C.hb2f = hb2;
+  C.hicf = hic;
+  // b1 = 2 (b1/2) and u_d/2 from the given values (exact scalings: the same
+  // relative bound)
   C.b1f = 2.0f * C.hb1f;
   C.hudf = 0.5f * C.uf[DIR];
 #pragma unroll
   for (int f = 0; f < NVAR; ++f) {
-    C.haf[f] = hi_float(alpha[f]);
-    C.mp[f] = C.mm[f] = 0.0f;
+    C.haf[f] = ha[f];
+    C.xm[f] = 0.0f;
   }
-  C.vmax = 0.0f;
+  C.hum = C.hpm = 0.0f;
+  C.dir = DIR;
 }
 
-// Point j: U_j (binary64 state, normal momentum already mirrored at a wall),
-// unj = u_d/2, pnj = p/2.  The split values follow the binary64
+template <int NDIM, int DIR>
+TENO_CERT_HD void cert_begin(const double (&u)[NDIM], double hb1, double hb2, double hic,
+                             const double (&alpha)[NDIM + 2], CertIfc<NDIM>& C) {
+  float uf[NDIM], ha[NDIM + 2];
+#pragma unroll
+  for (int k = 0; k < NDIM; ++k) uf[k] = hi_float(u[k]);
+#pragma unroll
+  for (int f = 0; f < NDIM + 2; ++f) ha[f] = hi_float(alpha[f]);
+  cert_begin_f<NDIM, DIR>(uf, hi_float(hb1), hi_float(hb2), hi_float(hic), ha, C);
+}
+
+// Point j: truncated values X of U_j (normal momentum already mirrored at a
+// wall), of u_d/2 and of p/2.  The split values follow the binary64
 // characteristic path: w = L U_j, t = (p/2) z, v+ = (u_d/2 + alpha) w + t,
 // v- = v+ - 2 alpha w.
 template <int NDIM, int DIR>
-TENO_CERT_HD void cert_point(int j, const double (&Uj)[NDIM + 2], double unj, double pnj, CertIfc<NDIM>& C) {
+TENO_CERT_HD void cert_point_f(int j, const float (&X)[NDIM + 2], float huf, float hpf, CertIfc<NDIM>& C) {
   constexpr int NVAR = NDIM + 2;
-  float X[NVAR], Xa[NVAR];
 #pragma unroll
-  for (int v = 0; v < NVAR; ++v) {
-    X[v] = hi_float(Uj[v]);
-    Xa[v] = fabsf(X[v]);
-  }
-  float Sv = -X[NVAR - 1], Sa = Xa[NVAR - 1];
+  for (int v = 0; v < NVAR; ++v) C.xm[v] = fmaxf(C.xm[v], fabsf(X[v]));
+  C.hum = fmaxf(C.hum, fabsf(huf));
+  C.hpm = fmaxf(C.hpm, fabsf(hpf));
+  float Sv = -X[NVAR - 1];
 #pragma unroll
-  for (int k = 0; k < NDIM; ++k) {
-    Sv = ffma(C.uf[k], X[1 + k], Sv);
-    Sa = ffma(fabsf(C.uf[k]), Xa[1 + k], Sa);
-  }
+  for (int k = 0; k < NDIM; ++k) Sv = ffma(C.uf[k], X[1 + k], Sv);
   const float A = ffma(C.hb2f, X[0], -fmul(C.hb1f, Sv));
-  const float Aa = ffma(fabsf(C.hb2f), Xa[0], fmul(fabsf(C.hb1f), Sa));
   const float B = fmul(ffma(C.uf[DIR], X[0], -X[1 + DIR]), C.hicf);
-  const float Ba = fmul(ffma(fabsf(C.uf[DIR]), Xa[0], Xa[1 + DIR]), fabsf(C.hicf));
-  float w[NVAR], wa[NVAR];
+  float w[NVAR];
   w[0] = fadd(A, B);
-  wa[0] = fadd(Aa, Ba);
   w[1] = ffma(-2.0f, A, X[0]);
-  wa[1] = ffma(2.0f, Aa, Xa[0]);
   {
     int f = 2;
 #pragma unroll
     for (int t = 0; t < NDIM; ++t) {
       if (t == DIR) continue;
       w[f] = ffma(-C.uf[t], X[0], X[1 + t]);
-      wa[f] = ffma(fabsf(C.uf[t]), Xa[0], Xa[1 + t]);
       ++f;
     }
   }
   w[NVAR - 1] = fsub(A, B);
-  wa[NVAR - 1] = fadd(Aa, Ba);
-  const float huf = hi_float(unj), hpf = hi_float(pnj);
   const float az = fmul(hpf, fmul(C.b1f, fsub(huf, C.hudf)));
-  const float aza = fmul(fabsf(hpf), fmul(fabsf(C.b1f), fadd(fabsf(huf), fabsf(C.hudf))));
-  const float bz = fmul(hpf, C.hicf), bza = fmul(fabsf(hpf), fabsf(C.hicf));
+  const float bz = fmul(hpf, C.hicf);
 #pragma unroll
   for (int f = 0; f < NVAR; ++f) {
-    const float t = (f == 0) ? fsub(az, bz) : (f == NVAR - 1) ? fadd(az, bz) : (f == 1) ? -2.0f * az : 0.0f;
-    const float ta = (f == 0 || f == NVAR - 1) ? fadd(aza, bza) : (f == 1) ? 2.0f * aza : 0.0f;
-    C.vp32[j][f] = ffma(fadd(huf, C.haf[f]), w[f], t);
+    const float t = (f == 0) ? fsub(az, bz) : (f == NVAR - 1) ? fadd(az, bz) : -2.0f * az;
+    const float s = fadd(huf, C.haf[f]);
+    C.vp32[j][f] = (f >= 2 && f < NVAR - 1) ? fmul(s, w[f]) : ffma(s, w[f], t);
     C.vm32[j][f] = ffma(-2.0f * C.haf[f], w[f], C.vp32[j][f]);
-    const float pa = ffma(fadd(fabsf(huf), C.haf[f]), wa[f], ta);
-    const float ma = ffma(2.0f * C.haf[f], wa[f], pa);
-    if (j <= 4) C.mp[f] = fmaxf(C.mp[f], pa);
-    if (j >= 1) C.mm[f] = fmaxf(C.mm[f], ma);
-    C.vmax = fmaxf(C.vmax, fmaxf(fabsf(C.vp32[j][f]), fabsf(C.vm32[j][f])));
   }
+}
+
+template <int NDIM, int DIR>
+TENO_CERT_HD void cert_point(int j, const double (&Uj)[NDIM + 2], double unj, double pnj, CertIfc<NDIM>& C) {
+  float X[NDIM + 2];
+#pragma unroll
+  for (int v = 0; v < NDIM + 2; ++v) X[v] = hi_float(Uj[v]);
+  cert_point_f<NDIM, DIR>(j, X, hi_float(unj), hi_float(pnj), C);
 }
 
 // cert_open: bit 2 f (side v+) and 2 f + 1 (side v-) set where the test does
@@ -367,16 +379,38 @@ TENO_CERT_HD void cert_point(int j, const double (&Uj)[NDIM + 2], double unj, do
 template <int NDIM>
 TENO_CERT_HD unsigned cert_open(const CertIfc<NDIM>& C, float thr_f, float eps4_f) {
   constexpr int NVAR = NDIM + 2;
-  const float kd = 8.0f * 0x1p-20f;
-  const float ku = ffma(8.0f * 0x1p-24f, C.vmax, 0x1p-100f);
+  // the absolute evaluation of cert_point_f's expressions at the maxima
+  float Sa = C.xm[NVAR - 1];
+#pragma unroll
+  for (int k = 0; k < NDIM; ++k) Sa = ffma(fabsf(C.uf[k]), C.xm[1 + k], Sa);
+  const float Aa = ffma(fabsf(C.hb2f), C.xm[0], fmul(fabsf(C.hb1f), Sa));
+  const float Ba = fmul(ffma(fabsf(C.uf[C.dir]), C.xm[0], C.xm[1 + C.dir]), fabsf(C.hicf));
+  float wa[NVAR];
+  wa[0] = wa[NVAR - 1] = fadd(Aa, Ba);
+  wa[1] = ffma(2.0f, Aa, C.xm[0]);
+  {
+    int f = 2;
+#pragma unroll
+    for (int t = 0; t < NDIM; ++t) {
+      if (t == C.dir) continue;
+      wa[f] = ffma(fabsf(C.uf[t]), C.xm[0], C.xm[1 + t]);
+      ++f;
+    }
+  }
+  const float aza = fmul(C.hpm, fmul(fabsf(C.b1f), fadd(C.hum, fabsf(C.hudf))));
+  const float bza = fmul(C.hpm, fabsf(C.hicf));
+  const float kd = 8.0f * 0x1p-20f + 8.0f * 0x1p-24f;
   unsigned open = 0u;
 #pragma unroll
   for (int f = 0; f < NVAR; ++f) {
+    const float ta = (f == 0 || f == NVAR - 1) ? fadd(aza, bza) : (f == 1) ? 2.0f * aza : 0.0f;
+    const float mp = ffma(fadd(C.hum, C.haf[f]), wa[f], ta);
+    const float mm = ffma(2.0f * C.haf[f], wa[f], mp);
     if (!certify_keep(C.vp32[0][f], C.vp32[1][f], C.vp32[2][f], C.vp32[3][f], C.vp32[4][f],
-                      ffma(kd, C.mp[f], ku), thr_f, eps4_f))
+                      ffma(kd, mp, 0x1p-100f), thr_f, eps4_f))
       open |= 1u << (2 * f);
     if (!certify_keep(C.vm32[5][f], C.vm32[4][f], C.vm32[3][f], C.vm32[2][f], C.vm32[1][f],
-                      ffma(kd, C.mm[f], ku), thr_f, eps4_f))
+                      ffma(kd, mm, 0x1p-100f), thr_f, eps4_f))
       open |= 2u << (2 * f);
   }
   return open;

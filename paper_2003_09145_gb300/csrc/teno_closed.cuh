@@ -1,0 +1,237 @@
+// teno_closed.cuh -- the closed form of an interface flux (every stencil kept)
+// with its certified test, as the two-pass flux kernels and the batched
+// kernel run it: the Roe state and the corrections in two binary32 values
+// (teno_df.cuh), U~ and the mass flux in 64-bit fixed point (teno_fixsum.cuh),
+// the other fluxes as binary64 chains.  FP64 instructions per interface: 25 of
+// the 3D sweep's (five per component, and the reciprocal, square root and
+// products of the Roe state gone), against 78 with the Roe state and the
+// corrections in binary64.
+#pragma once
+
+#include "teno_df.cuh"
+#include "teno_flux.cuh"
+
+namespace teno {
+
+// The speeds in the forms the closed form reads: halved, as two binary32
+// values (the middle one, and the sum and difference of the acoustic
+// ones' differences against it -- closed_out's amid, sg, df), as binary32, and
+// whether they lie in the range of teno_df's terms (2^-19 .. 2^30).
+struct FaceSpeeds {
+  teno_df::df amid, sg, dd;
+  float ha[3], amax;
+  bool in_range;
+};
+__device__ __forceinline__ FaceSpeeds face_speeds(const double (&a3)[3]) {
+  using namespace teno_df;
+  FaceSpeeds F;
+  const df am = from_double(a3[0]), a0 = from_double(a3[1]), ap = from_double(a3[2]);
+  const df d0 = add(am, neg(a0)), dE = add(ap, neg(a0));
+  F.amid = a0;
+  F.sg = add(d0, dE);
+  F.dd = add(d0, neg(dE));
+#pragma unroll
+  for (int s = 0; s < 3; ++s) F.ha[s] = hi_float(a3[s]);
+  F.amax = 2.0f * fmaxf(F.ha[0], F.ha[2]);
+  F.in_range = F.amax >= 0x1p-19f && F.amax <= 0x1p30f;
+  return F;
+}
+
+// The Roe state in two binary32 values, from the cells' sqrt(rho),
+// (E+p)/sqrt(rho) and m_k/sqrt(rho) (roe_interface's average): u~, |u~|^2, H~,
+// c~^2 and 1/c~.
+template <int NDIM>
+struct RoeDf {
+  teno_df::df u[NDIM], q2, H, c2, ic;
+};
+template <int NDIM>
+__device__ __forceinline__ void roe_df(double sr2, double sr3, double sh2, double sh3, const double (&su2)[NDIM],
+                                       const double (&su3)[NDIM], const Scheme& S, RoeDf<NDIM>& R) {
+  using namespace teno_df;
+  const df y = recip(add(from_double(sr2), from_double(sr3)));
+#pragma unroll
+  for (int k = 0; k < NDIM; ++k) {
+    R.u[k] = mul(add(from_double(su2[k]), from_double(su3[k])), y);
+    R.q2 = k == 0 ? sqr(R.u[0]) : add(R.q2, sqr(R.u[k]));
+  }
+  R.H = mul(add(from_double(sh2), from_double(sh3)), y);
+  R.c2 = mul(df{S.gm1_h, S.gm1_l}, add(R.H, scale(R.q2, -0.5f)));
+  R.ic = teno_df::rsqrt(R.c2);
+}
+
+// The certificate's view of that Roe state: its high parts lie within 2^-21
+// of the values where roe_df_ok holds, i.e. where c~^2 keeps 2^-6 of
+// (gamma - 1) H~ (Mach numbers below about 18 for gamma = 1.4; c~^2 is then
+// good to 2^-38).
+template <int NDIM, int DIR>
+__device__ __forceinline__ void cert_begin_df(const RoeDf<NDIM>& R, const float (&ha3)[3], const Scheme& S,
+                                              CertIfc<NDIM>& C) {
+  float uf[NDIM], ha[NDIM + 2];
+#pragma unroll
+  for (int k = 0; k < NDIM; ++k) uf[k] = R.u[k].h;
+#pragma unroll
+  for (int f = 0; f < NDIM + 2; ++f) ha[f] = ha3[f == 0 ? 0 : (f == NDIM + 1 ? 2 : 1)];
+  const float hb1 = teno_cert::fmul(0.5f * S.gm1_h, teno_cert::fmul(R.ic.h, R.ic.h));
+  teno_cert::cert_begin_f<NDIM, DIR>(uf, hb1, teno_cert::fmul(0.5f * hb1, R.q2.h), 0.5f * R.ic.h, ha, C);
+}
+template <int NDIM>
+__device__ __forceinline__ bool roe_df_ok(const RoeDf<NDIM>& R, const Scheme& S) {
+  return R.c2.h > 0x1p-6f * S.gm1_h * R.H.h;
+}
+
+// binary32 truncation of |x| < 2^127 (hi_float without its upper clamp):
+// magnitudes below 2^-126 become +-2^-126
+__device__ __forceinline__ float low_float(double x) {
+  const uint32_t hi = teno_fix::hi_word(x);
+  uint32_t m = hi << 1;
+  m = m < (897u << 21) ? (897u << 21) : m;
+  return __uint_as_float((m * 4u - (896u << 23)) | (hi & 0x80000000u));
+}
+
+// 2^-20 <= max rho < 2^30 and max E < 2^95 (from the high words' magnitudes,
+// shifted left by one) keep every term of the test and of teno_df in binary32's
+// range; |u| and c are bounded by the speeds.
+__device__ __forceinline__ bool df_range(uint32_t tr, uint32_t te) {
+  return tr >= (1003u << 21) && tr < (1053u << 21) && te < (1118u << 21);
+}
+
+// The flux of one interface with every stencil kept, and the mask of its open
+// reconstructions (see interface_flux_closed_wide, which takes over, all in
+// binary64, where the interface leaves teno_df's range or U~ is not small
+// against the flux scale, i.e. near shocks).  I: the cell index type, 32 bits
+// on the grid path; a3: the halved speeds, F: face_speeds of them.
+template <int NDIM, int DIR, bool GH, class I>
+__device__ __forceinline__ unsigned interface_flux_closed(const double* __restrict__ U,
+                                                          const double* __restrict__ aux,
+                                                          const double* __restrict__ fh, int64_t ncell,
+                                                          const I (&cells)[6], unsigned flips,
+                                                          const double (&a3)[3], const FaceSpeeds& F,
+                                                          const Scheme& S, double (&out)[NDIM + 2],
+                                                          int* __restrict__ status, const GhostCells& gc) {
+  using namespace teno_df;
+  constexpr int NVAR = NDIM + 2;
+  if (S.keep_idx < 0) return kRough | kAllOpen<NDIM>;
+  const double* gfh = GH ? gc.fh + DIR * (NVAR - 1) * kGhostSlots : nullptr;
+  RoeDf<NDIM> R;
+  {
+    double su2[NDIM], su3[NDIM];
+#pragma unroll
+    for (int k = 0; k < NDIM; ++k) {
+      su2[k] = ldc<GH>(aux, gc.aux, ncell, NDIM + 3 + k, cells[2]);
+      su3[k] = ldc<GH>(aux, gc.aux, ncell, NDIM + 3 + k, cells[3]);
+    }
+    su2[DIR] = flip_sign(su2[DIR], (flips >> 2) & 1u);
+    su3[DIR] = flip_sign(su3[DIR], (flips >> 3) & 1u);
+    roe_df<NDIM>(ldc<GH>(aux, gc.aux, ncell, NDIM + 1, cells[2]), ldc<GH>(aux, gc.aux, ncell, NDIM + 1, cells[3]),
+                 ldc<GH>(aux, gc.aux, ncell, NDIM + 2, cells[2]), ldc<GH>(aux, gc.aux, ncell, NDIM + 2, cells[3]),
+                 su2, su3, S, R);
+  }
+  bool range = F.in_range && roe_df_ok<NDIM>(R, S), wide = false;
+  // first pass: the certified test and the largest magnitudes of the summed
+  // components (a mirrored point changes signs only)
+  unsigned open;
+  float xm[NVAR];
+  {
+    CertIfc<NDIM> C;
+    cert_begin_df<NDIM, DIR>(R, F.ha, S, C);
+    uint32_t tr = 0u, te = 0u;   // the magnitudes of rho and E, not clamped
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+      const I c = cells[j];
+      const uint32_t fj = ((flips >> j) & 1u) << 31;
+      float X[NVAR];
+#pragma unroll
+      for (int v = 0; v < NVAR; ++v) {
+        const double x = ldc<GH>(U, gc.U, ncell, v, c);
+        X[v] = low_float(x);
+        if (v == 0) tr = max(tr, teno_fix::hi_word(x) << 1);
+        if (v == NVAR - 1) te = max(te, teno_fix::hi_word(x) << 1);
+      }
+      X[1 + DIR] = __uint_as_float(__float_as_uint(X[1 + DIR]) ^ fj);
+      const float huf = __uint_as_float(__float_as_uint(low_float(ldc<GH>(aux, gc.aux, ncell, DIR, c))) ^ fj);
+      teno_cert::cert_point_f<NDIM, DIR>(j, X, huf, low_float(ldc<GH>(aux, gc.aux, ncell, NDIM, c)), C);
+    }
+    range = range && df_range(tr, te);
+    open = cert_open<NDIM>(C, S);
+#pragma unroll
+    for (int v = 0; v < NVAR; ++v) xm[v] = C.xm[v];
+  }
+  if (range) {
+    // second pass: 60 U~ and the mass flux in fixed point on the grids of the
+    // components' largest exponents, the other fluxes as binary64 chains
+    // (see ClosedFix).  The points are taken in two rounds of three (fully
+    // unrolled, the sums' temporaries of all six points would not fit in
+    // the registers; the cell indices, read with a loop index, then sit in the
+    // stack frame).
+    uint32_t EU[NVAR];
+    int64_t AU[NVAR], AF = 0;
+    double Fd[NVAR];
+#pragma unroll
+    for (int v = 0; v < NVAR; ++v) {
+      EU[v] = (__float_as_uint(xm[v]) >> 23) + 896u;
+      AU[v] = 0;
+      Fd[v] = 0.0;
+    }
+#pragma unroll 3
+    for (int j = 0; j < 6; ++j) {
+      const I c = cells[j];
+      const bool fj = (flips >> j) & 1u;
+      const int cw = c_fix_w[0][j], mw = c_fix_w[1][j];
+      const double cd = c_fix_cd[j];
+#pragma unroll
+      for (int v = 0; v < NVAR; ++v) {
+        const double x = flip_sign(ldc<GH>(U, gc.U, ncell, v, c), fj && v == 1 + DIR);
+        const int64_t X = teno_fix::term(x, EU[v]);
+        AU[v] += mw * X;
+        if (v == 1 + DIR) AF += cw * X;
+      }
+#pragma unroll
+      for (int v = 1; v < NVAR; ++v) {
+        const double f = flip_sign(ldc<GH>(fh, gfh, ncell, v - 1, c), fj && v != 1 + DIR);
+        if (j == 0) Fd[v] = f;
+        else Fd[v] = fma(cd, f, Fd[v]);
+      }
+    }
+    df Ut[NVAR];
+    // U~ against the flux scale: |60 U~| <= 60 2^-8 (rho, alpha rho, E),
+    // tightened by c~^2 / ((gamma - 1) H~), the digits that c~^2 lost
+    const float gH = S.gm1_h * R.H.h, lim = (60.0f * 0x1p-8f) * R.c2.h;
+#pragma unroll
+    for (int v = 0; v < NVAR; ++v) {
+      Ut[v] = from_fixed(AU[v], EU[v]);
+      const float sc = v == 0 ? xm[0] : (v == NVAR - 1 ? xm[NVAR - 1] : xm[0] * F.amax);
+      wide = wide || !(fabsf(Ut[v].h) * gH <= lim * sc);
+    }
+    if (!wide) {
+      // closed_out with c~ eliminated: T = |u~|^2/2 U~_0 - u~.U~_m + U~_E,
+      // V = (u~_d U~_0 - U~_d)/2 = c~ B, t = c~ A = (gamma-1)/2 T / c~,
+      // gs = (sg t + df V) / c~, c~ ngd = df t + sg V
+      df T = mul(scale(R.q2, 0.5f), Ut[0]);
+#pragma unroll
+      for (int k = 0; k < NDIM; ++k) T = add(T, neg(mul(R.u[k], Ut[1 + k])));
+      T = add(T, Ut[NVAR - 1]);
+      const df V = scale(add(mul(R.u[DIR], Ut[0]), neg(Ut[1 + DIR])), 0.5f);
+      const df t = mul(mul(df{0.5f * S.gm1_h, 0.5f * S.gm1_l}, T), R.ic);
+      const df gs = mul(R.ic, add(mul(F.sg, t), mul(F.dd, V)));
+      const df cn = add(mul(F.dd, t), mul(F.sg, V));
+      out[0] = teno_fix::round(AF, EU[1 + DIR] - 1u) + to_double(add(mul(F.amid, Ut[0]), gs));
+#pragma unroll
+      for (int k = 0; k < NDIM; ++k) {
+        df o = add(mul(F.amid, Ut[1 + k]), mul(R.u[k], gs));
+        if (k == DIR) o = add(o, neg(cn));
+        out[1 + k] = Fd[1 + k] + to_double(o);
+      }
+      out[NVAR - 1] =
+          Fd[NVAR - 1] + to_double(add(add(mul(F.amid, Ut[NVAR - 1]), mul(R.H, gs)), neg(mul(R.u[DIR], cn))));
+    }
+  }
+  // out of range the binary64 form also decides; where only U~ is large it
+  // gives the flux
+  if (!range || wide) {
+    const unsigned w = interface_flux_closed_wide<NDIM, DIR, GH, I>(U, aux, fh, ncell, cells, flips, a3, S, out, status, gc);
+    if (!range || (w & kRough)) open = w;
+  }
+  return open;
+}
+
+}  // namespace teno

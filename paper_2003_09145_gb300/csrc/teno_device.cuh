@@ -98,6 +98,7 @@ struct Scheme {
   double eps_a;   // kSchemeTeno5A: eps of eq. 2.18
   double gamma;   // ratio of specific heats (eq. 4.7)
   double gm1;     // gamma - 1
+  float gm1_h, gm1_l;   // gamma - 1 as two binary32 values
   double eps;     // epsilon of eq. 2.8 / 3.2
   double eps4;    // 4 eps (the indicators are carried scaled by 4)
   int b_l, b_u;   // magnitude bounds of eq. 3.1

@@ -324,11 +324,22 @@ __device__ __forceinline__ void closed_out(const double (&Ft)[NDIM + 2], const d
   out[NVAR - 1] = fma(R.H, gs, fma(-(R.u[DIR] * R.cs), ngd, fma(amid, Ut[NVAR - 1], Ft[NVAR - 1])));
 }
 
+// the three halved speeds (a_-, a_mid, a_+) per field, and their negated doubles
+template <int NDIM>
+__device__ __forceinline__ void spread_speeds(const double (&a3)[3], double (&alpha)[NDIM + 2],
+                                              double (&nal)[NDIM + 2]) {
+#pragma unroll
+  for (int f = 0; f < NDIM + 2; ++f) {
+    alpha[f] = a3[f == 0 ? 0 : (f == NDIM + 1 ? 2 : 1)];
+    nal[f] = -2.0 * alpha[f];
+  }
+}
+
 // ---------------------------------------------------------------------------
 // The closed form alone, with the per-cell F_DIR/2 of the cell
 // pass (`fh`, momentum and energy components only: [nvar - 1][ncell]), in
 // two passes over the six stencil points: the FP32 test (and the exponents
-// of the sums), then the fixed-point sums, so that the test's state is dead
+// of the sums), then the sums, so that the test's state is dead
 // before the sums' state is live.  Returns the open reconstructions (bit
 // 2 s + side of field s, cert_open's mask): 0 -- the test keeps every stencil
 // and `out` is the flux (interface_flux's up to the rounding of the sums,
@@ -336,26 +347,29 @@ __device__ __forceinline__ void closed_out(const double (&Ft)[NDIM + 2], const d
 // the flux with every stencil kept, to which warp_correct adds the
 // open reconstructions' differences.  kRough: the fixed point does not cover
 // a sum and `out` is unwritten (warp_correct then sums every field).
+//
+// This form evaluates the Roe state and the corrections in binary64;
+// teno_closed.cuh's interface_flux_closed, which takes them in two binary32
+// values, falls back to it (out of line: rare, and the common form's code
+// stays small).
+// (GH: the sweep direction has fixed-state ghost cells, read from gc; the
+// half fluxes of the ghost block are taken at direction DIR's block.)
 // ---------------------------------------------------------------------------
 constexpr unsigned kRough = 1u << 15;
 template <int NDIM>
 constexpr unsigned kAllOpen = (1u << (2 * (NDIM + 2))) - 1u;
-// (GH: the sweep direction has fixed-state ghost cells, read from gc; the
-// half fluxes of the ghost block are taken at direction DIR's block.  With
-// `rout` the interface's Roe state is also returned, whatever the test
-// decides.)
-template <int NDIM, int DIR, bool GH = false>
-__device__ __forceinline__ unsigned interface_flux_closed(const double* __restrict__ U,
-                                                      const double* __restrict__ aux,
-                                                      const double* __restrict__ fh, int64_t ncell,
-                                                      const int64_t (&cells)[6], unsigned flips,
-                                                      const double (&alpha)[NDIM + 2],
-                                                      const double (&nal)[NDIM + 2], const Scheme& S,
-                                                      double (&out)[NDIM + 2], int* __restrict__ status,
-                                                      const GhostCells& gc = GhostCells(),
-                                                      RoeIfc<NDIM>* rout = nullptr) {
+
+template <int NDIM, int DIR, bool GH, class I>
+__device__ __noinline__ unsigned interface_flux_closed_wide(const double* __restrict__ U,
+                                                            const double* __restrict__ aux,
+                                                            const double* __restrict__ fh, int64_t ncell,
+                                                            const I (&cells)[6], unsigned flips,
+                                                            const double (&a3)[3], const Scheme& S,
+                                                            double (&out)[NDIM + 2], int* __restrict__ status,
+                                                            const GhostCells& gc) {
   constexpr int NVAR = NDIM + 2;
-  if (S.keep_idx < 0) return kRough | kAllOpen<NDIM>;
+  double alpha[NVAR], nal[NVAR];
+  spread_speeds<NDIM>(a3, alpha, nal);
   const double* gfh = GH ? gc.fh + DIR * (NVAR - 1) * kGhostSlots : nullptr;
   RoeIfc<NDIM> R;
   {
@@ -372,11 +386,10 @@ __device__ __forceinline__ unsigned interface_flux_closed(const double* __restri
                              ldc<GH>(aux, gc.aux, ncell, NDIM + 2, cells[2]),
                              ldc<GH>(aux, gc.aux, ncell, NDIM + 2, cells[3]), su2, su3, S, R, status);
   }
-  if (rout) *rout = R;
   // stencil point j: U with the normal momentum reversed at a mirrored wall
   // point, so u_d and every component of F_d/2 but the normal-momentum one
   // change sign
-  auto load_point = [&](int j, int64_t c, double (&Uj)[NVAR], double (&Fhj)[NVAR]) {
+  auto load_point = [&](int j, I c, double (&Uj)[NVAR], double (&Fhj)[NVAR]) {
     const bool fj = (flips >> j) & 1u;
 #pragma unroll
     for (int v = 0; v < NVAR; ++v) Uj[v] = ldc<GH>(U, gc.U, ncell, v, c);
@@ -396,7 +409,7 @@ __device__ __forceinline__ unsigned interface_flux_closed(const double* __restri
     cert_begin<NDIM, DIR>(R, alpha, C);
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
-      const int64_t c = cells[j];
+      const I c = cells[j];
       const bool fj = (flips >> j) & 1u;
       double Uj[NVAR];
 #pragma unroll
@@ -488,10 +501,10 @@ struct CorrectScratch {   // one per warp
   uint16_t item[2 * (NDIM + 2) * 32];   // owner | reconstruction << 5 | whole << 9
 };
 
-// cells_of(q, cells, flips) gives the stencil of interface q.  Every lane of
+// cells_of(q, cells, flips) gives the stencil of interface q (cell indices I).  Every lane of
 // the warp calls; `open` is 0 in lanes without an interface.  On entry `out`
 // is interface_flux_closed's (unset with kRough), on return the flux.
-template <int NDIM, int DIR, bool GH, class Cells>
+template <int NDIM, int DIR, bool GH, class I, class Cells>
 __device__ __forceinline__ void warp_correct(const double* __restrict__ U, const double* __restrict__ aux,
                                              int64_t ncell, const Cells& cells_of, uint32_t q,
                                              const double (&alpha)[NDIM + 2], const Scheme& S, unsigned open,
@@ -504,7 +517,7 @@ __device__ __forceinline__ void warp_correct(const double* __restrict__ U, const
   double q2 = 0.0;
   __syncwarp();
   if (open) {
-    int64_t cells[6];
+    I cells[6];
     unsigned flips;
     cells_of(q, cells, flips);
     RoeIfc<NDIM> R;
@@ -557,14 +570,14 @@ __device__ __forceinline__ void warp_correct(const double* __restrict__ U, const
     const unsigned it = W.item[i];
     const unsigned o = it & 31u, b = (it >> 5) & 15u, s = b >> 1;
     const bool minus = b & 1u;
-    int64_t cells[6];
+    I cells[6];
     unsigned flips;
     cells_of(W.q[o], cells, flips);
     double v[5];
     auto point = [&](int j, double (&Uj)[NVAR], double& un) {
       const int p = minus ? 5 - j : j;
       const bool fj = (flips >> p) & 1u;
-      const int64_t c = minus ? cells[5 - j] : cells[j];
+      const I c = minus ? cells[5 - j] : cells[j];
 #pragma unroll
       for (int k = 0; k < NVAR; ++k) Uj[k] = ldc<GH>(U, gc.U, ncell, k, c);
       Uj[1 + DIR] = flip_sign(Uj[1 + DIR], fj);
@@ -579,7 +592,7 @@ __device__ __forceinline__ void warp_correct(const double* __restrict__ U, const
       for (int j = 0; j < 5; ++j) {
         const int p = minus ? 5 - j : j;
         const bool fj = (flips >> p) & 1u;
-        const int64_t c = minus ? cells[5 - j] : cells[j];
+        const I c = minus ? cells[5 - j] : cells[j];
         const double w = fma(-ut, ldc<GH>(U, gc.U, ncell, 0, c), ldc<GH>(U, gc.U, ncell, 1 + t, c));
         v[j] = (flip_sign(ldc<GH>(aux, gc.aux, ncell, DIR, c), fj) + (minus ? -alpha[1] : alpha[1])) * w;
       }
@@ -673,10 +686,10 @@ constexpr unsigned kUndecided = 0xffu;
 
 // the certify-only instantiation ends early: its remaining code is unreachable
 #pragma nv_diag_suppress 128
-template <int NDIM, int DIR, bool WITH_FLAGS, int MODE = kFluxFull, bool GH = false>
+template <int NDIM, int DIR, bool WITH_FLAGS, int MODE = kFluxFull, bool GH = false, class I = int64_t>
 __device__ __forceinline__ void interface_flux(const double* __restrict__ U,
                                                const double* __restrict__ aux,
-                                               int64_t ncell, const int64_t (&cells)[6], unsigned flips,
+                                               int64_t ncell, const I (&cells)[6], unsigned flips,
                                                const double (&alpha)[NDIM + 2],
                                                const double (&nal)[NDIM + 2],
                                                const Scheme& S, double (&out)[NDIM + 2],
@@ -690,7 +703,7 @@ __device__ __forceinline__ void interface_flux(const double* __restrict__ U,
     double sr2, sr3, sh2, sh3, su2[NDIM], su3[NDIM];
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
-      const int64_t c = cells[j];
+      const I c = cells[j];
       const bool fj = (flips >> j) & 1u;   // mirrored wall point
 #pragma unroll
       for (int v = 0; v < NVAR; ++v) Ux[j][v] = ldc<GH>(U, gc.U, ncell, v, c);

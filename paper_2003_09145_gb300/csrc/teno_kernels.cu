@@ -17,6 +17,7 @@
 #include <cstring>
 #include <cuda_runtime.h>
 
+#include "teno_closed.cuh"
 #include "teno_device.cuh"
 #include "teno_flux.cuh"
 #include "teno_launch.h"
@@ -285,29 +286,42 @@ __global__ void __launch_bounds__(128, TENO_FLUX_MINBLOCKS) flux_kernel(
 #define TENO_CLOSED_Z_TILE 1
 #endif
 
-// GH: fixed-state faces along DIR, whose ghost points are the virtual cells
-// ncell + 2 DIR + side
+// The stencil of interface q (32-bit indices throughout: the C-ABI admits
+// fewer than 2^32 interfaces per direction).  GH: fixed-state faces along
+// DIR, whose ghost points are the virtual cells ncell + 2 DIR + side.
+// Interfaces three cells off both ends, nearly all, skip the boundary maps.
 template <int NDIM, int DIR, bool GH = false>
-__device__ __forceinline__ void interface_cells(int64_t q, const Grid& G, int64_t (&cells)[6], unsigned& flips) {
-  const int64_t m0 = G.n[0] + (DIR == 0), m1 = G.n[1] + (DIR == 1);
-  const int64_t stride_d = (DIR == 0) ? 1 : (DIR == 1 ? G.n[0] : G.n[0] * G.n[1]);
-  const int64_t i0 = q % m0;
-  const int64_t r = q / m0;
-  const int64_t i1 = r % m1;
-  const int64_t i2 = r / m1;
-  const int64_t id = (DIR == 0) ? i0 : (DIR == 1 ? i1 : i2);
-  const int64_t base = (DIR == 0) ? (i2 * G.n[1] + i1) * G.n[0]
-                     : (DIR == 1) ? i2 * G.n[1] * G.n[0] + i0
-                                  : i1 * G.n[0] + i0;
+__device__ __forceinline__ void interface_cells(uint32_t q, const Grid& G, uint32_t (&cells)[6], unsigned& flips) {
+  const uint32_t n0 = static_cast<uint32_t>(G.n[0]), n1 = static_cast<uint32_t>(G.n[1]);
+  const uint32_t nd = static_cast<uint32_t>(G.n[DIR]);
+  const uint32_t m0 = n0 + (DIR == 0), m1 = n1 + (DIR == 1);
+  const uint32_t sd = (DIR == 0) ? 1u : (DIR == 1 ? n0 : n0 * n1);
+  uint32_t i0 = q, i1 = 0, i2 = 0;
+  if (NDIM > 1) {
+    const uint32_t r = q / m0;
+    i0 = q - r * m0;
+    i1 = r;
+    if (NDIM > 2) {
+      i2 = r / m1;
+      i1 = r - i2 * m1;
+    }
+  }
+  const uint32_t id = (DIR == 0) ? i0 : (DIR == 1 ? i1 : i2);
+  const uint32_t base = (DIR == 0) ? (i2 * n1 + i1) * n0 : (DIR == 1) ? i2 * n1 * n0 + i0 : i1 * n0 + i0;
   flips = 0u;
+  if (id >= 3u && id + 3u <= nd) {
+#pragma unroll
+    for (int j = 0; j < 6; ++j) cells[j] = base + (id - 3u + j) * sd;
+    return;
+  }
 #pragma unroll
   for (int j = 0; j < 6; ++j) {
-    bool f;
-    const int64_t k = id - 3 + j;
-    if (GH && (k < 0 || k >= G.n[DIR])) {
-      cells[j] = G.ncell + 2 * DIR + (k >= G.n[DIR]);
+    const int64_t k = (int64_t)id - 3 + j;
+    if (GH && (k < 0 || k >= (int64_t)nd)) {
+      cells[j] = static_cast<uint32_t>(G.ncell) + 2 * DIR + (k >= (int64_t)nd);
     } else {
-      cells[j] = base + ghost(k, G.n[DIR], G.bc[DIR], f) * stride_d;
+      bool f;
+      cells[j] = base + static_cast<uint32_t>(ghost(k, G.n[DIR], G.bc[DIR], f)) * sd;
       flips |= unsigned(f) << j;
     }
   }
@@ -344,8 +358,10 @@ __global__ void __launch_bounds__(128, TENO_CLOSED_MINBLOCKS) flux_closed_kernel
     Scheme S, double* __restrict__ roe_out = nullptr) {
   constexpr int NVAR = NDIM + 2;
   const int64_t nifc = (G.n[0] + (DIR == 0)) * (G.n[1] + (DIR == 1)) * (G.n[2] + (DIR == 2));
-  double alpha[NVAR], nal[NVAR];
-  half_speeds<NDIM, DIR>(alpha_bits, alpha, nal);
+  double a3[3];
+#pragma unroll
+  for (int s = 0; s < 3; ++s) a3[s] = 0.5 * __longlong_as_double((long long)alpha_bits[DIR * 3 + s]);
+  const FaceSpeeds F = face_speeds(a3);
   const unsigned lane = threadIdx.x & 31u;
   // The z sweep takes its interfaces in tiles of 32 along x by 4 along z
   // (a block of 128 threads per tile, a warp per z): the six stencil planes
@@ -369,16 +385,25 @@ __global__ void __launch_bounds__(128, TENO_CLOSED_MINBLOCKS) flux_closed_kernel
       if (x >= n0 || z >= nz1) continue;
       q = ((int64_t)z * n1 + (r % n1)) * n0 + x;
     }
-    int64_t cells[6];
+    uint32_t cells[6];
     unsigned flips;
-    interface_cells<NDIM, DIR, WALL == 2>(q, G, cells, flips);
+    interface_cells<NDIM, DIR, WALL == 2>(static_cast<uint32_t>(q), G, cells, flips);
     double out[NVAR];
-    RoeIfc<NDIM> R;
     const unsigned open = interface_flux_closed<NDIM, DIR, WALL == 2>(
-        U, aux, fh + (int64_t)DIR * (NVAR - 1) * G.ncell, G.ncell, cells, WALL == 1 ? flips : 0u, alpha, nal, S,
-        out, status, GhostCells{G.gU, G.gaux, G.gfh}, ROE ? &R : nullptr);
+        U, aux, fh + (int64_t)DIR * (NVAR - 1) * G.ncell, G.ncell, cells, WALL == 1 ? flips : 0u, a3, F, S, out,
+        status, GhostCells{G.gU, G.gaux, G.gfh});
     if constexpr (ROE) {
       if (S.keep_idx >= 0) {
+        RoeIfc<NDIM> R;
+        double su2[NDIM], su3[NDIM];
+#pragma unroll
+        for (int k = 0; k < NDIM; ++k) {
+          su2[k] = aux[(NDIM + 3 + k) * G.ncell + cells[2]];
+          su3[k] = aux[(NDIM + 3 + k) * G.ncell + cells[3]];
+        }
+        roe_interface<NDIM, DIR>(aux[(NDIM + 1) * G.ncell + cells[2]], aux[(NDIM + 1) * G.ncell + cells[3]],
+                                 aux[(NDIM + 2) * G.ncell + cells[2]], aux[(NDIM + 2) * G.ncell + cells[3]], su2, su3,
+                                 S, R, status);
 #pragma unroll
         for (int k = 0; k < NDIM; ++k) roe_out[(int64_t)k * nifc + q] = R.u[k];
         roe_out[(int64_t)(NDIM + 0) * nifc + q] = R.q2;
@@ -430,7 +455,7 @@ __global__ void __launch_bounds__(128) flux_correct_kernel(
   if (blockIdx.x * (int64_t)(4 * per) >= n) return;
   double alpha[NVAR], nal[NVAR];
   half_speeds<NDIM, DIR>(alpha_bits, alpha, nal);
-  auto cells_of = [&](uint32_t q, int64_t (&cells)[6], unsigned& flips) {
+  auto cells_of = [&](uint32_t q, uint32_t (&cells)[6], unsigned& flips) {
     interface_cells<NDIM, DIR, GH>(q, G, cells, flips);
   };
   for (int64_t i0 = ((int64_t)blockIdx.x * 4 + warp) * per; i0 < n; i0 += nw * per) {
@@ -439,7 +464,7 @@ __global__ void __launch_bounds__(128) flux_correct_kernel(
     double out[NVAR];
 #pragma unroll
     for (int v = 0; v < NVAR; ++v) out[v] = e.y && !(e.y & kRough) ? Fhat[(int64_t)v * nifc + e.x] : 0.0;
-    warp_correct<NDIM, DIR, GH>(U, aux, G.ncell, cells_of, e.x, alpha, S, e.y, out, status, scratch[warp],
+    warp_correct<NDIM, DIR, GH, uint32_t>(U, aux, G.ncell, cells_of, e.x, alpha, S, e.y, out, status, scratch[warp],
                                 GhostCells{G.gU, G.gaux, G.gfh});
     if (e.y)
 #pragma unroll
@@ -460,9 +485,9 @@ __global__ void __launch_bounds__(128) flux_wenoz_kernel(
   double alpha[NVAR], nal[NVAR];
   half_speeds<NDIM, DIR>(alpha_bits, alpha, nal);
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nifc; q += (int64_t)gridDim.x * blockDim.x) {
-    int64_t cells[6];
+    uint32_t cells[6];
     unsigned flips;
-    interface_cells<NDIM, DIR, GH>(q, G, cells, flips);
+    interface_cells<NDIM, DIR, GH>(static_cast<uint32_t>(q), G, cells, flips);
     double out[NVAR];
     unsigned fl[NVAR][2];
     interface_flux<NDIM, DIR, false, kFluxChar, GH>(U, aux, G.ncell, cells, flips, alpha, nal, S, out, fl, status,
@@ -629,6 +654,8 @@ Scheme make_scheme(double gamma, double H, double eps, int b_l, int b_u, int var
   S.eps_a = kTeno5ACr * 0.9 / (1.0 - 0.9 * kTeno5ACr) * kTeno5AXi * kTeno5AXi;
   S.gamma = gamma;
   S.gm1 = gamma - 1.0;
+  S.gm1_h = static_cast<float>(S.gm1);
+  S.gm1_l = static_cast<float>(S.gm1 - static_cast<double>(S.gm1_h));
   S.eps = eps;
   S.eps4 = 4.0 * eps;
   S.b_l = b_l;
