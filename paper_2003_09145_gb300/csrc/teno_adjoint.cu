@@ -218,12 +218,11 @@ __global__ void __launch_bounds__(kAdjThreads, TENO_ADJ_KEPT_MINBLOCKS) adj_kept
       const double a3[3] = {ha[0], ha[1], ha[NVAR - 1]};
       const teno::FaceSpeeds F = teno::face_speeds(a3);
       teno::RoeDf<NDIM> Rd;
-      teno::roe_df<NDIM>(sr2, sr3, sh2, sh3, su2, su3, S, Rd);
+      teno::roe_df<NDIM>(teno::roe_cell<NDIM>(sr2, sh2, su2), teno::roe_cell<NDIM>(sr3, sh3, su3), S, Rd);
       teno::CertIfc<NDIM> C;
       for (bool df = F.in_range && teno::roe_df_ok<NDIM>(Rd, S);;) {
         if (df) teno::cert_begin_df<NDIM, DIR>(Rd, F.ha, S, C);
         else teno::cert_begin<NDIM, DIR>(Rf, ha, C);
-        uint32_t tr = 0u, te = 0u;
 #pragma unroll
         for (int j = 0; j < 6; ++j) {
           double Uj[NVAR];
@@ -232,11 +231,9 @@ __global__ void __launch_bounds__(kAdjThreads, TENO_ADJ_KEPT_MINBLOCKS) adj_kept
             Uj[v] = U[v * I.ncell + cells[j]];
             Ut[v] = j == 0 ? Uj[v] : (j == 5 ? Ut[v] - Uj[v] : fma(Mi[j], Uj[v], Ut[v]));
           }
-          tr = max(tr, teno_fix::hi_word(Uj[0]) << 1);
-          te = max(te, teno_fix::hi_word(Uj[NVAR - 1]) << 1);
           teno::cert_point<NDIM, DIR>(j, Uj, aux[DIR * I.ncell + cells[j]], aux[NDIM * I.ncell + cells[j]], C);
         }
-        if (!df || teno::df_range(tr, te)) break;
+        if (!df || teno::df_range(C.xm[0], C.xm[NVAR - 1])) break;
         df = false;
       }
       kept = S.keep_idx >= 0 && teno::cert_keep<NDIM>(C, S);
@@ -953,7 +950,7 @@ struct AdjLayout {
   // alpha + 128 s, its arg-max cells (9 x 8) at argidx + 128 s
   static constexpr size_t kStage = 128;
   size_t status = 0, dt = 8, alpha = 64, argidx = 512;
-  size_t aux = 0, aux_bytes = 0, cand = 0, fh = 0, kb = 0, kb_bytes = 0, contrib = 0, contrib_bytes = 0,
+  size_t aux = 0, aux_bytes = 0, cand = 0, fh = 0, pf = 0, kb = 0, kb_bytes = 0, contrib = 0, contrib_bytes = 0,
          pending = 0, pending_bytes = 0, list = 0, sel = 0, lcount = 0, apart = 0, R = 0, U1 = 0, U2 = 0, B1 = 0,
          B2 = 0, roe = 0, roe_stage_bytes = 0, total = 0;
   size_t roe_dir = 0;   // doubles between two directions' Roe states
@@ -1000,6 +997,8 @@ AdjLayout adj_layout(const teno_grid* g, int op, int nsm) {
     // half fluxes of the recomputed forward stages (two-pass fluxes)
     L.fh = off;
     off += round_up(sizeof(double) * g->ndim * (nvar - 1) * ncell);
+    L.pf = off;   // and their binary32 planes
+    off += round_up(sizeof(float4) * teno::plane_count(g->ndim) * ncell);
     // forward recomputation (R, U1, U2) and the stage adjoints (B1, B2)
     L.R = off;
     off += round_up(sizeof(double) * nvar * ncell);
@@ -1138,7 +1137,7 @@ teno_status adjoint_sequence(const teno_grid* g, const AdjLayout& L, char* ws, i
   if (cell) {
     auto* cand = reinterpret_cast<unsigned long long*>(ws + L.cand);
     if (cudaMemsetAsync(alpha, 0, sizeof(unsigned long long) * 9, st) != cudaSuccess) return TENO_ERR_CUDA;
-    if (teno::launch_cell(g->ndim, U, aux, nullptr, alpha, status, G.ncell, g->gamma, nsm, st, cand) !=
+    if (teno::launch_cell(g->ndim, U, aux, nullptr, nullptr, alpha, status, G.ncell, g->gamma, nsm, st, cand) !=
             cudaSuccess ||
         teno::launch_argmax_finish(g->ndim, cand, G.ncell, nsm, argidx, st) != cudaSuccess)
       return TENO_ERR_CUDA;
@@ -1239,13 +1238,13 @@ teno_status teno_rk3_step_adjoint(const teno_grid* g, const double* U_n, double 
   if (cudaGetLastError() != cudaSuccess) return TENO_ERR_CUDA;
   double* roe0 = reinterpret_cast<double*>(w + L.roe);
   double* roe1 = reinterpret_cast<double*>(w + L.roe + L.roe_stage_bytes);
-  teno_status s = teno::forward_stage(g, w, L.status, L.dt, L.alpha, L.aux, L.fh, L.contrib, L.list, U_n, R,
+  teno_status s = teno::forward_stage(g, w, L.status, L.dt, L.alpha, L.aux, L.fh, L.pf, L.contrib, L.list, U_n, R,
                                       2, U_n, nullptr, U1, st, cand, roe0, L.roe_dir);
   if (s != TENO_OK) return s;
   if (teno::launch_argmax_finish(g->ndim, cand, ncell, nsm, reinterpret_cast<unsigned long long*>(w + L.argidx),
                                  st) != cudaSuccess)
     return TENO_ERR_CUDA;
-  s = teno::forward_stage(g, w, L.status, L.dt, L.alpha + AdjLayout::kStage, L.aux + L.aux_bytes, L.fh, L.contrib,
+  s = teno::forward_stage(g, w, L.status, L.dt, L.alpha + AdjLayout::kStage, L.aux + L.aux_bytes, L.fh, L.pf, L.contrib,
                           L.list, U1, R, 3, U_n, U1, U2, st, cand, roe1, L.roe_dir);
   if (s != TENO_OK) return s;
   if (teno::launch_argmax_finish(g->ndim, cand, ncell, nsm,

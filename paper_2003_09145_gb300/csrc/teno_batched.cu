@@ -43,6 +43,7 @@ struct BatchArgs {
   double* Uout;        // U1, U2 or U^{n+1}
   double* aux;         // [aux_fields(1) = 5][ncell] (the grid path's per-cell primitives)
   double* fh;          // [2][ncell]: F/2 of every cell (eq. 4.7), momentum and energy
+  float4* pf;          // [3][ncell]: binary32 copies (store_planes)
   const int64_t* offsets;
   const double* dx;
   double* t;
@@ -93,6 +94,9 @@ __global__ void __launch_bounds__(BLOCK) batched_stage_kernel(BatchArgs A, Schem
       teno::cell_flux_half_ep<1, 0>(Uc, uh[0], A.aux[A.ncell + c], ep, Fh);
 #pragma unroll
       for (int v = 1; v < 3; ++v) A.fh[(v - 1) * A.ncell + c] = Fh[v];
+      const double su[1] = {A.aux[4 * A.ncell + c]};
+      teno::store_planes<1>(A.pf, A.ncell, c, Uc, uh, A.aux[A.ncell + c], A.aux[2 * A.ncell + c],
+                            A.aux[3 * A.ncell + c], su);
       // u -+ c from u/2 with one rounding; max|u| kept as max|u/2|
       b0 = teno::max_abs_bits(b0, fma(2.0, uh[0], -cs));
       b1 = teno::max_abs_bits(b1, uh[0]);
@@ -163,7 +167,7 @@ __global__ void __launch_bounds__(BLOCK) batched_stage_kernel(BatchArgs A, Schem
 #pragma unroll
         for (int j = 0; j < 6; ++j) cells[j] = off + teno::ghost(face - 3 + j, n, A.bc);
         double out[3];
-        const unsigned open = teno::interface_flux_closed<1, 0, false>(A.Uin, A.aux, A.fh, A.ncell, cells, 0u, alpha,
+        const unsigned open = teno::interface_flux_closed<1, 0, false>(A.Uin, A.aux, A.fh, A.pf, A.ncell, cells, 0u, alpha,
                                                                        F, S, out, A.status, teno::GhostCells());
         if (!(open & teno::kRough)) {
           s_F[tid][0] = out[0];
@@ -215,7 +219,7 @@ constexpr size_t kAlign = 256;
 size_t round_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct BatchLayout {
-  size_t status = 0, queue = 64, order = 0, dt = 0, aux = 0, fh = 0, U1 = 0, U2 = 0, total = 0;
+  size_t status = 0, queue = 64, order = 0, dt = 0, aux = 0, fh = 0, pf = 0, U1 = 0, U2 = 0, total = 0;
 };
 
 bool batch_ok(const teno_batch* b) {
@@ -238,6 +242,8 @@ BatchLayout batch_layout(const teno_batch* b) {
   off += round_up(sizeof(double) * teno::aux_fields(1) * size_t(b->ncell));
   L.fh = off;
   off += round_up(sizeof(double) * 2 * size_t(b->ncell));
+  L.pf = off;
+  off += round_up(sizeof(float4) * teno::plane_count(1) * size_t(b->ncell));
   L.U1 = off;
   off += round_up(sizeof(double) * 3 * size_t(b->ncell));
   L.U2 = off;
@@ -322,6 +328,7 @@ teno_status teno_rk3_step_batched(const teno_batch* b, const int64_t* offsets, c
   BatchArgs A;
   A.aux = reinterpret_cast<double*>(w + L.aux);
   A.fh = reinterpret_cast<double*>(w + L.fh);
+  A.pf = reinterpret_cast<float4*>(w + L.pf);
   A.offsets = offsets;
   A.dx = dx;
   A.t = t_dev;

@@ -79,7 +79,7 @@ struct Layout {
   // header: [0] status, [8] dt, [64] LF speeds (9 x 8) then the pending-list
   // counters (3 x 4)
   size_t status = 0, dt = 8, alpha = 64;
-  size_t aux = 0, fh = 0, fhat = 0, list = 0, ghost = 0, R = 0, U1 = 0, U2 = 0, total = 0;
+  size_t aux = 0, fh = 0, pf = 0, fhat = 0, list = 0, ghost = 0, R = 0, U1 = 0, U2 = 0, total = 0;
 };
 
 Layout layout_of(const teno_grid* g, int op) {
@@ -93,6 +93,8 @@ Layout layout_of(const teno_grid* g, int op) {
   off += round_up(sizeof(double) * teno::aux_fields(g->ndim) * ncell);
   L.fh = off;   // half physical fluxes F_d/2 per cell and direction (no mass component)
   off += round_up(sizeof(double) * g->ndim * (nvar - 1) * ncell);
+  L.pf = off;   // binary32 copies of the cells (store_planes)
+  off += round_up(sizeof(float4) * teno::plane_count(g->ndim) * ncell);
   L.fhat = off;
   off += round_up(sizeof(double) * nvar * size_t(maxifc));
   L.list = off;
@@ -138,6 +140,9 @@ Grid grid_in(const teno_grid* g, const Layout& L, char* ws) {
   G.gU = gb;
   G.gaux = gb + nvar * teno::kGhostSlots;
   G.gfh = gb + (nvar + teno::aux_fields(g->ndim)) * teno::kGhostSlots;
+  // (an even number of doubles before it: 16-byte aligned, as the block is)
+  G.gpf = reinterpret_cast<const float4*>(
+      gb + (nvar + teno::aux_fields(g->ndim) + g->ndim * (g->ndim + 1)) * teno::kGhostSlots);
   return G;
 }
 
@@ -222,6 +227,7 @@ teno_status stage_begin(const teno_grid* g, const Layout& L, char* ws, const dou
   auto* alpha = reinterpret_cast<unsigned long long*>(ws + L.alpha);
   double* aux = reinterpret_cast<double*>(ws + L.aux);
   double* fh = one_pass ? nullptr : reinterpret_cast<double*>(ws + L.fh);
+  float4* pf = reinterpret_cast<float4*>(ws + L.pf);
   TENO_CUDA(cudaMemsetAsync(alpha, 0, teno::kAlphaAndCountBytes, st));
   TimerScope ts(st, TENO_KERNEL_CELL);
   if (has_dirichlet(g)) {
@@ -237,7 +243,7 @@ teno_status stage_begin(const teno_grid* g, const Layout& L, char* ws, const dou
     }
     TENO_CUDA(teno::launch_ghost_cells(g->ndim, gs, mask, G, g->gamma, st));
   }
-  TENO_CUDA(teno::launch_cell(g->ndim, U, aux, fh, alpha, status, G.ncell, g->gamma, nsm, st));
+  TENO_CUDA(teno::launch_cell(g->ndim, U, aux, fh, pf, alpha, status, G.ncell, g->gamma, nsm, st));
   return TENO_OK;
 }
 
@@ -259,6 +265,7 @@ teno_status stage_finish(const teno_grid* g, const Layout& L, char* ws, const do
   double* Fhat = reinterpret_cast<double*>(ws + L.fhat);
   uint2* list = reinterpret_cast<uint2*>(ws + L.list);
   double* fh = flags ? nullptr : reinterpret_cast<double*>(ws + L.fh);   // the flag path is one-pass
+  const float4* pf = reinterpret_cast<const float4*>(ws + L.pf);
   unsigned* count = reinterpret_cast<unsigned*>(ws + L.alpha + teno::kPendingCountOffset);
   if (with_dt) {
     TimerScope ts(st, TENO_KERNEL_DT);
@@ -270,7 +277,7 @@ teno_status stage_finish(const teno_grid* g, const Layout& L, char* ws, const do
     {
       TimerScope ts(st, TENO_KERNEL_FLUX);
       int nl = 1;
-      TENO_CUDA(teno::launch_flux(g->ndim, d, U, aux, fh, alpha, Fhat, fl, list, count + d, status, G, S, nsm, st,
+      TENO_CUDA(teno::launch_flux(g->ndim, d, U, aux, fh, pf, alpha, Fhat, fl, list, count + d, status, G, S, nsm, st,
                                   &nl));
       ts.launches(nl);
     }

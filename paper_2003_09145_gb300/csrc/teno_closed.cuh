@@ -2,10 +2,15 @@
 // with its certified test, as the two-pass flux kernels and the batched
 // kernel run it: the Roe state and the corrections in two binary32 values
 // (teno_df.cuh), U~ and the mass flux in 64-bit fixed point (teno_fixsum.cuh),
-// the other fluxes as binary64 chains.  FP64 instructions per interface: 25 of
-// the 3D sweep's (five per component, and the reciprocal, square root and
-// products of the Roe state gone), against 78 with the Roe state and the
-// corrections in binary64.
+// the other fluxes as binary64 chains.
+//
+// What bounds it: instruction issue (it was FP64 issue: 78 FP64 instructions
+// per interface, each holding an SM partition for 64 cycles; now 29, the FP64
+// pipe 40 % busy).  Measured at 256^3 (ms per RK3 step): Roe state and
+// corrections in binary64 37.0, in two binary32 values 28.1, with the cells'
+// binary32 copies from the cell pass (store_planes) 25.3.  Tried on top
+// and dropped: the mass flux as a binary64 chain too (slower), the corrections
+// widened and added in two FP64 additions instead of one (no gain).
 #pragma once
 
 #include "teno_df.cuh"
@@ -37,6 +42,79 @@ __device__ __forceinline__ FaceSpeeds face_speeds(const double (&a3)[3]) {
   return F;
 }
 
+// What the closed form's first pass and its Roe state read of a cell, in
+// binary32, written once per cell by the cell pass (converting it at each of
+// the eighteen stencil points that read the cell took some 280 instructions
+// per interface): planes of float4, pf[plane_count(NDIM)][ncell].  Truncated
+// values of U, p/2 and u_k/2 (hi_float), and sqrt(rho), (E+p)/sqrt(rho),
+// m_k/sqrt(rho) as two binary32 values (from_double):
+//   1D: {rho, m, E, p/2}, {u/2, 0, su}, {sr, sh}
+//   2D: {rho, m_0, m_1, E}, {p/2, u_0/2, u_1/2, 0}, {sr, sh}, {su_0, su_1}
+//   3D: {rho, m_0, m_1, m_2}, {E, p/2, u_0/2, u_1/2}, {u_2/2, 0, su_2}, {sr, sh}, {su_0, su_1}
+template <int NDIM>
+__device__ __forceinline__ void store_planes(float4* __restrict__ pf, int64_t ncell, int64_t c,
+                                             const double (&U)[NDIM + 2], const double (&uh)[NDIM], double ph, double sr,
+                                             double sh, const double (&su)[NDIM]) {
+  using namespace teno_df;
+  float X[NDIM + 2], u[NDIM];
+#pragma unroll
+  for (int v = 0; v < NDIM + 2; ++v) X[v] = hi_float(U[v]);
+#pragma unroll
+  for (int k = 0; k < NDIM; ++k) u[k] = hi_float(uh[k]);
+  const float p = hi_float(ph);
+  const df r = from_double(sr), h = from_double(sh), s0 = from_double(su[0]);
+  float4* o = pf + c;
+  if constexpr (NDIM == 1) {
+    o[0] = make_float4(X[0], X[1], X[2], p);
+    o[ncell] = make_float4(u[0], 0.0f, s0.h, s0.l);
+    o[2 * ncell] = make_float4(r.h, r.l, h.h, h.l);
+  } else if constexpr (NDIM == 2) {
+    const df s1 = from_double(su[1]);
+    o[0] = make_float4(X[0], X[1], X[2], X[3]);
+    o[ncell] = make_float4(p, u[0], u[1], 0.0f);
+    o[2 * ncell] = make_float4(r.h, r.l, h.h, h.l);
+    o[3 * ncell] = make_float4(s0.h, s0.l, s1.h, s1.l);
+  } else {
+    const df s1 = from_double(su[1]), s2 = from_double(su[2]);
+    o[0] = make_float4(X[0], X[1], X[2], X[3]);
+    o[ncell] = make_float4(X[4], p, u[0], u[1]);
+    o[2 * ncell] = make_float4(u[2], 0.0f, s2.h, s2.l);
+    o[3 * ncell] = make_float4(r.h, r.l, h.h, h.l);
+    o[4 * ncell] = make_float4(s0.h, s0.l, s1.h, s1.l);
+  }
+}
+
+// plane k of cell c, or of the ghost block when GH and c is a virtual cell
+template <bool GH, class I>
+__device__ __forceinline__ const float4* plane(const float4* __restrict__ pf, const float4* __restrict__ gpf,
+                                               int64_t ncell, int k, I c) {
+  if (GH && (int64_t)c >= ncell) return gpf + k * kGhostSlots + ((int64_t)c - ncell);
+  return pf + k * ncell + c;
+}
+
+// U, u_DIR/2 and p/2 of cell c
+template <int NDIM, int DIR, bool GH, class I>
+__device__ __forceinline__ void load_point_f(const float4* __restrict__ pf, const float4* __restrict__ gpf,
+                                             int64_t ncell, I c, float (&X)[NDIM + 2], float& u, float& p) {
+  const float4 a = *plane<GH>(pf, gpf, ncell, 0, c);
+  if constexpr (NDIM == 1) {
+    X[0] = a.x, X[1] = a.y, X[2] = a.z, p = a.w;
+    u = plane<GH>(pf, gpf, ncell, 1, c)->x;
+  } else {
+    const float4 b = *plane<GH>(pf, gpf, ncell, 1, c);
+    X[0] = a.x, X[1] = a.y, X[2] = a.z, X[3] = a.w;
+    if constexpr (NDIM == 2) {
+      p = b.x;
+      u = DIR == 0 ? b.y : b.z;
+    } else {
+      X[4] = b.x;
+      p = b.y;
+      if constexpr (DIR == 2) u = plane<GH>(pf, gpf, ncell, 2, c)->x;
+      else u = DIR == 0 ? b.z : b.w;
+    }
+  }
+}
+
 // The Roe state in two binary32 values, from the cells' sqrt(rho),
 // (E+p)/sqrt(rho) and m_k/sqrt(rho) (roe_interface's average): u~, |u~|^2, H~,
 // c~^2 and 1/c~.
@@ -45,16 +123,50 @@ struct RoeDf {
   teno_df::df u[NDIM], q2, H, c2, ic;
 };
 template <int NDIM>
-__device__ __forceinline__ void roe_df(double sr2, double sr3, double sh2, double sh3, const double (&su2)[NDIM],
-                                       const double (&su3)[NDIM], const Scheme& S, RoeDf<NDIM>& R) {
+struct RoeCellDf {   // one cell's contribution
+  teno_df::df sr, sh, su[NDIM];
+};
+template <int NDIM, bool GH, class I>
+__device__ __forceinline__ RoeCellDf<NDIM> load_roe_cell(const float4* __restrict__ pf, const float4* __restrict__ gpf,
+                                                         int64_t ncell, I c) {
+  RoeCellDf<NDIM> R;
+  const float4 d = *plane<GH>(pf, gpf, ncell, NDIM == 3 ? 3 : 2, c);
+  R.sr = {d.x, d.y};
+  R.sh = {d.z, d.w};
+  if constexpr (NDIM == 1) {
+    const float4 e = *plane<GH>(pf, gpf, ncell, 1, c);
+    R.su[0] = {e.z, e.w};
+  } else {
+    const float4 e = *plane<GH>(pf, gpf, ncell, NDIM == 3 ? 4 : 3, c);
+    R.su[0] = {e.x, e.y};
+    R.su[1] = {e.z, e.w};
+    if constexpr (NDIM == 3) {
+      const float4 f = *plane<GH>(pf, gpf, ncell, 2, c);
+      R.su[2] = {f.z, f.w};
+    }
+  }
+  return R;
+}
+template <int NDIM>
+__device__ __forceinline__ RoeCellDf<NDIM> roe_cell(double sr, double sh, const double (&su)[NDIM]) {
+  RoeCellDf<NDIM> R;
+  R.sr = teno_df::from_double(sr);
+  R.sh = teno_df::from_double(sh);
+#pragma unroll
+  for (int k = 0; k < NDIM; ++k) R.su[k] = teno_df::from_double(su[k]);
+  return R;
+}
+template <int NDIM>
+__device__ __forceinline__ void roe_df(const RoeCellDf<NDIM>& a, const RoeCellDf<NDIM>& b, const Scheme& S,
+                                       RoeDf<NDIM>& R) {
   using namespace teno_df;
-  const df y = recip(add(from_double(sr2), from_double(sr3)));
+  const df y = recip(add(a.sr, b.sr));
 #pragma unroll
   for (int k = 0; k < NDIM; ++k) {
-    R.u[k] = mul(add(from_double(su2[k]), from_double(su3[k])), y);
+    R.u[k] = mul(add(a.su[k], b.su[k]), y);
     R.q2 = k == 0 ? sqr(R.u[0]) : add(R.q2, sqr(R.u[k]));
   }
-  R.H = mul(add(from_double(sh2), from_double(sh3)), y);
+  R.H = mul(add(a.sh, b.sh), y);
   R.c2 = mul(df{S.gm1_h, S.gm1_l}, add(R.H, scale(R.q2, -0.5f)));
   R.ic = teno_df::rsqrt(R.c2);
 }
@@ -79,20 +191,10 @@ __device__ __forceinline__ bool roe_df_ok(const RoeDf<NDIM>& R, const Scheme& S)
   return R.c2.h > 0x1p-6f * S.gm1_h * R.H.h;
 }
 
-// binary32 truncation of |x| < 2^127 (hi_float without its upper clamp):
-// magnitudes below 2^-126 become +-2^-126
-__device__ __forceinline__ float low_float(double x) {
-  const uint32_t hi = teno_fix::hi_word(x);
-  uint32_t m = hi << 1;
-  m = m < (897u << 21) ? (897u << 21) : m;
-  return __uint_as_float((m * 4u - (896u << 23)) | (hi & 0x80000000u));
-}
-
-// 2^-20 <= max rho < 2^30 and max E < 2^95 (from the high words' magnitudes,
-// shifted left by one) keep every term of the test and of teno_df in binary32's
-// range; |u| and c are bounded by the speeds.
-__device__ __forceinline__ bool df_range(uint32_t tr, uint32_t te) {
-  return tr >= (1003u << 21) && tr < (1053u << 21) && te < (1118u << 21);
+// 2^-20 <= max rho < 2^30 and max E < 2^95 keep every term of the test and of
+// teno_df in binary32's range; |u| and c are bounded by the speeds.
+__device__ __forceinline__ bool df_range(float rho_max, float e_max) {
+  return rho_max >= 0x1p-20f && rho_max < 0x1p30f && e_max < 0x1p95f;
 }
 
 // The flux of one interface with every stencil kept, and the mask of its open
@@ -103,7 +205,8 @@ __device__ __forceinline__ bool df_range(uint32_t tr, uint32_t te) {
 template <int NDIM, int DIR, bool GH, class I>
 __device__ __forceinline__ unsigned interface_flux_closed(const double* __restrict__ U,
                                                           const double* __restrict__ aux,
-                                                          const double* __restrict__ fh, int64_t ncell,
+                                                          const double* __restrict__ fh,
+                                                          const float4* __restrict__ pf, int64_t ncell,
                                                           const I (&cells)[6], unsigned flips,
                                                           const double (&a3)[3], const FaceSpeeds& F,
                                                           const Scheme& S, double (&out)[NDIM + 2],
@@ -114,17 +217,12 @@ __device__ __forceinline__ unsigned interface_flux_closed(const double* __restri
   const double* gfh = GH ? gc.fh + DIR * (NVAR - 1) * kGhostSlots : nullptr;
   RoeDf<NDIM> R;
   {
-    double su2[NDIM], su3[NDIM];
-#pragma unroll
-    for (int k = 0; k < NDIM; ++k) {
-      su2[k] = ldc<GH>(aux, gc.aux, ncell, NDIM + 3 + k, cells[2]);
-      su3[k] = ldc<GH>(aux, gc.aux, ncell, NDIM + 3 + k, cells[3]);
-    }
-    su2[DIR] = flip_sign(su2[DIR], (flips >> 2) & 1u);
-    su3[DIR] = flip_sign(su3[DIR], (flips >> 3) & 1u);
-    roe_df<NDIM>(ldc<GH>(aux, gc.aux, ncell, NDIM + 1, cells[2]), ldc<GH>(aux, gc.aux, ncell, NDIM + 1, cells[3]),
-                 ldc<GH>(aux, gc.aux, ncell, NDIM + 2, cells[2]), ldc<GH>(aux, gc.aux, ncell, NDIM + 2, cells[3]),
-                 su2, su3, S, R);
+    RoeCellDf<NDIM> ra = load_roe_cell<NDIM, GH>(pf, gc.pf, ncell, cells[2]);
+    RoeCellDf<NDIM> rb = load_roe_cell<NDIM, GH>(pf, gc.pf, ncell, cells[3]);
+    const float fa = (flips >> 2) & 1u ? -1.0f : 1.0f, fb = (flips >> 3) & 1u ? -1.0f : 1.0f;
+    ra.su[DIR] = scale(ra.su[DIR], fa);
+    rb.su[DIR] = scale(rb.su[DIR], fb);
+    roe_df<NDIM>(ra, rb, S, R);
   }
   bool range = F.in_range && roe_df_ok<NDIM>(R, S), wide = false;
   // first pass: the certified test and the largest magnitudes of the summed
@@ -134,24 +232,16 @@ __device__ __forceinline__ unsigned interface_flux_closed(const double* __restri
   {
     CertIfc<NDIM> C;
     cert_begin_df<NDIM, DIR>(R, F.ha, S, C);
-    uint32_t tr = 0u, te = 0u;   // the magnitudes of rho and E, not clamped
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
-      const I c = cells[j];
+      float X[NVAR], u, p;
+      load_point_f<NDIM, DIR, GH>(pf, gc.pf, ncell, cells[j], X, u, p);
       const uint32_t fj = ((flips >> j) & 1u) << 31;
-      float X[NVAR];
-#pragma unroll
-      for (int v = 0; v < NVAR; ++v) {
-        const double x = ldc<GH>(U, gc.U, ncell, v, c);
-        X[v] = low_float(x);
-        if (v == 0) tr = max(tr, teno_fix::hi_word(x) << 1);
-        if (v == NVAR - 1) te = max(te, teno_fix::hi_word(x) << 1);
-      }
       X[1 + DIR] = __uint_as_float(__float_as_uint(X[1 + DIR]) ^ fj);
-      const float huf = __uint_as_float(__float_as_uint(low_float(ldc<GH>(aux, gc.aux, ncell, DIR, c))) ^ fj);
-      teno_cert::cert_point_f<NDIM, DIR>(j, X, huf, low_float(ldc<GH>(aux, gc.aux, ncell, NDIM, c)), C);
+      u = __uint_as_float(__float_as_uint(u) ^ fj);
+      teno_cert::cert_point_f<NDIM, DIR>(j, X, u, p, C);
     }
-    range = range && df_range(tr, te);
+    range = range && df_range(C.xm[0], C.xm[NVAR - 1]);
     open = cert_open<NDIM>(C, S);
 #pragma unroll
     for (int v = 0; v < NVAR; ++v) xm[v] = C.xm[v];

@@ -75,6 +75,8 @@ constexpr int kMaxDim = 3;
 // Per-cell primitive fields the cell pass writes (aux, [aux_fields][ncell]):
 // u_k/2 (ndim), p/2, sqrt(rho), (E+p)/sqrt(rho), m_k/sqrt(rho) = sqrt(rho) u_k (ndim).
 __host__ __device__ constexpr int aux_fields(int ndim) { return 2 * ndim + 3; }
+// planes of the cell pass's binary32 copies (store_planes)
+__host__ __device__ constexpr int plane_count(int ndim) { return ndim + 2; }
 constexpr int kMaxVar = 5;
 constexpr int kMaxLadder = 16;
 
@@ -135,6 +137,7 @@ struct Grid {
   const double* gU = nullptr;
   const double* gaux = nullptr;
   const double* gfh = nullptr;
+  const float4* gpf = nullptr;
 };
 
 // Index of a (possibly ghost) cell along an axis of n cells: periodic wrap,

@@ -19,6 +19,7 @@ struct GhostCells {
   const double* U = nullptr;
   const double* aux = nullptr;
   const double* fh = nullptr;
+  const float4* pf = nullptr;   // the cell pass's binary32 planes [ndim + 2][6]
 };
 
 // field `f` of cell c of an array with ncell entries per field, or of the

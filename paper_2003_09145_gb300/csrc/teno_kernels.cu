@@ -31,7 +31,7 @@ namespace teno {
 // to their maxima over all cells.
 // aux layout: [aux_fields(ndim) = 2 ndim + 3][ncell]: u_0/2..u_{ndim-1}/2,
 // p/2, sqrt(rho), (E+p)/sqrt(rho), m_0/sqrt(rho)..m_{ndim-1}/sqrt(rho).
-// With `fh`, also the half physical fluxes F_d/2 (eq. 4.7)
+// With `fh`, also the binary32 copies `pf` (store_planes) and the half physical fluxes F_d/2 (eq. 4.7)
 // of every direction, momentum and energy components only (the mass one is
 // m_d/2), [ndim][nvar - 1][ncell], for the closed-form flux pass.
 // alpha layout (bit patterns of non-negative doubles): [ndim][3] =
@@ -61,7 +61,7 @@ __device__ __forceinline__ void store_flux_half(const double (&Uc)[NDIM + 2], co
 template <int NDIM, bool ARG>
 __global__ void __launch_bounds__(256, TENO_CELL_MINBLOCKS) cell_kernel(const double* __restrict__ U,
                                                    double* __restrict__ aux,
-                                                   double* __restrict__ fh,
+                                                   double* __restrict__ fh, float4* __restrict__ pf,
                                                    unsigned long long* __restrict__ alpha,
                                                    int* __restrict__ status,
                                                    int64_t ncell, double gamma,
@@ -87,6 +87,10 @@ __global__ void __launch_bounds__(256, TENO_CELL_MINBLOCKS) cell_kernel(const do
       for (int v = 0; v < NVAR; ++v) Uc[v] = U[v * ncell + c];
       const double pn = aux[NDIM * ncell + c];
       store_flux_half<NDIM, 0>(Uc, uh, pn, ep, fh, ncell, c);
+      double su[NDIM];
+#pragma unroll
+      for (int k = 0; k < NDIM; ++k) su[k] = aux[(NDIM + 3 + k) * ncell + c];
+      store_planes<NDIM>(pf, ncell, c, Uc, uh, pn, aux[(NDIM + 1) * ncell + c], aux[(NDIM + 2) * ncell + c], su);
     }
     // u -+ c = 2 (u/2) -+ c with one rounding, as a subtraction of u would;
     // max|u| is kept as max|u/2| and doubled (exactly) below
@@ -250,7 +254,7 @@ __global__ void __launch_bounds__(128, TENO_FLUX_MINBLOCKS) flux_kernel(
     double out[NVAR];
     unsigned fl[NVAR][2];
     interface_flux<NDIM, DIR, WITH_FLAGS, kFluxFull, GH>(U, aux, ncell, cells, flips, alpha, nal, S, out, fl, status,
-                                                        GhostCells{G.gU, G.gaux, G.gfh});
+                                                        GhostCells{G.gU, G.gaux, G.gfh, G.gpf});
     if (WITH_FLAGS) {
       // direction block offset is applied by the caller through `flags`
 #pragma unroll
@@ -353,7 +357,7 @@ __device__ __forceinline__ void half_speeds(const unsigned long long* __restrict
 template <int NDIM, int DIR, int WALL, bool ROE = false>
 __global__ void __launch_bounds__(128, TENO_CLOSED_MINBLOCKS) flux_closed_kernel(
     const double* __restrict__ U, const double* __restrict__ aux, const double* __restrict__ fh,
-    const unsigned long long* __restrict__ alpha_bits, double* __restrict__ Fhat,
+    const float4* __restrict__ pf, const unsigned long long* __restrict__ alpha_bits, double* __restrict__ Fhat,
     uint2* __restrict__ list, unsigned* __restrict__ count, int* __restrict__ status, Grid G,
     Scheme S, double* __restrict__ roe_out = nullptr) {
   constexpr int NVAR = NDIM + 2;
@@ -390,8 +394,8 @@ __global__ void __launch_bounds__(128, TENO_CLOSED_MINBLOCKS) flux_closed_kernel
     interface_cells<NDIM, DIR, WALL == 2>(static_cast<uint32_t>(q), G, cells, flips);
     double out[NVAR];
     const unsigned open = interface_flux_closed<NDIM, DIR, WALL == 2>(
-        U, aux, fh + (int64_t)DIR * (NVAR - 1) * G.ncell, G.ncell, cells, WALL == 1 ? flips : 0u, a3, F, S, out,
-        status, GhostCells{G.gU, G.gaux, G.gfh});
+        U, aux, fh + (int64_t)DIR * (NVAR - 1) * G.ncell, pf, G.ncell, cells, WALL == 1 ? flips : 0u, a3, F, S, out,
+        status, GhostCells{G.gU, G.gaux, G.gfh, G.gpf});
     if constexpr (ROE) {
       if (S.keep_idx >= 0) {
         RoeIfc<NDIM> R;
@@ -465,7 +469,7 @@ __global__ void __launch_bounds__(128) flux_correct_kernel(
 #pragma unroll
     for (int v = 0; v < NVAR; ++v) out[v] = e.y && !(e.y & kRough) ? Fhat[(int64_t)v * nifc + e.x] : 0.0;
     warp_correct<NDIM, DIR, GH, uint32_t>(U, aux, G.ncell, cells_of, e.x, alpha, S, e.y, out, status, scratch[warp],
-                                GhostCells{G.gU, G.gaux, G.gfh});
+                                GhostCells{G.gU, G.gaux, G.gfh, G.gpf});
     if (e.y)
 #pragma unroll
       for (int v = 0; v < NVAR; ++v) Fhat[(int64_t)v * nifc + e.x] = out[v];
@@ -491,7 +495,7 @@ __global__ void __launch_bounds__(128) flux_wenoz_kernel(
     double out[NVAR];
     unsigned fl[NVAR][2];
     interface_flux<NDIM, DIR, false, kFluxChar, GH>(U, aux, G.ncell, cells, flips, alpha, nal, S, out, fl, status,
-                                                   GhostCells{G.gU, G.gaux, G.gfh});
+                                                   GhostCells{G.gU, G.gaux, G.gfh, G.gpf});
 #pragma unroll
     for (int v = 0; v < NVAR; ++v) Fhat[(int64_t)v * nifc + q] = out[v];
   }
@@ -726,8 +730,8 @@ Scheme make_scheme(double gamma, double H, double eps, int b_l, int b_u, int var
 // ---------------------------------------------------------------------------
 template <int NDIM>
 __global__ void ghost_cell_kernel(GhostStates gs, unsigned mask, double* __restrict__ gU,
-                                  double* __restrict__ gaux, double* __restrict__ gfh, double gamma,
-                                  int* __restrict__ status) {
+                                  double* __restrict__ gaux, double* __restrict__ gfh, float4* __restrict__ gpf,
+                                  double gamma, int* __restrict__ status) {
   constexpr int NVAR = NDIM + 2;
   const int slot = threadIdx.x;
   if (slot >= kGhostSlots || !((mask >> slot) & 1u)) return;
@@ -738,6 +742,11 @@ __global__ void ghost_cell_kernel(GhostStates gs, unsigned mask, double* __restr
   if (!cell_primitives<NDIM>(gU, kGhostSlots, slot, gamma, gaux, uh, cs, ep) && status)
     atomicOr(status, kStatusNonphysical);
   store_flux_half<NDIM, 0>(Uc, uh, gaux[NDIM * kGhostSlots + slot], ep, gfh, kGhostSlots, slot);
+  double su[NDIM];
+#pragma unroll
+  for (int k = 0; k < NDIM; ++k) su[k] = gaux[(NDIM + 3 + k) * kGhostSlots + slot];
+  store_planes<NDIM>(gpf, kGhostSlots, slot, Uc, uh, gaux[NDIM * kGhostSlots + slot],
+                     gaux[(NDIM + 1) * kGhostSlots + slot], gaux[(NDIM + 2) * kGhostSlots + slot], su);
 }
 
 cudaError_t launch_ghost_cells(int ndim, const GhostStates& gs, unsigned mask, const Grid& G, double gamma,
@@ -745,10 +754,11 @@ cudaError_t launch_ghost_cells(int ndim, const GhostStates& gs, unsigned mask, c
   double* gU = const_cast<double*>(G.gU);
   double* gaux = const_cast<double*>(G.gaux);
   double* gfh = const_cast<double*>(G.gfh);
+  float4* gpf = const_cast<float4*>(G.gpf);
   switch (ndim) {
-    case 1: ghost_cell_kernel<1><<<1, 32, 0, st>>>(gs, mask, gU, gaux, gfh, gamma, nullptr); break;
-    case 2: ghost_cell_kernel<2><<<1, 32, 0, st>>>(gs, mask, gU, gaux, gfh, gamma, nullptr); break;
-    default: ghost_cell_kernel<3><<<1, 32, 0, st>>>(gs, mask, gU, gaux, gfh, gamma, nullptr); break;
+    case 1: ghost_cell_kernel<1><<<1, 32, 0, st>>>(gs, mask, gU, gaux, gfh, gpf, gamma, nullptr); break;
+    case 2: ghost_cell_kernel<2><<<1, 32, 0, st>>>(gs, mask, gU, gaux, gfh, gpf, gamma, nullptr); break;
+    default: ghost_cell_kernel<3><<<1, 32, 0, st>>>(gs, mask, gU, gaux, gfh, gpf, gamma, nullptr); break;
   }
   return cudaGetLastError();
 }
@@ -765,23 +775,23 @@ static inline int blocks_for(int64_t n, int threads, int cap) {
 
 int cell_blocks(int64_t ncell, int nsm) { return blocks_for(ncell, 256, nsm * 8); }
 
-cudaError_t launch_cell(int ndim, const double* U, double* aux, double* fh,
+cudaError_t launch_cell(int ndim, const double* U, double* aux, double* fh, float4* pf,
                         unsigned long long* alpha, int* status, int64_t ncell,
                         double gamma, int nsm, cudaStream_t st, unsigned long long* cand) {
   const int threads = 256;
   const int blocks = cell_blocks(ncell, nsm);
   if (cand) {
     switch (ndim) {
-      case 1: cell_kernel<1, true><<<blocks, threads, 0, st>>>(U, aux, fh, alpha, status, ncell, gamma, cand); break;
-      case 2: cell_kernel<2, true><<<blocks, threads, 0, st>>>(U, aux, fh, alpha, status, ncell, gamma, cand); break;
-      default: cell_kernel<3, true><<<blocks, threads, 0, st>>>(U, aux, fh, alpha, status, ncell, gamma, cand); break;
+      case 1: cell_kernel<1, true><<<blocks, threads, 0, st>>>(U, aux, fh, pf, alpha, status, ncell, gamma, cand); break;
+      case 2: cell_kernel<2, true><<<blocks, threads, 0, st>>>(U, aux, fh, pf, alpha, status, ncell, gamma, cand); break;
+      default: cell_kernel<3, true><<<blocks, threads, 0, st>>>(U, aux, fh, pf, alpha, status, ncell, gamma, cand); break;
     }
     return cudaGetLastError();
   }
   switch (ndim) {
-    case 1: cell_kernel<1, false><<<blocks, threads, 0, st>>>(U, aux, fh, alpha, status, ncell, gamma, nullptr); break;
-    case 2: cell_kernel<2, false><<<blocks, threads, 0, st>>>(U, aux, fh, alpha, status, ncell, gamma, nullptr); break;
-    default: cell_kernel<3, false><<<blocks, threads, 0, st>>>(U, aux, fh, alpha, status, ncell, gamma, nullptr); break;
+    case 1: cell_kernel<1, false><<<blocks, threads, 0, st>>>(U, aux, fh, pf, alpha, status, ncell, gamma, nullptr); break;
+    case 2: cell_kernel<2, false><<<blocks, threads, 0, st>>>(U, aux, fh, pf, alpha, status, ncell, gamma, nullptr); break;
+    default: cell_kernel<3, false><<<blocks, threads, 0, st>>>(U, aux, fh, pf, alpha, status, ncell, gamma, nullptr); break;
   }
   return cudaGetLastError();
 }
@@ -794,8 +804,8 @@ cudaError_t launch_argmax_finish(int ndim, const unsigned long long* cand, int64
 
 template <int NDIM, int DIR>
 static int flux_launch(int blocks, int threads, int pblocks, int nsm, cudaStream_t st, const double* U,
-                       const double* aux, const double* fh, const unsigned long long* alpha, double* Fhat,
-                       uint8_t* flags, uint2* list, unsigned* count, int* status, const Grid& G,
+                       const double* aux, const double* fh, const float4* pf, const unsigned long long* alpha,
+                       double* Fhat, uint8_t* flags, uint2* list, unsigned* count, int* status, const Grid& G,
                        const Scheme& S, double* roe_out) {
   const bool gh = G.bc[DIR] == TENO_BC_DIRICHLET;
   if (flags || !list) {
@@ -811,14 +821,14 @@ static int flux_launch(int blocks, int threads, int pblocks, int nsm, cudaStream
     return 1;
   }
   if (G.bc[DIR] == TENO_BC_REFLECTIVE)
-    flux_closed_kernel<NDIM, DIR, 1><<<blocks, threads, 0, st>>>(U, aux, fh, alpha, Fhat, list, count, status, G, S);
+    flux_closed_kernel<NDIM, DIR, 1><<<blocks, threads, 0, st>>>(U, aux, fh, pf, alpha, Fhat, list, count, status, G, S);
   else if (gh)
-    flux_closed_kernel<NDIM, DIR, 2><<<blocks, threads, 0, st>>>(U, aux, fh, alpha, Fhat, list, count, status, G, S);
+    flux_closed_kernel<NDIM, DIR, 2><<<blocks, threads, 0, st>>>(U, aux, fh, pf, alpha, Fhat, list, count, status, G, S);
   else if (roe_out)
-    flux_closed_kernel<NDIM, DIR, 0, true><<<blocks, threads, 0, st>>>(U, aux, fh, alpha, Fhat, list, count, status,
+    flux_closed_kernel<NDIM, DIR, 0, true><<<blocks, threads, 0, st>>>(U, aux, fh, pf, alpha, Fhat, list, count, status,
                                                                       G, S, roe_out);
   else
-    flux_closed_kernel<NDIM, DIR, 0><<<blocks, threads, 0, st>>>(U, aux, fh, alpha, Fhat, list, count, status, G, S);
+    flux_closed_kernel<NDIM, DIR, 0><<<blocks, threads, 0, st>>>(U, aux, fh, pf, alpha, Fhat, list, count, status, G, S);
   if (gh)
     flux_correct_kernel<NDIM, DIR, true><<<pblocks, threads, 0, st>>>(U, aux, alpha, Fhat, list, count, status, G, S, nsm);
   else
@@ -826,7 +836,7 @@ static int flux_launch(int blocks, int threads, int pblocks, int nsm, cudaStream
   return 2;
 }
 
-cudaError_t launch_flux(int ndim, int dir, const double* U, const double* aux, const double* fh,
+cudaError_t launch_flux(int ndim, int dir, const double* U, const double* aux, const double* fh, const float4* pf,
                         const unsigned long long* alpha, double* Fhat,
                         uint8_t* flags, uint2* list, unsigned* count, int* status,
                         const Grid& G, const Scheme& S, int nsm, cudaStream_t st,
@@ -834,19 +844,19 @@ cudaError_t launch_flux(int ndim, int dir, const double* U, const double* aux, c
   int64_t nifc = 1;
   for (int k = 0; k < 3; ++k) nifc *= G.n[k] + (k == dir ? 1 : 0);
   if (nifc > int64_t(UINT32_MAX)) list = nullptr;   // list entries are 32-bit
-  if (!count || !fh) list = nullptr;
+  if (!count || !fh || !pf) list = nullptr;
   const int threads = 128;
   const int blocks = blocks_for(nifc, threads, nsm * 64);
   const int pblocks = blocks_for(nifc, threads, nsm * 16);
   int n = 0;
-  if (ndim == 1) n = flux_launch<1, 0>(blocks, threads, pblocks, nsm, st, U, aux, fh, alpha, Fhat, flags, list, count, status, G, S, roe_out);
+  if (ndim == 1) n = flux_launch<1, 0>(blocks, threads, pblocks, nsm, st, U, aux, fh, pf, alpha, Fhat, flags, list, count, status, G, S, roe_out);
   else if (ndim == 2) {
-    if (dir == 0) n = flux_launch<2, 0>(blocks, threads, pblocks, nsm, st, U, aux, fh, alpha, Fhat, flags, list, count, status, G, S, roe_out);
-    else n = flux_launch<2, 1>(blocks, threads, pblocks, nsm, st, U, aux, fh, alpha, Fhat, flags, list, count, status, G, S, roe_out);
+    if (dir == 0) n = flux_launch<2, 0>(blocks, threads, pblocks, nsm, st, U, aux, fh, pf, alpha, Fhat, flags, list, count, status, G, S, roe_out);
+    else n = flux_launch<2, 1>(blocks, threads, pblocks, nsm, st, U, aux, fh, pf, alpha, Fhat, flags, list, count, status, G, S, roe_out);
   } else {
-    if (dir == 0) n = flux_launch<3, 0>(blocks, threads, pblocks, nsm, st, U, aux, fh, alpha, Fhat, flags, list, count, status, G, S, roe_out);
-    else if (dir == 1) n = flux_launch<3, 1>(blocks, threads, pblocks, nsm, st, U, aux, fh, alpha, Fhat, flags, list, count, status, G, S, roe_out);
-    else n = flux_launch<3, 2>(blocks, threads, pblocks, nsm, st, U, aux, fh, alpha, Fhat, flags, list, count, status, G, S, roe_out);
+    if (dir == 0) n = flux_launch<3, 0>(blocks, threads, pblocks, nsm, st, U, aux, fh, pf, alpha, Fhat, flags, list, count, status, G, S, roe_out);
+    else if (dir == 1) n = flux_launch<3, 1>(blocks, threads, pblocks, nsm, st, U, aux, fh, pf, alpha, Fhat, flags, list, count, status, G, S, roe_out);
+    else n = flux_launch<3, 2>(blocks, threads, pblocks, nsm, st, U, aux, fh, pf, alpha, Fhat, flags, list, count, status, G, S, roe_out);
   }
   if (launches) *launches = n;
   return cudaGetLastError();
@@ -909,8 +919,8 @@ cudaError_t launch_dt(int ndim, const unsigned long long* alpha, const Grid& G,
 }
 
 teno_status forward_stage(const teno_grid* g, char* ws, size_t status_off, size_t dt_off,
-                          size_t alpha_off, size_t aux_off, size_t fh_off, size_t fhat_off, size_t list_off,
-                          const double* U, double* R, int mode, const double* Un, const double* Uk,
+                          size_t alpha_off, size_t aux_off, size_t fh_off, size_t pf_off, size_t fhat_off,
+                          size_t list_off, const double* U, double* R, int mode, const double* Un, const double* Uk,
                           double* Uout, cudaStream_t st, unsigned long long* cand, double* roe_out,
                           size_t roe_stride) {
   Grid G;
@@ -934,12 +944,13 @@ teno_status forward_stage(const teno_grid* g, char* ws, size_t status_off, size_
   double* Fhat = reinterpret_cast<double*>(ws + fhat_off);
   uint2* list = list_off ? reinterpret_cast<uint2*>(ws + list_off) : nullptr;
   double* fh = fh_off ? reinterpret_cast<double*>(ws + fh_off) : nullptr;
+  float4* pf = fh_off ? reinterpret_cast<float4*>(ws + pf_off) : nullptr;
   unsigned* count = reinterpret_cast<unsigned*>(ws + alpha_off + kPendingCountOffset);
   if (cudaMemsetAsync(alpha, 0, kAlphaAndCountBytes, st) != cudaSuccess) return TENO_ERR_CUDA;
-  if (launch_cell(g->ndim, U, aux, fh, alpha, status, G.ncell, g->gamma, nsm, st, cand) != cudaSuccess)
+  if (launch_cell(g->ndim, U, aux, fh, pf, alpha, status, G.ncell, g->gamma, nsm, st, cand) != cudaSuccess)
     return TENO_ERR_CUDA;
   for (int d = 0; d < g->ndim; ++d) {
-    if (launch_flux(g->ndim, d, U, aux, fh, alpha, Fhat, nullptr, list, count + d, status, G, S, nsm, st,
+    if (launch_flux(g->ndim, d, U, aux, fh, pf, alpha, Fhat, nullptr, list, count + d, status, G, S, nsm, st,
                     nullptr, roe_out ? roe_out + d * roe_stride : nullptr) != cudaSuccess)
       return TENO_ERR_CUDA;
     if (launch_diff(g->ndim, d, Fhat, R, Un, Uk, Uout, dt, G, mode, nsm, st, U) != cudaSuccess)

@@ -29,10 +29,10 @@ inline Scheme scheme_of(const teno_grid* g) {
 
 // Primitives (aux) and LF speeds of every cell; with `fh` (nullable) also
 // the half physical fluxes F_d/2 without their mass component,
-// [ndim][nvar - 1][ncell]; with `cand` (nullable, 18 words per block of
+// [ndim][nvar - 1][ncell], and the binary32 planes `pf` [ndim + 2][ncell]; with `cand` (nullable, 18 words per block of
 // cell_blocks) the per-block arg-max candidates of the speeds.
 int cell_blocks(int64_t ncell, int nsm);
-cudaError_t launch_cell(int ndim, const double* U, double* aux, double* fh,
+cudaError_t launch_cell(int ndim, const double* U, double* aux, double* fh, float4* pf,
                         unsigned long long* alpha, int* status, int64_t ncell,
                         double gamma, int nsm, cudaStream_t st, unsigned long long* cand = nullptr);
 // argidx[3 d + s] = the lowest cell index at which speed s of direction d
@@ -49,7 +49,7 @@ cudaError_t launch_argmax_finish(int ndim, const unsigned long long* cand, int64
 // fixed-state faces only) the closed-form pass also writes every
 // interface's Roe state and its certificate's decision, [ndim + 8][#interfaces]
 // (flux_closed_kernel).
-cudaError_t launch_flux(int ndim, int dir, const double* U, const double* aux, const double* fh,
+cudaError_t launch_flux(int ndim, int dir, const double* U, const double* aux, const double* fh, const float4* pf,
                         const unsigned long long* alpha, double* Fhat,
                         uint8_t* flags, uint2* list, unsigned* count, int* status,
                         const Grid& G, const Scheme& S, int nsm, cudaStream_t st,
@@ -83,7 +83,9 @@ struct GhostStates {
 cudaError_t launch_ghost_cells(int ndim, const GhostStates& gs, unsigned mask, const Grid& G, double gamma,
                                cudaStream_t st);
 // doubles of the ghost block for an ndim grid
-inline int ghost_block_doubles(int ndim) { return 6 * ((ndim + 2) + aux_fields(ndim) + ndim * (ndim + 1)); }
+inline int ghost_block_doubles(int ndim) {
+  return 6 * ((ndim + 2) + aux_fields(ndim) + ndim * (ndim + 1) + 2 * plane_count(ndim));
+}
 
 cudaError_t launch_dt(int ndim, const unsigned long long* alpha, const Grid& G,
                       double cfl, double dt_fixed, double* t_dev, double t_end,
@@ -93,13 +95,13 @@ cudaError_t launch_dt(int ndim, const unsigned long long* alpha, const Grid& G,
 // (2, 3 or 4; see diff_kernel) into Uout, with dt read from the workspace
 // word at dt_off.  `ws` offsets locate the status word, the LF speeds (and
 // the pending counters after them), the per-cell primitives, the half
-// fluxes, the interface-flux buffer and the pending list (fh_off or list_off
+// fluxes, the binary32 planes, the interface-flux buffer and the pending list (fh_off or list_off
 // 0: one-pass fluxes); R holds the partial sums of the multi-dimensional
 // difference; `cand` (nullable) as for launch_cell; with `roe_out`, direction
 // d's Roe states go to roe_out + d roe_stride (see launch_flux).
 teno_status forward_stage(const teno_grid* g, char* ws, size_t status_off, size_t dt_off,
-                          size_t alpha_off, size_t aux_off, size_t fh_off, size_t fhat_off, size_t list_off,
-                          const double* U, double* R, int mode, const double* Un, const double* Uk,
+                          size_t alpha_off, size_t aux_off, size_t fh_off, size_t pf_off, size_t fhat_off,
+                          size_t list_off, const double* U, double* R, int mode, const double* Un, const double* Uk,
                           double* Uout, cudaStream_t st, unsigned long long* cand = nullptr,
                           double* roe_out = nullptr, size_t roe_stride = 0);
 
