@@ -143,6 +143,48 @@ TENO_CERT_HD bool certify_keep(float v0, float v1, float v2, float v3, float v4,
   return (dtau <= 1.0e38f) && (fadd(tau, dtau) <= fmul(thr_f, fmul(fsub(dmin, ddmin), 1.0f - 1e-5f)));
 }
 
+// certify_keep of two reconstructions at once (x and y: the same operations
+// in the same order, so the same outcomes), with two operations per
+// instruction where the hardware pairs them: bit 0 set where x is not proven
+// kept, bit 1 where y is not.
+#ifdef __CUDACC__
+__device__ __forceinline__ unsigned certify_open2(float2 v0, float2 v1, float2 v2, float2 v3, float2 v4, float2 d,
+                                                  float thr_f, float eps4_f) {
+  const float u = 0x1p-24f, k = 13.0f / 3.0f;
+  const float2 m1 = make_float2(-1.0f, -1.0f), two = make_float2(2.0f, 2.0f), kk = make_float2(k, k);
+  const float2 p3 = make_float2(3.0f, 3.0f), n3 = make_float2(-3.0f, -3.0f);
+  // x - y is exact as fma(y, -1, x)
+  const float2 e0 = __ffma2_rn(v0, m1, v1), e1 = __ffma2_rn(v1, m1, v2), e2 = __ffma2_rn(v2, m1, v3),
+               e3 = __ffma2_rn(v3, m1, v4);
+  const float2 a0 = __ffma2_rn(e0, m1, e1), a1 = __ffma2_rn(e1, m1, e2), a2 = __ffma2_rn(e2, m1, e3);
+  const float2 ne0 = make_float2(-e0.x, -e0.y);
+  const float2 c0 = __ffma2_rn(p3, e1, ne0), c1 = __fadd2_rn(e1, e2), c2 = __ffma2_rn(n3, e2, e3);
+  const float2 b0 = __ffma2_rn(__fmul2_rn(kk, a0), a0, __fmul2_rn(c0, c0));
+  const float2 b1 = __ffma2_rn(__fmul2_rn(kk, a1), a1, __fmul2_rn(c1, c1));
+  const float2 b2 = __ffma2_rn(__fmul2_rn(kk, a2), a2, __fmul2_rn(c2, c2));
+  const float2 da = __fmul2_rn(d, make_float2(4.0f, 4.0f)), dc = __fmul2_rn(d, make_float2(8.0f, 8.0f));
+  const float2 am = make_float2(fmaxf(fabsf(a0.x), fmaxf(fabsf(a1.x), fabsf(a2.x))),
+                                fmaxf(fabsf(a0.y), fmaxf(fabsf(a1.y), fabsf(a2.y))));
+  const float2 cm = make_float2(fmaxf(fabsf(c0.x), fmaxf(fabsf(c1.x), fabsf(c2.x))),
+                                fmaxf(fabsf(c0.y), fmaxf(fabsf(c1.y), fabsf(c2.y))));
+  const float2 bm = make_float2(fmaxf(b0.x, fmaxf(b1.x, b2.x)), fmaxf(b0.y, fmaxf(b1.y, b2.y)));
+  const float2 bn = make_float2(fminf(b0.x, fminf(b1.x, b2.x)), fminf(b0.y, fminf(b1.y, b2.y)));
+  const float2 db = __ffma2_rn(make_float2(4.0f * u, 4.0f * u), bm,
+                               __ffma2_rn(__fmul2_rn(kk, __ffma2_rn(two, am, da)), da,
+                                          __fmul2_rn(__ffma2_rn(two, cm, dc), dc)));
+  const float2 df = __ffma2_rn(b0, m1, b2);
+  const float2 tau = make_float2(fabsf(df.x), fabsf(df.y));
+  const float2 dtau = __ffma2_rn(make_float2(u, u), tau, __fadd2_rn(db, db));
+  const float2 dmin = __fadd2_rn(bn, make_float2(eps4_f, eps4_f));
+  const float2 ddmin = __ffma2_rn(make_float2(4.0f * u, 4.0f * u), dmin, db);
+  const float2 lhs = __fadd2_rn(tau, dtau);
+  const float2 rhs = __fmul2_rn(make_float2(thr_f, thr_f),
+                                __fmul2_rn(__ffma2_rn(ddmin, m1, dmin), make_float2(1.0f - 1e-5f, 1.0f - 1e-5f)));
+  const bool kx = dtau.x <= 1.0e38f && lhs.x <= rhs.x, ky = dtau.y <= 1.0e38f && lhs.y <= rhs.y;
+  return (kx ? 0u : 1u) | (ky ? 0u : 2u);
+}
+#endif
+
 // The same test on five binary64 values (one scalar reconstruction),
 // truncated by hi_float: |g_j - v_j| <= 2^-20 |v_j| + 2^-126 and
 // |v_j| <= |g_j| (1 + 2^-19), so r + 2uW <= 0x1.2p-20 W + 2^-126 (plus
@@ -406,12 +448,20 @@ TENO_CERT_HD unsigned cert_open(const CertIfc<NDIM>& C, float thr_f, float eps4_
     const float ta = (f == 0 || f == NVAR - 1) ? fadd(aza, bza) : (f == 1) ? 2.0f * aza : 0.0f;
     const float mp = ffma(fadd(C.hum, C.haf[f]), wa[f], ta);
     const float mm = ffma(2.0f * C.haf[f], wa[f], mp);
+#ifdef __CUDA_ARCH__
+    open |= certify_open2(make_float2(C.vp32[0][f], C.vm32[5][f]), make_float2(C.vp32[1][f], C.vm32[4][f]),
+                          make_float2(C.vp32[2][f], C.vm32[3][f]), make_float2(C.vp32[3][f], C.vm32[2][f]),
+                          make_float2(C.vp32[4][f], C.vm32[1][f]),
+                          make_float2(ffma(kd, mp, 0x1p-100f), ffma(kd, mm, 0x1p-100f)), thr_f, eps4_f)
+            << (2 * f);
+#else
     if (!certify_keep(C.vp32[0][f], C.vp32[1][f], C.vp32[2][f], C.vp32[3][f], C.vp32[4][f],
                       ffma(kd, mp, 0x1p-100f), thr_f, eps4_f))
       open |= 1u << (2 * f);
     if (!certify_keep(C.vm32[5][f], C.vm32[4][f], C.vm32[3][f], C.vm32[2][f], C.vm32[1][f],
                       ffma(kd, mm, 0x1p-100f), thr_f, eps4_f))
       open |= 2u << (2 * f);
+#endif
   }
   return open;
 }

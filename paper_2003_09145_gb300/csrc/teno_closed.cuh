@@ -8,7 +8,8 @@
 // per interface, each holding an SM partition for 64 cycles; now 29, the FP64
 // pipe 40 % busy).  Measured at 256^3 (ms per RK3 step): Roe state and
 // corrections in binary64 37.0, in two binary32 values 28.1, with the cells'
-// binary32 copies from the cell pass (store_planes) 25.3.  Tried on top
+// binary32 copies from the cell pass (store_planes) 25.3, with the
+// certificate's reconstructions in pairs (certify_open2) 24.3.  Tried on top
 // and dropped: the mass flux as a binary64 chain too (slower), the corrections
 // widened and added in two FP64 additions instead of one (no gain).
 #pragma once
