@@ -86,9 +86,10 @@ __global__ void __launch_bounds__(BLOCK) batched_stage_kernel(BatchArgs A, Schem
     unsigned long long b0 = 0ull, b1 = 0ull, b2 = 0ull;   // bit patterns of the maxima
     bool bad = false;
     for (int64_t i = tid; i < n; i += BLOCK) {
-      double uh[1], cs, ep;
+      double uh[1], ep, pc, hr, cs;
       const int64_t c = off + i;
-      if (!teno::cell_primitives<1>(A.Uin, A.ncell, c, A.gamma, A.aux, uh, cs, ep)) bad = true;
+      if (!teno::cell_primitives<1>(A.Uin, A.ncell, c, A.gamma, A.aux, uh, ep, pc, hr)) bad = true;
+      if (!teno::sound_speed(pc, hr, A.gamma, cs)) bad = true;
       const double Uc[3] = {A.Uin[c], A.Uin[A.ncell + c], A.Uin[2 * A.ncell + c]};
       double Fh[3];
       teno::cell_flux_half_ep<1, 0>(Uc, uh[0], A.aux[A.ncell + c], ep, Fh);

@@ -853,44 +853,89 @@ __device__ __forceinline__ void interface_flux(const double* __restrict__ U,
 // ---------------------------------------------------------------------------
 // Primitive variables of cell c from one reciprocal square root:
 // 1/sqrt(rho), sqrt(rho) = rho/sqrt(rho), 1/(2 rho) = (1/sqrt(rho))^2 / 2,
-// u/2 = m/(2 rho), p = (gamma-1)(E - 2 rho |u/2|^2) (eq. 4.7),
-// c = sqrt(gamma p / rho).  Writes the aux entries (u_k/2, p/2, sqrt(rho),
+// u/2 = m/(2 rho), p = (gamma-1)(E - 2 rho |u/2|^2) (eq. 4.7).
+// Writes the aux entries (u_k/2, p/2, sqrt(rho),
 // (E+p)/sqrt(rho), sqrt(rho) u_k = m_k/sqrt(rho) -- the Roe average's
 // weighted velocities)
-// and returns uh = u/2, c and E + p; false if the state is not physical
-// (rho <= 0, p <= 0 or non-finite).  Working with u/2 saves the halving
-// multiplies; every value equals the u-based evaluation's bit for bit,
-// since the factors of 2 are exact.
+// and returns uh = u/2, E + p, p and hr = 1/(2 rho); false if the state is not
+// physical (rho <= 0, p <= 0 or non-finite, but for p/rho: sound_speed).
+// Working with u/2 saves the halving multiplies, and the exact factors of 2
+// are applied on the integer pipe; every value equals the u-based evaluation's
+// bit for bit.
 // ---------------------------------------------------------------------------
+// x/2 and 2x of a finite x on the integer pipe (multiplied where an exponent
+// leaves the normal range)
+__device__ __forceinline__ double half_of(double x) {
+  const int hi = __double2hiint(x);
+  const unsigned e = (static_cast<unsigned>(hi) >> 20) & 0x7ffu;
+  return e - 2u < 2045u ? __hiloint2double(hi - 0x100000, __double2loint(x)) : 0.5 * x;
+}
+__device__ __forceinline__ double twice(double x) {
+  const int hi = __double2hiint(x);
+  const unsigned e = (static_cast<unsigned>(hi) >> 20) & 0x7ffu;
+  return e - 1u < 2045u ? __hiloint2double(hi + 0x100000, __double2loint(x)) : 2.0 * x;
+}
+
+// c = sqrt(gamma p / rho) as s / sqrt(s); false if s is not positive and finite
+__device__ __forceinline__ bool sound_speed(double p, double hr, double gamma, double& cs) {
+  const double gpr = (2.0 * gamma) * p * hr;
+  cs = gpr * rsqrt(gpr);
+  return pos_finite(gpr);
+}
+
 template <int NDIM>
 __device__ __forceinline__ bool cell_primitives(const double* __restrict__ U, int64_t ncell,
                                                 int64_t c, double gamma,
                                                 double* __restrict__ aux,
-                                                double (&uh)[NDIM], double& cs, double& ep) {
+                                                double (&uh)[NDIM], double& ep, double& p, double& hr) {
   constexpr int NVAR = NDIM + 2;
   const double rho = U[c];
   const double E = U[(NVAR - 1) * ncell + c];
   const double isr = rsqrt(rho);
   const double sr = rho * isr;
-  const double hr = (0.5 * isr) * isr;
+  hr = half_of(isr * isr);
   double q2h = 0.0;
 #pragma unroll
   for (int k = 0; k < NDIM; ++k) {
     uh[k] = U[(1 + k) * ncell + c] * hr;
-    q2h = fma(uh[k], uh[k], q2h);
+    q2h = k == 0 ? uh[0] * uh[0] : fma(uh[k], uh[k], q2h);
   }
-  const double p = (gamma - 1.0) * fma(-2.0 * rho, q2h, E);
-  const double gpr = (2.0 * gamma) * p * hr;
-  cs = gpr * rsqrt(gpr);
+  p = (gamma - 1.0) * fma(-twice(rho), q2h, E);
   ep = E + p;
 #pragma unroll
   for (int k = 0; k < NDIM; ++k) aux[k * ncell + c] = uh[k];
-  aux[NDIM * ncell + c] = 0.5 * p;
+  aux[NDIM * ncell + c] = half_of(p);
   aux[(NDIM + 1) * ncell + c] = sr;
   aux[(NDIM + 2) * ncell + c] = ep * isr;
 #pragma unroll
   for (int k = 0; k < NDIM; ++k) aux[(NDIM + 3 + k) * ncell + c] = U[(1 + k) * ncell + c] * isr;
-  return pos_finite(rho) && pos_finite(p) && is_finite(E) && is_finite(q2h) && pos_finite(gpr);
+  return pos_finite(rho) && pos_finite(p) && is_finite(E) && is_finite(q2h);
+}
+
+// Upper bounds of |u_k - c|, |u_k|, |u_k + c| in binary32 (of the values the
+// binary64 evaluation gives), for skipping cells that cannot reach the running
+// maxima: each truncated input is within 2^-20 of its value and the root and
+// products add a few ulps, so c is within 2^-19 and u - c, u + c within
+// 2^-18 (|u| + c) + 2^-120.  Infinite where a magnitude lies outside
+// 2^-60 .. 2^60 (and the caller then evaluates in binary64); negative for
+// u_k = 0, which no maximum takes.
+template <int NDIM>
+__device__ __forceinline__ void speed_bounds(const double (&uh)[NDIM], double p, double hr, float gamma_f,
+                                             float (&ub)[NDIM][3]) {
+  const unsigned ep = (static_cast<unsigned>(__double2hiint(p)) >> 20) - 963u;
+  const unsigned er = (static_cast<unsigned>(__double2hiint(hr)) >> 20) - 963u;
+  const bool in = ep < 120u && er < 120u;   // (positive too: the sign bit would exceed)
+  const float c = sqrtf(2.0f * gamma_f * hi_float(p) * hi_float(hr));
+#pragma unroll
+  for (int k = 0; k < NDIM; ++k) {
+    const float u = 2.0f * hi_float(uh[k]);
+    const float au = fabsf(u);
+    const float m = fmaf(0x1p-18f, au + c, 0x1p-120f);
+    const bool ok = in && au < 0x1p60f;
+    ub[k][0] = ok ? fabsf(u - c) + m : __int_as_float(0x7f800000);
+    ub[k][1] = (dbits(uh[k]) << 1) == 0ull ? -2.0f : ok ? fmaf(0x1p-18f, au, au + 0x1p-120f) : __int_as_float(0x7f800000);
+    ub[k][2] = ok ? fabsf(u + c) + m : __int_as_float(0x7f800000);
+  }
 }
 
 // SSP-RK3 stage value (eq. 4.1-4.3) of element e from d = L(U^(k))_e:

@@ -38,6 +38,8 @@ namespace teno {
 // max|u_d - c|, max|u_d|, max|u_d + c|.
 // ---------------------------------------------------------------------------
 // F_d/2 of cell c for d = D..NDIM-1 into fh[d][v - 1][c], v = 1..nvar-1.
+// The off-diagonal momentum fluxes rho u_d u_k are formed once, as (u_d/2) m_k
+// of the lower d, for both directions.
 template <int NDIM, int D>
 __device__ __forceinline__ void store_flux_half(const double (&Uc)[NDIM + 2], const double (&uh)[NDIM], double pn,
                                                 double ep, double* __restrict__ fh, int64_t ncell, int64_t c) {
@@ -45,6 +47,8 @@ __device__ __forceinline__ void store_flux_half(const double (&Uc)[NDIM + 2], co
     constexpr int NVAR = NDIM + 2;
     double Fh[NVAR];
     cell_flux_half_ep<NDIM, D>(Uc, uh[D], pn, ep, Fh);
+#pragma unroll
+    for (int k = 0; k < D; ++k) Fh[1 + k] = uh[k] * Uc[1 + D];
 #pragma unroll
     for (int v = 1; v < NVAR; ++v) fh[(int64_t)(D * (NVAR - 1) + v - 1) * ncell + c] = Fh[v];
     store_flux_half<NDIM, D + 1>(Uc, uh, pn, ep, fh, ncell, c);
@@ -77,10 +81,15 @@ __global__ void __launch_bounds__(256, TENO_CELL_MINBLOCKS) cell_kernel(const do
       arg[d][s] = ncell;
     }
   bool bad = false;
+  // the block's running maxima so far, as binary32 values not above them
+  __shared__ volatile float low[NDIM * 3];
+  if (threadIdx.x < NDIM * 3) low[threadIdx.x] = -1.0f;
+  __syncthreads();
+  const float gamma_f = static_cast<float>(gamma);
   for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < ncell;
        c += (int64_t)gridDim.x * blockDim.x) {
-    double uh[NDIM], cs, ep;
-    if (!cell_primitives<NDIM>(U, ncell, c, gamma, aux, uh, cs, ep)) bad = true;
+    double uh[NDIM], p, hr, ep;
+    if (!cell_primitives<NDIM>(U, ncell, c, gamma, aux, uh, ep, p, hr)) bad = true;
     if (fh) {
       double Uc[NVAR];
 #pragma unroll
@@ -92,6 +101,23 @@ __global__ void __launch_bounds__(256, TENO_CELL_MINBLOCKS) cell_kernel(const do
       for (int k = 0; k < NDIM; ++k) su[k] = aux[(NDIM + 3 + k) * ncell + c];
       store_planes<NDIM>(pf, ncell, c, Uc, uh, pn, aux[(NDIM + 1) * ncell + c], aux[(NDIM + 2) * ncell + c], su);
     }
+    // The wave speeds only enter through their maxima: a cell whose binary32
+    // upper bounds all lie below the block's maxima is skipped (15 of a 3D
+    // cell's FP64 instructions; with the halvings and doublings on the integer
+    // pipe and the off-diagonal momentum fluxes formed once the pass fell from
+    // 476 to 406 us at 160^3, FP64 pipe 82 % busy, and a 256^3 step from 24.3
+    // to 22.5 ms).  Anything not certainly below -- NaN too -- is
+    // evaluated, so the maxima are those of all cells, bit for bit.
+    float ub[NDIM][3];
+    speed_bounds<NDIM>(uh, p, hr, gamma_f, ub);
+    bool below = true;
+#pragma unroll
+    for (int d = 0; d < NDIM; ++d)
+#pragma unroll
+      for (int s = 0; s < 3; ++s) below = below && ub[d][s] < low[d * 3 + s];
+    if (below) continue;
+    double cs;
+    if (!sound_speed(p, hr, gamma, cs)) bad = true;
     // u -+ c = 2 (u/2) -+ c with one rounding, as a subtraction of u would;
     // max|u| is kept as max|u/2| and doubled (exactly) below
 #pragma unroll
@@ -99,12 +125,15 @@ __global__ void __launch_bounds__(256, TENO_CELL_MINBLOCKS) cell_kernel(const do
       const double x[3] = {fma(2.0, uh[d], -cs), uh[d], fma(2.0, uh[d], cs)};
 #pragma unroll
       for (int s = 0; s < 3; ++s) {
-        if constexpr (ARG) {
-          const unsigned long long m = max_abs_bits(lam[d][s], x[s]);
+        const unsigned long long m = max_abs_bits(lam[d][s], x[s]);
+        if constexpr (ARG)
           if (m != lam[d][s]) arg[d][s] = c;
+        if (m != lam[d][s]) {
           lam[d][s] = m;
-        } else {
-          lam[d][s] = max_abs_bits(lam[d][s], x[s]);
+          // (hi_float truncates, so the published value is not above the
+          // maximum; a lost update only leaves a lower bound)
+          const float f = (s == 1 ? 2.0f : 1.0f) * hi_float(__longlong_as_double(static_cast<long long>(m)));
+          if (f > low[d * 3 + s] && f > 0x1p-100f && f < 0x1p100f) low[d * 3 + s] = f;
         }
       }
     }
@@ -738,9 +767,9 @@ __global__ void ghost_cell_kernel(GhostStates gs, unsigned mask, double* __restr
   double Uc[NVAR];
 #pragma unroll
   for (int v = 0; v < NVAR; ++v) gU[v * kGhostSlots + slot] = Uc[v] = gs.U[slot][v];
-  double uh[NDIM], cs, ep;
-  if (!cell_primitives<NDIM>(gU, kGhostSlots, slot, gamma, gaux, uh, cs, ep) && status)
-    atomicOr(status, kStatusNonphysical);
+  double uh[NDIM], ep, p, hr, cs;
+  const bool ok = cell_primitives<NDIM>(gU, kGhostSlots, slot, gamma, gaux, uh, ep, p, hr);
+  if (!(sound_speed(p, hr, gamma, cs) && ok) && status) atomicOr(status, kStatusNonphysical);
   store_flux_half<NDIM, 0>(Uc, uh, gaux[NDIM * kGhostSlots + slot], ep, gfh, kGhostSlots, slot);
   double su[NDIM];
 #pragma unroll
@@ -773,7 +802,10 @@ static inline int blocks_for(int64_t n, int threads, int cap) {
   return static_cast<int>(b);
 }
 
-int cell_blocks(int64_t ncell, int nsm) { return blocks_for(ncell, 256, nsm * 8); }
+// The cell pass's grid: the blocks that are resident at once, so that a block
+// sees many cells and its running maxima settle (2 per SM against 8: 22.49
+// against 22.62 ms per 256^3 step, 3.70 against 3.77 at 2048^2).
+int cell_blocks(int64_t ncell, int nsm) { return blocks_for(ncell, 256, nsm * TENO_CELL_MINBLOCKS); }
 
 cudaError_t launch_cell(int ndim, const double* U, double* aux, double* fh, float4* pf,
                         unsigned long long* alpha, int* status, int64_t ncell,
