@@ -250,10 +250,9 @@ __device__ __forceinline__ unsigned interface_flux_closed(const double* __restri
   if (range) {
     // second pass: 60 U~ and the mass flux in fixed point on the grids of the
     // components' largest exponents, the other fluxes as binary64 chains
-    // (see ClosedFix).  The points are taken in two rounds of three (fully
-    // unrolled, the sums' temporaries of all six points would not fit in
-    // the registers; the cell indices, read with a loop index, then sit in the
-    // stack frame).
+    // (see ClosedFix), fully unrolled: the weights are constants (22.1 ms per
+    // 256^3 step against 22.5 in two rounds of three and 24.0 rolled).
+    constexpr int kC[6] = {1, -8, 37, 37, -8, 1}, kM[6] = {1, -5, 10, -10, 5, -1};
     uint32_t EU[NVAR];
     int64_t AU[NVAR], AF = 0;
     double Fd[NVAR];
@@ -263,24 +262,23 @@ __device__ __forceinline__ unsigned interface_flux_closed(const double* __restri
       AU[v] = 0;
       Fd[v] = 0.0;
     }
-#pragma unroll 3
+#pragma unroll
     for (int j = 0; j < 6; ++j) {
       const I c = cells[j];
       const bool fj = (flips >> j) & 1u;
-      const int cw = c_fix_w[0][j], mw = c_fix_w[1][j];
-      const double cd = c_fix_cd[j];
 #pragma unroll
       for (int v = 0; v < NVAR; ++v) {
         const double x = flip_sign(ldc<GH>(U, gc.U, ncell, v, c), fj && v == 1 + DIR);
         const int64_t X = teno_fix::term(x, EU[v]);
-        AU[v] += mw * X;
-        if (v == 1 + DIR) AF += cw * X;
+        AU[v] += kM[j] * X;
+        if (v == 1 + DIR) AF += kC[j] * X;
       }
 #pragma unroll
       for (int v = 1; v < NVAR; ++v) {
         const double f = flip_sign(ldc<GH>(fh, gfh, ncell, v - 1, c), fj && v != 1 + DIR);
         if (j == 0) Fd[v] = f;
-        else Fd[v] = fma(cd, f, Fd[v]);
+        else if (j == 5) Fd[v] += f;
+        else Fd[v] = fma(double(kC[j]), f, Fd[v]);
       }
     }
     df Ut[NVAR];
