@@ -216,6 +216,22 @@ struct TimerScope {
     if ((call) != cudaSuccess) return TENO_ERR_CUDA;     \
   } while (0)
 
+// the fixed-state ghost cells of the grid, if it has any, into the ghost block
+cudaError_t ghost_cells(const teno_grid* g, const Grid& G, cudaStream_t st) {
+  if (!has_dirichlet(g)) return cudaSuccess;
+  teno::GhostStates gs;
+  std::memset(&gs, 0, sizeof(gs));
+  unsigned mask = 0;
+  for (int d = 0; d < g->ndim; ++d) {
+    if (g->bc[d] != TENO_BC_DIRICHLET) continue;
+    for (int side = 0; side < 2; ++side) {
+      for (int v = 0; v < g->ndim + 2; ++v) gs.U[2 * d + side][v] = g->bc_state[d][side][v];
+      mask |= 1u << (2 * d + side);
+    }
+  }
+  return teno::launch_ghost_cells(g->ndim, gs, mask, G, g->gamma, st);
+}
+
 // The first half of a right-hand-side evaluation of state `U`: clear the LF
 // speeds and pending counters, then the cell pass (primitives, half fluxes
 // for the two-pass flux evaluation, this grid's LF speeds).
@@ -230,19 +246,7 @@ teno_status stage_begin(const teno_grid* g, const Layout& L, char* ws, const dou
   float4* pf = reinterpret_cast<float4*>(ws + L.pf);
   TENO_CUDA(cudaMemsetAsync(alpha, 0, teno::kAlphaAndCountBytes, st));
   TimerScope ts(st, TENO_KERNEL_CELL);
-  if (has_dirichlet(g)) {
-    teno::GhostStates gs;
-    std::memset(&gs, 0, sizeof(gs));
-    unsigned mask = 0;
-    for (int d = 0; d < g->ndim; ++d) {
-      if (g->bc[d] != TENO_BC_DIRICHLET) continue;
-      for (int side = 0; side < 2; ++side) {
-        for (int v = 0; v < g->ndim + 2; ++v) gs.U[2 * d + side][v] = g->bc_state[d][side][v];
-        mask |= 1u << (2 * d + side);
-      }
-    }
-    TENO_CUDA(teno::launch_ghost_cells(g->ndim, gs, mask, G, g->gamma, st));
-  }
+  TENO_CUDA(ghost_cells(g, G, st));
   TENO_CUDA(teno::launch_cell(g->ndim, U, aux, fh, pf, alpha, status, G.ncell, g->gamma, nsm, st));
   return TENO_OK;
 }
@@ -367,6 +371,29 @@ teno_status teno_rk3_step(const teno_grid* g, double* U, double cfl, double dt_f
   double* R = reinterpret_cast<double*>(w + L.R);
   double* U1 = reinterpret_cast<double*>(w + L.U1);
   double* U2 = reinterpret_cast<double*>(w + L.U2);
+  const Grid G = grid_in(g, L, w);
+  const Scheme S = make_scheme(g);
+  if (teno::small_step_applies(G, S)) {
+    TimerScope ts(st, TENO_KERNEL_FLUX);
+    TENO_CUDA(ghost_cells(g, G, st));
+    teno::SmallStep A;
+    A.U = U;
+    A.U1 = U1;
+    A.U2 = U2;
+    A.aux = reinterpret_cast<double*>(w + L.aux);
+    A.fh = reinterpret_cast<double*>(w + L.fh);
+    A.pf = reinterpret_cast<float4*>(w + L.pf);
+    A.alpha = reinterpret_cast<unsigned long long*>(w + L.alpha);
+    A.status = reinterpret_cast<int*>(w + L.status);
+    A.t = t_dev;
+    A.dt_ws = reinterpret_cast<double*>(w + L.dt);
+    A.dt_out = dt_dev;
+    A.cfl = cfl;
+    A.dt_fixed = dt_fixed;
+    A.t_end = t_end;
+    TENO_CUDA(teno::launch_step1d(A, G, S, st));
+    return TENO_OK;
+  }
   teno_status s;
   // eq. 4.1: U1 = U + dt L(U); dt from U^n (eq. dt1 / dt2)
   s = rhs_sequence(g, L, w, U, R, nullptr, 2, U, nullptr, U1, st, true, cfl, dt_fixed, t_dev,

@@ -91,6 +91,21 @@ cudaError_t launch_dt(int ndim, const unsigned long long* alpha, const Grid& G,
                       double cfl, double dt_fixed, double* t_dev, double t_end,
                       double* dt_ws, double* dt_out, cudaStream_t st);
 
+// A whole SSP-RK3 step of a small 1D grid in one launch (teno_small.cu): the
+// caller's state and scalars, and the step workspace's arrays.
+struct SmallStep {
+  double *U, *U1, *U2;
+  double *aux, *fh;
+  float4* pf;
+  unsigned long long* alpha;
+  int* status;
+  double *t, *dt_ws, *dt_out;
+  double cfl, dt_fixed, t_end;
+};
+constexpr int64_t kSmallStepMax = 16384;
+bool small_step_applies(const Grid& G, const Scheme& S);
+cudaError_t launch_step1d(const SmallStep& A, const Grid& G, const Scheme& S, cudaStream_t st);
+
 // One right-hand-side evaluation of U fused with the SSP-RK3 stage `mode`
 // (2, 3 or 4; see diff_kernel) into Uout, with dt read from the workspace
 // word at dt_off.  `ws` offsets locate the status word, the LF speeds (and
