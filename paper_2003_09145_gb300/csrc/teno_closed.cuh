@@ -198,10 +198,48 @@ __device__ __forceinline__ bool df_range(float rho_max, float e_max) {
   return rho_max >= 0x1p-20f && rho_max < 0x1p30f && e_max < 0x1p95f;
 }
 
+// The closed form's Roe state and corrections in binary64, on sums already
+// formed (60 U~ and the mass flux in fixed point, the other fluxes): where U~
+// is not small against the flux scale, i.e. at shocks.  Out of line, on copies
+// of its inputs, so that the common form's values stay in registers.
+template <int NDIM>
+struct ClosedSums {
+  uint32_t EU[NDIM + 2];
+  int64_t AU[NDIM + 2], AF;
+  double Fd[NDIM + 2];
+};
+template <int NDIM, int DIR, bool GH, class I>
+__device__ __noinline__ void closed_rough(const double* __restrict__ aux, int64_t ncell, I ca, I cb, unsigned flips,
+                                          double am, double a0, double ap, const Scheme& S, const ClosedSums<NDIM>& X,
+                                          double (&out)[NDIM + 2], int* __restrict__ status, const GhostCells& gc) {
+  constexpr int NVAR = NDIM + 2;
+  const double a3[3] = {am, a0, ap};
+  double alpha[NVAR], nal[NVAR], su2[NDIM], su3[NDIM];
+  spread_speeds<NDIM>(a3, alpha, nal);
+  RoeIfc<NDIM> R;
+#pragma unroll
+  for (int k = 0; k < NDIM; ++k) {
+    su2[k] = ldc<GH>(aux, gc.aux, ncell, NDIM + 3 + k, ca);
+    su3[k] = ldc<GH>(aux, gc.aux, ncell, NDIM + 3 + k, cb);
+  }
+  su2[DIR] = flip_sign(su2[DIR], (flips >> 2) & 1u);
+  su3[DIR] = flip_sign(su3[DIR], (flips >> 3) & 1u);
+  roe_interface<NDIM, DIR>(ldc<GH>(aux, gc.aux, ncell, NDIM + 1, ca), ldc<GH>(aux, gc.aux, ncell, NDIM + 1, cb),
+                           ldc<GH>(aux, gc.aux, ncell, NDIM + 2, ca), ldc<GH>(aux, gc.aux, ncell, NDIM + 2, cb), su2,
+                           su3, S, R, status);
+  double Ft[NVAR], Ut[NVAR];
+#pragma unroll
+  for (int v = 0; v < NVAR; ++v) {
+    Ft[v] = v == 0 ? teno_fix::round(X.AF, X.EU[1 + DIR]) : X.Fd[v];
+    Ut[v] = teno_fix::round(X.AU[v], X.EU[v]);
+  }
+  closed_out<NDIM, DIR>(Ft, Ut, R, nal, out);
+}
+
 // The flux of one interface with every stencil kept, and the mask of its open
 // reconstructions (see interface_flux_closed_wide, which takes over, all in
-// binary64, where the interface leaves teno_df's range or U~ is not small
-// against the flux scale, i.e. near shocks).  I: the cell index type, 32 bits
+// binary64, where the interface leaves teno_df's range; closed_rough: near
+// shocks).  I: the cell index type, 32 bits
 // on the grid path; a3: the halved speeds, F: face_speeds of them.
 template <int NDIM, int DIR, bool GH, class I>
 __device__ __forceinline__ unsigned interface_flux_closed(const double* __restrict__ U,
@@ -225,7 +263,7 @@ __device__ __forceinline__ unsigned interface_flux_closed(const double* __restri
     rb.su[DIR] = scale(rb.su[DIR], fb);
     roe_df<NDIM>(ra, rb, S, R);
   }
-  bool range = F.in_range && roe_df_ok<NDIM>(R, S), wide = false;
+  bool range = F.in_range && roe_df_ok<NDIM>(R, S);
   // first pass: the certified test and the largest magnitudes of the summed
   // components (a mirrored point changes signs only)
   unsigned open;
@@ -282,6 +320,7 @@ __device__ __forceinline__ unsigned interface_flux_closed(const double* __restri
       }
     }
     df Ut[NVAR];
+    bool rough = false;
     // U~ against the flux scale: |60 U~| <= 60 2^-8 (rho, alpha rho, E),
     // tightened by c~^2 / ((gamma - 1) H~), the digits that c~^2 lost
     const float gH = S.gm1_h * R.H.h, lim = (60.0f * 0x1p-8f) * R.c2.h;
@@ -289,9 +328,9 @@ __device__ __forceinline__ unsigned interface_flux_closed(const double* __restri
     for (int v = 0; v < NVAR; ++v) {
       Ut[v] = from_fixed(AU[v], EU[v]);
       const float sc = v == 0 ? xm[0] : (v == NVAR - 1 ? xm[NVAR - 1] : xm[0] * F.amax);
-      wide = wide || !(fabsf(Ut[v].h) * gH <= lim * sc);
+      rough = rough || !(fabsf(Ut[v].h) * gH <= lim * sc);
     }
-    if (!wide) {
+    if (!rough) {
       // closed_out with c~ eliminated: T = |u~|^2/2 U~_0 - u~.U~_m + U~_E,
       // V = (u~_d U~_0 - U~_d)/2 = c~ B, t = c~ A = (gamma-1)/2 T / c~,
       // gs = (sg t + df V) / c~, c~ ngd = df t + sg V
@@ -312,13 +351,28 @@ __device__ __forceinline__ unsigned interface_flux_closed(const double* __restri
       }
       out[NVAR - 1] =
           Fd[NVAR - 1] + to_double(add(add(mul(F.amid, Ut[NVAR - 1]), mul(R.H, gs)), neg(mul(R.u[DIR], cn))));
+    } else {
+      ClosedSums<NDIM> X;
+      double o[NVAR];
+#pragma unroll
+      for (int v = 0; v < NVAR; ++v) {
+        X.EU[v] = EU[v];
+        X.AU[v] = AU[v];
+        X.Fd[v] = Fd[v];
+      }
+      X.AF = AF;
+      closed_rough<NDIM, DIR, GH, I>(aux, ncell, cells[2], cells[3], flips, a3[0], a3[1], a3[2], S, X, o, status, gc);
+#pragma unroll
+      for (int v = 0; v < NVAR; ++v) out[v] = o[v];
     }
-  }
-  // out of range the binary64 form also decides; where only U~ is large it
-  // gives the flux
-  if (!range || wide) {
-    const unsigned w = interface_flux_closed_wide<NDIM, DIR, GH, I>(U, aux, fh, ncell, cells, flips, a3, S, out, status, gc);
-    if (!range || (w & kRough)) open = w;
+  } else {
+    I cc[6];
+    double aa[3] = {a3[0], a3[1], a3[2]}, o[NVAR];
+#pragma unroll
+    for (int j = 0; j < 6; ++j) cc[j] = cells[j];
+    open = interface_flux_closed_wide<NDIM, DIR, GH, I>(U, aux, fh, ncell, cc, flips, aa, S, o, status, gc);
+#pragma unroll
+    for (int v = 0; v < NVAR; ++v) out[v] = o[v];
   }
   return open;
 }

@@ -119,15 +119,23 @@ __global__ void __launch_bounds__(kSmallThreads) step1d_kernel(SmallStep A, Grid
       s_max[tid] = m;
     }
     cluster.sync();
-    if (tid < 3) {
-      unsigned long long m = 0ull;
-      for (unsigned r = 0; r < ncta; ++r) {
-        const unsigned long long x = *cluster.map_shared_rank(&s_max[tid], r);
-        m = m > x ? m : x;
+    if (warp == 0) {   // lane r reads CTA r's maxima
+      unsigned long long m[3];
+#pragma unroll
+      for (int s = 0; s < 3; ++s) m[s] = lane < int(ncta) ? *cluster.map_shared_rank(&s_max[s], lane) : 0ull;
+#pragma unroll
+      for (int o = kSmallCtas / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int s = 0; s < 3; ++s) {
+          const unsigned long long x = __shfl_xor_sync(0xffffffffu, m[s], o);
+          m[s] = m[s] > x ? m[s] : x;
+        }
+      if (lane < 3) {
+        const unsigned long long x = lane == 0 ? m[0] : (lane == 1 ? m[1] : m[2]);
+        s_red[0][lane] = x;
+        s_a[lane] = 0.5 * __longlong_as_double(static_cast<long long>(x));
+        if (rank == 0) A.alpha[lane] = x;
       }
-      s_red[0][tid] = m;
-      s_a[tid] = 0.5 * __longlong_as_double(static_cast<long long>(m));
-      if (rank == 0) A.alpha[tid] = m;
     }
     __syncthreads();
     if (stage == 0) {
