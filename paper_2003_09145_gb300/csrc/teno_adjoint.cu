@@ -231,7 +231,15 @@ __global__ void __launch_bounds__(kAdjThreads, TENO_ADJ_KEPT_MINBLOCKS) adj_kept
             Uj[v] = U[v * I.ncell + cells[j]];
             Ut[v] = j == 0 ? Uj[v] : (j == 5 ? Ut[v] - Uj[v] : fma(Mi[j], Uj[v], Ut[v]));
           }
-          teno::cert_point<NDIM, DIR>(j, Uj, aux[DIR * I.ncell + cells[j]], aux[NDIM * I.ncell + cells[j]], C);
+          const double un = aux[DIR * I.ncell + cells[j]], pn = aux[NDIM * I.ncell + cells[j]];
+          if (df) {
+            float X[NVAR];
+#pragma unroll
+            for (int v = 0; v < NVAR; ++v) X[v] = teno::near_float(Uj[v]);
+            teno_cert::cert_point_f<NDIM, DIR>(j, X, teno::near_float(un), teno::near_float(pn), C);
+          } else {
+            teno::cert_point<NDIM, DIR>(j, Uj, un, pn, C);
+          }
         }
         if (!df || teno::df_range(C.xm[0], C.xm[NVAR - 1])) break;
         df = false;

@@ -320,25 +320,36 @@ TENO_CERT_HD bool select_diffs(double f0, double f1, double f2, double f3, float
 // from below by at most the same relative amount).  The absolute evaluation
 // is monotone in every input, so cert_open forms it once per interface, from
 // the largest magnitudes over the six points, instead of at every point; it
-// also bounds max|v| (FP32 rounding is monotone).  Inputs below 2^-126 add
-// an absolute error below 2^-100 for any physical scale.  cert_open passes
-// d = (8 2^-20 + 8 u) |.|_abs + 2^-100, more than 1.7 times the r + 2 u W that
+// also bounds max|v| (FP32 rounding is monotone).  Inputs below 2^-100 add
+// an absolute error below 2^-90 for any physical scale.  cert_open passes
+// d = (8 2^-20 + 8 u) |.|_abs + 2^-90, more than 1.7 times the r + 2 u W that
 // certify_keep needs, and at least 2^-21 W.
+//
+// The grid path's inputs are not truncated but rounded (cert_begin_f): U, u_d/2,
+// p/2, u~, alpha and 1/c~ within 1 u, b1/2 within 5 u and b2/2 within 7 u.  The
+// longest chain ((u_d/2 + alpha) b1/2 (u~.m - E)) then stays within 20 u, and
+// d = 32 u |.|_abs + 2^-90 leaves the same slack.  The bound matters where the
+// variation is small against the values (large pressures): with 8 2^-20 the
+// test proved nothing for |.|_abs above about 50, with 32 u about 190.
 // ---------------------------------------------------------------------------
 template <int NDIM>
 struct CertIfc {
   float uf[NDIM], hb1f, hb2f, hicf, b1f, hudf, haf[NDIM + 2];
   float vp32[6][NDIM + 2], vm32[6][NDIM + 2];
   float xm[NDIM + 2], hum, hpm;   // largest |U_v|, |u_d/2|, |p/2| over the points
+  float kd;                       // relative bound of the split values' errors
   int dir;                        // sweep direction (a constant once inlined)
 };
 
-// From binary32 values of the Roe state (u~, b1/2, b2/2, 1/(2c), each within
-// 2^-20 relative of the exact one) and of the halved speeds.
+// From binary32 values of the Roe state (u~, b1/2, b2/2, 1/(2c)) and of the
+// halved speeds; kd: kCertRounded for inputs rounded as above, kCertTruncated
+// for truncated ones (hi_float).
+constexpr float kCertTruncated = 8.0f * 0x1p-20f + 8.0f * 0x1p-24f, kCertRounded = 32.0f * 0x1p-24f;
 template <int NDIM, int DIR>
 TENO_CERT_HD void cert_begin_f(const float (&u)[NDIM], float hb1, float hb2, float hic, const float (&ha)[NDIM + 2],
-                               CertIfc<NDIM>& C) {
+                               float kd, CertIfc<NDIM>& C) {
   constexpr int NVAR = NDIM + 2;
+  C.kd = kd;
 #pragma unroll
   for (int k = 0; k < NDIM; ++k) C.uf[k] = u[k];
   C.hb1f = hb1;
@@ -365,10 +376,10 @@ TENO_CERT_HD void cert_begin(const double (&u)[NDIM], double hb1, double hb2, do
   for (int k = 0; k < NDIM; ++k) uf[k] = hi_float(u[k]);
 #pragma unroll
   for (int f = 0; f < NDIM + 2; ++f) ha[f] = hi_float(alpha[f]);
-  cert_begin_f<NDIM, DIR>(uf, hi_float(hb1), hi_float(hb2), hi_float(hic), ha, C);
+  cert_begin_f<NDIM, DIR>(uf, hi_float(hb1), hi_float(hb2), hi_float(hic), ha, kCertTruncated, C);
 }
 
-// Point j: truncated values X of U_j (normal momentum already mirrored at a
+// Point j: binary32 values X of U_j (normal momentum already mirrored at a
 // wall), of u_d/2 and of p/2.  The split values follow the binary64
 // characteristic path: w = L U_j, t = (p/2) z, v+ = (u_d/2 + alpha) w + t,
 // v- = v+ - 2 alpha w.
@@ -441,7 +452,7 @@ TENO_CERT_HD unsigned cert_open(const CertIfc<NDIM>& C, float thr_f, float eps4_
   }
   const float aza = fmul(C.hpm, fmul(fabsf(C.b1f), fadd(C.hum, fabsf(C.hudf))));
   const float bza = fmul(C.hpm, fabsf(C.hicf));
-  const float kd = 8.0f * 0x1p-20f + 8.0f * 0x1p-24f;
+  const float kd = C.kd;
   unsigned open = 0u;
 #pragma unroll
   for (int f = 0; f < NVAR; ++f) {
@@ -452,14 +463,14 @@ TENO_CERT_HD unsigned cert_open(const CertIfc<NDIM>& C, float thr_f, float eps4_
     open |= certify_open2(make_float2(C.vp32[0][f], C.vm32[5][f]), make_float2(C.vp32[1][f], C.vm32[4][f]),
                           make_float2(C.vp32[2][f], C.vm32[3][f]), make_float2(C.vp32[3][f], C.vm32[2][f]),
                           make_float2(C.vp32[4][f], C.vm32[1][f]),
-                          make_float2(ffma(kd, mp, 0x1p-100f), ffma(kd, mm, 0x1p-100f)), thr_f, eps4_f)
+                          make_float2(ffma(kd, mp, 0x1p-90f), ffma(kd, mm, 0x1p-90f)), thr_f, eps4_f)
             << (2 * f);
 #else
     if (!certify_keep(C.vp32[0][f], C.vp32[1][f], C.vp32[2][f], C.vp32[3][f], C.vp32[4][f],
-                      ffma(kd, mp, 0x1p-100f), thr_f, eps4_f))
+                      ffma(kd, mp, 0x1p-90f), thr_f, eps4_f))
       open |= 1u << (2 * f);
     if (!certify_keep(C.vm32[5][f], C.vm32[4][f], C.vm32[3][f], C.vm32[2][f], C.vm32[1][f],
-                      ffma(kd, mm, 0x1p-100f), thr_f, eps4_f))
+                      ffma(kd, mm, 0x1p-90f), thr_f, eps4_f))
       open |= 2u << (2 * f);
 #endif
   }

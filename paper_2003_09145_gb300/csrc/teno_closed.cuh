@@ -19,6 +19,16 @@
 
 namespace teno {
 
+// x rounded to binary32 (within 2^-24 and a bit, relative) by integer and FP32
+// operations, for 2^-100 <= |x| < 2^100; beyond that hi_float's clamped
+// truncation
+__device__ __forceinline__ float near_float(double x) {
+  const uint32_t e = (teno_fix::hi_word(x) >> 20) & 0x7FFu;
+  if (e - 923u >= 200u) return hi_float(x);
+  const teno_df::df d = teno_df::from_double(x);
+  return teno_cert::fadd(d.h, d.l);
+}
+
 // The speeds in the forms the closed form reads: halved, as two binary32
 // values (the middle one, and the sum and difference of the acoustic
 // ones' differences against it -- closed_out's amid, sg, df), as binary32, and
@@ -37,7 +47,7 @@ __device__ __forceinline__ FaceSpeeds face_speeds(const double (&a3)[3]) {
   F.sg = add(d0, dE);
   F.dd = add(d0, neg(dE));
 #pragma unroll
-  for (int s = 0; s < 3; ++s) F.ha[s] = hi_float(a3[s]);
+  for (int s = 0; s < 3; ++s) F.ha[s] = near_float(a3[s]);
   F.amax = 2.0f * fmaxf(F.ha[0], F.ha[2]);
   F.in_range = F.amax >= 0x1p-19f && F.amax <= 0x1p30f;
   return F;
@@ -46,8 +56,8 @@ __device__ __forceinline__ FaceSpeeds face_speeds(const double (&a3)[3]) {
 // What the closed form's first pass and its Roe state read of a cell, in
 // binary32, written once per cell by the cell pass (converting it at each of
 // the eighteen stencil points that read the cell took some 280 instructions
-// per interface): planes of float4, pf[plane_count(NDIM)][ncell].  Truncated
-// values of U, p/2 and u_k/2 (hi_float), and sqrt(rho), (E+p)/sqrt(rho),
+// per interface): planes of float4, pf[plane_count(NDIM)][ncell].  Rounded
+// values of U, p/2 and u_k/2 (near_float), and sqrt(rho), (E+p)/sqrt(rho),
 // m_k/sqrt(rho) as two binary32 values (from_double):
 //   1D: {rho, m, E, p/2}, {u/2, 0, su}, {sr, sh}
 //   2D: {rho, m_0, m_1, E}, {p/2, u_0/2, u_1/2, 0}, {sr, sh}, {su_0, su_1}
@@ -59,10 +69,10 @@ __device__ __forceinline__ void store_planes(float4* __restrict__ pf, int64_t nc
   using namespace teno_df;
   float X[NDIM + 2], u[NDIM];
 #pragma unroll
-  for (int v = 0; v < NDIM + 2; ++v) X[v] = hi_float(U[v]);
+  for (int v = 0; v < NDIM + 2; ++v) X[v] = near_float(U[v]);
 #pragma unroll
-  for (int k = 0; k < NDIM; ++k) u[k] = hi_float(uh[k]);
-  const float p = hi_float(ph);
+  for (int k = 0; k < NDIM; ++k) u[k] = near_float(uh[k]);
+  const float p = near_float(ph);
   const df r = from_double(sr), h = from_double(sh), s0 = from_double(su[0]);
   float4* o = pf + c;
   if constexpr (NDIM == 1) {
@@ -172,20 +182,23 @@ __device__ __forceinline__ void roe_df(const RoeCellDf<NDIM>& a, const RoeCellDf
   R.ic = teno_df::rsqrt(R.c2);
 }
 
-// The certificate's view of that Roe state: its high parts lie within 2^-21
-// of the values where roe_df_ok holds, i.e. where c~^2 keeps 2^-6 of
-// (gamma - 1) H~ (Mach numbers below about 18 for gamma = 1.4; c~^2 is then
-// good to 2^-38).
+// The certificate's view of that Roe state, rounded to binary32, where
+// roe_df_ok holds, i.e. where c~^2 keeps 2^-6 of (gamma - 1) H~ (Mach numbers
+// below about 18 for gamma = 1.4; c~^2 is then good to 2^-38).
 template <int NDIM, int DIR>
 __device__ __forceinline__ void cert_begin_df(const RoeDf<NDIM>& R, const float (&ha3)[3], const Scheme& S,
                                               CertIfc<NDIM>& C) {
+  using teno_cert::fadd;
+  using teno_cert::fmul;
   float uf[NDIM], ha[NDIM + 2];
 #pragma unroll
-  for (int k = 0; k < NDIM; ++k) uf[k] = R.u[k].h;
+  for (int k = 0; k < NDIM; ++k) uf[k] = fadd(R.u[k].h, R.u[k].l);
 #pragma unroll
   for (int f = 0; f < NDIM + 2; ++f) ha[f] = ha3[f == 0 ? 0 : (f == NDIM + 1 ? 2 : 1)];
-  const float hb1 = teno_cert::fmul(0.5f * S.gm1_h, teno_cert::fmul(R.ic.h, R.ic.h));
-  teno_cert::cert_begin_f<NDIM, DIR>(uf, hb1, teno_cert::fmul(0.5f * hb1, R.q2.h), 0.5f * R.ic.h, ha, C);
+  const float ic = fadd(R.ic.h, R.ic.l);
+  const float hb1 = fmul(0.5f * S.gm1_h, fmul(ic, ic));
+  teno_cert::cert_begin_f<NDIM, DIR>(uf, hb1, fmul(0.5f * hb1, fadd(R.q2.h, R.q2.l)), 0.5f * ic, ha,
+                                     teno_cert::kCertRounded, C);
 }
 template <int NDIM>
 __device__ __forceinline__ bool roe_df_ok(const RoeDf<NDIM>& R, const Scheme& S) {

@@ -102,7 +102,7 @@ struct SmallStep {
   double *t, *dt_ws, *dt_out;
   double cfl, dt_fixed, t_end;
 };
-constexpr int64_t kSmallStepMax = 16384;
+constexpr int64_t kSmallStepMax = 6144;
 bool small_step_applies(const Grid& G, const Scheme& S);
 cudaError_t launch_step1d(const SmallStep& A, const Grid& G, const Scheme& S, cudaStream_t st);
 
