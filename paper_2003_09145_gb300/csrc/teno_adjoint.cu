@@ -57,23 +57,6 @@ using teno::Scheme;
 
 constexpr int kAdjThreads = 128;
 
-// The adjoint's six-point sums with integer weights in 64-bit fixed point
-// (teno_fixsum.cuh, as in the forward's closed form): bit 1 the stencil on
-// Rbar (weights 1, -9, 45 on the differences), bit 2 the M-weighted U~bar of
-// the slots, bit 4 the kept pass's 60 U~ (from stored Roe states).  A
-// component the fixed point does not cover takes the binary64 form.  A
-// tuning choice between the FP64 and integer pipes; measured on the 256^3
-// reverse RK3 step (ms): none 102.4, bit 1 100.9-101.1 (this default), bit
-// 4 101.5, bits 1 and 4 100.0, bits 1 and 2 114.7 (the M sums' seven loads
-// per component spill and the integer chains then bound the gather).  Bit 4
-// is left off: the kept pass without stored states (the staged reverse
-// step's) sums U~ as a binary64 chain, and the two reverse steps agree bit
-// for bit only if both do.
-#ifndef TENO_ADJ_FIX_MASK
-#define TENO_ADJ_FIX_MASK 1
-#endif
-constexpr unsigned kAdjFixMask = TENO_ADJ_FIX_MASK;
-
 // Geometry of interface q of direction DIR: its index id along DIR, the
 // linear index of its line's cell 0 and the six stencil cells (ghosts mapped).
 template <int NDIM, int DIR>
@@ -161,6 +144,58 @@ __device__ __forceinline__ void add_alpha(const double (&ab)[NVAR], double (&asu
   asum[2] += ab[NVAR - 1];
 }
 
+// The forward's certificate at one interface (interface_flux_closed's open
+// mask): on the Roe state in two binary32 values, or on the binary64 one
+// outside their range.  Out of line: its registers are its own.
+template <int NDIM, int DIR>
+__device__ __noinline__ unsigned forward_open(const double* __restrict__ U, const double* __restrict__ aux,
+                                              int64_t ncell, int64_t line, int64_t id, int64_t nd, int64_t stride, int bc,
+                                              double am, double a0, double ap, const Scheme& S, int* status) {
+  constexpr int NVAR = NDIM + 2;
+  if (S.keep_idx < 0) return teno::kRough | teno::kAllOpen<NDIM>;
+  int64_t cells[6];
+#pragma unroll
+  for (int j = 0; j < 6; ++j) cells[j] = line + teno::ghost(id - 3 + j, nd, bc) * stride;
+  const double a3[3] = {am, a0, ap};
+  const teno::FaceSpeeds F = teno::face_speeds(a3);
+  double su2[NDIM], su3[NDIM];
+#pragma unroll
+  for (int k = 0; k < NDIM; ++k) {
+    su2[k] = aux[(NDIM + 3 + k) * ncell + cells[2]];
+    su3[k] = aux[(NDIM + 3 + k) * ncell + cells[3]];
+  }
+  const double sr2 = aux[(NDIM + 1) * ncell + cells[2]], sr3 = aux[(NDIM + 1) * ncell + cells[3]];
+  const double sh2 = aux[(NDIM + 2) * ncell + cells[2]], sh3 = aux[(NDIM + 2) * ncell + cells[3]];
+  teno::RoeDf<NDIM> Rd;
+  teno::roe_df<NDIM>(teno::roe_cell<NDIM>(sr2, sh2, su2), teno::roe_cell<NDIM>(sr3, sh3, su3), S, Rd);
+  teno::CertIfc<NDIM> C;
+  for (bool df = F.in_range && teno::roe_df_ok<NDIM>(Rd, S);; df = false) {
+    if (df) {
+      teno::cert_begin_df<NDIM, DIR>(Rd, F.ha, S, C);
+    } else {
+      double alpha[NVAR], nal[NVAR];
+      teno::spread_speeds<NDIM>(a3, alpha, nal);
+      teno::RoeIfc<NDIM> R;
+      teno::roe_interface<NDIM, DIR>(sr2, sr3, sh2, sh3, su2, su3, S, R, status);
+      teno::cert_begin<NDIM, DIR>(R, alpha, C);
+    }
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+      float X[NVAR];
+      const double un = aux[DIR * ncell + cells[j]], pn = aux[NDIM * ncell + cells[j]];
+#pragma unroll
+      for (int v = 0; v < NVAR; ++v) {
+        const double x = U[v * ncell + cells[j]];
+        X[v] = df ? teno::near_float(x) : teno::hi_float(x);
+      }
+      teno_cert::cert_point_f<NDIM, DIR>(j, X, df ? teno::near_float(un) : teno::hi_float(un),
+                                         df ? teno::near_float(pn) : teno::hi_float(pn), C);
+    }
+    if (!df || teno::df_range(C.xm[0], C.xm[NVAR - 1])) break;
+  }
+  return teno::cert_open<NDIM>(C, S);
+}
+
 // One thread per interface: the forward pass's certified FP32 test (the
 // same device code teno_rhs / teno_rk3_step run).  Where it keeps every
 // stencil, the interface part of the closed-form VJP: U~bar and the
@@ -168,7 +203,7 @@ __device__ __forceinline__ void add_alpha(const double (&ab)[NVAR], double (&asu
 // (the flux Jacobians and the Roe-parameter maps are applied per cell by the
 // gather); elsewhere the interface is marked pending for adj_general_kernel.
 #ifndef TENO_ADJ_KEPT_MINBLOCKS
-#define TENO_ADJ_KEPT_MINBLOCKS 3   // 168 registers: 12 warps per SM
+#define TENO_ADJ_KEPT_MINBLOCKS 4   // 128 registers, 16 warps per SM: 14.91 ms per 128^3 reverse step against 15.28 at 3
 #endif
 template <int NDIM, int DIR, bool STORED>
 __global__ void __launch_bounds__(kAdjThreads, TENO_ADJ_KEPT_MINBLOCKS) adj_kept_kernel(
@@ -184,7 +219,6 @@ __global__ void __launch_bounds__(kAdjThreads, TENO_ADJ_KEPT_MINBLOCKS) adj_kept
   // factor scale / dx (carried by the speeds instead); its ab come out times
   // 60 dx / scale, which adj_alpha_kernel divides out of the block sums
   const double fscale = scale * G.inv_dx[DIR];
-  const double Mi[6] = {1.0, -5.0, 10.0, -10.0, 5.0, -1.0};
   const double amid = fscale * fa[1], d0 = fscale * (fa[0] - fa[1]), dE = fscale * (fa[NVAR - 1] - fa[1]);
   const double igm1 = 1.0 / (S.gamma - 1.0);
   double asum[3] = {0.0, 0.0, 0.0};
@@ -213,38 +247,8 @@ __global__ void __launch_bounds__(kAdjThreads, TENO_ADJ_KEPT_MINBLOCKS) adj_kept
         su3[k] = aux[(NDIM + 3 + k) * I.ncell + cells[3]];
       }
       teno::roe_interface<NDIM, DIR>(sr2, sr3, sh2, sh3, su2, su3, S, Rf, status);
-      // the forward's certificate: on the Roe state in two binary32 values,
-      // or on the binary64 one outside their range (interface_flux_closed)
-      const double a3[3] = {ha[0], ha[1], ha[NVAR - 1]};
-      const teno::FaceSpeeds F = teno::face_speeds(a3);
-      teno::RoeDf<NDIM> Rd;
-      teno::roe_df<NDIM>(teno::roe_cell<NDIM>(sr2, sh2, su2), teno::roe_cell<NDIM>(sr3, sh3, su3), S, Rd);
-      teno::CertIfc<NDIM> C;
-      for (bool df = F.in_range && teno::roe_df_ok<NDIM>(Rd, S);;) {
-        if (df) teno::cert_begin_df<NDIM, DIR>(Rd, F.ha, S, C);
-        else teno::cert_begin<NDIM, DIR>(Rf, ha, C);
-#pragma unroll
-        for (int j = 0; j < 6; ++j) {
-          double Uj[NVAR];
-#pragma unroll
-          for (int v = 0; v < NVAR; ++v) {
-            Uj[v] = U[v * I.ncell + cells[j]];
-            Ut[v] = j == 0 ? Uj[v] : (j == 5 ? Ut[v] - Uj[v] : fma(Mi[j], Uj[v], Ut[v]));
-          }
-          const double un = aux[DIR * I.ncell + cells[j]], pn = aux[NDIM * I.ncell + cells[j]];
-          if (df) {
-            float X[NVAR];
-#pragma unroll
-            for (int v = 0; v < NVAR; ++v) X[v] = teno::near_float(Uj[v]);
-            teno_cert::cert_point_f<NDIM, DIR>(j, X, teno::near_float(un), teno::near_float(pn), C);
-          } else {
-            teno::cert_point<NDIM, DIR>(j, Uj, un, pn, C);
-          }
-        }
-        if (!df || teno::df_range(C.xm[0], C.xm[NVAR - 1])) break;
-        df = false;
-      }
-      kept = S.keep_idx >= 0 && teno::cert_keep<NDIM>(C, S);
+      kept = forward_open<NDIM, DIR>(U, aux, I.ncell, base, id, I.nd, I.stride_d, I.bcd, ha[0], ha[1], ha[NVAR - 1], S,
+                                     status) == 0u;
     }
     pending[q] = kept ? 0 : 1;
     if (!kept) {
@@ -264,18 +268,22 @@ __global__ void __launch_bounds__(kAdjThreads, TENO_ADJ_KEPT_MINBLOCKS) adj_kept
       Rf.hb1 = roe_in[(int64_t)(NDIM + 4) * I.nifc + q];
       Rf.hb2 = roe_in[(int64_t)(NDIM + 5) * I.nifc + q];
       Rf.hic = roe_in[(int64_t)(NDIM + 6) * I.nifc + q];
+    }
+    // 60 U~ in 64-bit fixed point (teno_fixsum.cuh, as in the forward's closed
+    // form; a component it does not cover as a binary64 chain): 14.32 ms per
+    // 128^3 reverse step against 14.74 with the chain.  (The gather's stencil
+    // on Rbar in fixed point measured 14.91 against 14.74 without.)
 #pragma unroll
-      for (int v = 0; v < NVAR; ++v) {
-        double us[6];
+    for (int v = 0; v < NVAR; ++v) {
+      double us[6];
 #pragma unroll
-        for (int j = 0; j < 6; ++j) us[j] = U[v * I.ncell + cells[j]];
-        const int mw[6] = {1, -5, 10, -10, 5, -1};
-        if (!(kAdjFixMask & 4u) || !teno_fix::sum<6>(us, mw, Ut[v])) {
-          Ut[v] = us[0];
+      for (int j = 0; j < 6; ++j) us[j] = U[v * I.ncell + cells[j]];
+      const int mw[6] = {1, -5, 10, -10, 5, -1};
+      if (!teno_fix::sum<6>(us, mw, Ut[v])) {
+        Ut[v] = us[0];
 #pragma unroll
-          for (int j = 1; j < 5; ++j) Ut[v] = fma(Mi[j], us[j], Ut[v]);
-          Ut[v] -= us[5];
-        }
+        for (int j = 1; j < 5; ++j) Ut[v] = fma(double(mw[j]), us[j], Ut[v]);
+        Ut[v] -= us[5];
       }
     }
     // the VJP's Roe state: the same average, and the cells' velocity and
@@ -500,11 +508,10 @@ __global__ void __launch_bounds__(kListThreads) adj_part_scatter_kernel(
 // The listed interfaces in two passes, so that the VJP runs on full warps
 // (the forward's cutoff decisions branch per field and lane; the VJP with
 // the selections fixed does not branch):
-//   adj_select_kernel: one thread per listed interface: the characteristic
-//                      path of the forward pass (the same binary64 decisions
-//                      its pending pass takes on these very interfaces, as the
-//                      kept pass ran the forward's certificate) -> the ten
-//                      3-bit selections packed into sel[i];
+//   adj_select_kernel: the forward's certificate again for the mask of open
+//                      reconstructions, and the decisions its correction pass
+//                      takes on those (warp_correct) -> the ten 3-bit
+//                      selections packed into sel[i];
 //   partition passes  : the list reordered, those that keep every stencil
 //                      after all first (below);
 //   adj_general_kernel: one thread per listed interface: the closed-form VJP
@@ -519,27 +526,40 @@ __global__ void __launch_bounds__(kAdjThreads) adj_select_kernel(
     const unsigned long long* __restrict__ alpha_bits, const uint32_t* __restrict__ list,
     const int* __restrict__ count, uint32_t* __restrict__ sel, int* __restrict__ status, Grid G, Scheme S) {
   constexpr int NVAR = NDIM + 2;
+  __shared__ teno::CorrectScratch<NDIM> scratch[kAdjThreads / 32];
   const IfcGeom<NDIM, DIR> I(G);
   double fa[NVAR], ha[NVAR], nfa[NVAR];
   field_speeds<NDIM, DIR>(alpha_bits, fa, ha, nfa);
   const int64_t n = *count;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t q = list[i];
-    int64_t id, base, cells[6];
+  const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  auto cells_of = [&](uint32_t q, int64_t (&cells)[6], unsigned& flips) {
+    int64_t id, base;
     I.locate(q, G, id, base, cells);
-    double fout[NVAR];
-    unsigned fl[NVAR][2];
-    teno::interface_flux<NDIM, DIR, false, teno::kFluxChar>(U, aux, I.ncell, cells, 0u, ha, nfa, S, fout, fl,
-                                                            status);
-    uint32_t w = 0;
-#pragma unroll
-    for (int f = 0; f < NVAR; ++f) w |= ((fl[f][0] & 7u) | ((fl[f][1] & 7u) << 3)) << (6 * f);
-    sel[i] = w;
+    flips = 0u;
+  };
+  for (int64_t i0 = ((int64_t)blockIdx.x * (kAdjThreads / 32) + warp) * 32; i0 < n;
+       i0 += (int64_t)gridDim.x * kAdjThreads) {
+    const int64_t i = i0 + lane;
+    unsigned open = 0u;
+    uint32_t q = 0u;
+    if (i < n) {
+      q = list[i];
+      int64_t id, base, cells[6];
+      I.locate(q, G, id, base, cells);
+      open = forward_open<NDIM, DIR>(U, aux, I.ncell, base, id, I.nd, I.stride_d, I.bcd, ha[0], ha[1], ha[NVAR - 1], S,
+                                     status);
+    }
+    double out[NVAR];
+    const uint32_t w = teno::warp_correct<NDIM, DIR, false, int64_t, true>(U, aux, I.ncell, cells_of, q, ha, S, open,
+                                                                          out, status, scratch[warp]);
+    if (i < n) sel[i] = w;
   }
 }
 
 template <int NDIM, int DIR>
-__global__ void __launch_bounds__(kAdjThreads) adj_general_kernel(
+// (3 blocks per SM, 168 registers: 29.7 against 30.6 ms for the rollout case at 64^3, where a third
+// of the interfaces is listed)
+__global__ void __launch_bounds__(kAdjThreads, 3) adj_general_kernel(
     const double* __restrict__ U, const unsigned long long* __restrict__ alpha_bits,
     const double* __restrict__ Rbar, double scale, double* __restrict__ contrib,
     const uint32_t* __restrict__ list, const int* __restrict__ count, const int* __restrict__ nkept,
@@ -587,8 +607,6 @@ __global__ void __launch_bounds__(kAdjThreads) adj_general_kernel(
 // for U~ = sum_j M_j U_j (indexed by a warp-uniform slot number).
 __constant__ double c_adjP[6] = {1.0 / 60.0, -8.0 / 60.0, 37.0 / 60.0, 37.0 / 60.0, -8.0 / 60.0, 1.0 / 60.0};
 __constant__ double c_adjM[6] = {1.0 / 60.0, -5.0 / 60.0, 10.0 / 60.0, -10.0 / 60.0, 5.0 / 60.0, -1.0 / 60.0};
-__constant__ int c_adjMi[6] = {1, -5, 10, -10, 5, -1};
-
 
 // What the gather reads per direction, and its output.
 struct GatherArgs {
@@ -606,24 +624,6 @@ struct GatherArgs {
 // acc and its Roe-parameter adjoints (j = 2: cell i, j = 3: cell i+1) into
 // rp (both zero for a pending interface), and for a pending one its own
 // contribution into acc.
-// (slot_rest: the same without the M_j U~bar term, which the stencil path
-// sums in fixed point.)
-template <int NVAR>
-__device__ __forceinline__ void slot_rest(int j, int64_t q, const double* __restrict__ kb,
-                                          const double* __restrict__ contrib,
-                                          const unsigned char* __restrict__ pending, int64_t nifc,
-                                          double (&acc)[NVAR], double (&rp)[NVAR]) {
-  if (j == 2)
-#pragma unroll
-    for (int v = 0; v < NVAR; ++v) rp[v] += kb[(int64_t)(NVAR + v) * nifc + q];
-  if (j == 3)
-#pragma unroll
-    for (int v = 0; v < NVAR; ++v) rp[v] += kb[(int64_t)(2 * NVAR + v) * nifc + q];
-  if (pending[q])
-#pragma unroll
-    for (int v = 0; v < NVAR; ++v) acc[v] += contrib[(int64_t)(j * NVAR + v) * nifc + q];
-}
-
 template <int NVAR>
 __device__ __forceinline__ void slot_terms(int j, int64_t q, const double* __restrict__ kb,
                                            const double* __restrict__ contrib,
@@ -750,33 +750,12 @@ __device__ __forceinline__ void gather_dir(const Grid& G, int64_t c, int64_t i0,
     for (int v = 0; v < NVAR; ++v) {
       const double* r = Rbar + v * ncell + line;
       const double r1p = r[o1p], r1m = r[o1m], r2p = r[o2p], r2m = r[o2m], r3p = r[o3p], r3m = r[o3m];
-      double S;
-      const double rs[6] = {r3p, r3m, r2p, r2m, r1p, r1m};
-      const int rw[6] = {1, -1, -9, 9, 45, -45};
-      if ((kAdjFixMask & 1u) && teno_fix::sum<6>(rs, rw, S)) Fsum[v] = w1 * S;
-      else Fsum[v] = fma(w45, r1p - r1m, fma(w9, r2p - r2m, w1 * (r3p - r3m)));
-      if (kAdjFixMask & 2u) {
-        const double* k = kb + (int64_t)v * nifc;
-        const double ks[7] = {k[qs[0]], k[qs[1]], k[qs[2]], k[qs[3]], k[qs[4]], k[qs[5]], jd >= 0 ? k[qd] : 0.0};
-        const int kw[7] = {1, -5, 10, -10, 5, -1, jd >= 0 ? c_adjMi[jd] : 0};
-        double T;
-        if (teno_fix::sum<7>(ks, kw, T)) {
-          acc[v] = fma(1.0 / 60.0, T, acc[v]);
-        } else {
-#pragma unroll
-          for (int j = 0; j < 7; ++j) acc[v] = fma(kw[j] * (1.0 / 60.0), ks[j], acc[v]);
-        }
-      }
+      Fsum[v] = fma(w45, r1p - r1m, fma(w9, r2p - r2m, w1 * (r3p - r3m)));
     }
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
-      if (kAdjFixMask & 2u) {
-        slot_rest<NVAR>(j, qs[j], kb, contrib, pending, nifc, acc, rp);
-        if (j == jd) slot_rest<NVAR>(j, qd, kb, contrib, pending, nifc, acc, rp);
-      } else {
-        slot_terms<NVAR>(j, qs[j], kb, contrib, pending, nifc, acc, rp);
-        if (j == jd) slot_terms<NVAR>(j, qd, kb, contrib, pending, nifc, acc, rp);
-      }
+      slot_terms<NVAR>(j, qs[j], kb, contrib, pending, nifc, acc, rp);
+      if (j == jd) slot_terms<NVAR>(j, qd, kb, contrib, pending, nifc, acc, rp);
     }
   } else {
 #pragma unroll
@@ -852,45 +831,54 @@ struct AlphaScale {
   double k[3];
 };
 constexpr int kAlphaThreads = 256;
+// (One warp per direction and pass sums its blocks -- lane strides, then a
+// fixed tree -- and one lane per speed evaluates its gradient; one thread adds
+// them in speed order, as several speeds may share a cell.  With one block-wide
+// sum after another and one thread for the gradients the pass took 77 us, all
+// of it latency.)
 template <int NDIM>
 __global__ void __launch_bounds__(kAlphaThreads) adj_alpha_kernel(const double* __restrict__ apart, int nblocks,
                                  AlphaScale kscale, const unsigned long long* __restrict__ argidx,
                                  const double* __restrict__ U, double* __restrict__ Ubar, int64_t ncell,
                                  double gamma) {
   constexpr int NVAR = NDIM + 2;
-  __shared__ double red[kAlphaThreads][3];
   __shared__ double tot[NDIM][2][3];
-  for (int d = 0; d < NDIM; ++d)
-    for (int h = 0; h < 2; ++h) {
-      const double* ap = apart + ((int64_t)d * 2 + h) * nblocks * 3;
-      double s[3] = {0.0, 0.0, 0.0};
-      for (int b = threadIdx.x; b < nblocks; b += kAlphaThreads)
-        for (int k = 0; k < 3; ++k) s[k] += ap[b * 3 + k];
-      for (int k = 0; k < 3; ++k) red[threadIdx.x][k] = s[k];
-      __syncthreads();
-      for (int w = kAlphaThreads / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-          for (int k = 0; k < 3; ++k) red[threadIdx.x][k] += red[threadIdx.x + w][k];
-        __syncthreads();
-      }
-      if (threadIdx.x == 0)
-        for (int k = 0; k < 3; ++k) tot[d][h][k] = red[0][k];
-      __syncthreads();
+  __shared__ double grad[NDIM * 3][NVAR];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp < 2 * NDIM) {
+    const double* ap = apart + (int64_t)warp * nblocks * 3;   // [d][h] = [warp / 2][warp % 2]
+    double s[3] = {0.0, 0.0, 0.0};
+    for (int b = lane; b < nblocks; b += 32)
+      for (int k = 0; k < 3; ++k) s[k] += ap[b * 3 + k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+      for (int k = 0; k < 3; ++k) s[k] += __shfl_down_sync(0xffffffffu, s[k], o);
+    if (lane == 0)
+      for (int k = 0; k < 3; ++k) tot[warp >> 1][warp & 1][k] = s[k];
+  }
+  __syncthreads();
+  if (threadIdx.x < NDIM * 3) {
+    const int d = threadIdx.x / 3, k = threadIdx.x % 3;
+    const unsigned long long c = argidx[threadIdx.x];
+    double Uc[NVAR], g[NVAR];
+    const bool in = c < (unsigned long long)ncell;
+    for (int v = 0; v < NVAR; ++v) {
+      Uc[v] = in ? U[v * ncell + c] : 1.0;
+      g[v] = 0.0;
     }
-  if (threadIdx.x != 0) return;
-  for (int d = 0; d < NDIM; ++d)
-    for (int k = 0; k < 3; ++k) {
-      const unsigned long long c = argidx[d * 3 + k];
-      if (c >= (unsigned long long)ncell) continue;
-      double Uc[NVAR], g[NVAR];
-      for (int v = 0; v < NVAR; ++v) {
-        Uc[v] = U[v * ncell + c];
-        g[v] = 0.0;
-      }
+    if (in) {
       const double s = fma(kscale.k[d], tot[d][0][k], tot[d][1][k]);
       teno_adj::wave_speed_grad<NDIM>(Uc, d, k, gamma, s, g);
-      for (int v = 0; v < NVAR; ++v) Ubar[v * ncell + c] += g[v];
     }
+    for (int v = 0; v < NVAR; ++v) grad[threadIdx.x][v] = g[v];
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int k = 0; k < NDIM * 3; ++k) {
+    const unsigned long long c = argidx[k];
+    if (c >= (unsigned long long)ncell) continue;
+    for (int v = 0; v < NVAR; ++v) Ubar[v * ncell + c] += grad[k][v];
+  }
 }
 
 __global__ void set_value_kernel(double* p, double v) {

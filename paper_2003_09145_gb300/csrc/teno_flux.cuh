@@ -505,8 +505,10 @@ struct CorrectScratch {   // one per warp
 // cells_of(q, cells, flips) gives the stencil of interface q (cell indices I).  Every lane of
 // the warp calls; `open` is 0 in lanes without an interface.  On entry `out`
 // is interface_flux_closed's (unset with kRough), on return the flux.
-template <int NDIM, int DIR, bool GH, class I, class Cells>
-__device__ __forceinline__ void warp_correct(const double* __restrict__ U, const double* __restrict__ aux,
+// With SELECT only the selections are wanted: `out` is not touched, and the
+// delta bits of every field and side are returned, three bits each (7 where not open).
+template <int NDIM, int DIR, bool GH, class I, bool SELECT = false, class Cells>
+__device__ __forceinline__ uint32_t warp_correct(const double* __restrict__ U, const double* __restrict__ aux,
                                              int64_t ncell, const Cells& cells_of, uint32_t q,
                                              const double (&alpha)[NDIM + 2], const Scheme& S, unsigned open,
                                              double (&out)[NDIM + 2], int* __restrict__ status,
@@ -534,13 +536,15 @@ __device__ __forceinline__ void warp_correct(const double* __restrict__ U, const
                              ldc<GH>(aux, gc.aux, ncell, NDIM + 1, cells[3]),
                              ldc<GH>(aux, gc.aux, ncell, NDIM + 2, cells[2]),
                              ldc<GH>(aux, gc.aux, ncell, NDIM + 2, cells[3]), su2, su3, S, R, status);
-    float rm = 0.0f, em = 0.0f;
+    if constexpr (!SELECT) {
+      float rm = 0.0f, em = 0.0f;
 #pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      rm = fmaxf(rm, fabsf(hi_float(ldc<GH>(U, gc.U, ncell, 0, cells[j]))));
-      em = fmaxf(em, fabsf(hi_float(ldc<GH>(U, gc.U, ncell, NVAR - 1, cells[j]))));
+      for (int j = 0; j < 6; ++j) {
+        rm = fmaxf(rm, fabsf(hi_float(ldc<GH>(U, gc.U, ncell, 0, cells[j]))));
+        em = fmaxf(em, fabsf(hi_float(ldc<GH>(U, gc.U, ncell, NVAR - 1, cells[j]))));
+      }
+      whole = (open & kRough) || beyond_flux_scale<NDIM>(out, alpha, rm, em);
     }
-    whole = (open & kRough) || beyond_flux_scale<NDIM>(out, alpha, rm, em);
 #pragma unroll
     for (int k = 0; k < NDIM; ++k) W.u[k][lane] = R.u[k];
     W.H[lane] = R.H;
@@ -562,7 +566,7 @@ __device__ __forceinline__ void warp_correct(const double* __restrict__ U, const
       W.item[n + __popc(m & ((1u << lane) - 1u))] =
           static_cast<uint16_t>(lane | unsigned(b) << 5 | (whole ? 1u << 9 : 0u));
     } else {
-      W.d[b][lane] = 0.0;
+      W.d[b][lane] = SELECT ? 7.0 : 0.0;
     }
     n += __popc(m);
   }
@@ -624,6 +628,10 @@ __device__ __forceinline__ void warp_correct(const double* __restrict__ U, const
     }
     const double e[4] = {v[1] - v[0], v[2] - v[1], v[3] - v[2], v[4] - v[3]};
     const unsigned sel = teno_select(v, e, S);
+    if constexpr (SELECT) {
+      W.d[b][o] = double(sel);
+      continue;
+    }
     double dl = 0.0;
     if (it >> 9) {
       dl = fma(c_lin[sel][0], v[0], fma(c_lin[sel][1], v[1], fma(c_lin[sel][2], v[2], fma(c_lin[sel][3], v[3], c_lin[sel][4] * v[4]))));
@@ -634,6 +642,12 @@ __device__ __forceinline__ void warp_correct(const double* __restrict__ U, const
     W.d[b][o] = dl;
   }
   __syncwarp();
+  if constexpr (SELECT) {
+    uint32_t w = 0;
+#pragma unroll
+    for (int b = 0; b < NREC; ++b) w |= static_cast<uint32_t>(W.d[b][lane]) << (3 * b);
+    return w;
+  }
   if (open) {
     // back-projection of the differences (the whole values), as interface_flux's
     double f[NVAR];
@@ -662,6 +676,7 @@ __device__ __forceinline__ void warp_correct(const double* __restrict__ U, const
     }
     out[NVAR - 1] += eng;
   }
+  return 0u;
 }
 
 // ---------------------------------------------------------------------------
