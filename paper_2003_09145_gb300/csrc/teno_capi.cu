@@ -80,6 +80,7 @@ struct Layout {
   // counters (3 x 4)
   size_t status = 0, dt = 8, alpha = 64;
   size_t aux = 0, fh = 0, pf = 0, fhat = 0, list = 0, ghost = 0, R = 0, U1 = 0, U2 = 0, total = 0;
+  int64_t fstride = 0, lstride = 0;   // per-direction flux buffers and lists (kMultiCells); 0: shared
 };
 
 Layout layout_of(const teno_grid* g, int op) {
@@ -95,10 +96,15 @@ Layout layout_of(const teno_grid* g, int op) {
   off += round_up(sizeof(double) * g->ndim * (nvar - 1) * ncell);
   L.pf = off;   // binary32 copies of the cells (store_planes)
   off += round_up(sizeof(float4) * teno::plane_count(g->ndim) * ncell);
+  const int copies = ncell <= size_t(teno::kMultiCells) ? g->ndim : 1;
+  if (copies > 1) {
+    L.fstride = nvar * maxifc;
+    L.lstride = maxifc;
+  }
   L.fhat = off;
-  off += round_up(sizeof(double) * nvar * size_t(maxifc));
+  off += round_up(sizeof(double) * nvar * size_t(maxifc) * copies);
   L.list = off;
-  off += round_up(sizeof(uint2) * size_t(maxifc));
+  off += round_up(sizeof(uint2) * size_t(maxifc) * copies);
   L.ghost = off;   // fixed-state ghost cells (state, primitives, half fluxes of 6 face slots)
   off += round_up(sizeof(double) * size_t(teno::ghost_block_doubles(g->ndim)));
   if (op == TENO_OP_RK3) {
@@ -274,6 +280,27 @@ teno_status stage_finish(const teno_grid* g, const Layout& L, char* ws, const do
   if (with_dt) {
     TimerScope ts(st, TENO_KERNEL_DT);
     TENO_CUDA(teno::launch_dt(g->ndim, alpha, G, cfl, dt_fixed, t_dev, t_end, dt_ws, dt_out, st));
+  }
+  if (L.fstride && !flags) {
+    {
+      TimerScope ts(st, TENO_KERNEL_FLUX);
+      int nl = 0;
+      for (int d = 0; d < g->ndim; ++d) {
+        int k = 1;
+        TENO_CUDA(teno::launch_flux(g->ndim, d, U, aux, fh, pf, alpha, Fhat + d * L.fstride, nullptr,
+                                    list + d * L.lstride, count + d, status, G, S, nsm, st, &k, nullptr, false));
+        nl += k;
+      }
+      if (S.variant != teno::kSchemeWenoZ) {
+        TENO_CUDA(teno::launch_correct_all(g->ndim, U, aux, alpha, Fhat, L.fstride, list, L.lstride, count, status, G,
+                                           S, nsm, st));
+        ++nl;
+      }
+      ts.launches(nl);
+    }
+    TimerScope ts(st, TENO_KERNEL_DIFF);
+    TENO_CUDA(teno::launch_diff_all(g->ndim, Fhat, L.fstride, R, Un, Uk, Uout, dt_ws, G, mode_last, nsm, st, U));
+    return TENO_OK;
   }
   int64_t foff = 0;
   for (int d = 0; d < g->ndim; ++d) {

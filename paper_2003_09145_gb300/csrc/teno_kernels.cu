@@ -190,37 +190,30 @@ __global__ void __launch_bounds__(256, TENO_CELL_MINBLOCKS) cell_kernel(const do
 // The arg-max cells of the nine LF speeds from the cell pass's per-block
 // candidates: the largest value of each speed and the lowest cell index
 // attaining it (entries of unused directions stay as they are).
-constexpr int kArgThreads = 256;
+// One warp per speed (one block-wide reduction after another took 16 us).
+constexpr int kArgThreads = 288;
 __global__ void __launch_bounds__(kArgThreads) argmax_finish_kernel(const unsigned long long* __restrict__ cand,
                                                                     int nblocks, int nspeed,
                                                                     unsigned long long* __restrict__ argidx) {
-  __shared__ unsigned long long sv[kArgThreads];
-  __shared__ unsigned long long sa[kArgThreads];
-  for (int k = 0; k < nspeed; ++k) {
-    unsigned long long v = 0, a = ~0ull;
-    for (int b = threadIdx.x; b < nblocks; b += kArgThreads) {
-      const unsigned long long x = cand[(b * 9 + k) * 2], i = cand[(b * 9 + k) * 2 + 1];
-      if (x > v || (x == v && i < a)) {
-        v = x;
-        a = i;
-      }
+  const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
+  if (k >= nspeed) return;
+  unsigned long long v = 0, a = ~0ull;
+  for (int b = lane; b < nblocks; b += 32) {
+    const unsigned long long x = cand[(b * 9 + k) * 2], i = cand[(b * 9 + k) * 2 + 1];
+    if (x > v || (x == v && i < a)) {
+      v = x;
+      a = i;
     }
-    sv[threadIdx.x] = v;
-    sa[threadIdx.x] = a;
-    __syncthreads();
-    for (int w = kArgThreads / 2; w > 0; w >>= 1) {
-      if (threadIdx.x < w) {
-        const unsigned long long x = sv[threadIdx.x + w], i = sa[threadIdx.x + w];
-        if (x > sv[threadIdx.x] || (x == sv[threadIdx.x] && i < sa[threadIdx.x])) {
-          sv[threadIdx.x] = x;
-          sa[threadIdx.x] = i;
-        }
-      }
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) argidx[k] = sa[0];
-    __syncthreads();
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long x = __shfl_down_sync(0xffffffffu, v, o), i = __shfl_down_sync(0xffffffffu, a, o);
+    if (x > v || (x == v && i < a)) {
+      v = x;
+      a = i;
+    }
+  }
+  if (lane == 0) argidx[k] = a;
 }
 
 // ---------------------------------------------------------------------------
@@ -472,15 +465,13 @@ __global__ void __launch_bounds__(128, TENO_CLOSED_MINBLOCKS) flux_closed_kernel
 // the chip, and fewer (2, 4, 8, 16) when the list is short: a short list is
 // bound by one warp's chain, and few interfaces finish in a single round.
 template <int NDIM, int DIR, bool GH>
-__global__ void __launch_bounds__(128) flux_correct_kernel(
-    const double* __restrict__ U, const double* __restrict__ aux,
-    const unsigned long long* __restrict__ alpha_bits, double* __restrict__ Fhat,
-    const uint2* __restrict__ list, const unsigned* __restrict__ count, int* __restrict__ status,
-    Grid G, Scheme S, int nsm) {
+__device__ __forceinline__ void correct_list(const double* __restrict__ U, const double* __restrict__ aux,
+                                             const unsigned long long* __restrict__ alpha_bits,
+                                             double* __restrict__ Fhat, const uint2* __restrict__ list, int64_t n,
+                                             int* __restrict__ status, const Grid& G, const Scheme& S, int nsm,
+                                             CorrectScratch<NDIM>& W) {
   constexpr int NVAR = NDIM + 2;
-  __shared__ CorrectScratch<NDIM> scratch[4];
   const int64_t nifc = (G.n[0] + (DIR == 0)) * (G.n[1] + (DIR == 1)) * (G.n[2] + (DIR == 2));
-  const int64_t n = *count;
   const int64_t nw = (int64_t)gridDim.x * 4;
   int per = 2;
   while (per < 32 && n > (int64_t)per * 4 * nsm) per *= 2;
@@ -488,8 +479,10 @@ __global__ void __launch_bounds__(128) flux_correct_kernel(
   if (blockIdx.x * (int64_t)(4 * per) >= n) return;
   double alpha[NVAR], nal[NVAR];
   half_speeds<NDIM, DIR>(alpha_bits, alpha, nal);
+  const bool ghost_dir = GH && G.bc[DIR] == TENO_BC_DIRICHLET;
   auto cells_of = [&](uint32_t q, uint32_t (&cells)[6], unsigned& flips) {
-    interface_cells<NDIM, DIR, GH>(q, G, cells, flips);
+    if (ghost_dir) interface_cells<NDIM, DIR, GH>(q, G, cells, flips);
+    else interface_cells<NDIM, DIR, false>(q, G, cells, flips);
   };
   for (int64_t i0 = ((int64_t)blockIdx.x * 4 + warp) * per; i0 < n; i0 += nw * per) {
     const int64_t i = i0 + lane;
@@ -497,12 +490,43 @@ __global__ void __launch_bounds__(128) flux_correct_kernel(
     double out[NVAR];
 #pragma unroll
     for (int v = 0; v < NVAR; ++v) out[v] = e.y && !(e.y & kRough) ? Fhat[(int64_t)v * nifc + e.x] : 0.0;
-    warp_correct<NDIM, DIR, GH, uint32_t>(U, aux, G.ncell, cells_of, e.x, alpha, S, e.y, out, status, scratch[warp],
-                                GhostCells{G.gU, G.gaux, G.gfh, G.gpf});
+    warp_correct<NDIM, DIR, GH, uint32_t>(U, aux, G.ncell, cells_of, e.x, alpha, S, e.y, out, status, W,
+                                          GhostCells{G.gU, G.gaux, G.gfh, G.gpf});
     if (e.y)
 #pragma unroll
       for (int v = 0; v < NVAR; ++v) Fhat[(int64_t)v * nifc + e.x] = out[v];
   }
+}
+
+template <int NDIM, int DIR, bool GH>
+__global__ void __launch_bounds__(128) flux_correct_kernel(
+    const double* __restrict__ U, const double* __restrict__ aux,
+    const unsigned long long* __restrict__ alpha_bits, double* __restrict__ Fhat,
+    const uint2* __restrict__ list, const unsigned* __restrict__ count, int* __restrict__ status,
+    Grid G, Scheme S, int nsm) {
+  __shared__ CorrectScratch<NDIM> scratch[4];
+  correct_list<NDIM, DIR, GH>(U, aux, alpha_bits, Fhat, list, *count, status, G, S, nsm, scratch[threadIdx.x >> 5]);
+}
+
+// The lists of every direction in one launch (blockIdx.y: the direction), each
+// with its own fluxes and list (stages of small and medium grids).
+template <int NDIM, bool GH>
+__global__ void __launch_bounds__(128) flux_correct_all_kernel(
+    const double* __restrict__ U, const double* __restrict__ aux,
+    const unsigned long long* __restrict__ alpha_bits, double* __restrict__ Fhat, int64_t fstride,
+    const uint2* __restrict__ list, int64_t lstride, const unsigned* __restrict__ count, int* __restrict__ status,
+    Grid G, Scheme S, int nsm) {
+  __shared__ CorrectScratch<NDIM> scratch[4];
+  CorrectScratch<NDIM>& W = scratch[threadIdx.x >> 5];
+  const int d = blockIdx.y;
+  const int64_t n = count[d];
+  Fhat += d * fstride;
+  list += d * lstride;
+  if (d == 0) correct_list<NDIM, 0, GH>(U, aux, alpha_bits, Fhat, list, n, status, G, S, nsm, W);
+  if constexpr (NDIM > 1)
+    if (d == 1) correct_list<NDIM, 1, GH>(U, aux, alpha_bits, Fhat, list, n, status, G, S, nsm, W);
+  if constexpr (NDIM > 2)
+    if (d == 2) correct_list<NDIM, 2, GH>(U, aux, alpha_bits, Fhat, list, n, status, G, S, nsm, W);
 }
 
 template <int NDIM, int DIR, bool GH>
@@ -632,6 +656,79 @@ __global__ void __launch_bounds__(256) diff_kernel(
 #pragma unroll
       for (int v = 0; v < NVAR; ++v) Uout[v * ncell + cc] = o[v];
     }
+  }
+}
+
+// The differences of every direction and the last one's MODE in one pass
+// (kDiffRhs or a stage 2, 3, 4), from one flux buffer per direction: the
+// per-direction passes' operations in their order, with the partial sum in a
+// register instead of R -- the same results bit for bit in one launch
+// instead of ndim.
+template <int NDIM, int DIR>
+__device__ __forceinline__ void add_direction(const double* __restrict__ Fhat, int64_t fstride, const Grid& G,
+                                              uint32_t c, double (&s)[NDIM + 2]) {
+  if constexpr (DIR < NDIM) {
+    const uint32_t n0 = static_cast<uint32_t>(G.n[0]), n01 = n0 * static_cast<uint32_t>(G.n[1]);
+    const int64_t m0 = G.n[0] + (DIR == 0), m1 = G.n[1] + (DIR == 1);
+    const int64_t nifc = m0 * m1 * (G.n[2] + (DIR == 2));
+    const int64_t left = DIR == 0 ? (int64_t)c + c / n0 : (DIR == 1 ? (int64_t)c + (int64_t)(c / n01) * n0 : (int64_t)c);
+    const int64_t right = left + (DIR == 0 ? 1 : (DIR == 1 ? m0 : m0 * m1));
+    const double* F = Fhat + DIR * fstride;
+#pragma unroll
+    for (int v = 0; v < NDIM + 2; ++v) {
+      const double t = F[v * nifc + left] - F[v * nifc + right];
+      s[v] = DIR == 0 ? t : fma(G.rdx[DIR], t, s[v]);
+    }
+    add_direction<NDIM, DIR + 1>(Fhat, fstride, G, c, s);
+  }
+}
+
+template <int NDIM, int MODE, bool GRAV>
+__global__ void __launch_bounds__(256) diff_all_kernel(const double* __restrict__ Fhat, int64_t fstride,
+                                                       double* R, const double* Un, const double* Uk, double* Uout,
+                                                       const double* __restrict__ dt_ptr, Grid G,
+                                                       const double* Usrc) {
+  constexpr bool stage = MODE != kDiffRhs;
+  constexpr int NVAR = NDIM + 2;
+  const int64_t ncell = G.ncell;
+  const double idf = G.inv_dx[0] / kFluxScale;
+  double c = 0.0;
+  if (stage) {
+    const double dt = *dt_ptr;
+    if (!(dt > 0.0)) {   // as diff_kernel
+      if (MODE <= 3)
+        for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < NVAR * ncell;
+             e += (int64_t)gridDim.x * blockDim.x)
+          Uout[e] = Un[e];
+      return;
+    }
+    c = dt * idf;
+  }
+  for (int64_t cc = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; cc < ncell;
+       cc += (int64_t)gridDim.x * blockDim.x) {
+    double s[NVAR], src[NVAR];
+    add_direction<NDIM, 0>(Fhat, fstride, G, static_cast<uint32_t>(cc), s);
+    if (GRAV) {
+      const double rho = Usrc[cc];
+      double w = 0.0;
+      src[0] = 0.0;
+#pragma unroll
+      for (int k = 0; k < NDIM; ++k) {
+        src[1 + k] = rho * G.grav[k];
+        w = fma(Usrc[(1 + k) * ncell + cc], G.grav[k], w);
+      }
+      src[NVAR - 1] = w;
+      if (stage)
+#pragma unroll
+        for (int v = 1; v < NVAR; ++v) s[v] = fma(kFluxScale * G.dx[0], src[v], s[v]);
+    }
+    double o[NVAR];
+#pragma unroll
+    for (int v = 0; v < NVAR; ++v)
+      o[v] = stage ? stage_value(MODE, c, s[v], Un, Uk, v * ncell + cc) : (GRAV ? fma(s[v], idf, src[v]) : s[v] * idf);
+    double* out = stage ? Uout : R;
+#pragma unroll
+    for (int v = 0; v < NVAR; ++v) out[v * ncell + cc] = o[v];
   }
 }
 
@@ -838,7 +935,7 @@ template <int NDIM, int DIR>
 static int flux_launch(int blocks, int threads, int pblocks, int nsm, cudaStream_t st, const double* U,
                        const double* aux, const double* fh, const float4* pf, const unsigned long long* alpha,
                        double* Fhat, uint8_t* flags, uint2* list, unsigned* count, int* status, const Grid& G,
-                       const Scheme& S, double* roe_out) {
+                       const Scheme& S, double* roe_out, bool correct) {
   const bool gh = G.bc[DIR] == TENO_BC_DIRICHLET;
   if (flags || !list) {
     if (flags && gh) flux_kernel<NDIM, DIR, true, true><<<blocks, threads, 0, st>>>(U, aux, alpha, Fhat, flags, status, G, S);
@@ -861,6 +958,7 @@ static int flux_launch(int blocks, int threads, int pblocks, int nsm, cudaStream
                                                                       G, S, roe_out);
   else
     flux_closed_kernel<NDIM, DIR, 0><<<blocks, threads, 0, st>>>(U, aux, fh, pf, alpha, Fhat, list, count, status, G, S);
+  if (!correct) return 1;
   if (gh)
     flux_correct_kernel<NDIM, DIR, true><<<pblocks, threads, 0, st>>>(U, aux, alpha, Fhat, list, count, status, G, S, nsm);
   else
@@ -872,7 +970,7 @@ cudaError_t launch_flux(int ndim, int dir, const double* U, const double* aux, c
                         const unsigned long long* alpha, double* Fhat,
                         uint8_t* flags, uint2* list, unsigned* count, int* status,
                         const Grid& G, const Scheme& S, int nsm, cudaStream_t st,
-                        int* launches, double* roe_out) {
+                        int* launches, double* roe_out, bool correct) {
   int64_t nifc = 1;
   for (int k = 0; k < 3; ++k) nifc *= G.n[k] + (k == dir ? 1 : 0);
   if (nifc > int64_t(UINT32_MAX)) list = nullptr;   // list entries are 32-bit
@@ -881,16 +979,66 @@ cudaError_t launch_flux(int ndim, int dir, const double* U, const double* aux, c
   const int blocks = blocks_for(nifc, threads, nsm * 64);
   const int pblocks = blocks_for(nifc, threads, nsm * 16);
   int n = 0;
-  if (ndim == 1) n = flux_launch<1, 0>(blocks, threads, pblocks, nsm, st, U, aux, fh, pf, alpha, Fhat, flags, list, count, status, G, S, roe_out);
+  if (ndim == 1) n = flux_launch<1, 0>(blocks, threads, pblocks, nsm, st, U, aux, fh, pf, alpha, Fhat, flags, list, count, status, G, S, roe_out, correct);
   else if (ndim == 2) {
-    if (dir == 0) n = flux_launch<2, 0>(blocks, threads, pblocks, nsm, st, U, aux, fh, pf, alpha, Fhat, flags, list, count, status, G, S, roe_out);
-    else n = flux_launch<2, 1>(blocks, threads, pblocks, nsm, st, U, aux, fh, pf, alpha, Fhat, flags, list, count, status, G, S, roe_out);
+    if (dir == 0) n = flux_launch<2, 0>(blocks, threads, pblocks, nsm, st, U, aux, fh, pf, alpha, Fhat, flags, list, count, status, G, S, roe_out, correct);
+    else n = flux_launch<2, 1>(blocks, threads, pblocks, nsm, st, U, aux, fh, pf, alpha, Fhat, flags, list, count, status, G, S, roe_out, correct);
   } else {
-    if (dir == 0) n = flux_launch<3, 0>(blocks, threads, pblocks, nsm, st, U, aux, fh, pf, alpha, Fhat, flags, list, count, status, G, S, roe_out);
-    else if (dir == 1) n = flux_launch<3, 1>(blocks, threads, pblocks, nsm, st, U, aux, fh, pf, alpha, Fhat, flags, list, count, status, G, S, roe_out);
-    else n = flux_launch<3, 2>(blocks, threads, pblocks, nsm, st, U, aux, fh, pf, alpha, Fhat, flags, list, count, status, G, S, roe_out);
+    if (dir == 0) n = flux_launch<3, 0>(blocks, threads, pblocks, nsm, st, U, aux, fh, pf, alpha, Fhat, flags, list, count, status, G, S, roe_out, correct);
+    else if (dir == 1) n = flux_launch<3, 1>(blocks, threads, pblocks, nsm, st, U, aux, fh, pf, alpha, Fhat, flags, list, count, status, G, S, roe_out, correct);
+    else n = flux_launch<3, 2>(blocks, threads, pblocks, nsm, st, U, aux, fh, pf, alpha, Fhat, flags, list, count, status, G, S, roe_out, correct);
   }
   if (launches) *launches = n;
+  return cudaGetLastError();
+}
+
+cudaError_t launch_correct_all(int ndim, const double* U, const double* aux, const unsigned long long* alpha,
+                               double* Fhat, int64_t fstride, const uint2* list, int64_t lstride,
+                               const unsigned* count, int* status, const Grid& G, const Scheme& S, int nsm,
+                               cudaStream_t st) {
+  int64_t nifc = 0;
+  bool gh = false;
+  for (int d = 0; d < ndim; ++d) {
+    int64_t m = 1;
+    for (int k = 0; k < 3; ++k) m *= G.n[k] + (k == d ? 1 : 0);
+    nifc = m > nifc ? m : nifc;
+    gh = gh || G.bc[d] == TENO_BC_DIRICHLET;
+  }
+  const dim3 grid(unsigned(blocks_for(nifc, 128, nsm * 16)), unsigned(ndim));
+  if (ndim == 1) {
+    if (gh) flux_correct_all_kernel<1, true><<<grid, 128, 0, st>>>(U, aux, alpha, Fhat, fstride, list, lstride, count, status, G, S, nsm);
+    else flux_correct_all_kernel<1, false><<<grid, 128, 0, st>>>(U, aux, alpha, Fhat, fstride, list, lstride, count, status, G, S, nsm);
+  } else if (ndim == 2) {
+    if (gh) flux_correct_all_kernel<2, true><<<grid, 128, 0, st>>>(U, aux, alpha, Fhat, fstride, list, lstride, count, status, G, S, nsm);
+    else flux_correct_all_kernel<2, false><<<grid, 128, 0, st>>>(U, aux, alpha, Fhat, fstride, list, lstride, count, status, G, S, nsm);
+  } else {
+    if (gh) flux_correct_all_kernel<3, true><<<grid, 128, 0, st>>>(U, aux, alpha, Fhat, fstride, list, lstride, count, status, G, S, nsm);
+    else flux_correct_all_kernel<3, false><<<grid, 128, 0, st>>>(U, aux, alpha, Fhat, fstride, list, lstride, count, status, G, S, nsm);
+  }
+  return cudaGetLastError();
+}
+
+template <int NDIM, bool GRAV>
+static void diff_all_launch(int blocks, cudaStream_t st, const double* Fhat, int64_t fstride, double* R,
+                            const double* Un, const double* Uk, double* Uout, const double* dt, const Grid& G, int mode,
+                            const double* Usrc) {
+  switch (mode) {
+    case 0: diff_all_kernel<NDIM, kDiffRhs, GRAV><<<blocks, 256, 0, st>>>(Fhat, fstride, R, Un, Uk, Uout, dt, G, Usrc); break;
+    case 2: diff_all_kernel<NDIM, 2, GRAV><<<blocks, 256, 0, st>>>(Fhat, fstride, R, Un, Uk, Uout, dt, G, Usrc); break;
+    case 3: diff_all_kernel<NDIM, 3, GRAV><<<blocks, 256, 0, st>>>(Fhat, fstride, R, Un, Uk, Uout, dt, G, Usrc); break;
+    default: diff_all_kernel<NDIM, 4, GRAV><<<blocks, 256, 0, st>>>(Fhat, fstride, R, Un, Uk, Uout, dt, G, Usrc); break;
+  }
+}
+
+cudaError_t launch_diff_all(int ndim, const double* Fhat, int64_t fstride, double* R, const double* Un,
+                            const double* Uk, double* Uout, const double* dt, const Grid& G, int mode, int nsm,
+                            cudaStream_t st, const double* Usrc) {
+  if (mode != 0 && (mode < 2 || mode > 4)) return cudaErrorInvalidValue;
+  const int blocks = blocks_for(G.ncell, 256, nsm * 16);
+  const bool g = G.has_grav;
+  if (ndim == 1) (g ? diff_all_launch<1, true> : diff_all_launch<1, false>)(blocks, st, Fhat, fstride, R, Un, Uk, Uout, dt, G, mode, Usrc);
+  else if (ndim == 2) (g ? diff_all_launch<2, true> : diff_all_launch<2, false>)(blocks, st, Fhat, fstride, R, Un, Uk, Uout, dt, G, mode, Usrc);
+  else (g ? diff_all_launch<3, true> : diff_all_launch<3, false>)(blocks, st, Fhat, fstride, R, Un, Uk, Uout, dt, G, mode, Usrc);
   return cudaGetLastError();
 }
 
