@@ -74,7 +74,8 @@ cudaError_t launch_diff(int ndim, int dir, const double* Fhat, double* R,
                         const double* dt, const Grid& G, int mode,
                         int nsm, cudaStream_t st, const double* Usrc);
 
-// Small and medium grids (up to kMultiCells cells) keep one flux buffer and
+// Grids up to kMultiCells cells (a 256^3 step: 21.59 against 21.40 ms; beyond
+// that the buffers' memory counts) keep one flux buffer and
 // one list per direction (fstride, lstride entries apart): the lists of all
 // directions are corrected in one launch and the differences taken in one
 // pass, instead of ndim launches each of which is a few microseconds of
@@ -82,7 +83,7 @@ cudaError_t launch_diff(int ndim, int dir, const double* Fhat, double* R,
 // 512^2 step 438 against 407, 129 x 515 with walls and gravity 253 against
 // 203, a 64^3 step 959 against 862, a 97 x 61 x 45 right-hand side 407
 // against 354.
-constexpr int64_t kMultiCells = int64_t(1) << 22;
+constexpr int64_t kMultiCells = int64_t(1) << 25;
 cudaError_t launch_correct_all(int ndim, const double* U, const double* aux, const unsigned long long* alpha,
                                double* Fhat, int64_t fstride, const uint2* list, int64_t lstride,
                                const unsigned* count, int* status, const Grid& G, const Scheme& S, int nsm,
