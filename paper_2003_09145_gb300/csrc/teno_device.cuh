@@ -268,6 +268,40 @@ __device__ __forceinline__ int teno5a_magnitude(double e0, double e1, double e2,
 }
 
 // ---------------------------------------------------------------------------
+// WENO-Z on the indicator terms a_k, c_k (see teno5_lad): omega_k = a_k / sum_j
+// a_j with a_k = c_k (1 + tau / D_k), D_k = beta_k + eps (carried times 4; the
+// factor cancels).  eps enters the indicators' own sums, and tau = |D_2 - D_0|
+// (off by the D's rounding only, which 1 + tau / D_k has anyway).  With N_k =
+// D_k + tau and A_k = 10 c_k N_k prod_{j != k} D_j, omega_k = A_k / sum A (three
+// divisions where the products leave the range).  The weights enter f^ = v2 +
+// sum_k w_k e_k (see c_cut) unnormalised,
+//   6 sum A sum_k w_k e_k = -2 A0 e0 + (5 A0 + A1) e1 + (2 A1 + 4 A2) e2 - A2 e3,
+// and one reciprocal of 6 sum A divides: every interface takes this path on
+// every field and side, bound by FP64 issue, and this is 17 instructions fewer
+// than three weights by a division and four coefficients.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ double weno_z(double e0, double e1, double e2, double e3, double a0, double a1, double a2,
+                                         double c0, double c1, double c2, double v2, double acc, double eps4,
+                                         unsigned& flag) {
+  const double k13_3 = 13.0 / 3.0;
+  const double d0 = fma(k13_3 * a0, a0, fma(c0, c0, eps4));
+  const double d1 = fma(k13_3 * a1, a1, fma(c1, c1, eps4));
+  const double d2 = fma(k13_3 * a2, a2, fma(c2, c2, eps4));
+  const double tau = fabs(d2 - d0);
+  double A0 = (d0 + tau) * (d1 * d2), A1 = 6.0 * ((d1 + tau) * (d0 * d2)), A2 = 3.0 * ((d2 + tau) * (d0 * d1));
+  double As = A0 + A1 + A2;
+  if (!pos_finite(As)) {
+    A0 = 1.0 + tau / d0;
+    A1 = 6.0 * (1.0 + tau / d1);
+    A2 = 3.0 * (1.0 + tau / d2);
+    As = A0 + A1 + A2;
+  }
+  flag = 7u;
+  const double q = fma(-2.0 * A0, e0, fma(fma(5.0, A0, A1), e1, fma(fma(4.0, A2, 2.0 * A1), e2, -A2 * e3)));
+  return fma(q, recip_pos(6.0 * As), v2 + acc);
+}
+
+// ---------------------------------------------------------------------------
 // TENO5-LAD scalar reconstruction of the interface value from five values
 // v0..v4 = (f_{i-2}, ..., f_{i+2}).  Returns acc + f^ (eq. 2.7); `flag`
 // receives delta bits 0..2 and m in bits 3..6.
@@ -311,6 +345,7 @@ __device__ __forceinline__ double teno5_lad(double v0, double v1, double v2,
   const double c0 = fma(3.0, e1, -e0);
   const double c1 = e1 + e2;
   const double c2 = fma(-3.0, e2, e3);
+  if (S.variant == kSchemeWenoZ) return weno_z(e0, e1, e2, e3, a0, a1, a2, c0, c1, c2, v2, acc, S.eps4, flag);
   const double beta0 = fma(k13_3 * a0, a0, c0 * c0);
   const double beta1 = fma(k13_3 * a1, a1, c1 * c1);
   const double beta2 = fma(k13_3 * a2, a2, c2 * c2);
@@ -322,29 +357,6 @@ __device__ __forceinline__ double teno5_lad(double v0, double v1, double v2,
   const unsigned long long btau = dbits(tau);
   unsigned sel = 7u;
   int m = S.b_u;
-  if (S.variant == kSchemeWenoZ) {
-    // WENO-Z: omega_k = a_k / sum_j a_j with a_k = c_k (1 + tau / D_k),
-    // D_k = beta_k + eps (the common factor 4 cancels); with N_k = D_k + tau
-    // and A_k = 10 c_k N_k prod_{j != k} D_j = 10 a_k D_0 D_1 D_2, omega_k =
-    // A_k / sum A (three divisions where the products leave the range).  The
-    // weights enter f^ = v2 + sum_k w_k e_k (see c_cut) unnormalised,
-    //   6 sum A sum_k w_k e_k = -2 A0 e0 + (5 A0 + A1) e1 + (2 A1 + 4 A2) e2 - A2 e3,
-    // and one reciprocal of 6 sum A divides: every interface takes this path
-    // ten times, bound by FP64 issue, and this is 14 instructions fewer than
-    // a division, three weights and four coefficients.
-    const double d0 = beta0 + S.eps4, d1 = beta1 + S.eps4, d2 = beta2 + S.eps4;
-    double A0 = (d0 + tau) * (d1 * d2), A1 = 6.0 * ((d1 + tau) * (d0 * d2)), A2 = 3.0 * ((d2 + tau) * (d0 * d1));
-    double As = A0 + A1 + A2;
-    if (!pos_finite(As)) {
-      A0 = 1.0 + tau / d0;
-      A1 = 6.0 * (1.0 + tau / d1);
-      A2 = 3.0 * (1.0 + tau / d2);
-      As = A0 + A1 + A2;
-    }
-    flag = 7u;
-    const double q = fma(-2.0 * A0, e0, fma(fma(5.0, A0, A1), e1, fma(fma(4.0, A2, 2.0 * A1), e2, -A2 * e3)));
-    return fma(q, recip_pos(6.0 * As), v2 + acc);
-  }
   if (!WITH_M && S.keep_idx >= 0 && btau <= dbits(S.thr[S.keep_idx] * dmin)) {
     // tau below the keep-all threshold: every stencil is kept (for LAD, m
     // lies in the keep-all range, a suffix of B_l..B_u; for TENO5 and
