@@ -285,7 +285,13 @@ teno_status stage_finish(const teno_grid* g, const Layout& L, char* ws, const do
     {
       TimerScope ts(st, TENO_KERNEL_FLUX);
       int nl = 0;
-      for (int d = 0; d < g->ndim; ++d) {
+      const bool one = g->ndim > 1 && S.variant != teno::kSchemeWenoZ && G.ncell <= teno::kClosedAllCells;
+      if (one) {
+        TENO_CUDA(teno::launch_closed_all(g->ndim, U, aux, fh, pf, alpha, Fhat, L.fstride, list, L.lstride, count,
+                                          status, G, S, nsm, st));
+        nl = 1;
+      }
+      for (int d = 0; d < (one ? 0 : g->ndim); ++d) {
         int k = 1;
         TENO_CUDA(teno::launch_flux(g->ndim, d, U, aux, fh, pf, alpha, Fhat + d * L.fstride, nullptr,
                                     list + d * L.lstride, count + d, status, G, S, nsm, st, &k, nullptr, false));

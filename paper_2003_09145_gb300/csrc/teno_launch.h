@@ -83,7 +83,11 @@ cudaError_t launch_diff(int ndim, int dir, const double* Fhat, double* R,
 // 512^2 step 438 against 407, 129 x 515 with walls and gravity 253 against
 // 203, a 64^3 step 959 against 862, a 97 x 61 x 45 right-hand side 407
 // against 354.
-constexpr int64_t kMultiCells = int64_t(1) << 25;
+constexpr int64_t kMultiCells = int64_t(1) << 25, kClosedAllCells = int64_t(1) << 17;
+cudaError_t launch_closed_all(int ndim, const double* U, const double* aux, const double* fh, const float4* pf,
+                              const unsigned long long* alpha, double* Fhat, int64_t fstride, uint2* list,
+                              int64_t lstride, unsigned* count, int* status, const Grid& G, const Scheme& S, int nsm,
+                              cudaStream_t st);
 cudaError_t launch_correct_all(int ndim, const double* U, const double* aux, const unsigned long long* alpha,
                                double* Fhat, int64_t fstride, const uint2* list, int64_t lstride,
                                const unsigned* count, int* status, const Grid& G, const Scheme& S, int nsm,
