@@ -50,7 +50,10 @@ FP64_FLOP_PER_CLK_PER_SM = 4          # 2 FP64 FMA lanes per SM per clock
 #   (exact terms, one rounding: teno_fixsum.cuh) and the other four
 #   P-weighted sums as binary64 chains that skip the products with weights
 #   +-1 (9 of their 12 flops), so 187 - 6 x 12 - 4 x 3 = 103 flops per
-#   interface run on the FP64 pipe: fp64_flops_per_interface.  The roofline keeps the
+#   interface are left to the FP64 pipe where the Roe state and the
+#   corrections run in binary64 too (FP64_CLOSED_3D: near shocks).  Elsewhere
+#   those run as two binary32 values (teno_df.cuh) and 4 x (9 + 1) + 1 = 41
+#   remain: FP64_PIPE_3D, fp64_flops_per_interface.  The roofline keeps the
 #   algorithmic count against the FP64 peak, the rate at which binary64
 #   could evaluate the same arithmetic.
 # * Otherwise the characteristic path: Roe 27, projection 6 x 20, split 6 x 28,
@@ -74,6 +77,7 @@ def alg_counts(ndim: int):
 
 ALG_CLOSED_3D, ALG_FIXED_3D = alg_counts(3)
 FP64_CLOSED_3D = ALG_CLOSED_3D - 6 * 12 - 4 * 3   # the closed form's flops on the FP64 pipe
+FP64_PIPE_3D = 41
 ALG_PER_RECON_KEEP = 9
 ALG_PER_RECON = 38
 ALG_CUTOFF = 21
@@ -646,7 +650,7 @@ def main() -> None:
                                f"{sm_max:.0f} MHz (max SM clock)",
                 "fp64_probe_tflops": probe,
                 "alg_flops_per_interface": alg_per_ifc,
-                "fp64_flops_per_interface": alg_per_ifc - (ALG_CLOSED_3D - FP64_CLOSED_3D) * closed_frac,
+                "fp64_flops_per_interface": alg_per_ifc - (ALG_CLOSED_3D - FP64_PIPE_3D) * closed_frac,
                 "fixed_point_sums": "closed form: the five M-weighted sums (60 U~) and the mass flux's "
                                     "P-weighted sum in 64-bit fixed point on the integer pipes (terms "
                                     "truncated 3 bits below the largest value's ulp, summed exactly, "
