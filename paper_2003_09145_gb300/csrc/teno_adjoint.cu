@@ -146,9 +146,12 @@ __device__ __forceinline__ void add_alpha(const double (&ab)[NVAR], double (&asu
 
 // The forward's certificate at one interface (interface_flux_closed's open
 // mask): on the Roe state in two binary32 values, or on the binary64 one
-// outside their range.  Out of line: its registers are its own.
+// outside their range.  Out of line: its registers are its own.  pf: the cell
+// pass's binary32 planes of U where it wrote them (else the same values are
+// converted here).
 template <int NDIM, int DIR>
 __device__ __noinline__ unsigned forward_open(const double* __restrict__ U, const double* __restrict__ aux,
+                                              const float4* __restrict__ pf,
                                               int64_t ncell, int64_t line, int64_t id, int64_t nd, int64_t stride, int bc,
                                               double am, double a0, double ap, const Scheme& S, int* status) {
   constexpr int NVAR = NDIM + 2;
@@ -167,7 +170,11 @@ __device__ __noinline__ unsigned forward_open(const double* __restrict__ U, cons
   const double sr2 = aux[(NDIM + 1) * ncell + cells[2]], sr3 = aux[(NDIM + 1) * ncell + cells[3]];
   const double sh2 = aux[(NDIM + 2) * ncell + cells[2]], sh3 = aux[(NDIM + 2) * ncell + cells[3]];
   teno::RoeDf<NDIM> Rd;
-  teno::roe_df<NDIM>(teno::roe_cell<NDIM>(sr2, sh2, su2), teno::roe_cell<NDIM>(sr3, sh3, su3), S, Rd);
+  if (pf)
+    teno::roe_df<NDIM>(teno::load_roe_cell<NDIM, false>(pf, nullptr, ncell, cells[2]),
+                       teno::load_roe_cell<NDIM, false>(pf, nullptr, ncell, cells[3]), S, Rd);
+  else
+    teno::roe_df<NDIM>(teno::roe_cell<NDIM>(sr2, sh2, su2), teno::roe_cell<NDIM>(sr3, sh3, su3), S, Rd);
   teno::CertIfc<NDIM> C;
   for (bool df = F.in_range && teno::roe_df_ok<NDIM>(Rd, S);; df = false) {
     if (df) {
@@ -182,6 +189,12 @@ __device__ __noinline__ unsigned forward_open(const double* __restrict__ U, cons
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
       float X[NVAR];
+      if (pf && df) {
+        float u, p;
+        teno::load_point_f<NDIM, DIR, false>(pf, nullptr, ncell, cells[j], X, u, p);
+        teno_cert::cert_point_f<NDIM, DIR>(j, X, u, p, C);
+        continue;
+      }
       const double un = aux[DIR * ncell + cells[j]], pn = aux[NDIM * ncell + cells[j]];
 #pragma unroll
       for (int v = 0; v < NVAR; ++v) {
@@ -210,7 +223,8 @@ __global__ void __launch_bounds__(kAdjThreads, TENO_ADJ_KEPT_MINBLOCKS) adj_kept
     const double* __restrict__ U, const double* __restrict__ aux,
     const unsigned long long* __restrict__ alpha_bits, const double* __restrict__ Rbar, double scale,
     double* __restrict__ kb, unsigned char* __restrict__ pending, double* __restrict__ apart,
-    int* __restrict__ status, Grid G, Scheme S, const double* __restrict__ roe_in) {
+    int* __restrict__ status, Grid G, Scheme S, const double* __restrict__ roe_in,
+    const float4* __restrict__ pf) {
   constexpr int NVAR = NDIM + 2;
   const IfcGeom<NDIM, DIR> I(G);
   double fa[NVAR], ha[NVAR], nfa[NVAR];
@@ -247,7 +261,7 @@ __global__ void __launch_bounds__(kAdjThreads, TENO_ADJ_KEPT_MINBLOCKS) adj_kept
         su3[k] = aux[(NDIM + 3 + k) * I.ncell + cells[3]];
       }
       teno::roe_interface<NDIM, DIR>(sr2, sr3, sh2, sh3, su2, su3, S, Rf, status);
-      kept = forward_open<NDIM, DIR>(U, aux, I.ncell, base, id, I.nd, I.stride_d, I.bcd, ha[0], ha[1], ha[NVAR - 1], S,
+      kept = forward_open<NDIM, DIR>(U, aux, pf, I.ncell, base, id, I.nd, I.stride_d, I.bcd, ha[0], ha[1], ha[NVAR - 1], S,
                                      status) == 0u;
     }
     pending[q] = kept ? 0 : 1;
@@ -524,7 +538,8 @@ template <int NDIM, int DIR>
 __global__ void __launch_bounds__(kAdjThreads) adj_select_kernel(
     const double* __restrict__ U, const double* __restrict__ aux,
     const unsigned long long* __restrict__ alpha_bits, const uint32_t* __restrict__ list,
-    const int* __restrict__ count, uint32_t* __restrict__ sel, int* __restrict__ status, Grid G, Scheme S) {
+    const int* __restrict__ count, uint32_t* __restrict__ sel, int* __restrict__ status, Grid G, Scheme S,
+    const float4* __restrict__ pf) {
   constexpr int NVAR = NDIM + 2;
   __shared__ teno::CorrectScratch<NDIM> scratch[kAdjThreads / 32];
   const IfcGeom<NDIM, DIR> I(G);
@@ -546,7 +561,7 @@ __global__ void __launch_bounds__(kAdjThreads) adj_select_kernel(
       q = list[i];
       int64_t id, base, cells[6];
       I.locate(q, G, id, base, cells);
-      open = forward_open<NDIM, DIR>(U, aux, I.ncell, base, id, I.nd, I.stride_d, I.bcd, ha[0], ha[1], ha[NVAR - 1], S,
+      open = forward_open<NDIM, DIR>(U, aux, pf, I.ncell, base, id, I.nd, I.stride_d, I.bcd, ha[0], ha[1], ha[NVAR - 1], S,
                                      status);
     }
     double out[NVAR];
@@ -1053,13 +1068,14 @@ template <int NDIM, int DIR>
 void launch_adj_dir(int nblk, int nsm, cudaStream_t st, const double* U, const double* aux,
                     const unsigned long long* alpha, const double* Rbar, double scale, double* kb,
                     double* contrib, unsigned char* pending, uint32_t* list, int* lcount, uint32_t* sel,
-                    double* apart, int* status, const Grid& G, const Scheme& S, const double* roe_in) {
+                    double* apart, int* status, const Grid& G, const Scheme& S, const double* roe_in,
+                    const float4* pf) {
   if (roe_in)
     adj_kept_kernel<NDIM, DIR, true><<<nblk, kAdjThreads, 0, st>>>(U, aux, alpha, Rbar, scale, kb, pending, apart,
-                                                                  status, G, S, roe_in);
+                                                                  status, G, S, roe_in, nullptr);
   else
     adj_kept_kernel<NDIM, DIR, false><<<nblk, kAdjThreads, 0, st>>>(U, aux, alpha, Rbar, scale, kb, pending, apart,
-                                                                   status, G, S, nullptr);
+                                                                   status, G, S, nullptr, pf);
   int64_t nifc = 1;
   for (int k = 0; k < 3; ++k) nifc *= G.n[k] + (k == DIR ? 1 : 0);
   const int lblk = adj_list_blocks(nsm);
@@ -1069,7 +1085,7 @@ void launch_adj_dir(int nblk, int nsm, cudaStream_t st, const double* U, const d
   adj_count_kernel<<<lblk, kListThreads, 0, st>>>(pending, nifc, bcount);
   adj_scan_kernel<<<1, kListThreads, 0, st>>>(bcount, lblk, boff, total);
   adj_scatter_kernel<<<lblk, kListThreads, 0, st>>>(pending, nifc, boff, list);
-  adj_select_kernel<NDIM, DIR><<<nblk, kAdjThreads, 0, st>>>(U, aux, alpha, list, total, sel, status, G, S);
+  adj_select_kernel<NDIM, DIR><<<nblk, kAdjThreads, 0, st>>>(U, aux, alpha, list, total, sel, status, G, S, pf);
   // the partition reuses the counts and offsets; its own total (the number
   // of all-kept entries) goes to the slot after the list's
   int* nkept = total + 1;
@@ -1086,7 +1102,7 @@ template <int NDIM>
 void launch_adj_all(int nblk, int nsm, cudaStream_t st, const double* U, const double* aux,
                     const unsigned long long* alpha, const unsigned long long* argidx, const double* Rbar,
                     double scale, const AdjLayout& L, char* ws, int* status, GatherArgs A, const Grid& G,
-                    const Scheme& S, const double* roe_in) {
+                    const Scheme& S, const double* roe_in, const float4* pf) {
   auto* list = reinterpret_cast<uint32_t*>(ws + L.list);
   auto* lcount = reinterpret_cast<int*>(ws + L.lcount);
   auto* sel = reinterpret_cast<uint32_t*>(ws + L.sel);
@@ -1097,11 +1113,11 @@ void launch_adj_all(int nblk, int nsm, cudaStream_t st, const double* U, const d
     auto* pending = reinterpret_cast<unsigned char*>(ws + L.pending + d * L.pending_bytes);
     double* ap = apart + 6 * nblk * d;
     const double* rin = roe_in ? roe_in + d * L.roe_dir : nullptr;
-    if (d == 0) launch_adj_dir<NDIM, 0>(nblk, nsm, st, U, aux, alpha, Rbar, scale, kb, contrib, pending, list, lcount, sel, ap, status, G, S, rin);
+    if (d == 0) launch_adj_dir<NDIM, 0>(nblk, nsm, st, U, aux, alpha, Rbar, scale, kb, contrib, pending, list, lcount, sel, ap, status, G, S, rin, pf);
     if constexpr (NDIM > 1)
-      if (d == 1) launch_adj_dir<NDIM, 1>(nblk, nsm, st, U, aux, alpha, Rbar, scale, kb, contrib, pending, list, lcount, sel, ap, status, G, S, rin);
+      if (d == 1) launch_adj_dir<NDIM, 1>(nblk, nsm, st, U, aux, alpha, Rbar, scale, kb, contrib, pending, list, lcount, sel, ap, status, G, S, rin, pf);
     if constexpr (NDIM > 2)
-      if (d == 2) launch_adj_dir<NDIM, 2>(nblk, nsm, st, U, aux, alpha, Rbar, scale, kb, contrib, pending, list, lcount, sel, ap, status, G, S, rin);
+      if (d == 2) launch_adj_dir<NDIM, 2>(nblk, nsm, st, U, aux, alpha, Rbar, scale, kb, contrib, pending, list, lcount, sel, ap, status, G, S, rin, pf);
     A.kb[d] = kb;
     A.contrib[d] = contrib;
     A.pending[d] = pending;
@@ -1130,10 +1146,13 @@ teno_status adjoint_sequence(const teno_grid* g, const AdjLayout& L, char* ws, i
   auto* alpha = reinterpret_cast<unsigned long long*>(ws + L.alpha + stage * AdjLayout::kStage);
   auto* argidx = reinterpret_cast<unsigned long long*>(ws + L.argidx + stage * AdjLayout::kStage);
   double* aux = reinterpret_cast<double*>(ws + L.aux + stage * L.aux_bytes);
+  // this stage input's binary32 planes, where its cell pass runs here and the
+  // workspace has room for them
+  float4* pf = cell && L.pf ? reinterpret_cast<float4*>(ws + L.pf) : nullptr;
   if (cell) {
     auto* cand = reinterpret_cast<unsigned long long*>(ws + L.cand);
     if (cudaMemsetAsync(alpha, 0, sizeof(unsigned long long) * 9, st) != cudaSuccess) return TENO_ERR_CUDA;
-    if (teno::launch_cell(g->ndim, U, aux, nullptr, nullptr, alpha, status, G.ncell, g->gamma, nsm, st, cand) !=
+    if (teno::launch_cell(g->ndim, U, aux, nullptr, pf, alpha, status, G.ncell, g->gamma, nsm, st, cand) !=
             cudaSuccess ||
         teno::launch_argmax_finish(g->ndim, cand, G.ncell, nsm, argidx, st) != cudaSuccess)
       return TENO_ERR_CUDA;
@@ -1149,9 +1168,9 @@ teno_status adjoint_sequence(const teno_grid* g, const AdjLayout& L, char* ws, i
   const double* roe_in = (!cell && L.roe && stage < 2 && S.keep_idx >= 0)
                              ? reinterpret_cast<const double*>(ws + L.roe + stage * L.roe_stage_bytes)
                              : nullptr;
-  if (g->ndim == 1) launch_adj_all<1>(nblk, nsm, st, U, aux, alpha, argidx, Rbar, scale, L, ws, status, A, G, S, roe_in);
-  else if (g->ndim == 2) launch_adj_all<2>(nblk, nsm, st, U, aux, alpha, argidx, Rbar, scale, L, ws, status, A, G, S, roe_in);
-  else launch_adj_all<3>(nblk, nsm, st, U, aux, alpha, argidx, Rbar, scale, L, ws, status, A, G, S, roe_in);
+  if (g->ndim == 1) launch_adj_all<1>(nblk, nsm, st, U, aux, alpha, argidx, Rbar, scale, L, ws, status, A, G, S, roe_in, pf);
+  else if (g->ndim == 2) launch_adj_all<2>(nblk, nsm, st, U, aux, alpha, argidx, Rbar, scale, L, ws, status, A, G, S, roe_in, pf);
+  else launch_adj_all<3>(nblk, nsm, st, U, aux, alpha, argidx, Rbar, scale, L, ws, status, A, G, S, roe_in, pf);
   return cudaGetLastError() == cudaSuccess ? TENO_OK : TENO_ERR_CUDA;
 }
 

@@ -249,7 +249,7 @@ teno_status stage_begin(const teno_grid* g, const Layout& L, char* ws, const dou
   auto* alpha = reinterpret_cast<unsigned long long*>(ws + L.alpha);
   double* aux = reinterpret_cast<double*>(ws + L.aux);
   double* fh = one_pass ? nullptr : reinterpret_cast<double*>(ws + L.fh);
-  float4* pf = reinterpret_cast<float4*>(ws + L.pf);
+  float4* pf = one_pass ? nullptr : reinterpret_cast<float4*>(ws + L.pf);
   TENO_CUDA(cudaMemsetAsync(alpha, 0, teno::kAlphaAndCountBytes, st));
   TimerScope ts(st, TENO_KERNEL_CELL);
   TENO_CUDA(ghost_cells(g, G, st));

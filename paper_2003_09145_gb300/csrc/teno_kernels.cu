@@ -98,10 +98,15 @@ __global__ void __launch_bounds__(256, TENO_CELL_MINBLOCKS) cell_kernel(const do
       for (int v = 0; v < NVAR; ++v) Uc[v] = U[v * ncell + c];
       const double pn = aux[NDIM * ncell + c];
       store_flux_half<NDIM, 0>(Uc, uh, pn, ep, fh, ncell, c);
-      double su[NDIM];
+    }
+    if (pf) {
+      double Uc[NVAR], su[NDIM];
+#pragma unroll
+      for (int v = 0; v < NVAR; ++v) Uc[v] = U[v * ncell + c];
 #pragma unroll
       for (int k = 0; k < NDIM; ++k) su[k] = aux[(NDIM + 3 + k) * ncell + c];
-      store_planes<NDIM>(pf, ncell, c, Uc, uh, pn, aux[(NDIM + 1) * ncell + c], aux[(NDIM + 2) * ncell + c], su);
+      store_planes<NDIM>(pf, ncell, c, Uc, uh, aux[NDIM * ncell + c], aux[(NDIM + 1) * ncell + c],
+                         aux[(NDIM + 2) * ncell + c], su);
     }
     // The wave speeds only enter through their maxima: a cell whose binary32
     // upper bounds all lie below the block's maxima is skipped (15 of a 3D
