@@ -406,7 +406,7 @@ teno_status teno_rk3_step(const teno_grid* g, double* U, double cfl, double dt_f
   double* U2 = reinterpret_cast<double*>(w + L.U2);
   const Grid G = grid_in(g, L, w);
   const Scheme S = make_scheme(g);
-  if (teno::small_step_applies(G, S)) {
+  if (teno::small_step_applies(g->ndim, G, S)) {
     TimerScope ts(st, TENO_KERNEL_FLUX);
     TENO_CUDA(ghost_cells(g, G, st));
     teno::SmallStep A;

@@ -126,7 +126,7 @@ struct SmallStep {
   double cfl, dt_fixed, t_end;
 };
 constexpr int64_t kSmallStepMax = 6144;
-bool small_step_applies(const Grid& G, const Scheme& S);
+bool small_step_applies(int ndim, const Grid& G, const Scheme& S);
 cudaError_t launch_step1d(const SmallStep& A, const Grid& G, const Scheme& S, cudaStream_t st);
 
 // One right-hand-side evaluation of U fused with the SSP-RK3 stage `mode`

@@ -237,8 +237,10 @@ __global__ void __launch_bounds__(kSmallThreads) step1d_kernel(SmallStep A, Grid
 
 }  // namespace
 
-bool small_step_applies(const Grid& G, const Scheme& S) {
-  return G.n[1] == 1 && G.n[2] == 1 && G.ncell <= kSmallStepMax && S.variant != kSchemeWenoZ;
+// (ndim, not the extents: a 2D or 3D grid of one cell across still has the
+// other momenta and their directions' speeds)
+bool small_step_applies(int ndim, const Grid& G, const Scheme& S) {
+  return ndim == 1 && G.ncell <= kSmallStepMax && S.variant != kSchemeWenoZ;
 }
 
 cudaError_t launch_step1d(const SmallStep& A, const Grid& G, const Scheme& S, cudaStream_t st) {

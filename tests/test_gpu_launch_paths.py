@@ -61,6 +61,26 @@ def test_small_step_equals_staged_step(api, n, bc):
         assert S.status() == E.status() == 0
 
 
+@pytest.mark.parametrize("n", [(200, 1), (1, 200), (6144, 1), (1, 1), (200, 1, 1), (1, 200, 1), (1, 1, 200), (3, 1, 40)])
+@pytest.mark.parametrize("bc", [0, 1, 2])
+def test_one_cell_across_equals_staged_step(api, n, bc):
+    """2D and 3D grids of one cell across are no 1D grids: every momentum counts."""
+    ndim = len(n)
+    U = inputs.random_discontinuous_state(ndim, n, seed=sum(n))
+    U[2:-1] += 0.3 * U[0]
+    U[-1] += 0.5 * (U[1:-1] ** 2).sum(0) / U[0]
+    U0 = torch.from_numpy(np.ascontiguousarray(U)).cuda()
+    grid = api.EulerGrid(n, (0.01,) * ndim, (bc,) * ndim)
+    S, E = api.Solver(grid), api.SlabEngine(grid)
+    U, U1, U2, V = U0.clone(), torch.empty_like(U0), torch.empty_like(U0), U0.clone()
+    S.step(U)
+    for k, (a, b) in enumerate(((U0, U1), (U1, U2), (U2, V)), start=1):
+        E.begin(a)
+        E.end(k, a, U0, b, float("inf"), 0.0)
+    assert torch.equal(U, V) and torch.equal(S.dt, E.dt)
+    assert S.status() == E.status() == 0
+
+
 def test_small_step_past_t_end_and_nonphysical(api):
     n = 300
     U0 = torch.from_numpy(_line(n, 3)).cuda()
