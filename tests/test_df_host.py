@@ -97,3 +97,9 @@ def test_fixed_sums(lib):
     for a, e, (h, l) in zip(A.tolist(), E.tolist(), out):
         want = F(a) * (F(2) ** (e - 1078))
         assert abs(F(float(h)) + F(float(l)) - want) <= abs(want) * F(1, 2**46), (a, e, h, l)
+
+
+def test_zero_is_zero(lib):
+    a = np.array([0.0, -0.0, 2.0**-1000, -(2.0**-101), 2.0**-100])
+    out = _run(lib, 0, a, a)
+    assert np.all(out[:4] == 0.0) and out[4, 0] == 2.0**-100 and out[4, 1] == 0.0

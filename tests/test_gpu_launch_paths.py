@@ -132,3 +132,28 @@ def test_closed_form_in_and_out_of_range(api, ndim, n, krho, ku):
     b = api.rhs(grid, Ut)
     assert torch.isfinite(b).all()
     assert rel_max_err(b.cpu().numpy(), a.cpu().numpy(), flux_scale(U, n, dx)) <= 1e-13
+
+
+@pytest.mark.parametrize("ndim", [2, 3])
+@pytest.mark.parametrize("axis", [0, 1, 2])
+@pytest.mark.parametrize("p0", [1.0, 1e5, 1e9])
+def test_a_direction_at_rest_stays_at_rest(api, ndim, axis, p0):
+    """A rough wave along one axis, uniform along the others: their momenta get exact zeros."""
+    if axis >= ndim:
+        pytest.skip("axis")
+    rng = np.random.default_rng(axis)
+    n = tuple(96 if k == axis else 7 for k in range(ndim))
+    x = np.arange(96) / 96
+    shape = tuple(96 if ndim - 1 - k == axis else 1 for k in range(ndim))
+    wave = (np.sin(2.0 * np.pi * x) + 0.2 * rng.uniform(-1, 1, 96)).reshape(shape)
+    full = tuple(reversed(n))
+    rho = np.broadcast_to(1.0 + 0.01 * wave, full)
+    vel = [np.broadcast_to((0.3 + 0.01 * wave) * np.sqrt(p0) if k == axis else 0.0 * wave, full) for k in range(ndim)]
+    p = np.broadcast_to(p0 * (1.0 + 0.01 * wave), full)
+    U = torch.from_numpy(np.ascontiguousarray(inputs.prim_to_cons(rho, vel, p))).cuda()
+    grid = api.EulerGrid(n, (0.1,) * ndim, (0,) * ndim)
+    R = api.rhs(grid, U)
+    assert torch.isfinite(R).all() and R[1 + axis].abs().max() > 0
+    for k in range(ndim):
+        if k != axis:
+            assert torch.count_nonzero(R[1 + k]).item() == 0
