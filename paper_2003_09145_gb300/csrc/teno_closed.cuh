@@ -25,7 +25,7 @@ namespace teno {
 __device__ __forceinline__ float near_float(double x) {
   const uint32_t e = (teno_fix::hi_word(x) >> 20) & 0x7FFu;
   if (e - 923u >= 200u) return hi_float(x);
-  const teno_df::df d = teno_df::from_double(x);
+  const teno_df::df d = teno_df::split(x);
   return teno_cert::fadd(d.h, d.l);
 }
 

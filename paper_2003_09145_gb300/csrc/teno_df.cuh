@@ -57,16 +57,21 @@ TENO_CERT_HD df neg(df a) { return {-a.h, -a.l}; }
 // exact scaling by a power of two
 TENO_CERT_HD df scale(df a, float p) { return {fmul(a.h, p), fmul(a.l, p)}; }
 
-// x truncated to 46 bits (24 in h, the next 23 in l), |x| < 2^127; magnitudes
-// below 2^-100 become 0 (a direction at rest stays at rest exactly)
-TENO_CERT_HD df from_double(double x) {
+// x truncated to 46 bits (24 in h, the next 23 in l), 2^-100 <= |x| < 2^127
+TENO_CERT_HD df split(double x) {
   const uint32_t hi = teno_fix::hi_word(x), lo = teno_fix::lo_word(x);
   const uint32_t m = hi << 1;
-  if (m < (923u << 21)) return {0.0f, 0.0f};
   const uint32_t h = (m * 4u - (896u << 23)) | (hi & 0x80000000u) | (lo >> 29);
   const uint32_t b = (h & 0xFF800000u) - (23u << 23);   // the low part's unit, with the sign
   const uint32_t r = (lo >> 6) & 0x7FFFFFu;
   return {from_bits(h), fsub(from_bits(b | r), from_bits(b))};
+}
+// the same; magnitudes below 2^-100 become 0 (a direction at rest stays at
+// rest exactly)
+TENO_CERT_HD df from_double(double x) {
+  const df d = split(x);
+  const bool zero = (teno_fix::hi_word(x) & 0x7FFFFFFFu) < (923u << 20);
+  return {zero ? 0.0f : d.h, zero ? 0.0f : d.l};
 }
 
 TENO_CERT_HD df add(df a, df b) {
