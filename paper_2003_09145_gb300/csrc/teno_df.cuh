@@ -138,26 +138,27 @@ TENO_CERT_HD df from_fixed(int64_t A, uint32_t E) {
   return {fmul(h, pow2_field(f + 21)), fmul(l, pow2_field(f))};
 }
 
-// h + l in binary64 with integer operations, to 2^-46 relative: h + l is
-// renormalised, h moved one ulp towards zero where l points back (l then rounds
-// once), and l fills the significand's low 29 bits.  Values below 2^-100
-// become 0.  (Two FP64 additions of the widened parts would hold the FP64
+// h + l in binary64 with integer operations, to 2^-46 relative (and 2^-125, as
+// l ends at 2^-126 and smaller values become 0): h + l is renormalised, h
+// moved one ulp towards zero where l points back (l then rounds once), and l's
+// significand, shifted to h's exponent, fills the result's low 29 bits.  (Two FP64 additions of the widened parts would hold the FP64
 // pipe for 128 cycles a warp; this is some 20 instructions.)
 TENO_CERT_HD double to_double(df a) {
   const float s = fadd(a.h, a.l), t = fsub(s, a.h);
   float l = fadd(fsub(a.h, fsub(s, t)), fsub(a.l, t));
   uint32_t hb = bits(s);
-  if ((hb & 0x7FFFFFFFu) < (27u << 23)) return 0.0;
+  if ((hb & 0x7FFFFFFFu) < (2u << 23)) return 0.0;
   const bool back = l != 0.0f && ((bits(l) ^ hb) >> 31);
   const float h = from_bits(hb - (back ? 1u : 0u));
   l = fadd(l, fsub(s, h));
   hb = bits(h);
   const uint32_t mag = hb & 0x7FFFFFFFu;
-  // |l| / 2^(e - 52) with e the exponent of h: below 2^29
-  const int f = 306 - static_cast<int>(mag >> 23);
-  float n = fmul(fabsf(l), pow2_field(f > 254 ? 254 : f));
-  uint32_t q = static_cast<uint32_t>(n);
-  q = q > 0x1FFFFFFFu ? 0x1FFFFFFFu : q;
+  // |l| / 2^(e - 52) with e the exponent of h: its 24-bit significand times
+  // 2^(e_l - e + 29), e_l <= e - 23
+  const uint32_t lm = bits(l) & 0x7FFFFFFFu, el = lm >> 23;
+  const uint32_t sh = (mag >> 23) - el - 23u;
+  uint32_t q = ((lm & 0x7FFFFFu) | 0x800000u) << 6 >> (sh < 31u ? sh : 31u);
+  q = el == 0u ? 0u : (q > 0x1FFFFFFFu ? 0x1FFFFFFFu : q);
   const uint32_t hi = (hb & 0x80000000u) | ((mag >> 3) + (896u << 20));
   const uint32_t lo = (mag << 29) | q;
   return teno_fix::from_bits((static_cast<uint64_t>(hi) << 32) | lo);

@@ -103,3 +103,15 @@ def test_zero_is_zero(lib):
     a = np.array([0.0, -0.0, 2.0**-1000, -(2.0**-101), 2.0**-100])
     out = _run(lib, 0, a, a)
     assert np.all(out[:4] == 0.0) and out[4, 0] == 2.0**-100 and out[4, 1] == 0.0
+
+
+def test_to_double_of_small_values(lib):
+    """Down to the end of binary32's normal range: h rounds nothing, l is cut
+    at 2^-46 of h, and bits of l below 2^-126 are lost."""
+    rng = np.random.default_rng(9)
+    a = _values(rng, 6000, -124, -30)
+    b = a * (2.0**-25 * rng.uniform(-1, 1, len(a)))
+    for op in (5, 1):
+        for x, y, (h, l, d) in zip(a, b, _run(lib, op, a, b)):
+            s = F(float(h)) + F(float(l))
+            assert abs(F(float(d)) - s) <= abs(s) * F(1, 2**46) + F(1, 2**125), (op, x, y, h, l, d)
