@@ -161,6 +161,7 @@ __device__ __noinline__ unsigned forward_open(const double* __restrict__ U, cons
   for (int j = 0; j < 6; ++j) cells[j] = line + teno::ghost(id - 3 + j, nd, bc) * stride;
   const double a3[3] = {am, a0, ap};
   const teno::FaceSpeeds F = teno::face_speeds(a3);
+  const teno_df::df gm1 = teno::gm1_df(S);
   double su2[NDIM], su3[NDIM];
 #pragma unroll
   for (int k = 0; k < NDIM; ++k) {
@@ -172,13 +173,13 @@ __device__ __noinline__ unsigned forward_open(const double* __restrict__ U, cons
   teno::RoeDf<NDIM> Rd;
   if (pf)
     teno::roe_df<NDIM>(teno::load_roe_cell<NDIM, false>(pf, nullptr, ncell, cells[2]),
-                       teno::load_roe_cell<NDIM, false>(pf, nullptr, ncell, cells[3]), S, Rd);
+                       teno::load_roe_cell<NDIM, false>(pf, nullptr, ncell, cells[3]), gm1, Rd);
   else
-    teno::roe_df<NDIM>(teno::roe_cell<NDIM>(sr2, sh2, su2), teno::roe_cell<NDIM>(sr3, sh3, su3), S, Rd);
+    teno::roe_df<NDIM>(teno::roe_cell<NDIM>(sr2, sh2, su2), teno::roe_cell<NDIM>(sr3, sh3, su3), gm1, Rd);
   teno::CertIfc<NDIM> C;
-  for (bool df = F.in_range && teno::roe_df_ok<NDIM>(Rd, S);; df = false) {
+  for (bool df = F.in_range && teno::roe_df_ok<NDIM>(Rd, gm1);; df = false) {
     if (df) {
-      teno::cert_begin_df<NDIM, DIR>(Rd, F.ha, S, C);
+      teno::cert_begin_df<NDIM, DIR>(Rd, F.ha, gm1, C);
     } else {
       double alpha[NVAR], nal[NVAR];
       teno::spread_speeds<NDIM>(a3, alpha, nal);

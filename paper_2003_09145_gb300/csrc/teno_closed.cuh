@@ -14,44 +14,12 @@
 // widened and added in two FP64 additions instead of one (no gain).
 #pragma once
 
-#include "teno_df.cuh"
+#include "teno_closed_core.cuh"
 #include "teno_flux.cuh"
 
 namespace teno {
 
-// x rounded to binary32 (within 2^-24 and a bit, relative) by integer and FP32
-// operations, for 2^-100 <= |x| < 2^100; beyond that hi_float's clamped
-// truncation
-__device__ __forceinline__ float near_float(double x) {
-  const uint32_t e = (teno_fix::hi_word(x) >> 20) & 0x7FFu;
-  if (e - 923u >= 200u) return hi_float(x);
-  const teno_df::df d = teno_df::split(x);
-  return teno_cert::fadd(d.h, d.l);
-}
-
-// The speeds in the forms the closed form reads: halved, as two binary32
-// values (the middle one, and the sum and difference of the acoustic
-// ones' differences against it -- closed_out's amid, sg, df), as binary32, and
-// whether they lie in the range of teno_df's terms (2^-19 .. 2^30).
-struct FaceSpeeds {
-  teno_df::df amid, sg, dd;
-  float ha[3], amax;
-  bool in_range;
-};
-__device__ __forceinline__ FaceSpeeds face_speeds(const double (&a3)[3]) {
-  using namespace teno_df;
-  FaceSpeeds F;
-  const df am = from_double(a3[0]), a0 = from_double(a3[1]), ap = from_double(a3[2]);
-  const df d0 = add(am, neg(a0)), dE = add(ap, neg(a0));
-  F.amid = a0;
-  F.sg = add(d0, dE);
-  F.dd = add(d0, neg(dE));
-#pragma unroll
-  for (int s = 0; s < 3; ++s) F.ha[s] = near_float(a3[s]);
-  F.amax = 2.0f * fmaxf(F.ha[0], F.ha[2]);
-  F.in_range = F.amax >= 0x1p-19f && F.amax <= 0x1p30f;
-  return F;
-}
+__device__ __forceinline__ teno_df::df gm1_df(const Scheme& S) { return {S.gm1_h, S.gm1_l}; }
 
 // What the closed form's first pass and its Roe state read of a cell, in
 // binary32, written once per cell by the cell pass (converting it at each of
@@ -126,17 +94,6 @@ __device__ __forceinline__ void load_point_f(const float4* __restrict__ pf, cons
   }
 }
 
-// The Roe state in two binary32 values, from the cells' sqrt(rho),
-// (E+p)/sqrt(rho) and m_k/sqrt(rho) (roe_interface's average): u~, |u~|^2, H~,
-// c~^2 and 1/c~.
-template <int NDIM>
-struct RoeDf {
-  teno_df::df u[NDIM], q2, H, c2, ic;
-};
-template <int NDIM>
-struct RoeCellDf {   // one cell's contribution
-  teno_df::df sr, sh, su[NDIM];
-};
 template <int NDIM, bool GH, class I>
 __device__ __forceinline__ RoeCellDf<NDIM> load_roe_cell(const float4* __restrict__ pf, const float4* __restrict__ gpf,
                                                          int64_t ncell, I c) {
@@ -158,62 +115,10 @@ __device__ __forceinline__ RoeCellDf<NDIM> load_roe_cell(const float4* __restric
   }
   return R;
 }
-template <int NDIM>
-__device__ __forceinline__ RoeCellDf<NDIM> roe_cell(double sr, double sh, const double (&su)[NDIM]) {
-  RoeCellDf<NDIM> R;
-  R.sr = teno_df::from_double(sr);
-  R.sh = teno_df::from_double(sh);
-#pragma unroll
-  for (int k = 0; k < NDIM; ++k) R.su[k] = teno_df::from_double(su[k]);
-  return R;
-}
-template <int NDIM>
-__device__ __forceinline__ void roe_df(const RoeCellDf<NDIM>& a, const RoeCellDf<NDIM>& b, const Scheme& S,
-                                       RoeDf<NDIM>& R) {
-  using namespace teno_df;
-  const df y = recip(add(a.sr, b.sr));
-#pragma unroll
-  for (int k = 0; k < NDIM; ++k) {
-    R.u[k] = mul(add(a.su[k], b.su[k]), y);
-    R.q2 = k == 0 ? sqr(R.u[0]) : add(R.q2, sqr(R.u[k]));
-  }
-  R.H = mul(add(a.sh, b.sh), y);
-  R.c2 = mul(df{S.gm1_h, S.gm1_l}, add(R.H, scale(R.q2, -0.5f)));
-  R.ic = teno_df::rsqrt(R.c2);
-}
-
-// The certificate's view of that Roe state, rounded to binary32, where
-// roe_df_ok holds, i.e. where c~^2 keeps 2^-6 of (gamma - 1) H~ (Mach numbers
-// below about 18 for gamma = 1.4; c~^2 is then good to 2^-38).
-template <int NDIM, int DIR>
-__device__ __forceinline__ void cert_begin_df(const RoeDf<NDIM>& R, const float (&ha3)[3], const Scheme& S,
-                                              CertIfc<NDIM>& C) {
-  using teno_cert::fadd;
-  using teno_cert::fmul;
-  float uf[NDIM], ha[NDIM + 2];
-#pragma unroll
-  for (int k = 0; k < NDIM; ++k) uf[k] = fadd(R.u[k].h, R.u[k].l);
-#pragma unroll
-  for (int f = 0; f < NDIM + 2; ++f) ha[f] = ha3[f == 0 ? 0 : (f == NDIM + 1 ? 2 : 1)];
-  const float ic = fadd(R.ic.h, R.ic.l);
-  const float hb1 = fmul(0.5f * S.gm1_h, fmul(ic, ic));
-  teno_cert::cert_begin_f<NDIM, DIR>(uf, hb1, fmul(0.5f * hb1, fadd(R.q2.h, R.q2.l)), 0.5f * ic, ha,
-                                     teno_cert::kCertRounded, C);
-}
-template <int NDIM>
-__device__ __forceinline__ bool roe_df_ok(const RoeDf<NDIM>& R, const Scheme& S) {
-  return R.c2.h > 0x1p-6f * S.gm1_h * R.H.h;
-}
-
-// 2^-20 <= max rho < 2^30 and max E < 2^95 keep every term of the test and of
-// teno_df in binary32's range; |u| and c are bounded by the speeds.
-__device__ __forceinline__ bool df_range(float rho_max, float e_max) {
-  return rho_max >= 0x1p-20f && rho_max < 0x1p30f && e_max < 0x1p95f;
-}
-
 // The closed form's Roe state and corrections in binary64, on sums already
-// formed (60 U~ and the mass flux in fixed point, the other fluxes): where U~
-// is not small against the flux scale, i.e. at shocks.  Out of line, on copies
+// formed (60 U~ and the mass flux in fixed point, the other fluxes): where the
+// corrections are not small against the flux scale (closed_df_rough), i.e. at
+// shocks.  Out of line, on copies
 // of its inputs, so that the common form's values stay in registers.
 template <int NDIM>
 struct ClosedSums {
@@ -267,6 +172,7 @@ __device__ __forceinline__ unsigned interface_flux_closed(const double* __restri
   constexpr int NVAR = NDIM + 2;
   if (S.keep_idx < 0) return kRough | kAllOpen<NDIM>;
   const double* gfh = GH ? gc.fh + DIR * (NVAR - 1) * kGhostSlots : nullptr;
+  const df gm1 = gm1_df(S);
   RoeDf<NDIM> R;
   {
     RoeCellDf<NDIM> ra = load_roe_cell<NDIM, GH>(pf, gc.pf, ncell, cells[2]);
@@ -274,16 +180,16 @@ __device__ __forceinline__ unsigned interface_flux_closed(const double* __restri
     const float fa = (flips >> 2) & 1u ? -1.0f : 1.0f, fb = (flips >> 3) & 1u ? -1.0f : 1.0f;
     ra.su[DIR] = scale(ra.su[DIR], fa);
     rb.su[DIR] = scale(rb.su[DIR], fb);
-    roe_df<NDIM>(ra, rb, S, R);
+    roe_df<NDIM>(ra, rb, gm1, R);
   }
-  bool range = F.in_range && roe_df_ok<NDIM>(R, S);
+  bool range = F.in_range && roe_df_ok<NDIM>(R, gm1);
   // first pass: the certified test and the largest magnitudes of the summed
   // components (a mirrored point changes signs only)
   unsigned open;
   float xm[NVAR];
   {
     CertIfc<NDIM> C;
-    cert_begin_df<NDIM, DIR>(R, F.ha, S, C);
+    cert_begin_df<NDIM, DIR>(R, F.ha, gm1, C);
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
       float X[NVAR], u, p;
@@ -333,37 +239,14 @@ __device__ __forceinline__ unsigned interface_flux_closed(const double* __restri
       }
     }
     df Ut[NVAR];
-    bool rough = false;
-    // U~ against the flux scale: |60 U~| <= 60 2^-8 (rho, alpha rho, E),
-    // tightened by c~^2 / ((gamma - 1) H~), the digits that c~^2 lost
-    const float gH = S.gm1_h * R.H.h, lim = (60.0f * 0x1p-8f) * R.c2.h;
 #pragma unroll
-    for (int v = 0; v < NVAR; ++v) {
-      Ut[v] = from_fixed(AU[v], EU[v]);
-      const float sc = v == 0 ? xm[0] : (v == NVAR - 1 ? xm[NVAR - 1] : xm[0] * F.amax);
-      rough = rough || !(fabsf(Ut[v].h) * gH <= lim * sc);
-    }
-    if (!rough) {
-      // closed_out with c~ eliminated: T = |u~|^2/2 U~_0 - u~.U~_m + U~_E,
-      // V = (u~_d U~_0 - U~_d)/2 = c~ B, t = c~ A = (gamma-1)/2 T / c~,
-      // gs = (sg t + df V) / c~, c~ ngd = df t + sg V
-      df T = mul(scale(R.q2, 0.5f), Ut[0]);
+    for (int v = 0; v < NVAR; ++v) Ut[v] = from_fixed(AU[v], EU[v]);
+    if (!closed_df_rough<NDIM, DIR>(Ut, R, gm1, F.amax, xm[0], xm[NVAR - 1])) {
+      df o[NVAR];
+      closed_df<NDIM, DIR>(Ut, R, F, gm1, o);
+      out[0] = teno_fix::round(AF, EU[1 + DIR] - 1u) + to_double(o[0]);
 #pragma unroll
-      for (int k = 0; k < NDIM; ++k) T = add(T, neg(mul(R.u[k], Ut[1 + k])));
-      T = add(T, Ut[NVAR - 1]);
-      const df V = scale(add(mul(R.u[DIR], Ut[0]), neg(Ut[1 + DIR])), 0.5f);
-      const df t = mul(mul(df{0.5f * S.gm1_h, 0.5f * S.gm1_l}, T), R.ic);
-      const df gs = mul(R.ic, add(mul(F.sg, t), mul(F.dd, V)));
-      const df cn = add(mul(F.dd, t), mul(F.sg, V));
-      out[0] = teno_fix::round(AF, EU[1 + DIR] - 1u) + to_double(add(mul(F.amid, Ut[0]), gs));
-#pragma unroll
-      for (int k = 0; k < NDIM; ++k) {
-        df o = add(mul(F.amid, Ut[1 + k]), mul(R.u[k], gs));
-        if (k == DIR) o = add(o, neg(cn));
-        out[1 + k] = Fd[1 + k] + to_double(o);
-      }
-      out[NVAR - 1] =
-          Fd[NVAR - 1] + to_double(add(add(mul(F.amid, Ut[NVAR - 1]), mul(R.H, gs)), neg(mul(R.u[DIR], cn))));
+      for (int v = 1; v < NVAR; ++v) out[v] = Fd[v] + to_double(o[v]);
     } else {
       ClosedSums<NDIM> X;
       double o[NVAR];

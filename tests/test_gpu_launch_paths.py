@@ -157,3 +157,31 @@ def test_a_direction_at_rest_stays_at_rest(api, ndim, axis, p0):
     for k in range(ndim):
         if k != axis:
             assert torch.count_nonzero(R[1 + k]).item() == 0
+
+
+@pytest.mark.parametrize("ndim,n", [(1, (500,)), (2, (61, 47)), (3, (23, 19, 17))])
+@pytest.mark.parametrize("krho,ku", [(-19, -18), (-10, -18), (-15, -15), (-20, -19), (-18, -10), (28, -18)])
+def test_closed_form_with_both_scales_moved(api, ndim, n, krho, ku):
+    """As above: the energy flux goes with rho u^3."""
+    test_closed_form_in_and_out_of_range(api, ndim, n, krho, ku)
+
+
+@pytest.mark.parametrize("ndim,n", [(1, (512,)), (2, (64, 40)), (3, (48, 16, 12))])
+@pytest.mark.parametrize("p_cold", [1e-2, 1e-4, 1e-6, 1e-10, 1e-14, 1e-18, 1e-22, 1e-26, 1e-30])
+def test_cold_region_beside_a_fast_one(api, ndim, n, p_cold):
+    """The speeds are set by the fast half; in the cold one 1/c multiplies the corrections."""
+    rng = np.random.default_rng(3)
+    full = tuple(reversed(n))
+    x = np.broadcast_to(np.arange(n[0]) / n[0], full)
+    cold = (x > 0.25) & (x < 0.85)
+    f = [1.0 + 0.02 * np.sin(2 * np.pi * (5 * x + rng.uniform())) + 0.01 * rng.uniform(-1, 1, full) for _ in range(3)]
+    rho = f[0]
+    p = np.where(cold, p_cold, 1.0) * f[1]
+    vel = [np.where(cold, np.sqrt(p_cold) * 0.01 * rng.uniform(-1, 1, full), 0.7 * f[2]) for _ in range(ndim)]
+    U = inputs.prim_to_cons(rho, vel, p)
+    grid = api.EulerGrid(n, (1.0,) * ndim, (0,) * ndim)
+    Ut = torch.from_numpy(np.ascontiguousarray(U)).cuda()
+    a, _ = api.rhs(grid, Ut, want_flags=True)
+    b = api.rhs(grid, Ut)
+    assert torch.isfinite(b).all()
+    assert rel_max_err(b.cpu().numpy(), a.cpu().numpy(), flux_scale(U, n, (1.0,) * ndim)) <= 1e-13
