@@ -272,8 +272,10 @@ __device__ __forceinline__ int teno5a_magnitude(double e0, double e1, double e2,
 // a_j with a_k = c_k (1 + tau / D_k), D_k = beta_k + eps (carried times 4; the
 // factor cancels).  eps enters the indicators' own sums, and tau = |D_2 - D_0|
 // (off by the D's rounding only, which 1 + tau / D_k has anyway).  With N_k =
-// D_k + tau and A_k = 10 c_k N_k prod_{j != k} D_j, omega_k = A_k / sum A (three
-// divisions where the products leave the range).  The weights enter f^ = v2 +
+// D_k + tau and A_k = 10 c_k N_k prod_{j != k} D_j, omega_k = A_k / sum A (by
+// divisions, normalised, where sum A, which goes with e^6, is not between 2^-400 and 2^860: the
+// products A_k e of the next line and 6 sum A then stay normal numbers).  The
+// weights enter f^ = v2 +
 // sum_k w_k e_k (see c_cut) unnormalised,
 //   6 sum A sum_k w_k e_k = -2 A0 e0 + (5 A0 + A1) e1 + (2 A1 + 4 A2) e2 - A2 e3,
 // and one reciprocal of 6 sum A divides: every interface takes this path on
@@ -290,11 +292,15 @@ __device__ __forceinline__ double weno_z(double e0, double e1, double e2, double
   const double tau = fabs(d2 - d0);
   double A0 = (d0 + tau) * (d1 * d2), A1 = 6.0 * ((d1 + tau) * (d0 * d2)), A2 = 3.0 * ((d2 + tau) * (d0 * d1));
   double As = A0 + A1 + A2;
-  if (!pos_finite(As)) {
+  if (!(dbits(As) - (623ull << 52) < (1260ull << 52))) {
     A0 = 1.0 + tau / d0;
     A1 = 6.0 * (1.0 + tau / d1);
     A2 = 3.0 * (1.0 + tau / d2);
-    As = A0 + A1 + A2;
+    const double r = 1.0 / (A0 + A1 + A2);
+    A0 *= r;
+    A1 *= r;
+    A2 *= r;
+    As = 1.0;
   }
   flag = 7u;
   const double q = fma(-2.0 * A0, e0, fma(fma(5.0, A0, A1), e1, fma(fma(4.0, A2, 2.0 * A1), e2, -A2 * e3)));

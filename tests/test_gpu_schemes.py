@@ -125,3 +125,21 @@ def test_teno5_fixed_equals_lad_with_one_magnitude(api):
     b, fb = api.rhs(api.EulerGrid(P.n, P.dx, P.bc, api.Scheme(b_l=7, b_u=8)), U, want_flags=True)
     assert torch.equal(a, b)
     assert torch.equal(fa & 7, fb & 7)
+
+
+@pytest.mark.parametrize("k", [-480, -300, -170, -146, -130, -60, 0, 60, 130, 143, 146, 150, 155, 170, 330, 480])
+@pytest.mark.parametrize("fixed_eps", [False, True])
+def test_wenoz_at_any_scale(api, k, fixed_eps):
+    """WENO-Z is homogeneous in (u, sqrt(eps)): data times 2^k with eps times 4^k
+    give 2^k times the right-hand side (the products of the weights round alike up
+    to their range's ends; 1e-14 covers the divided weights beyond)."""
+    rng = np.random.default_rng(4)
+    n = 300
+    u = np.sin(2 * np.pi * np.arange(n) / 40.0) + (np.arange(n) > 150) + 0.1 * rng.standard_normal(n)
+    e0, ek = (1e-6 * 4.0**-k, 1e-6) if fixed_eps else (1e-6, 1e-6 * 4.0**k)
+    R = []
+    for s, eps in ((0, e0), (k, ek)):
+        adv = api.ScalarAdvection(n, 1.0 / n, scheme=api.Scheme(scheme="wenoz", eps=eps))
+        R.append(adv.rhs(torch.from_numpy(u * 2.0**s).cuda()).cpu().numpy())
+    assert np.isfinite(R[1]).all()
+    assert np.max(np.abs(R[1] * 2.0**-k - R[0])) <= 1e-14 * n * np.max(np.abs(u))
