@@ -22,8 +22,9 @@ static __constant__ float c_lad_f[16] = {1e-0f, 1e-1f, 1e-2f,  1e-3f,  1e-4f,  1
 
 // TENO weights of eq. 2.15 for each selection pattern sel = delta_0 |
 // delta_1 << 1 | delta_2 << 2, with the linear weights c = (0.1, 0.6, 0.3):
-// omega_k = delta_k c_k / sum_j delta_j c_j.  Pattern 0 cannot occur (the
-// largest chi_k is at least 1/3 > C_T).
+// omega_k = delta_k c_k / sum_j delta_j c_j.  Pattern 0 only occurs with C_T = 1
+// (B_l = 0, m = 0; else the largest chi_k, at least 1/3, exceeds C_T): eq. 2.15 is
+// 0/0 there, and the field's value is 0.
 static __constant__ double c_omega[8][3] = {
     {0.0, 0.0, 0.0},
     {0.1 / 0.1, 0.0, 0.0},
@@ -39,7 +40,8 @@ static __constant__ double c_omega[8][3] = {
 // w = (-omega_0/3, 5 omega_0/6 + omega_1/6, omega_1/3 + 2 omega_2/3, -omega_2/6)
 // (candidates of eq. 2.4-2.6 relative to v2: (5 e1/6 - e0/3), (e1/6 + e2/3),
 // (2 e2/3 - e3/6)); with every stencil kept this is eq. 2.3.  The table holds
-// w[sel] - w[7]: what the selection changes against keeping every stencil.
+// w[sel] - w[7]: what the selection changes against keeping every stencil (not
+// for pattern 0, whose weights do not add up to 1).
 #define TENO_CUT_ROW(o0, o1, o2)                                                                       \
   {-((o0) - 0.1) / 3.0, 5.0 * ((o0) - 0.1) / 6.0 + ((o1) - 0.6) / 6.0,                                 \
    ((o1) - 0.6) / 3.0 + 2.0 * ((o2) - 0.3) / 3.0, -((o2) - 0.3) / 6.0}
@@ -420,6 +422,8 @@ __device__ __forceinline__ double teno5_lad(double v0, double v1, double v2,
   }
   if (cut) {
     if (sel == 7u) return acc;
+    if (sel == 0u)   // less the whole all-kept value
+      return acc - fma(c_lin[7][0], v0, fma(c_lin[7][1], v1, fma(c_lin[7][2], v2, fma(c_lin[7][3], v3, c_lin[7][4] * v4))));
     return fma(c_cut[sel][0], e0, fma(c_cut[sel][1], e1, fma(c_cut[sel][2], e2, fma(c_cut[sel][3], e3, acc))));
   }
   // eq. 2.4-2.7 with the weights of eq. 2.15 (c_lin)

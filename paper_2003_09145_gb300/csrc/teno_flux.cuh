@@ -633,8 +633,10 @@ __device__ __forceinline__ uint32_t warp_correct(const double* __restrict__ U, c
       continue;
     }
     double dl = 0.0;
-    if (it >> 9) {
-      dl = fma(c_lin[sel][0], v[0], fma(c_lin[sel][1], v[1], fma(c_lin[sel][2], v[2], fma(c_lin[sel][3], v[3], c_lin[sel][4] * v[4]))));
+    if ((it >> 9) || sel == 0u) {   // the whole value; for no stencil at all, less the all-kept one
+      const unsigned r = it >> 9 ? sel : 7u;
+      dl = fma(c_lin[r][0], v[0], fma(c_lin[r][1], v[1], fma(c_lin[r][2], v[2], fma(c_lin[r][3], v[3], c_lin[r][4] * v[4]))));
+      if (!(it >> 9)) dl = -dl;
     } else if (sel != 7u) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) dl = fma(c_cut[sel][j], e[j], dl);

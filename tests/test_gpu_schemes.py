@@ -143,3 +143,66 @@ def test_wenoz_at_any_scale(api, k, fixed_eps):
         R.append(adv.rhs(torch.from_numpy(u * 2.0**s).cuda()).cpu().numpy())
     assert np.isfinite(R[1]).all()
     assert np.max(np.abs(R[1] * 2.0**-k - R[0])) <= 1e-14 * n * np.max(np.abs(u))
+
+
+def _flux_from_flags(U, bc, flags, gamma=1.4):
+    """The 1D fluxes with the selections of ``flags`` (the flag layout of teno.h),
+    every step from the paper's equations; no stencil at all gives a field 0."""
+    n = U.shape[1]
+    i = np.arange(-3, n + 3)
+    P = U[:, i % n if bc == 0 else np.clip(i, 0, n - 1)]
+    rho, m, E = P
+    u = m / rho
+    p = (gamma - 1) * (E - 0.5 * rho * u * u)
+    c = np.sqrt(gamma * p / rho)
+    al = [np.abs(u - c).max(), np.abs(u).max(), np.abs(u + c).max()]
+    F = np.array([m, m * u + p, u * (E + p)])
+    a, b = slice(2, n + 3), slice(3, n + 4)
+    sa, sb = np.sqrt(rho[a]), np.sqrt(rho[b])
+    ut = (sa * u[a] + sb * u[b]) / (sa + sb)
+    H = (sa * (E[a] + p[a]) / rho[a] + sb * (E[b] + p[b]) / rho[b]) / (sa + sb)
+    c2 = (gamma - 1) * (H - 0.5 * ut * ut)
+    cs, b1 = np.sqrt(c2), (gamma - 1) / c2
+
+    def left(X):
+        A = 0.5 * b1 * (0.5 * ut * ut * X[0] - ut * X[1] + X[2])
+        B = 0.5 * (ut * X[0] - X[1]) / cs
+        return [A + B, X[0] - 2 * A, A - B]
+
+    def omega(sel):
+        d = np.array([(sel >> k) & 1 for k in range(3)]) * np.array([0.1, 0.6, 0.3])[:, None]
+        s = d.sum(0)
+        return d / np.where(s > 0, s, 1.0)
+
+    sel = flags.reshape(3, 2, n + 1) & 7
+    W = [left(P[:, j:j + n + 1]) for j in range(6)]
+    G = [left(F[:, j:j + n + 1]) for j in range(6)]
+    f = []
+    for s in range(3):
+        tot = 0.0
+        for side, sgn, order in ((0, 1.0, range(5)), (1, -1.0, range(5, 0, -1))):
+            v = [0.5 * (G[j][s] + sgn * al[s] * W[j][s]) for j in order]
+            o = omega(sel[s, side])
+            tot = tot + (o[0] * (2 * v[0] - 7 * v[1] + 11 * v[2]) + o[1] * (-v[1] + 5 * v[2] + 2 * v[3]) +
+                         o[2] * (2 * v[2] + 5 * v[3] - v[4])) / 6.0
+        f.append(tot)
+    mass = f[0] + f[1] + f[2]
+    return np.array([mass, ut * mass + cs * (f[2] - f[0]),
+                     f[0] * (H - ut * cs) + 0.5 * ut * ut * f[1] + f[2] * (H + ut * cs)]), sel
+
+
+def test_selection_of_no_stencil(api):
+    """B_l = 0 gives C_T = 1 at strong jumps, where no chi_k reaches it: the field
+    contributes nothing, on the flag path and on the flag-free one (which the steps take) alike."""
+    P = inputs.shock_tube(200)
+    grid = api.EulerGrid(P.n, P.dx, P.bc, api.Scheme(b_l=0, b_u=4))
+    U0 = P.U0 * (1.0 + 1e-3 * np.random.default_rng(1).standard_normal(P.U0.shape))
+    U = torch.from_numpy(np.ascontiguousarray(U0)).cuda()
+    a, flags = api.rhs(grid, U, want_flags=True)
+    b = api.rhs(grid, U)
+    F, sel = _flux_from_flags(U0, 1, flags.cpu().numpy())
+    assert np.count_nonzero(sel == 0) >= 4
+    want = (F[:, :-1] - F[:, 1:]) / P.dx[0]
+    scale = flux_scale(U0, P.n, P.dx)
+    assert rel_max_err(a.cpu().numpy(), want, scale) <= RHS_RTOL
+    assert rel_max_err(b.cpu().numpy(), want, scale) <= RHS_RTOL
