@@ -962,7 +962,7 @@ struct AdjLayout {
   // alpha + 128 s, its arg-max cells (9 x 8) at argidx + 128 s
   static constexpr size_t kStage = 128;
   size_t status = 0, dt = 8, alpha = 64, argidx = 512;
-  size_t aux = 0, aux_bytes = 0, cand = 0, fh = 0, pf = 0, kb = 0, kb_bytes = 0, contrib = 0, contrib_bytes = 0,
+  size_t aux = 0, aux_bytes = 0, cand = 0, fh = 0, kb = 0, kb_bytes = 0, contrib = 0, contrib_bytes = 0,
          pending = 0, pending_bytes = 0, list = 0, sel = 0, lcount = 0, apart = 0, R = 0, U1 = 0, U2 = 0, B1 = 0,
          B2 = 0, roe = 0, roe_stage_bytes = 0, total = 0;
   size_t roe_dir = 0;   // doubles between two directions' Roe states
@@ -1006,11 +1006,10 @@ AdjLayout adj_layout(const teno_grid* g, int op, int nsm) {
   L.apart = off;   // [ndim][2 blocks][3]: d/dalpha per block of the kept and general passes
   off += round_up(sizeof(double) * 3 * 2 * size_t(adj_blocks(nsm)) * g->ndim);
   if (op == TENO_OP_RK3_ADJOINT) {
-    // half fluxes of the recomputed forward stages (two-pass fluxes)
+    // half fluxes of the recomputed forward stages (two-pass fluxes; their
+    // binary32 planes lie in kb, which the reverse passes fill later)
     L.fh = off;
     off += round_up(sizeof(double) * g->ndim * (nvar - 1) * ncell);
-    L.pf = off;   // and their binary32 planes
-    off += round_up(sizeof(float4) * teno::plane_count(g->ndim) * ncell);
     // forward recomputation (R, U1, U2) and the stage adjoints (B1, B2)
     L.R = off;
     off += round_up(sizeof(double) * nvar * ncell);
@@ -1147,9 +1146,10 @@ teno_status adjoint_sequence(const teno_grid* g, const AdjLayout& L, char* ws, i
   auto* alpha = reinterpret_cast<unsigned long long*>(ws + L.alpha + stage * AdjLayout::kStage);
   auto* argidx = reinterpret_cast<unsigned long long*>(ws + L.argidx + stage * AdjLayout::kStage);
   double* aux = reinterpret_cast<double*>(ws + L.aux + stage * L.aux_bytes);
-  // this stage input's binary32 planes, where its cell pass runs here and the
-  // workspace has room for them
-  float4* pf = cell && L.pf ? reinterpret_cast<float4*>(ws + L.pf) : nullptr;
+  // this stage input's binary32 planes, where its cell pass runs here and there is
+  // room for them: in fh and R, which the forward stages have left by then (6 + 4
+  // and 12 + 5 doubles a cell in 2D and 3D, for planes of 8 and 10)
+  float4* pf = cell && L.fh && g->ndim > 1 ? reinterpret_cast<float4*>(ws + L.fh) : nullptr;
   if (cell) {
     auto* cand = reinterpret_cast<unsigned long long*>(ws + L.cand);
     if (cudaMemsetAsync(alpha, 0, sizeof(unsigned long long) * 9, st) != cudaSuccess) return TENO_ERR_CUDA;
@@ -1254,13 +1254,13 @@ teno_status teno_rk3_step_adjoint(const teno_grid* g, const double* U_n, double 
   if (cudaGetLastError() != cudaSuccess) return TENO_ERR_CUDA;
   double* roe0 = reinterpret_cast<double*>(w + L.roe);
   double* roe1 = reinterpret_cast<double*>(w + L.roe + L.roe_stage_bytes);
-  teno_status s = teno::forward_stage(g, w, L.status, L.dt, L.alpha, L.aux, L.fh, L.pf, L.contrib, L.list, U_n, R,
+  teno_status s = teno::forward_stage(g, w, L.status, L.dt, L.alpha, L.aux, L.fh, L.kb, L.contrib, L.list, U_n, R,
                                       2, U_n, nullptr, U1, st, cand, roe0, L.roe_dir);
   if (s != TENO_OK) return s;
   if (teno::launch_argmax_finish(g->ndim, cand, ncell, nsm, reinterpret_cast<unsigned long long*>(w + L.argidx),
                                  st) != cudaSuccess)
     return TENO_ERR_CUDA;
-  s = teno::forward_stage(g, w, L.status, L.dt, L.alpha + AdjLayout::kStage, L.aux + L.aux_bytes, L.fh, L.pf, L.contrib,
+  s = teno::forward_stage(g, w, L.status, L.dt, L.alpha + AdjLayout::kStage, L.aux + L.aux_bytes, L.fh, L.kb, L.contrib,
                           L.list, U1, R, 3, U_n, U1, U2, st, cand, roe1, L.roe_dir);
   if (s != TENO_OK) return s;
   if (teno::launch_argmax_finish(g->ndim, cand, ncell, nsm,

@@ -94,8 +94,11 @@ Layout layout_of(const teno_grid* g, int op) {
   off += round_up(sizeof(double) * teno::aux_fields(g->ndim) * ncell);
   L.fh = off;   // half physical fluxes F_d/2 per cell and direction (no mass component)
   off += round_up(sizeof(double) * g->ndim * (nvar - 1) * ncell);
-  L.pf = off;   // binary32 copies of the cells (store_planes)
-  off += round_up(sizeof(float4) * teno::plane_count(g->ndim) * ncell);
+  const bool planes = ncell <= size_t(teno::kPlaneCells);
+  if (planes) {
+    L.pf = off;   // binary32 copies of the cells (store_planes)
+    off += round_up(sizeof(float4) * teno::plane_count(g->ndim) * ncell);
+  }
   const int copies = ncell <= size_t(teno::kMultiCells) ? g->ndim : 1;
   if (copies > 1) {
     L.fstride = nvar * maxifc;
@@ -104,7 +107,7 @@ Layout layout_of(const teno_grid* g, int op) {
   L.fhat = off;
   off += round_up(sizeof(double) * nvar * size_t(maxifc) * copies);
   L.list = off;
-  off += round_up(sizeof(uint2) * size_t(maxifc) * copies);
+  off += round_up((planes ? sizeof(uint2) : sizeof(uint32_t)) * size_t(maxifc) * copies);
   L.ghost = off;   // fixed-state ghost cells (state, primitives, half fluxes of 6 face slots)
   off += round_up(sizeof(double) * size_t(teno::ghost_block_doubles(g->ndim)));
   if (op == TENO_OP_RK3) {
@@ -249,7 +252,7 @@ teno_status stage_begin(const teno_grid* g, const Layout& L, char* ws, const dou
   auto* alpha = reinterpret_cast<unsigned long long*>(ws + L.alpha);
   double* aux = reinterpret_cast<double*>(ws + L.aux);
   double* fh = one_pass ? nullptr : reinterpret_cast<double*>(ws + L.fh);
-  float4* pf = one_pass ? nullptr : reinterpret_cast<float4*>(ws + L.pf);
+  float4* pf = one_pass || !L.pf ? nullptr : reinterpret_cast<float4*>(ws + L.pf);
   TENO_CUDA(cudaMemsetAsync(alpha, 0, teno::kAlphaAndCountBytes, st));
   TimerScope ts(st, TENO_KERNEL_CELL);
   TENO_CUDA(ghost_cells(g, G, st));
@@ -275,7 +278,7 @@ teno_status stage_finish(const teno_grid* g, const Layout& L, char* ws, const do
   double* Fhat = reinterpret_cast<double*>(ws + L.fhat);
   uint2* list = reinterpret_cast<uint2*>(ws + L.list);
   double* fh = flags ? nullptr : reinterpret_cast<double*>(ws + L.fh);   // the flag path is one-pass
-  const float4* pf = reinterpret_cast<const float4*>(ws + L.pf);
+  const float4* pf = L.pf ? reinterpret_cast<const float4*>(ws + L.pf) : nullptr;
   unsigned* count = reinterpret_cast<unsigned*>(ws + L.alpha + teno::kPendingCountOffset);
   if (with_dt) {
     TimerScope ts(st, TENO_KERNEL_DT);

@@ -115,6 +115,26 @@ __device__ __forceinline__ RoeCellDf<NDIM> load_roe_cell(const float4* __restric
   }
   return R;
 }
+// The same from the binary64 arrays, for grids that keep no planes: the values
+// that store_planes would have written.
+template <int NDIM, int DIR, bool GH, class I>
+__device__ __forceinline__ void load_point_d(const double* __restrict__ U, const double* __restrict__ aux,
+                                             const GhostCells& gc, int64_t ncell, I c, float (&X)[NDIM + 2], float& u,
+                                             float& p) {
+#pragma unroll
+  for (int v = 0; v < NDIM + 2; ++v) X[v] = near_float(ldc<GH>(U, gc.U, ncell, v, c));
+  u = near_float(ldc<GH>(aux, gc.aux, ncell, DIR, c));
+  p = near_float(ldc<GH>(aux, gc.aux, ncell, NDIM, c));
+}
+template <int NDIM, bool GH, class I>
+__device__ __forceinline__ RoeCellDf<NDIM> load_roe_cell_d(const double* __restrict__ aux, const GhostCells& gc,
+                                                           int64_t ncell, I c) {
+  double su[NDIM];
+#pragma unroll
+  for (int k = 0; k < NDIM; ++k) su[k] = ldc<GH>(aux, gc.aux, ncell, NDIM + 3 + k, c);
+  return roe_cell<NDIM>(ldc<GH>(aux, gc.aux, ncell, NDIM + 1, c), ldc<GH>(aux, gc.aux, ncell, NDIM + 2, c), su);
+}
+
 // The closed form's Roe state and corrections in binary64, on sums already
 // formed (60 U~ and the mass flux in fixed point, the other fluxes): where the
 // corrections are not small against the flux scale (closed_df_rough), i.e. at
@@ -158,8 +178,9 @@ __device__ __noinline__ void closed_rough(const double* __restrict__ aux, int64_
 // reconstructions (see interface_flux_closed_wide, which takes over, all in
 // binary64, where the interface leaves teno_df's range; closed_rough: near
 // shocks).  I: the cell index type, 32 bits
-// on the grid path; a3: the halved speeds, F: face_speeds of them.
-template <int NDIM, int DIR, bool GH, class I>
+// on the grid path; a3: the halved speeds, F: face_speeds of them.  PF: the cells'
+// binary32 values from the planes pf, else converted here.
+template <int NDIM, int DIR, bool GH, bool PF = true, class I>
 __device__ __forceinline__ unsigned interface_flux_closed(const double* __restrict__ U,
                                                           const double* __restrict__ aux,
                                                           const double* __restrict__ fh,
@@ -175,8 +196,14 @@ __device__ __forceinline__ unsigned interface_flux_closed(const double* __restri
   const df gm1 = gm1_df(S);
   RoeDf<NDIM> R;
   {
-    RoeCellDf<NDIM> ra = load_roe_cell<NDIM, GH>(pf, gc.pf, ncell, cells[2]);
-    RoeCellDf<NDIM> rb = load_roe_cell<NDIM, GH>(pf, gc.pf, ncell, cells[3]);
+    RoeCellDf<NDIM> ra, rb;
+    if constexpr (PF) {
+      ra = load_roe_cell<NDIM, GH>(pf, gc.pf, ncell, cells[2]);
+      rb = load_roe_cell<NDIM, GH>(pf, gc.pf, ncell, cells[3]);
+    } else {
+      ra = load_roe_cell_d<NDIM, GH>(aux, gc, ncell, cells[2]);
+      rb = load_roe_cell_d<NDIM, GH>(aux, gc, ncell, cells[3]);
+    }
     const float fa = (flips >> 2) & 1u ? -1.0f : 1.0f, fb = (flips >> 3) & 1u ? -1.0f : 1.0f;
     ra.su[DIR] = scale(ra.su[DIR], fa);
     rb.su[DIR] = scale(rb.su[DIR], fb);
@@ -193,7 +220,8 @@ __device__ __forceinline__ unsigned interface_flux_closed(const double* __restri
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
       float X[NVAR], u, p;
-      load_point_f<NDIM, DIR, GH>(pf, gc.pf, ncell, cells[j], X, u, p);
+      if constexpr (PF) load_point_f<NDIM, DIR, GH>(pf, gc.pf, ncell, cells[j], X, u, p);
+      else load_point_d<NDIM, DIR, GH>(U, aux, gc, ncell, cells[j], X, u, p);
       const uint32_t fj = ((flips >> j) & 1u) << 31;
       X[1 + DIR] = __uint_as_float(__float_as_uint(X[1 + DIR]) ^ fj);
       u = __uint_as_float(__float_as_uint(u) ^ fj);

@@ -1,7 +1,7 @@
 // teno_closed_all.cu -- the closed-form pass of every direction in one launch,
-// for grids whose interfaces of one direction do not fill the chip (a
-// translation unit of its own: the three directions' loops compile in parallel
-// with the per-direction kernels).
+// for grids whose interfaces of one direction do not fill the chip, and the
+// passes without binary32 planes for the largest grids (a translation unit of
+// its own: it compiles in parallel with the per-direction kernels).
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -56,6 +56,49 @@ cudaError_t launch_closed_all(int ndim, const double* U, const double* aux, cons
     else flux_closed_all_kernel<3, 3><<<grid, 128, 0, st>>>(U, aux, fh, pf, alpha, Fhat, fstride, list, lstride, count, status, G, S);
   }
   return cudaGetLastError();
+}
+
+// One direction on a grid of more than kPlaneCells cells, which keeps no planes
+// and a list of indices: the conversions at each of the stencil's points, and
+// every reconstruction of a listed interface decided -- the same fluxes.
+template <int NDIM, int DIR, int WALL>
+__global__ void __launch_bounds__(128, 3) flux_closed_noplanes_kernel(
+    const double* __restrict__ U, const double* __restrict__ aux, const double* __restrict__ fh,
+    const unsigned long long* __restrict__ alpha_bits, double* __restrict__ Fhat, uint32_t* __restrict__ list,
+    unsigned* __restrict__ count, int* __restrict__ status, Grid G, Scheme S) {
+  closed_faces<NDIM, DIR, WALL, false, false>(U, aux, fh, nullptr, alpha_bits, Fhat, list, count, status, G, S,
+                                              nullptr);
+}
+template <int NDIM, int DIR, bool GH>
+__global__ void __launch_bounds__(128) flux_correct_noplanes_kernel(
+    const double* __restrict__ U, const double* __restrict__ aux,
+    const unsigned long long* __restrict__ alpha_bits, double* __restrict__ Fhat, const uint32_t* __restrict__ list,
+    const unsigned* __restrict__ count, int* __restrict__ status, Grid G, Scheme S, int nsm) {
+  __shared__ CorrectScratch<NDIM> scratch[4];
+  correct_list<NDIM, DIR, GH>(U, aux, alpha_bits, Fhat, list, *count, status, G, S, nsm, scratch[threadIdx.x >> 5]);
+}
+
+template <int NDIM, int DIR>
+static void noplanes_dir(const double* U, const double* aux, const double* fh, const unsigned long long* alpha,
+                         double* Fhat, uint32_t* list, unsigned* count, int* status, const Grid& G, const Scheme& S,
+                         int nsm, int blocks, int cblocks, cudaStream_t st) {
+  // (WALL 1 also covers plain boundaries: the mirror flags are then 0)
+  if (G.bc[DIR] == TENO_BC_DIRICHLET) {
+    flux_closed_noplanes_kernel<NDIM, DIR, 2><<<blocks, 128, 0, st>>>(U, aux, fh, alpha, Fhat, list, count, status, G, S);
+    flux_correct_noplanes_kernel<NDIM, DIR, true><<<cblocks, 128, 0, st>>>(U, aux, alpha, Fhat, list, count, status, G, S, nsm);
+  } else {
+    flux_closed_noplanes_kernel<NDIM, DIR, 1><<<blocks, 128, 0, st>>>(U, aux, fh, alpha, Fhat, list, count, status, G, S);
+    flux_correct_noplanes_kernel<NDIM, DIR, false><<<cblocks, 128, 0, st>>>(U, aux, alpha, Fhat, list, count, status, G, S, nsm);
+  }
+}
+
+void launch_flux_noplanes(int ndim, int dir, const double* U, const double* aux, const double* fh,
+                          const unsigned long long* alpha, double* Fhat, uint32_t* list, unsigned* count, int* status,
+                          const Grid& G, const Scheme& S, int nsm, int blocks, int cblocks, cudaStream_t st) {
+  auto* f = ndim == 1 ? noplanes_dir<1, 0>
+            : ndim == 2 ? (dir == 0 ? noplanes_dir<2, 0> : noplanes_dir<2, 1>)
+                        : (dir == 0 ? noplanes_dir<3, 0> : (dir == 1 ? noplanes_dir<3, 1> : noplanes_dir<3, 2>));
+  f(U, aux, fh, alpha, Fhat, list, count, status, G, S, nsm, blocks, cblocks, st);
 }
 
 }  // namespace teno

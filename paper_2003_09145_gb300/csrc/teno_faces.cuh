@@ -112,12 +112,14 @@ __device__ __forceinline__ void half_speeds(const unsigned long long* __restrict
 // certificate and the adjoint's closed-form VJP read: u~, |u~|^2, H~, c~,
 // b1, b1/2, b2/2, 1/(2c~)) and the certificate's decision (1 kept, 0
 // pending) also go to roe_out[ndim + 8][nifc], for the adjoint of this
-// stage.
-template <int NDIM, int DIR, int WALL, bool ROE>
+// stage.  PF: with the cells' binary32 planes; without them (the largest grids)
+// the list holds indices alone, its reconstructions all count as open, and a
+// face whose flux stays unwritten (kRough) is marked by a NaN.
+template <int NDIM, int DIR, int WALL, bool ROE, bool PF = true, class Entry = uint2>
 __device__ __forceinline__ void closed_faces(
     const double* __restrict__ U, const double* __restrict__ aux, const double* __restrict__ fh,
     const float4* __restrict__ pf, const unsigned long long* __restrict__ alpha_bits, double* __restrict__ Fhat,
-    uint2* __restrict__ list, unsigned* __restrict__ count, int* __restrict__ status, const Grid& G,
+    Entry* __restrict__ list, unsigned* __restrict__ count, int* __restrict__ status, const Grid& G,
     const Scheme& S, double* __restrict__ roe_out) {
   constexpr int NVAR = NDIM + 2;
   const int64_t nifc = (G.n[0] + (DIR == 0)) * (G.n[1] + (DIR == 1)) * (G.n[2] + (DIR == 2));
@@ -156,7 +158,7 @@ __device__ __forceinline__ void closed_faces(
     else
       interface_cells<NDIM, DIR, false>(static_cast<uint32_t>(q), G, cells, flips);
     double out[NVAR];
-    const unsigned open = interface_flux_closed<NDIM, DIR, (WALL >= 2)>(
+    const unsigned open = interface_flux_closed<NDIM, DIR, (WALL >= 2), PF>(
         U, aux, fh + (int64_t)DIR * (NVAR - 1) * G.ncell, pf, G.ncell, cells, WALL & 1 ? flips : 0u, a3, F, S, out,
         status, GhostCells{G.gU, G.gaux, G.gfh, G.gpf});
     if constexpr (ROE) {
@@ -183,7 +185,12 @@ __device__ __forceinline__ void closed_faces(
         roe_out[(int64_t)(NDIM + 7) * nifc + q] = open ? 0.0 : 1.0;
       }
     }
-    if (!(open & kRough)) {
+    if constexpr (!PF) {
+      if (open & kRough)
+#pragma unroll
+        for (int v = 0; v < NVAR; ++v) out[v] = __longlong_as_double(0x7FF8000000000000ll);
+    }
+    if (!PF || !(open & kRough)) {
 #pragma unroll
       for (int v = 0; v < NVAR; ++v) Fhat[(int64_t)v * nifc + q] = out[v];
     }
@@ -195,8 +202,55 @@ __device__ __forceinline__ void closed_faces(
       unsigned at = 0;
       if (lane == leader) at = atomicAdd(count, __popc(m));
       at = __shfl_sync(act, at, leader);
-      if (open) list[at + __popc(m & ((1u << lane) - 1u))] = make_uint2(static_cast<uint32_t>(q), open);
+      if (open) {
+        Entry& e = list[at + __popc(m & ((1u << lane) - 1u))];
+        if constexpr (PF) e = make_uint2(static_cast<uint32_t>(q), open);
+        else e = static_cast<uint32_t>(q);
+      }
     }
+  }
+}
+
+// An FP64 instruction holds its SM partition's pipe for 64 cycles whatever
+// lanes are active, so a warp's time is its FP64 instruction count.  A warp
+// takes 32 listed interfaces when there are enough for every partition of
+// the chip, and fewer (2, 4, 8, 16) when the list is short: a short list is
+// bound by one warp's chain, and few interfaces finish in a single round.
+template <int NDIM, int DIR, bool GH, class Entry>
+__device__ __forceinline__ void correct_list(const double* __restrict__ U, const double* __restrict__ aux,
+                                             const unsigned long long* __restrict__ alpha_bits,
+                                             double* __restrict__ Fhat, const Entry* __restrict__ list, int64_t n,
+                                             int* __restrict__ status, const Grid& G, const Scheme& S, int nsm,
+                                             CorrectScratch<NDIM>& W) {
+  constexpr int NVAR = NDIM + 2;
+  const int64_t nifc = (G.n[0] + (DIR == 0)) * (G.n[1] + (DIR == 1)) * (G.n[2] + (DIR == 2));
+  const int64_t nw = (int64_t)gridDim.x * 4;
+  int per = 2;
+  while (per < 32 && n > (int64_t)per * 4 * nsm) per *= 2;
+  const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  if (blockIdx.x * (int64_t)(4 * per) >= n) return;
+  double alpha[NVAR], nal[NVAR];
+  half_speeds<NDIM, DIR>(alpha_bits, alpha, nal);
+  const bool ghost_dir = GH && G.bc[DIR] == TENO_BC_DIRICHLET;
+  auto cells_of = [&](uint32_t q, uint32_t (&cells)[6], unsigned& flips) {
+    if (ghost_dir) interface_cells<NDIM, DIR, GH>(q, G, cells, flips);
+    else interface_cells<NDIM, DIR, false>(q, G, cells, flips);
+  };
+  for (int64_t i0 = ((int64_t)blockIdx.x * 4 + warp) * per; i0 < n; i0 += nw * per) {
+    const int64_t i = i0 + lane;
+    uint2 e = make_uint2(0u, 0u);
+    if (lane < per && i < n) {
+      if constexpr (sizeof(Entry) == sizeof(uint2)) e = list[i];
+      else e = make_uint2(list[i], kAllOpen<NDIM>);
+    }
+    double out[NVAR];
+#pragma unroll
+    for (int v = 0; v < NVAR; ++v) out[v] = e.y && !(e.y & kRough) ? Fhat[(int64_t)v * nifc + e.x] : 0.0;
+    warp_correct<NDIM, DIR, GH, uint32_t>(U, aux, G.ncell, cells_of, e.x, alpha, S, e.y, out, status, W,
+                                          GhostCells{G.gU, G.gaux, G.gfh, G.gpf});
+    if (e.y)
+#pragma unroll
+      for (int v = 0; v < NVAR; ++v) Fhat[(int64_t)v * nifc + e.x] = out[v];
   }
 }
 

@@ -306,45 +306,6 @@ __global__ void __launch_bounds__(128, TENO_CLOSED_MINBLOCKS) flux_closed_kernel
   closed_faces<NDIM, DIR, WALL, ROE>(U, aux, fh, pf, alpha_bits, Fhat, list, count, status, G, S, roe_out);
 }
 
-// An FP64 instruction holds its SM partition's pipe for 64 cycles whatever
-// lanes are active, so a warp's time is its FP64 instruction count.  A warp
-// takes 32 listed interfaces when there are enough for every partition of
-// the chip, and fewer (2, 4, 8, 16) when the list is short: a short list is
-// bound by one warp's chain, and few interfaces finish in a single round.
-template <int NDIM, int DIR, bool GH>
-__device__ __forceinline__ void correct_list(const double* __restrict__ U, const double* __restrict__ aux,
-                                             const unsigned long long* __restrict__ alpha_bits,
-                                             double* __restrict__ Fhat, const uint2* __restrict__ list, int64_t n,
-                                             int* __restrict__ status, const Grid& G, const Scheme& S, int nsm,
-                                             CorrectScratch<NDIM>& W) {
-  constexpr int NVAR = NDIM + 2;
-  const int64_t nifc = (G.n[0] + (DIR == 0)) * (G.n[1] + (DIR == 1)) * (G.n[2] + (DIR == 2));
-  const int64_t nw = (int64_t)gridDim.x * 4;
-  int per = 2;
-  while (per < 32 && n > (int64_t)per * 4 * nsm) per *= 2;
-  const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-  if (blockIdx.x * (int64_t)(4 * per) >= n) return;
-  double alpha[NVAR], nal[NVAR];
-  half_speeds<NDIM, DIR>(alpha_bits, alpha, nal);
-  const bool ghost_dir = GH && G.bc[DIR] == TENO_BC_DIRICHLET;
-  auto cells_of = [&](uint32_t q, uint32_t (&cells)[6], unsigned& flips) {
-    if (ghost_dir) interface_cells<NDIM, DIR, GH>(q, G, cells, flips);
-    else interface_cells<NDIM, DIR, false>(q, G, cells, flips);
-  };
-  for (int64_t i0 = ((int64_t)blockIdx.x * 4 + warp) * per; i0 < n; i0 += nw * per) {
-    const int64_t i = i0 + lane;
-    const uint2 e = lane < per && i < n ? list[i] : make_uint2(0u, 0u);
-    double out[NVAR];
-#pragma unroll
-    for (int v = 0; v < NVAR; ++v) out[v] = e.y && !(e.y & kRough) ? Fhat[(int64_t)v * nifc + e.x] : 0.0;
-    warp_correct<NDIM, DIR, GH, uint32_t>(U, aux, G.ncell, cells_of, e.x, alpha, S, e.y, out, status, W,
-                                          GhostCells{G.gU, G.gaux, G.gfh, G.gpf});
-    if (e.y)
-#pragma unroll
-      for (int v = 0; v < NVAR; ++v) Fhat[(int64_t)v * nifc + e.x] = out[v];
-  }
-}
-
 template <int NDIM, int DIR, bool GH>
 __global__ void __launch_bounds__(128) flux_correct_kernel(
     const double* __restrict__ U, const double* __restrict__ aux,
@@ -796,6 +757,11 @@ static int flux_launch(int blocks, int threads, int pblocks, int nsm, cudaStream
     else flux_wenoz_kernel<NDIM, DIR, false><<<pblocks, threads, 0, st>>>(U, aux, alpha, Fhat, status, G, S);
     return 1;
   }
+  if (!pf) {
+    launch_flux_noplanes(NDIM, DIR, U, aux, fh, alpha, Fhat, reinterpret_cast<uint32_t*>(list), count, status, G, S,
+                         nsm, blocks, pblocks, st);
+    return 2;
+  }
   if (G.bc[DIR] == TENO_BC_REFLECTIVE)
     flux_closed_kernel<NDIM, DIR, 1><<<blocks, threads, 0, st>>>(U, aux, fh, pf, alpha, Fhat, list, count, status, G, S);
   else if (gh)
@@ -821,7 +787,7 @@ cudaError_t launch_flux(int ndim, int dir, const double* U, const double* aux, c
   int64_t nifc = 1;
   for (int k = 0; k < 3; ++k) nifc *= G.n[k] + (k == dir ? 1 : 0);
   if (nifc > int64_t(UINT32_MAX)) list = nullptr;   // list entries are 32-bit
-  if (!count || !fh || !pf) list = nullptr;
+  if (!count || !fh) list = nullptr;
   const int threads = 128;
   const int blocks = blocks_for(nifc, threads, nsm * 64);
   const int pblocks = blocks_for(nifc, threads, nsm * 16);

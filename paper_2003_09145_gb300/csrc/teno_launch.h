@@ -43,8 +43,8 @@ cudaError_t launch_argmax_finish(int ndim, const unsigned long long* cand, int64
 // The interface fluxes of direction `dir` into Fhat.  With `flags`, or
 // without a pending list or the cell pass's half fluxes `fh`, one pass; with
 // `list` (room for one entry per interface: its index and the mask of its
-// open reconstructions), its counter `count` (zero on entry) and `fh`, the
-// closed-form pass and the pass that corrects the listed interfaces.  `launches` (optional) receives the number
+// open reconstructions; without `pf` its index alone, 32 bits), its counter
+// `count` (zero on entry) and `fh`, the closed-form pass and the pass that corrects the listed interfaces.  `launches` (optional) receives the number
 // of kernels launched.  With `roe_out` (two-pass fluxes without reflecting or
 // fixed-state faces only) the closed-form pass also writes every
 // interface's Roe state and its certificate's decision, [ndim + 8][#interfaces]
@@ -73,6 +73,17 @@ cudaError_t launch_diff(int ndim, int dir, const double* Fhat, double* R,
                         const double* Un, const double* Uk, double* Uout,
                         const double* dt, const Grid& G, int mode,
                         int nsm, cudaStream_t st, const double* Usrc);
+
+// Grids of more than kPlaneCells cells keep no binary32 planes and lists of
+// indices alone (4 instead of 8 bytes an interface): 372 instead of 456 bytes a
+// cell for a 3D step and its state, so that boxes up to 7.9e8 cells fit instead
+// of 6.4e8.  The planes pay where there is room (a 400^3 step 93 ms with, 123
+// without; 640^3 338, 440), so the line lies where a step and its state take two
+// thirds of the memory with them (184 GB).
+constexpr int64_t kPlaneCells = int64_t(3) << 27;
+void launch_flux_noplanes(int ndim, int dir, const double* U, const double* aux, const double* fh,
+                          const unsigned long long* alpha, double* Fhat, uint32_t* list, unsigned* count, int* status,
+                          const Grid& G, const Scheme& S, int nsm, int blocks, int cblocks, cudaStream_t st);
 
 // Grids up to kMultiCells cells (a 256^3 step: 21.59 against 21.40 ms; beyond
 // that the buffers' memory counts) keep one flux buffer and
