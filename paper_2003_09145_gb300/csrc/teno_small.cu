@@ -17,10 +17,15 @@
 //
 // Range of sizes: an FP64 instruction holds an SM partition for 64 cycles per
 // warp, so 16 CTAs fall behind 152 SMs once a partition has many warps.
-// Measured (us per step, one launch against one per pass; smooth tube, and a
-// Mach-3 shock into waves): 55 / 63 against 114 / 194 at 100 cells, 64 / 78
-// against 105 / 148 at 4096, 90 / 122 against 105 / 129 at 8192, 131 / 228
-// against 105 / 117 at 16384; the line is drawn at 16 CTAs of 384 cells.
+// Measured, us per step, one launch against one per pass, on a smooth tube and on a
+// Mach-3 shock into waves (plain calls; in brackets inside a CUDA graph):
+//     200 cells   54 / 100 (49 / 78)     68 / 159 (63 / 138)
+//    4096         65 / 107 (58 / 84)     78 / 160 (72 / 134)
+//    6144         81 / 107 (76 / 84)    113 / 120 (107 / 97)
+//    8192         92 / 107 (86 / 84)    130 / 121 (124 / 98)
+//   16384        135 / 108 (129 / 84)   228 / 114 (222 / 89)
+// so the line is drawn at 16 CTAs of 384 cells.
+#include <atomic>
 #include <cmath>
 #include <cooperative_groups.h>
 #include <cstdint>
@@ -237,40 +242,78 @@ __global__ void __launch_bounds__(kSmallThreads) step1d_kernel(SmallStep A, Grid
 
 }  // namespace
 
-// (ndim, not the extents: a 2D or 3D grid of one cell across still has the
-// other momenta and their directions' speeds)
-bool small_step_applies(int ndim, const Grid& G, const Scheme& S) {
-  return ndim == 1 && G.ncell <= kSmallStepMax && S.variant != kSchemeWenoZ;
-}
+namespace {
 
-cudaError_t launch_step1d(const SmallStep& A, const Grid& G, const Scheme& S, cudaStream_t st) {
-  const bool wall = G.bc[0] == TENO_BC_REFLECTIVE, gh = G.bc[0] == TENO_BC_DIRICHLET;
-  void (*k)(SmallStep, Grid, Scheme) = wall ? step1d_kernel<1> : (gh ? step1d_kernel<2> : step1d_kernel<0>);
-  // one warp per SM partition (127 cells a CTA) while 16 CTAs last, then
-  // equal shares in as few tiles as 384 threads allow
-  const int64_t n = G.ncell;
+struct SmallShape {
+  unsigned ctas, threads;
+};
+// one warp per SM partition (127 cells a CTA) while 16 CTAs last, then equal
+// shares in as few tiles as 384 threads allow
+SmallShape small_shape(int64_t n) {
   int64_t ctas = (n + 126) / 127;
   if (ctas > kSmallCtas) ctas = kSmallCtas;
   const int64_t per = (n + ctas - 1) / ctas;
   const int64_t tiles = (per + kSmallThreads - 2) / (kSmallThreads - 1);
   int threads = int(((per + tiles - 1) / tiles + 1 + 31) / 32 * 32);
   if (threads > kSmallThreads) threads = kSmallThreads;
-  if (ctas > 8) {
-    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-  }
+  return {unsigned(ctas), unsigned(threads)};
+}
+
+using SmallKernel = void (*)(SmallStep, Grid, Scheme);
+// 0 plain, 1 reflecting, 2 fixed-state faces
+int small_wall(const Grid& G) { return G.bc[0] == TENO_BC_REFLECTIVE ? 1 : (G.bc[0] == TENO_BC_DIRICHLET ? 2 : 0); }
+SmallKernel small_kernel(int wall) {
+  return wall == 1 ? step1d_kernel<1> : (wall == 2 ? step1d_kernel<2> : step1d_kernel<0>);
+}
+
+struct SmallLaunch {   // (the attribute is referred to by address)
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(unsigned(ctas));
-  cfg.blockDim = dim3(unsigned(threads));
-  cfg.stream = st;
   cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = unsigned(ctas);
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k, A, G, S);
+  SmallLaunch(SmallShape s, cudaStream_t st) {
+    cfg.gridDim = dim3(s.ctas);
+    cfg.blockDim = dim3(s.threads);
+    cfg.stream = st;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = s.ctas;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+  }
+};
+
+// Whether the current device can hold the cluster at all (more than eight CTAs
+// are beyond the portable size, and a device or context with few SMs may not
+// schedule them together).  Asked once per device, kernel and shape.
+bool cluster_fits(int wall, SmallShape s) {
+  static std::atomic<signed char> known[64][3][kSmallCtas + 1][kSmallThreads / 32 + 1];   // 0 not asked, 1, -1
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  std::atomic<signed char>* k = dev < 64 ? &known[dev][wall][s.ctas][s.threads / 32] : nullptr;
+  if (k && k->load(std::memory_order_relaxed)) return k->load(std::memory_order_relaxed) > 0;
+  const SmallKernel f = small_kernel(wall);
+  const SmallLaunch l(s, nullptr);
+  int n = 0;
+  const bool ok = (s.ctas <= 8 ||
+                   cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) &&
+                  cudaOccupancyMaxActiveClusters(&n, f, &l.cfg) == cudaSuccess && n > 0;
+  if (!ok) cudaGetLastError();   // no error of the step: it takes a launch per pass
+  if (k) k->store(ok ? 1 : -1, std::memory_order_relaxed);
+  return ok;
+}
+
+}  // namespace
+
+// (ndim, not the extents: a 2D or 3D grid of one cell across still has the
+// other momenta and their directions' speeds)
+bool small_step_applies(int ndim, const Grid& G, const Scheme& S) {
+  return ndim == 1 && G.ncell <= kSmallStepMax && S.variant != kSchemeWenoZ &&
+         cluster_fits(small_wall(G), small_shape(G.ncell));
+}
+
+cudaError_t launch_step1d(const SmallStep& A, const Grid& G, const Scheme& S, cudaStream_t st) {
+  const SmallLaunch l(small_shape(G.ncell), st);
+  return cudaLaunchKernelEx(&l.cfg, small_kernel(small_wall(G)), A, G, S);
 }
 
 }  // namespace teno

@@ -185,3 +185,27 @@ def test_cold_region_beside_a_fast_one(api, ndim, n, p_cold):
     b = api.rhs(grid, Ut)
     assert torch.isfinite(b).all()
     assert rel_max_err(b.cpu().numpy(), a.cpu().numpy(), flux_scale(U, n, (1.0,) * ndim)) <= 1e-13
+
+
+def _launches(api, grid, U):
+    import ctypes
+    lib, S = grid.lib, api.Solver(grid)
+    ms, n = (ctypes.c_double * 4)(), (ctypes.c_int64 * 4)()
+    lib.teno_timer_begin()
+    S.step(U.clone())
+    torch.cuda.synchronize()
+    lib.teno_timer_end(ms, n)
+    return sum(n)
+
+
+@pytest.mark.parametrize("n", [1, 127, 128, 1016, 1017, 2032, 6144])
+@pytest.mark.parametrize("bc", [0, 2, 3])
+def test_small_steps_are_one_launch(api, n, bc):
+    """The comparison above is of two paths: up to the rule's limit one launch, then several."""
+    face = [[[1.2, 0.1, 2.9], [0.9, -0.2, 2.4]]] if bc == 3 else None
+    U = torch.from_numpy(_line(n, 5)).cuda()
+    assert _launches(api, api.EulerGrid((n,), (1.0 / n,), (bc,), None, None, face), U) == 1
+    U = torch.from_numpy(_line(6145, 5)).cuda()
+    assert _launches(api, api.EulerGrid((6145,), (1.0,), (bc,), None, None, face), U) >= 12
+    U = torch.from_numpy(_line(n, 5)).cuda()
+    assert _launches(api, api.EulerGrid((n,), (1.0 / n,), (bc,), api.Scheme(scheme="wenoz"), None, face), U) >= 9
