@@ -251,7 +251,7 @@ teno_status stage_begin(const teno_grid* g, const Layout& L, char* ws, const dou
   int* status = reinterpret_cast<int*>(ws + L.status);
   auto* alpha = reinterpret_cast<unsigned long long*>(ws + L.alpha);
   double* aux = reinterpret_cast<double*>(ws + L.aux);
-  double* fh = one_pass ? nullptr : reinterpret_cast<double*>(ws + L.fh);
+  double* fh = reinterpret_cast<double*>(ws + L.fh);
   float4* pf = one_pass || !L.pf ? nullptr : reinterpret_cast<float4*>(ws + L.pf);
   TENO_CUDA(cudaMemsetAsync(alpha, 0, teno::kAlphaAndCountBytes, st));
   TimerScope ts(st, TENO_KERNEL_CELL);
@@ -277,7 +277,7 @@ teno_status stage_finish(const teno_grid* g, const Layout& L, char* ws, const do
   double* aux = reinterpret_cast<double*>(ws + L.aux);
   double* Fhat = reinterpret_cast<double*>(ws + L.fhat);
   uint2* list = reinterpret_cast<uint2*>(ws + L.list);
-  double* fh = flags ? nullptr : reinterpret_cast<double*>(ws + L.fh);   // the flag path is one-pass
+  double* fh = reinterpret_cast<double*>(ws + L.fh);
   const float4* pf = L.pf ? reinterpret_cast<const float4*>(ws + L.pf) : nullptr;
   unsigned* count = reinterpret_cast<unsigned*>(ws + L.alpha + teno::kPendingCountOffset);
   if (with_dt) {

@@ -18,12 +18,9 @@ namespace teno {
 // closed form with every stencil kept, and its certified FP32 test; the
 // interfaces with reconstructions that the test does not prove to be kept go
 // to `list` with the mask of those (one atomic per warp), and
-// flux_correct_kernel adds their differences (warp_correct).  Against
-// the one-pass kernel the closed form's six-point sums are fixed-point sums
-// rounded once (teno_fixsum.cuh: terms on a grid of an eighth of the largest
-// value's ulp, added exactly) where that one chains binary64 operations; the
-// closed-form pass stays small (registers, instruction cache) and its warps
-// do not diverge into the rare slow path.
+// flux_correct_kernel adds their differences (warp_correct).  The
+// closed-form pass stays small (registers, instruction cache) and its warps do
+// not diverge into the rare slow path, as they do in the one-pass kernel.
 // WENO-Z, which keeps no stencil exactly linear, takes flux_wenoz_kernel: the
 // characteristic path at every interface, no list.
 // ---------------------------------------------------------------------------

@@ -133,19 +133,16 @@ __device__ __forceinline__ unsigned cert_open(const CertIfc<NDIM>& C, const Sche
 // R L = I and alpha takes three values, so
 //   F^ = F~ + a_mid U~ + (a_0 - a_mid)(l_0.U~) r_0 + (a_E - a_mid)(l_E.U~) r_E.
 // cell_flux_half gives F_d(U)/2 of one cell (eq. 4.7) from its half u_d and
-// half p -- the grid path stores it per cell and direction, the one-pass
-// path forms it per stencil point, with the same rounding; closed_point adds
-// point j to F~ and U~ as a binary64 chain (the one-pass form's sums; the
-// two-pass kernels use the fixed-point sums below); closed_out forms F^.
+// half p -- the grid path stores it per cell and direction, teno_rhs_noalloc
+// forms it per stencil point, with the same rounding; closed_out forms F^.
 //
 // The sums are kept in integer weights, 30 F~ = sum_j c_j F_j/2 with
 // c = (1,-8,37,37,-8,1) and 60 U~ = sum_j m_j U_j with m = (1,-5,10,-10,5,-1),
-// so that point 0 enters by assignment and point 5 by an add (a multiply
-// fewer per component than with the fractional weights), and every interface
+// so that point 0 enters by assignment and point 5 by an add, and every interface
 // flux is stored as 30 F^ (kFluxScale): the speeds enter closed_out halved,
 // 30 a U~ = (a/2) 60 U~, and the difference pass divides by 30 together with
-// dx (Grid::inv_dx_f).  The mass component of F_d/2 is m_d/2: closed_point
-// sums c_j m_d and closed_out halves it, so the half fluxes need only the
+// dx (Grid::inv_dx_f).  The mass component of F_d/2 is m_d/2: the
+// sum is of c_j m_d and closed_out halves it, so the half fluxes need only the
 // momentum and energy components (v = 1..nvar-1).
 // ---------------------------------------------------------------------------
 // cell_flux_half_ep takes E + p as given (the cell pass has it);
@@ -169,29 +166,6 @@ __device__ __forceinline__ void cell_flux_half(const double (&Uc)[NDIM + 2], dou
   // momentum (u_d/2) m_k (+ p/2 for k = d), energy (u_d/2)(E + p); E + p
   // is formed as E + 2 (p/2), which doubles exactly
   cell_flux_half_ep<NDIM, DIR>(Uc, un, pn, fma(2.0, pn, Uc[NVAR - 1]), Fh);
-}
-
-// (Fhj[0] is not read: the mass sum is sum_j c_j m_d.)
-template <int NDIM, int DIR>
-__device__ __forceinline__ void closed_point(int j, const double (&Uj)[NDIM + 2], const double (&Fhj)[NDIM + 2],
-                                             double (&Ft)[NDIM + 2], double (&Ut)[NDIM + 2]) {
-  constexpr int NVAR = NDIM + 2;
-  const double C[6] = {1.0, -8.0, 37.0, 37.0, -8.0, 1.0};
-  const double Mw[6] = {1.0, -5.0, 10.0, -10.0, 5.0, -1.0};
-#pragma unroll
-  for (int v = 0; v < NVAR; ++v) {
-    const double f = v == 0 ? Uj[1 + DIR] : Fhj[v];
-    if (j == 0) {
-      Ft[v] = f;
-      Ut[v] = Uj[v];
-    } else if (j == 5) {
-      Ft[v] += f;
-      Ut[v] -= Uj[v];
-    } else {
-      Ft[v] = fma(C[j], f, Ft[v]);
-      Ut[v] = fma(Mw[j], Uj[v], Ut[v]);
-    }
-  }
 }
 
 // The same two sums in 64-bit fixed point (teno_fixsum.cuh): integer sums
@@ -325,6 +299,43 @@ __device__ __forceinline__ void closed_out(const double (&Ft)[NDIM + 2], const d
   out[NVAR - 1] = fma(R.H, gs, fma(-(R.u[DIR] * R.cs), ngd, fma(amid, Ut[NVAR - 1], Ft[NVAR - 1])));
 }
 
+// The all-kept flux of a stencil that is in registers (the one-pass form): 60 U~
+// and the mass flux in fixed point, which leaves 30 of its FP64 instructions to the
+// integer pipes, the other fluxes as binary64 chains; where the fixed point does
+// not cover a component, chains throughout.  half(j, Fhj) gives point j's F/2.
+template <int NDIM, int DIR, class Half>
+__device__ __forceinline__ void closed_in_registers(const double (&Ux)[6][NDIM + 2], const Half& half,
+                                                    const RoeIfc<NDIM>& R, const double (&nal)[NDIM + 2],
+                                                    double (&out)[NDIM + 2]) {
+  constexpr int NVAR = NDIM + 2;
+  constexpr int kC[6] = {1, -8, 37, 37, -8, 1}, kM[6] = {1, -5, 10, -10, 5, -1};
+  double Ft[NVAR], Ut[NVAR];
+#pragma unroll
+  for (int j = 0; j < 6; ++j) {
+    double Fhj[NVAR];
+    half(j, Fhj);
+#pragma unroll
+    for (int v = 1; v < NVAR; ++v) Ft[v] = j == 0 ? Fhj[v] : (j == 5 ? Ft[v] + Fhj[v] : fma(double(kC[j]), Fhj[v], Ft[v]));
+  }
+#pragma unroll
+  for (int v = 0; v < NVAR; ++v) {
+    double x[6];
+#pragma unroll
+    for (int j = 0; j < 6; ++j) x[j] = Ux[j][v];
+    if (!teno_fix::sum<6>(x, kM, Ut[v])) {
+      Ut[v] = x[0] - x[5];
+#pragma unroll
+      for (int j = 1; j < 5; ++j) Ut[v] = fma(double(kM[j]), x[j], Ut[v]);
+    }
+    if (v == 1 + DIR && !teno_fix::sum<6>(x, kC, Ft[0])) {
+      Ft[0] = x[0] + x[5];
+#pragma unroll
+      for (int j = 1; j < 5; ++j) Ft[0] = fma(double(kC[j]), x[j], Ft[0]);
+    }
+  }
+  closed_out<NDIM, DIR>(Ft, Ut, R, nal, out);
+}
+
 // the three halved speeds (a_-, a_mid, a_+) per field, and their negated doubles
 template <int NDIM>
 __device__ __forceinline__ void spread_speeds(const double (&a3)[3], double (&alpha)[NDIM + 2],
@@ -343,8 +354,7 @@ __device__ __forceinline__ void spread_speeds(const double (&a3)[3], double (&al
 // of the sums), then the sums, so that the test's state is dead
 // before the sums' state is live.  Returns the open reconstructions (bit
 // 2 s + side of field s, cert_open's mask): 0 -- the test keeps every stencil
-// and `out` is the flux (interface_flux's up to the rounding of the sums,
-// which that one-pass form evaluates as binary64 chains); else `out` holds
+// and `out` is the flux (interface_flux's); else `out` holds
 // the flux with every stencil kept, to which warp_correct adds the
 // open reconstructions' differences.  kRough: the fixed point does not cover
 // a sum and `out` is unwritten (warp_correct then sums every field).
@@ -713,7 +723,8 @@ __device__ __forceinline__ void interface_flux(const double* __restrict__ U,
                                                const Scheme& S, double (&out)[NDIM + 2],
                                                unsigned (&fl)[NDIM + 2][2],
                                                int* __restrict__ status,
-                                               const GhostCells& gc = GhostCells()) {
+                                               const GhostCells& gc = GhostCells(),
+                                               const double* __restrict__ fh = nullptr) {
   constexpr int NVAR = NDIM + 2;
   {
     // six-point stencil i-2..i+3 with i = id - 1
@@ -747,6 +758,17 @@ __device__ __forceinline__ void interface_flux(const double* __restrict__ U,
     const double (&u)[NDIM] = R.u;
     const double q2 = R.q2, H = R.H, cs = R.cs, b1 = R.b1;
     const double hb1 = R.hb1, hb2 = R.hb2, hic = R.hic, hud = R.hud;
+    // F/2 of stencil point j: the cell pass's with flags, else formed here
+    auto half = [&](int j, double (&Fhj)[NVAR]) {
+      if constexpr (WITH_FLAGS) {
+        const bool fj = (flips >> j) & 1u;
+#pragma unroll
+        for (int v = 1; v < NVAR; ++v)
+          Fhj[v] = flip_sign(ldc<GH>(fh, gc.fh, ncell, DIR * (NVAR - 1) + v - 1, cells[j]), fj && v != 1 + DIR);
+      } else {
+        cell_flux_half<NDIM, DIR>(Ux[j], un[j], pn[j], Fhj);
+      }
+    };
 
     if (!WITH_FLAGS && MODE != kFluxChar && S.keep_idx >= 0) {
       CertIfc<NDIM> C;
@@ -761,16 +783,7 @@ __device__ __forceinline__ void interface_flux(const double* __restrict__ U,
         return;
       }
       if (keep) {
-        // (the sums as binary64 chains: this one-pass form holds the whole
-        // stencil in registers already)
-        double Ft[NVAR], Ut[NVAR];
-#pragma unroll
-        for (int j = 0; j < 6; ++j) {
-          double Fhj[NVAR];
-          cell_flux_half<NDIM, DIR>(Ux[j], un[j], pn[j], Fhj);
-          closed_point<NDIM, DIR>(j, Ux[j], Fhj, Ft, Ut);
-        }
-        closed_out<NDIM, DIR>(Ft, Ut, R, nal, out);
+        closed_in_registers<NDIM, DIR>(Ux, half, R, nal, out);
 #pragma unroll
         for (int f = 0; f < NVAR; ++f) fl[f][0] = fl[f][1] = 7u;
         return;
@@ -786,17 +799,13 @@ __device__ __forceinline__ void interface_flux(const double* __restrict__ U,
     // (WENO-Z keeps no stencil exactly linear: always the whole values).
     bool cut = S.variant != kSchemeWenoZ;
     if (cut) {
-      double Ft[NVAR], Ut[NVAR];
       float rm = 0.0f, em = 0.0f;
 #pragma unroll
       for (int j = 0; j < 6; ++j) {
-        double Fhj[NVAR];
-        cell_flux_half<NDIM, DIR>(Ux[j], un[j], pn[j], Fhj);
-        closed_point<NDIM, DIR>(j, Ux[j], Fhj, Ft, Ut);
         rm = fmaxf(rm, fabsf(hi_float(Ux[j][0])));
         em = fmaxf(em, fabsf(hi_float(Ux[j][NVAR - 1])));
       }
-      closed_out<NDIM, DIR>(Ft, Ut, R, nal, out);
+      closed_in_registers<NDIM, DIR>(Ux, half, R, nal, out);
       cut = !beyond_flux_scale<NDIM>(out, alpha, rm, em);
     }
     if (!cut)
@@ -838,6 +847,12 @@ __device__ __forceinline__ void interface_flux(const double* __restrict__ U,
     for (int s = 0; s < NVAR; ++s) {
       const double hp = teno5_lad<WITH_FLAGS>(vp[0][s], vp[1][s], vp[2][s], vp[3][s], vp[4][s], 0.0, S, fl[s][0], cut);
       fchar[s] = teno5_lad<WITH_FLAGS>(vm[5][s], vm[4][s], vm[3][s], vm[2][s], vm[1][s], hp, S, fl[s][1], cut);
+    }
+    if (cut) {   // every stencil kept: the differences are zeros
+      bool none = true;
+#pragma unroll
+      for (int s = 0; s < NVAR; ++s) none = none && (dbits(fchar[s]) << 1) == 0ull;
+      if (none) return;
     }
     // back-projection F^ = R f^char, columns r_0 = (1, u - c e_n, H - u_n c),
     // r_1 = (1, u, q2/2), r_t = (0, e_t, u_t), r_{nvar-1} = (1, u + c e_n, H + u_n c),

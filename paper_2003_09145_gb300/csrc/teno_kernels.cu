@@ -227,13 +227,19 @@ __global__ void __launch_bounds__(kArgThreads) argmax_finish_kernel(const unsign
 // Interface fluxes of direction DIR.
 // ---------------------------------------------------------------------------
 
+// What bounds it: FP64 issue.  Against the whole characteristic values at every
+// interface (whose error on a 1e5 Pa state is 1.2e-13 of the flux scale, not 3e-14)
+// the all-kept flux costs up to a tenth where many selections cut and nothing
+// where few do: right-hand sides with flags at 160^3 12.7 against 12.8 ms, 1024^2
+// 1.97 / 1.91, 64^3 1.20 / 1.09, 4096 cells 39 / 37 us; with the all-kept sums as
+// chains of half fluxes formed here 14.1, 2.18, 1.21 ms, 40 us.
 #ifndef TENO_FLUX_MINBLOCKS
 #define TENO_FLUX_MINBLOCKS 4
 #endif
 
 template <int NDIM, int DIR, bool WITH_FLAGS, bool GH>
 __global__ void __launch_bounds__(128, TENO_FLUX_MINBLOCKS) flux_kernel(
-    const double* __restrict__ U, const double* __restrict__ aux,
+    const double* __restrict__ U, const double* __restrict__ aux, const double* __restrict__ fh,
     const unsigned long long* __restrict__ alpha_bits, double* __restrict__ Fhat,
     uint8_t* __restrict__ flags, int* __restrict__ status, Grid G, Scheme S) {
   constexpr int NVAR = NDIM + 2;
@@ -283,7 +289,7 @@ __global__ void __launch_bounds__(128, TENO_FLUX_MINBLOCKS) flux_kernel(
     double out[NVAR];
     unsigned fl[NVAR][2];
     interface_flux<NDIM, DIR, WITH_FLAGS, kFluxFull, GH>(U, aux, ncell, cells, flips, alpha, nal, S, out, fl, status,
-                                                        GhostCells{G.gU, G.gaux, G.gfh, G.gpf});
+                                                        GhostCells{G.gU, G.gaux, G.gfh, G.gpf}, fh);
     if (WITH_FLAGS) {
       // direction block offset is applied by the caller through `flags`
 #pragma unroll
@@ -746,10 +752,10 @@ static int flux_launch(int blocks, int threads, int pblocks, int nsm, cudaStream
                        const Scheme& S, double* roe_out, bool correct) {
   const bool gh = G.bc[DIR] == TENO_BC_DIRICHLET;
   if (flags || !list) {
-    if (flags && gh) flux_kernel<NDIM, DIR, true, true><<<blocks, threads, 0, st>>>(U, aux, alpha, Fhat, flags, status, G, S);
-    else if (flags) flux_kernel<NDIM, DIR, true, false><<<blocks, threads, 0, st>>>(U, aux, alpha, Fhat, flags, status, G, S);
-    else if (gh) flux_kernel<NDIM, DIR, false, true><<<blocks, threads, 0, st>>>(U, aux, alpha, Fhat, flags, status, G, S);
-    else flux_kernel<NDIM, DIR, false, false><<<blocks, threads, 0, st>>>(U, aux, alpha, Fhat, flags, status, G, S);
+    if (flags && gh) flux_kernel<NDIM, DIR, true, true><<<blocks, threads, 0, st>>>(U, aux, fh, alpha, Fhat, flags, status, G, S);
+    else if (flags) flux_kernel<NDIM, DIR, true, false><<<blocks, threads, 0, st>>>(U, aux, fh, alpha, Fhat, flags, status, G, S);
+    else if (gh) flux_kernel<NDIM, DIR, false, true><<<blocks, threads, 0, st>>>(U, aux, fh, alpha, Fhat, flags, status, G, S);
+    else flux_kernel<NDIM, DIR, false, false><<<blocks, threads, 0, st>>>(U, aux, fh, alpha, Fhat, flags, status, G, S);
     return 1;
   }
   if (S.variant == kSchemeWenoZ) {
