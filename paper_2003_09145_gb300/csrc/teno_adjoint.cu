@@ -12,15 +12,16 @@
 //   cell pass        : primitives, speeds and their arg-max cells (skipped
 //                      where the recomputed forward stage already made them);
 //   per direction d:
-//     adj_kept_kernel  : one thread per interface: the forward pass's certified
-//                        FP32 test; where it keeps every stencil, the
-//                        closed-form interface VJP (teno_adjoint_core.cuh)
+//     adj_open_kernel  : the forward pass's certified FP32 test at every interface
+//                        (skipped where the recomputed forward stage stored it);
+//     adj_kept_kernel  : one thread per interface: where the test keeps every
+//                        stencil, the closed-form interface VJP (teno_adjoint_core.cuh)
 //                        with Fbar from Rbar (eq. 2.2): U~bar and the adjoints
 //                        of the two Roe cells' parameters go to kb_d; the
 //                        rest is marked pending;
 //     list passes      : the pending interfaces in one list, index order;
 //     adj_select_kernel: the listed interfaces' selections by the forward
-//                        pass's binary64 decisions;
+//                        pass's decisions;
 //     partition passes : the list reordered stably, the interfaces that keep
 //                        every stencil after all first;
 //     adj_general_kernel: the listed interfaces' VJP with those selections
@@ -47,6 +48,7 @@
 #include "teno_adjoint_core.cuh"
 #include "teno_closed.cuh"
 #include "teno_device.cuh"
+#include "teno_faces.cuh"
 #include "teno_flux.cuh"
 #include "teno_launch.h"
 
@@ -144,74 +146,88 @@ __device__ __forceinline__ void add_alpha(const double (&ab)[NVAR], double (&asu
   asum[2] += ab[NVAR - 1];
 }
 
-// The forward's certificate at one interface (interface_flux_closed's open
-// mask): on the Roe state in two binary32 values, or on the binary64 one
-// outside their range.  Out of line: its registers are its own.  pf: the cell
-// pass's binary32 planes of U where it wrote them (else the same values are
-// converted here).
+// The forward's certificate at one interface outside the range of its
+// two-binary32 Roe state (interface_flux_closed_wide's mask).  Out of line: rare.
 template <int NDIM, int DIR>
-__device__ __noinline__ unsigned forward_open(const double* __restrict__ U, const double* __restrict__ aux,
-                                              const float4* __restrict__ pf,
-                                              int64_t ncell, int64_t line, int64_t id, int64_t nd, int64_t stride, int bc,
-                                              double am, double a0, double ap, const Scheme& S, int* status) {
+__device__ __noinline__ unsigned open_wide(const double* __restrict__ U, const double* __restrict__ aux, int64_t ncell,
+                                           const uint32_t (&cells)[6], const double (&a3)[3], const Scheme& S,
+                                           int* status) {
   constexpr int NVAR = NDIM + 2;
-  if (S.keep_idx < 0) return teno::kRough | teno::kAllOpen<NDIM>;
-  int64_t cells[6];
-#pragma unroll
-  for (int j = 0; j < 6; ++j) cells[j] = line + teno::ghost(id - 3 + j, nd, bc) * stride;
-  const double a3[3] = {am, a0, ap};
-  const teno::FaceSpeeds F = teno::face_speeds(a3);
-  const teno_df::df gm1 = teno::gm1_df(S);
-  double su2[NDIM], su3[NDIM];
+  double alpha[NVAR], nal[NVAR], su2[NDIM], su3[NDIM];
+  teno::spread_speeds<NDIM>(a3, alpha, nal);
 #pragma unroll
   for (int k = 0; k < NDIM; ++k) {
     su2[k] = aux[(NDIM + 3 + k) * ncell + cells[2]];
     su3[k] = aux[(NDIM + 3 + k) * ncell + cells[3]];
   }
-  const double sr2 = aux[(NDIM + 1) * ncell + cells[2]], sr3 = aux[(NDIM + 1) * ncell + cells[3]];
-  const double sh2 = aux[(NDIM + 2) * ncell + cells[2]], sh3 = aux[(NDIM + 2) * ncell + cells[3]];
-  teno::RoeDf<NDIM> Rd;
-  if (pf)
-    teno::roe_df<NDIM>(teno::load_roe_cell<NDIM, false>(pf, nullptr, ncell, cells[2]),
-                       teno::load_roe_cell<NDIM, false>(pf, nullptr, ncell, cells[3]), gm1, Rd);
-  else
-    teno::roe_df<NDIM>(teno::roe_cell<NDIM>(sr2, sh2, su2), teno::roe_cell<NDIM>(sr3, sh3, su3), gm1, Rd);
+  teno::RoeIfc<NDIM> R;
+  teno::roe_interface<NDIM, DIR>(aux[(NDIM + 1) * ncell + cells[2]], aux[(NDIM + 1) * ncell + cells[3]],
+                                 aux[(NDIM + 2) * ncell + cells[2]], aux[(NDIM + 2) * ncell + cells[3]], su2, su3, S, R,
+                                 status);
   teno::CertIfc<NDIM> C;
-  for (bool df = F.in_range && teno::roe_df_ok<NDIM>(Rd, gm1);; df = false) {
-    if (df) {
-      teno::cert_begin_df<NDIM, DIR>(Rd, F.ha, gm1, C);
-    } else {
-      double alpha[NVAR], nal[NVAR];
-      teno::spread_speeds<NDIM>(a3, alpha, nal);
-      teno::RoeIfc<NDIM> R;
-      teno::roe_interface<NDIM, DIR>(sr2, sr3, sh2, sh3, su2, su3, S, R, status);
-      teno::cert_begin<NDIM, DIR>(R, alpha, C);
-    }
+  teno::cert_begin<NDIM, DIR>(R, alpha, C);
 #pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      float X[NVAR];
-      if (pf && df) {
-        float u, p;
-        teno::load_point_f<NDIM, DIR, false>(pf, nullptr, ncell, cells[j], X, u, p);
-        teno_cert::cert_point_f<NDIM, DIR>(j, X, u, p, C);
-        continue;
-      }
-      const double un = aux[DIR * ncell + cells[j]], pn = aux[NDIM * ncell + cells[j]];
+  for (int j = 0; j < 6; ++j) {
+    double Uj[NVAR];
 #pragma unroll
-      for (int v = 0; v < NVAR; ++v) {
-        const double x = U[v * ncell + cells[j]];
-        X[v] = df ? teno::near_float(x) : teno::hi_float(x);
-      }
-      teno_cert::cert_point_f<NDIM, DIR>(j, X, df ? teno::near_float(un) : teno::hi_float(un),
-                                         df ? teno::near_float(pn) : teno::hi_float(pn), C);
-    }
-    if (!df || teno::df_range(C.xm[0], C.xm[NVAR - 1])) break;
+    for (int v = 0; v < NVAR; ++v) Uj[v] = U[v * ncell + cells[j]];
+    teno::cert_point<NDIM, DIR>(j, Uj, aux[DIR * ncell + cells[j]], aux[NDIM * ncell + cells[j]], C);
   }
   return teno::cert_open<NDIM>(C, S);
 }
 
-// One thread per interface: the forward pass's certified FP32 test (the
-// same device code teno_rhs / teno_rk3_step run).  Where it keeps every
+// The forward's certificate at every interface of a stage whose forward pass has
+// not stored it: the masks of open reconstructions (interface_flux_closed's), for
+// the kept and the selecting pass.  A pass of its own: it issues FP32 and integer
+// instructions only, and inside the kept pass it was an out of line call per
+// interface (and again per listed one): a staged reverse step at 192^3 40.5 against
+// 34.8 ms, a right-hand-side adjoint there 16.0 against 11.6, at 512^2 742 against
+// 624 us.
+template <int NDIM, int DIR>
+__global__ void __launch_bounds__(kAdjThreads, 5) adj_open_kernel(
+    const double* __restrict__ U, const double* __restrict__ aux, const float4* __restrict__ pf,
+    const unsigned long long* __restrict__ alpha_bits, uint32_t* __restrict__ mask, int* __restrict__ status, Grid G,
+    Scheme S) {
+  constexpr int NVAR = NDIM + 2;
+  const int64_t nifc = (G.n[0] + (DIR == 0)) * (G.n[1] + (DIR == 1)) * (G.n[2] + (DIR == 2));
+  double a3[3];
+#pragma unroll
+  for (int s = 0; s < 3; ++s) a3[s] = 0.5 * __longlong_as_double((long long)alpha_bits[DIR * 3 + s]);
+  const teno::FaceSpeeds F = teno::face_speeds(a3);
+  const teno_df::df gm1 = teno::gm1_df(S);
+  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nifc; q += (int64_t)gridDim.x * blockDim.x) {
+    if (S.keep_idx < 0) {
+      mask[q] = teno::kRough | teno::kAllOpen<NDIM>;
+      continue;
+    }
+    uint32_t cells[6];
+    unsigned flips;
+    teno::interface_cells<NDIM, DIR, false>(static_cast<uint32_t>(q), G, cells, flips);
+    teno::RoeDf<NDIM> R;
+    teno::roe_df<NDIM>(teno::load_roe_cell<NDIM, false>(pf, nullptr, G.ncell, cells[2]),
+                       teno::load_roe_cell<NDIM, false>(pf, nullptr, G.ncell, cells[3]), gm1, R);
+    teno::CertIfc<NDIM> C;
+    teno::cert_begin_df<NDIM, DIR>(R, F.ha, gm1, C);
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+      float X[NVAR], u, p;
+      teno::load_point_f<NDIM, DIR, false>(pf, nullptr, G.ncell, cells[j], X, u, p);
+      teno_cert::cert_point_f<NDIM, DIR>(j, X, u, p, C);
+    }
+    if (F.in_range && teno::roe_df_ok<NDIM>(R, gm1) && teno::df_range(C.xm[0], C.xm[NVAR - 1])) {
+      mask[q] = teno::cert_open<NDIM>(C, S);
+    } else {
+      uint32_t cc[6];
+      double aa[3] = {a3[0], a3[1], a3[2]};
+#pragma unroll
+      for (int j = 0; j < 6; ++j) cc[j] = cells[j];
+      mask[q] = open_wide<NDIM, DIR>(U, aux, G.ncell, cc, aa, S, status);
+    }
+  }
+}
+
+// One thread per interface.  Where the forward pass's certified FP32 test (its
+// mask from the forward stage, roe_in, or from adj_open_kernel) keeps every
 // stencil, the interface part of the closed-form VJP: U~bar and the
 // adjoints of the Roe parameters of cells i and i+1 go to kb[3 nvar][nifc]
 // (the flux Jacobians and the Roe-parameter maps are applied per cell by the
@@ -225,7 +241,7 @@ __global__ void __launch_bounds__(kAdjThreads, TENO_ADJ_KEPT_MINBLOCKS) adj_kept
     const unsigned long long* __restrict__ alpha_bits, const double* __restrict__ Rbar, double scale,
     double* __restrict__ kb, unsigned char* __restrict__ pending, double* __restrict__ apart,
     int* __restrict__ status, Grid G, Scheme S, const double* __restrict__ roe_in,
-    const float4* __restrict__ pf) {
+    const uint32_t* __restrict__ mask) {
   constexpr int NVAR = NDIM + 2;
   const IfcGeom<NDIM, DIR> I(G);
   double fa[NVAR], ha[NVAR], nfa[NVAR];
@@ -241,30 +257,7 @@ __global__ void __launch_bounds__(kAdjThreads, TENO_ADJ_KEPT_MINBLOCKS) adj_kept
        q += (int64_t)gridDim.x * blockDim.x) {
     int64_t id, base, cells[6];
     I.locate(q, G, id, base, cells);
-    // The forward pass's Roe state (roe_interface on the cell pass's
-    // primitives) and its certified FP32 test: a pass keeps every stencil
-    // exactly where the forward's closed-form pass did.  U~ is accumulated
-    // over the same stencil loads.  With STORED the recomputed forward
-    // stage's closed-form pass has stored both (roe_in), so neither is
-    // evaluated again.
-    const double sr2 = aux[(NDIM + 1) * I.ncell + cells[2]], sr3 = aux[(NDIM + 1) * I.ncell + cells[3]];
-    const double sh2 = aux[(NDIM + 2) * I.ncell + cells[2]], sh3 = aux[(NDIM + 2) * I.ncell + cells[3]];
-    teno::RoeIfc<NDIM> Rf;
-    double Ut[NVAR];
-    bool kept;
-    if constexpr (STORED) {
-      kept = roe_in[(int64_t)(NDIM + 7) * I.nifc + q] != 0.0;
-    } else {
-      double su2[NDIM], su3[NDIM];
-#pragma unroll
-      for (int k = 0; k < NDIM; ++k) {
-        su2[k] = aux[(NDIM + 3 + k) * I.ncell + cells[2]];
-        su3[k] = aux[(NDIM + 3 + k) * I.ncell + cells[3]];
-      }
-      teno::roe_interface<NDIM, DIR>(sr2, sr3, sh2, sh3, su2, su3, S, Rf, status);
-      kept = forward_open<NDIM, DIR>(U, aux, pf, I.ncell, base, id, I.nd, I.stride_d, I.bcd, ha[0], ha[1], ha[NVAR - 1], S,
-                                     status) == 0u;
-    }
+    const bool kept = STORED ? roe_in[(int64_t)(NDIM + 7) * I.nifc + q] == 0.0 : mask[q] == 0u;
     pending[q] = kept ? 0 : 1;
     if (!kept) {
       // a pending interface's terms come from adj_general_kernel; zeros
@@ -273,6 +266,11 @@ __global__ void __launch_bounds__(kAdjThreads, TENO_ADJ_KEPT_MINBLOCKS) adj_kept
       for (int v = 0; v < 3 * NVAR; ++v) kb[(int64_t)v * I.nifc + q] = 0.0;
       continue;
     }
+    // the forward pass's Roe state (roe_interface on the cell pass's primitives)
+    const double sr2 = aux[(NDIM + 1) * I.ncell + cells[2]], sr3 = aux[(NDIM + 1) * I.ncell + cells[3]];
+    const double sh2 = aux[(NDIM + 2) * I.ncell + cells[2]], sh3 = aux[(NDIM + 2) * I.ncell + cells[3]];
+    teno::RoeIfc<NDIM> Rf;
+    double Ut[NVAR];
     if constexpr (STORED) {
 #pragma unroll
       for (int k = 0; k < NDIM; ++k) Rf.u[k] = roe_in[(int64_t)k * I.nifc + q];
@@ -283,6 +281,14 @@ __global__ void __launch_bounds__(kAdjThreads, TENO_ADJ_KEPT_MINBLOCKS) adj_kept
       Rf.hb1 = roe_in[(int64_t)(NDIM + 4) * I.nifc + q];
       Rf.hb2 = roe_in[(int64_t)(NDIM + 5) * I.nifc + q];
       Rf.hic = roe_in[(int64_t)(NDIM + 6) * I.nifc + q];
+    } else {
+      double su2[NDIM], su3[NDIM];
+#pragma unroll
+      for (int k = 0; k < NDIM; ++k) {
+        su2[k] = aux[(NDIM + 3 + k) * I.ncell + cells[2]];
+        su3[k] = aux[(NDIM + 3 + k) * I.ncell + cells[3]];
+      }
+      teno::roe_interface<NDIM, DIR>(sr2, sr3, sh2, sh3, su2, su3, S, Rf, status);
     }
     // 60 U~ in 64-bit fixed point (teno_fixsum.cuh, as in the forward's closed
     // form; a component it does not cover as a binary64 chain): 14.32 ms per
@@ -523,10 +529,9 @@ __global__ void __launch_bounds__(kListThreads) adj_part_scatter_kernel(
 // The listed interfaces in two passes, so that the VJP runs on full warps
 // (the forward's cutoff decisions branch per field and lane; the VJP with
 // the selections fixed does not branch):
-//   adj_select_kernel: the forward's certificate again for the mask of open
-//                      reconstructions, and the decisions its correction pass
-//                      takes on those (warp_correct) -> the ten 3-bit
-//                      selections packed into sel[i];
+//   adj_select_kernel: the decisions that the forward's correction pass takes
+//                      on the open reconstructions of the mask (warp_correct)
+//                      -> the ten 3-bit selections packed into sel[i];
 //   partition passes  : the list reordered, those that keep every stencil
 //                      after all first (below);
 //   adj_general_kernel: one thread per listed interface: the closed-form VJP
@@ -540,7 +545,7 @@ __global__ void __launch_bounds__(kAdjThreads) adj_select_kernel(
     const double* __restrict__ U, const double* __restrict__ aux,
     const unsigned long long* __restrict__ alpha_bits, const uint32_t* __restrict__ list,
     const int* __restrict__ count, uint32_t* __restrict__ sel, int* __restrict__ status, Grid G, Scheme S,
-    const float4* __restrict__ pf) {
+    const double* __restrict__ roe_in, const uint32_t* __restrict__ mask) {
   constexpr int NVAR = NDIM + 2;
   __shared__ teno::CorrectScratch<NDIM> scratch[kAdjThreads / 32];
   const IfcGeom<NDIM, DIR> I(G);
@@ -560,10 +565,7 @@ __global__ void __launch_bounds__(kAdjThreads) adj_select_kernel(
     uint32_t q = 0u;
     if (i < n) {
       q = list[i];
-      int64_t id, base, cells[6];
-      I.locate(q, G, id, base, cells);
-      open = forward_open<NDIM, DIR>(U, aux, pf, I.ncell, base, id, I.nd, I.stride_d, I.bcd, ha[0], ha[1], ha[NVAR - 1], S,
-                                     status);
+      open = roe_in ? static_cast<unsigned>(roe_in[(int64_t)(NDIM + 7) * I.nifc + q]) : mask[q];
     }
     double out[NVAR];
     const uint32_t w = teno::warp_correct<NDIM, DIR, false, int64_t, true>(U, aux, I.ncell, cells_of, q, ha, S, open,
@@ -1070,14 +1072,21 @@ void launch_adj_dir(int nblk, int nsm, cudaStream_t st, const double* U, const d
                     double* contrib, unsigned char* pending, uint32_t* list, int* lcount, uint32_t* sel,
                     double* apart, int* status, const Grid& G, const Scheme& S, const double* roe_in,
                     const float4* pf) {
-  if (roe_in)
-    adj_kept_kernel<NDIM, DIR, true><<<nblk, kAdjThreads, 0, st>>>(U, aux, alpha, Rbar, scale, kb, pending, apart,
-                                                                  status, G, S, roe_in, nullptr);
-  else
-    adj_kept_kernel<NDIM, DIR, false><<<nblk, kAdjThreads, 0, st>>>(U, aux, alpha, Rbar, scale, kb, pending, apart,
-                                                                   status, G, S, nullptr, pf);
   int64_t nifc = 1;
   for (int k = 0; k < 3; ++k) nifc *= G.n[k] + (k == DIR ? 1 : 0);
+  // the masks of open reconstructions lie in the first plane of contrib, which
+  // the general pass writes after their last use
+  auto* mask = reinterpret_cast<uint32_t*>(contrib);
+  if (roe_in) {
+    adj_kept_kernel<NDIM, DIR, true><<<nblk, kAdjThreads, 0, st>>>(U, aux, alpha, Rbar, scale, kb, pending, apart,
+                                                                  status, G, S, roe_in, nullptr);
+  } else {
+    int64_t ob = (nifc + kAdjThreads - 1) / kAdjThreads;
+    if (ob > int64_t(nsm) * 64) ob = int64_t(nsm) * 64;
+    adj_open_kernel<NDIM, DIR><<<unsigned(ob), kAdjThreads, 0, st>>>(U, aux, pf, alpha, mask, status, G, S);
+    adj_kept_kernel<NDIM, DIR, false><<<nblk, kAdjThreads, 0, st>>>(U, aux, alpha, Rbar, scale, kb, pending, apart,
+                                                                   status, G, S, nullptr, mask);
+  }
   const int lblk = adj_list_blocks(nsm);
   int* bcount = lcount;
   int* boff = lcount + lblk;
@@ -1085,7 +1094,8 @@ void launch_adj_dir(int nblk, int nsm, cudaStream_t st, const double* U, const d
   adj_count_kernel<<<lblk, kListThreads, 0, st>>>(pending, nifc, bcount);
   adj_scan_kernel<<<1, kListThreads, 0, st>>>(bcount, lblk, boff, total);
   adj_scatter_kernel<<<lblk, kListThreads, 0, st>>>(pending, nifc, boff, list);
-  adj_select_kernel<NDIM, DIR><<<nblk, kAdjThreads, 0, st>>>(U, aux, alpha, list, total, sel, status, G, S, pf);
+  adj_select_kernel<NDIM, DIR><<<nblk, kAdjThreads, 0, st>>>(U, aux, alpha, list, total, sel, status, G, S, roe_in,
+                                                            mask);
   // the partition reuses the counts and offsets; its own total (the number
   // of all-kept entries) goes to the slot after the list's
   int* nkept = total + 1;
@@ -1146,10 +1156,14 @@ teno_status adjoint_sequence(const teno_grid* g, const AdjLayout& L, char* ws, i
   auto* alpha = reinterpret_cast<unsigned long long*>(ws + L.alpha + stage * AdjLayout::kStage);
   auto* argidx = reinterpret_cast<unsigned long long*>(ws + L.argidx + stage * AdjLayout::kStage);
   double* aux = reinterpret_cast<double*>(ws + L.aux + stage * L.aux_bytes);
-  // this stage input's binary32 planes, where its cell pass runs here and there is
-  // room for them: in fh and R, which the forward stages have left by then (6 + 4
-  // and 12 + 5 doubles a cell in 2D and 3D, for planes of 8 and 10)
-  float4* pf = cell && L.fh && g->ndim > 1 ? reinterpret_cast<float4*>(ws + L.fh) : nullptr;
+  // this stage input's binary32 planes, where its cell pass runs here: behind the
+  // masks in the last direction's contrib, which its general pass writes after
+  // their last use (16 nvar bytes a cell of 48 nvar an interface, 8 for the masks)
+  int64_t maxifc = 0;
+  for (int d = 0; d < g->ndim; ++d) maxifc = nifc_of(g, d) > maxifc ? nifc_of(g, d) : maxifc;
+  float4* pf = cell ? reinterpret_cast<float4*>(ws + L.contrib + (g->ndim - 1) * L.contrib_bytes +
+                                                round_up(sizeof(double) * size_t(maxifc)))
+                    : nullptr;
   if (cell) {
     auto* cand = reinterpret_cast<unsigned long long*>(ws + L.cand);
     if (cudaMemsetAsync(alpha, 0, sizeof(unsigned long long) * 9, st) != cudaSuccess) return TENO_ERR_CUDA;

@@ -105,11 +105,11 @@ __device__ __forceinline__ void half_speeds(const unsigned long long* __restrict
 // WALL: 1 -- the sweep direction has a reflecting wall, so stencil points may
 // be mirrored; 2 -- fixed-state faces (ghost points read from the ghost
 // block); 0 -- neither: the mirror flags are the constant 0 and their sign
-// flips fold away; 3 -- whichever the grid has (the launch over all directions).  With ROE every interface's Roe state (the fields the
-// certificate and the adjoint's closed-form VJP read: u~, |u~|^2, H~, c~,
-// b1, b1/2, b2/2, 1/(2c~)) and the certificate's decision (1 kept, 0
-// pending) also go to roe_out[ndim + 8][nifc], for the adjoint of this
-// stage.  PF: with the cells' binary32 planes; without them (the largest grids)
+// flips fold away; 3 -- whichever the grid has (the launch over all directions).
+// With ROE every interface's Roe state (the fields that the adjoint's closed-form
+// VJP reads: u~, |u~|^2, H~, c~, b1, b1/2, b2/2, 1/(2c~)) and the certificate's
+// mask (0: every stencil kept) also go to roe_out[ndim + 8][nifc], for the
+// adjoint of this stage.  PF: with the cells' binary32 planes; without them (the largest grids)
 // the list holds indices alone, its reconstructions all count as open, and a
 // face whose flux stays unwritten (kRough) is marked by a NaN.
 template <int NDIM, int DIR, int WALL, bool ROE, bool PF = true, class Entry = uint2>
@@ -179,7 +179,7 @@ __device__ __forceinline__ void closed_faces(
         roe_out[(int64_t)(NDIM + 4) * nifc + q] = R.hb1;
         roe_out[(int64_t)(NDIM + 5) * nifc + q] = R.hb2;
         roe_out[(int64_t)(NDIM + 6) * nifc + q] = R.hic;
-        roe_out[(int64_t)(NDIM + 7) * nifc + q] = open ? 0.0 : 1.0;
+        roe_out[(int64_t)(NDIM + 7) * nifc + q] = double(open);
       }
     }
     if constexpr (!PF) {

@@ -47,7 +47,7 @@ cudaError_t launch_argmax_finish(int ndim, const unsigned long long* cand, int64
 // `count` (zero on entry) and `fh`, the closed-form pass and the pass that corrects the listed interfaces.  `launches` (optional) receives the number
 // of kernels launched.  With `roe_out` (two-pass fluxes without reflecting or
 // fixed-state faces only) the closed-form pass also writes every
-// interface's Roe state and its certificate's decision, [ndim + 8][#interfaces]
+// interface's Roe state and its certificate's mask, [ndim + 8][#interfaces]
 // (flux_closed_kernel).  Without `correct` the listed interfaces are left to
 // launch_correct_all.
 cudaError_t launch_flux(int ndim, int dir, const double* U, const double* aux, const double* fh, const float4* pf,
