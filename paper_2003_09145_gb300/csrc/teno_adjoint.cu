@@ -292,8 +292,7 @@ __global__ void __launch_bounds__(kAdjThreads, TENO_ADJ_KEPT_MINBLOCKS) adj_kept
     }
     // 60 U~ in 64-bit fixed point (teno_fixsum.cuh, as in the forward's closed
     // form; a component it does not cover as a binary64 chain): 14.32 ms per
-    // 128^3 reverse step against 14.74 with the chain.  (The gather's stencil
-    // on Rbar in fixed point measured 14.91 against 14.74 without.)
+    // 128^3 reverse step against 14.74 with the chain.
 #pragma unroll
     for (int v = 0; v < NVAR; ++v) {
       double us[6];
@@ -768,7 +767,13 @@ __device__ __forceinline__ void gather_dir(const Grid& G, int64_t c, int64_t i0,
     for (int v = 0; v < NVAR; ++v) {
       const double* r = Rbar + v * ncell + line;
       const double r1p = r[o1p], r1m = r[o1m], r2p = r[o2p], r2m = r[o2m], r3p = r[o3p], r3m = r[o3m];
-      Fsum[v] = fma(w45, r1p - r1m, fma(w9, r2p - r2m, w1 * (r3p - r3m)));
+      // (in fixed point: exact sum, one rounding; a reverse step at 192^3 37.4
+      // against 38.2 ms with a chain, at 128^3 13.56 against 13.45)
+      const double rs[6] = {r3p, r3m, r2p, r2m, r1p, r1m};
+      constexpr int rw[6] = {1, -1, -9, 9, 45, -45};
+      double S;
+      if (teno_fix::sum<6>(rs, rw, S)) Fsum[v] = w1 * S;
+      else Fsum[v] = fma(w45, r1p - r1m, fma(w9, r2p - r2m, w1 * (r3p - r3m)));
     }
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
