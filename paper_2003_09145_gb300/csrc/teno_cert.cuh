@@ -147,8 +147,14 @@ TENO_CERT_HD bool certify_keep(float v0, float v1, float v2, float v3, float v4,
 // in the same order, so the same outcomes), with two operations per
 // instruction where the hardware pairs them: bit 0 set where x is not proven
 // kept, bit 1 where y is not.
+// (On the host a test supplies float2 and the paired operations.)
+#if defined(__CUDACC__) || defined(TENO_CERT_PAIRS)
 #ifdef __CUDACC__
-__device__ __forceinline__ unsigned certify_open2(float2 v0, float2 v1, float2 v2, float2 v3, float2 v4, float2 d,
+__device__ __forceinline__
+#else
+inline
+#endif
+unsigned certify_open2(float2 v0, float2 v1, float2 v2, float2 v3, float2 v4, float2 d,
                                                   float thr_f, float eps4_f) {
   const float u = 0x1p-24f, k = 13.0f / 3.0f;
   const float2 m1 = make_float2(-1.0f, -1.0f), two = make_float2(2.0f, 2.0f), kk = make_float2(k, k);
@@ -328,7 +334,7 @@ TENO_CERT_HD bool select_diffs(double f0, double f1, double f2, double f3, float
 // The grid path's inputs are not truncated but rounded (cert_begin_f): U, u_d/2,
 // p/2, u~, alpha and 1/c~ within 1 u, b1/2 within 5 u and b2/2 within 7 u.  The
 // longest chain ((u_d/2 + alpha) b1/2 (u~.m - E)) then stays within 20 u, and
-// d = 32 u |.|_abs + 2^-90 leaves the same slack.  The bound matters where the
+// d = 32 u |.|_abs + 2^-90 is 1.45 times the r + 2 u W of 22 u.  The bound matters where the
 // variation is small against the values (large pressures): with 8 2^-20 the
 // test proved nothing for |.|_abs above about 50, with 32 u about 190.
 // ---------------------------------------------------------------------------
