@@ -701,19 +701,11 @@ __device__ __forceinline__ uint32_t warp_correct(const double* __restrict__ U, c
 // mirrored wall point (reflecting boundary: normal velocity reversed).
 // `fl` receives the flag bytes when WITH_FLAGS
 // (without flags, bits 0..2 still hold the selections used).
-// MODE kFluxFull computes the flux.  kFluxSelect only wants the selections:
-// it returns without the flux when the certified test keeps every stencil.
-// kFluxCertify stops after the certified test: fl = 7 everywhere if it keeps
-// every stencil, else fl[0][0] = kUndecided and nothing else is written.
-// kFluxChar skips the certified test and takes the characteristic path (for
-// interfaces the test has already left undecided: the flux equals
-// kFluxFull's).
+// MODE kFluxFull computes the flux; kFluxChar skips the certified test and takes
+// the characteristic path (WENO-Z, which has no such test).
 // ---------------------------------------------------------------------------
-constexpr int kFluxFull = 0, kFluxSelect = 1, kFluxCertify = 2, kFluxChar = 4;
-constexpr unsigned kUndecided = 0xffu;
+constexpr int kFluxFull = 0, kFluxChar = 1;
 
-// the certify-only instantiation ends early: its remaining code is unreachable
-#pragma nv_diag_suppress 128
 template <int NDIM, int DIR, bool WITH_FLAGS, int MODE = kFluxFull, bool GH = false, class I = int64_t>
 __device__ __forceinline__ void interface_flux(const double* __restrict__ U,
                                                const double* __restrict__ aux,
@@ -776,22 +768,12 @@ __device__ __forceinline__ void interface_flux(const double* __restrict__ U,
 #pragma unroll
       for (int j = 0; j < 6; ++j) cert_point<NDIM, DIR>(j, Ux[j], un[j], pn[j], C);
       const bool keep = cert_keep<NDIM>(C, S);
-      if ((MODE == kFluxSelect || MODE == kFluxCertify) && keep) {
-        // only the selections are wanted: every stencil kept
-#pragma unroll
-        for (int f = 0; f < NVAR; ++f) fl[f][0] = fl[f][1] = 7u;
-        return;
-      }
       if (keep) {
         closed_in_registers<NDIM, DIR>(Ux, half, R, nal, out);
 #pragma unroll
         for (int f = 0; f < NVAR; ++f) fl[f][0] = fl[f][1] = 7u;
         return;
       }
-    }
-    if (MODE == kFluxCertify) {
-      fl[0][0] = kUndecided;
-      return;
     }
 
     // As in warp_correct: the flux with every stencil kept plus the fields'
@@ -880,7 +862,6 @@ __device__ __forceinline__ void interface_flux(const double* __restrict__ U,
     out[NVAR - 1] += eng;
   }
 }
-#pragma nv_diag_default 128
 
 // ---------------------------------------------------------------------------
 // Primitive variables of cell c from one reciprocal square root:

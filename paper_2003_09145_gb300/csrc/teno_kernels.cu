@@ -824,10 +824,7 @@ cudaError_t launch_correct_all(int ndim, const double* U, const double* aux, con
     gh = gh || G.bc[d] == TENO_BC_DIRICHLET;
   }
   const dim3 grid(unsigned(blocks_for(nifc, 128, nsm * 16)), unsigned(ndim));
-  if (ndim == 1) {
-    if (gh) flux_correct_all_kernel<1, true><<<grid, 128, 0, st>>>(U, aux, alpha, Fhat, fstride, list, lstride, count, status, G, S, nsm);
-    else flux_correct_all_kernel<1, false><<<grid, 128, 0, st>>>(U, aux, alpha, Fhat, fstride, list, lstride, count, status, G, S, nsm);
-  } else if (ndim == 2) {
+  if (ndim == 2) {
     if (gh) flux_correct_all_kernel<2, true><<<grid, 128, 0, st>>>(U, aux, alpha, Fhat, fstride, list, lstride, count, status, G, S, nsm);
     else flux_correct_all_kernel<2, false><<<grid, 128, 0, st>>>(U, aux, alpha, Fhat, fstride, list, lstride, count, status, G, S, nsm);
   } else {
@@ -855,8 +852,7 @@ cudaError_t launch_diff_all(int ndim, const double* Fhat, int64_t fstride, doubl
   if (mode != 0 && (mode < 2 || mode > 4)) return cudaErrorInvalidValue;
   const int blocks = blocks_for(G.ncell, 256, nsm * 16);
   const bool g = G.has_grav;
-  if (ndim == 1) (g ? diff_all_launch<1, true> : diff_all_launch<1, false>)(blocks, st, Fhat, fstride, R, Un, Uk, Uout, dt, G, mode, Usrc);
-  else if (ndim == 2) (g ? diff_all_launch<2, true> : diff_all_launch<2, false>)(blocks, st, Fhat, fstride, R, Un, Uk, Uout, dt, G, mode, Usrc);
+  if (ndim == 2) (g ? diff_all_launch<2, true> : diff_all_launch<2, false>)(blocks, st, Fhat, fstride, R, Un, Uk, Uout, dt, G, mode, Usrc);
   else (g ? diff_all_launch<3, true> : diff_all_launch<3, false>)(blocks, st, Fhat, fstride, R, Un, Uk, Uout, dt, G, mode, Usrc);
   return cudaGetLastError();
 }
