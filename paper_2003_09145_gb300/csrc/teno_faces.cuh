@@ -243,6 +243,8 @@ __device__ __forceinline__ void correct_list(const double* __restrict__ U, const
     double out[NVAR];
 #pragma unroll
     for (int v = 0; v < NVAR; ++v) out[v] = e.y && !(e.y & kRough) ? Fhat[(int64_t)v * nifc + e.x] : 0.0;
+    if constexpr (sizeof(Entry) != sizeof(uint2))
+      if (e.y && out[0] != out[0]) e.y |= kRough;   // the mark of an unwritten flux
     warp_correct<NDIM, DIR, GH, uint32_t>(U, aux, G.ncell, cells_of, e.x, alpha, S, e.y, out, status, W,
                                           GhostCells{G.gU, G.gaux, G.gfh, G.gpf});
     if (e.y)

@@ -112,3 +112,15 @@ def test_tiles_equal_the_small_grid(api, case, k):
     assert _same_in_every_tile(B, V, n, reps)
     del B, S
     torch.cuda.empty_cache()
+
+
+def test_tiles_beyond_the_fixed_points_range(api):
+    """Fluxes that the closed form leaves unwritten (values above 2^1007), on a list of indices."""
+    n, reps = (96,), (4194400,)
+    U0 = torch.from_numpy(_tile_state(n, (PERIODIC,), seed=1) * 2.0**1012).cuda()
+    small = api.EulerGrid(n, (1.0,), (PERIODIC,))
+    big = api.EulerGrid((n[0] * reps[0],), (1.0,), (PERIODIC,))
+    _need(int(1.05 * (2 * 24 * big.ncell + big.workspace_bytes(0))))
+    R0 = api.rhs(small, U0)
+    assert torch.isfinite(R0).all() and R0.abs().max() > 2.0**1000
+    assert _same_in_every_tile(api.rhs(big, U0.repeat((1, reps[0]))), R0, n, reps)
