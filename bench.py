@@ -52,10 +52,11 @@ FP64_FLOP_PER_CLK_PER_SM = 4          # 2 FP64 FMA lanes per SM per clock
 #   +-1 (9 of their 12 flops), so 187 - 6 x 12 - 4 x 3 = 103 flops per
 #   interface are left to the FP64 pipe where the Roe state and the
 #   corrections run in binary64 too (FP64_CLOSED_3D: near shocks).  Elsewhere
-#   those run as two binary32 values (teno_df.cuh) and 4 x (9 + 1) + 1 = 41
-#   remain: FP64_PIPE_3D, fp64_flops_per_interface.  The roofline keeps the
-#   algorithmic count against the FP64 peak, the rate at which binary64
-#   could evaluate the same arithmetic.
+#   those run as two binary32 values (teno_closed_core.cuh) and 4 x (9 + 1) + 1
+#   = 41 remain (pipe_flops; fp64_flops_per_interface).  The roofline holds
+#   these against the FP64 peak; the algorithmic count's rate, which exceeds
+#   that peak, is reported beside it, and so is the share of issue slots, which
+#   is what bounds the pass.
 # * Otherwise the characteristic path: Roe 27, projection 6 x 20, split 6 x 28,
 #   sum 5, back-projection 21 (= 341), plus per scalar reconstruction 9 when
 #   its own FP32 pre-test keeps every stencil, else 38 for the binary64
@@ -77,7 +78,14 @@ def alg_counts(ndim: int):
 
 ALG_CLOSED_3D, ALG_FIXED_3D = alg_counts(3)
 FP64_CLOSED_3D = ALG_CLOSED_3D - 6 * 12 - 4 * 3   # the closed form's flops on the FP64 pipe
-FP64_PIPE_3D = 41
+
+
+def pipe_flops(ndim: int) -> int:
+    """FP64-pipe flops of a closed-form interface: ndim + 1 chains of nine and an
+    addition each, and the mass flux's addition."""
+    return 10 * (ndim + 1) + 1
+
+
 ALG_PER_RECON_KEEP = 9
 ALG_PER_RECON = 38
 ALG_CUTOFF = 21
@@ -173,7 +181,8 @@ class ClockSampler:
                 "reasons": reasons, "samples": len(rows)}
 
 
-FLUX_KERNEL_SOURCES = ("teno_cert.cuh", "teno_device.cuh", "teno_fixsum.cuh", "teno_flux.cuh", "teno_kernels.cu")
+FLUX_KERNEL_SOURCES = ("teno_cert.cuh", "teno_closed.cuh", "teno_closed_all.cu", "teno_closed_core.cuh", "teno_device.cuh",
+                       "teno_df.cuh", "teno_faces.cuh", "teno_fixsum.cuh", "teno_flux.cuh", "teno_kernels.cu")
 
 
 def _source_hash() -> str:
@@ -186,9 +195,10 @@ def _source_hash() -> str:
     return h.hexdigest()[:16]
 
 
-def _traffic_per_launch():
-    """DRAM bytes per flux-kernel launch at the benchmark size, from the committed
-    ncu summary, if that was taken on the current kernel sources; else None."""
+def _captured():
+    """(DRAM bytes per flux-kernel launch at the benchmark size, warp instructions
+    per interface) from the committed ncu summary, if that was taken on the
+    current kernel sources; else (None, None)."""
     path = os.path.join(ROOT, "profiles", "flux_kernel_traffic.txt")
     rec = {}
     try:
@@ -198,13 +208,13 @@ def _traffic_per_launch():
                     k, v = line.split(":", 1)
                     rec[k.strip()] = v.strip()
     except OSError:
-        return None
+        return None, None
     if rec.get("source_hash") != _source_hash():
-        return None
+        return None, None
     try:
-        return float(rec["bytes_per_launch_256"])
+        return float(rec["bytes_per_launch_256"]), float(rec["warp_inst_per_launch_160"]) / float(rec["interfaces_160"])
     except (KeyError, ValueError):
-        return None
+        return None, None
 
 
 def cpu_baseline(sample_n: int = 96, steps: int = 2) -> dict:
@@ -337,7 +347,8 @@ def bench_riemann2d(api, lib, device, steps: int, warm_steps: int, peak: float) 
     nifc = (P.n[0] + 1) * P.n[1] + P.n[0] * (P.n[1] + 1)
     # one flux evaluation = both passes of one direction in one RK stage
     flux_s_per_step = flux_ms / steps * 1e-3
-    achieved = alg * nifc * 3 / flux_s_per_step / 1e12
+    rate = nifc * 3 / flux_s_per_step / 1e12
+    achieved = (alg - (alg_counts(2)[0] - pipe_flops(2)) * (1.0 - off)) * rate
     return {"value": grid.ncell / (ms * 1e-3) / 1e9, "unit": UNIT, "ms_per_step": ms,
             "workload": "2D four-quadrant Riemann problem (split (0.8, 0.8)), 2048^2, TENO5-LAD, SSP-RK3 "
                         f"CFL 0.5, timed from t = {t_start:.4f} (after {warm_steps} steps)",
@@ -345,7 +356,7 @@ def bench_riemann2d(api, lib, device, steps: int, warm_steps: int, peak: float) 
             "alg_flops_per_interface": alg,
             "kernel_ms_per_step": {k: v[0] / steps for k, v in kinds.items()},
             "flux_roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                              "frac": achieved / peak}}
+                              "frac": achieved / peak, "algorithmic_tflops": alg * rate}}
 
 
 def bench_schemes(api, lib, device, steps: int, workloads) -> dict:
@@ -637,9 +648,13 @@ def main() -> None:
     flux_evals = args.steps * 3 * 3
     nifc = (n + 1) * n * n
     flux_avg_s = flux_ms / flux_evals * 1e-3
-    achieved = alg_per_ifc * nifc / flux_avg_s / 1e12
+    fp64_per_ifc = alg_per_ifc - (ALG_CLOSED_3D - pipe_flops(3)) * closed_frac
+    achieved = fp64_per_ifc * nifc / flux_avg_s / 1e12
     probe = fp64_probe(api, device) / 1e12
-    traffic = _traffic_per_launch()
+    traffic, inst = _captured()
+    # one warp instruction per cycle on each of an SM's four partitions
+    issue_peak = SM_COUNT * 4 * (clk["sm_mhz"] or sm_max) * 1e6
+    issue_frac = inst * nifc / flux_avg_s / issue_peak if inst else None
     total_kernel_ms = sum(kms)
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": traffic,
@@ -650,12 +665,14 @@ def main() -> None:
                                f"{sm_max:.0f} MHz (max SM clock)",
                 "fp64_probe_tflops": probe,
                 "alg_flops_per_interface": alg_per_ifc,
-                "fp64_flops_per_interface": alg_per_ifc - (ALG_CLOSED_3D - FP64_PIPE_3D) * closed_frac,
-                "fixed_point_sums": "closed form: the five M-weighted sums (60 U~) and the mass flux's "
-                                    "P-weighted sum in 64-bit fixed point on the integer pipes (terms "
-                                    "truncated 3 bits below the largest value's ulp, summed exactly, "
-                                    "rounded once to binary64); the momentum and energy P-sums as "
-                                    "binary64 chains",
+                "fp64_flops_per_interface": fp64_per_ifc,
+                "algorithmic_tflops": alg_per_ifc * nifc / flux_avg_s / 1e12,
+                "issue_frac": issue_frac,
+                "fixed_point_sums": "closed form: the five M-weighted sums (60 U~, to 48 bits) and the mass "
+                                    "flux's P-weighted sum (rounded once to binary64) in 64-bit fixed point "
+                                    "on the integer pipes (terms truncated 3 bits below the largest value's "
+                                    "ulp, summed exactly); Roe state and corrections as sums of two binary32 "
+                                    "values; the momentum and energy P-sums as binary64 chains",
                 "cutoff_evaluated_fraction": cut_frac,
                 "straightforward_count_tflops": STRAIGHTFORWARD_FLOPS_PER_IFACE_3D * nifc / flux_avg_s / 1e12}
 

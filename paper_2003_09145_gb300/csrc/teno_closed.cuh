@@ -5,13 +5,14 @@
 // the other fluxes as binary64 chains.
 //
 // What bounds it: instruction issue (it was FP64 issue: 78 FP64 instructions
-// per interface, each holding an SM partition for 64 cycles; now 29, the FP64
-// pipe 40 % busy).  Measured at 256^3 (ms per RK3 step): Roe state and
-// corrections in binary64 37.0, in two binary32 values 28.1, with the cells'
-// binary32 copies from the cell pass (store_planes) 25.3, with the
-// certificate's reconstructions in pairs (certify_open2) 24.3.  Tried on top
-// and dropped: the mass flux as a binary64 chain too (slower), the corrections
-// widened and added in two FP64 additions instead of one (no gain).
+// per interface, each holding an SM partition for 64 cycles; now 26 of some
+// 2200, the FP64 pipe 45 to 48 % busy, issue 61 to 64 %).  Measured at 256^3 (ms
+// per RK3 step): Roe state and corrections in binary64 37.0, in two binary32
+// values 28.1, with the cells' binary32 copies from the cell pass (store_planes)
+// 25.3, with the certificate's reconstructions in pairs (certify_open2) 24.3,
+// with the other passes as they are now 21.3.  Tried on top and dropped: the mass
+// flux as a binary64 chain too (slower), the corrections widened and added in two
+// FP64 additions instead of one (no gain).
 #pragma once
 
 #include "teno_closed_core.cuh"
