@@ -488,20 +488,47 @@ __device__ __noinline__ unsigned interface_flux_closed_wide(const double* __rest
 // Where the all-kept flux is much larger than the flux scale (alpha rho,
 // alpha^2 rho, alpha E of the stencil -- a strong pressure jump seen from its
 // cold side), subtracting it back would cancel digits: such an interface,
-// and one with kRough, opens every reconstruction and sums the whole values.
+// and one with kRough, opens every reconstruction and sums the whole values; so,
+// in a second round, does one whose fields' differences are.
 // ---------------------------------------------------------------------------
-// Whether a flux (stored as 30 F^) exceeds the flux scale twice, in single
-// precision: the halved speeds, and the stencil's largest density and energy.
+// The flux scale twice, in single precision, as fluxes are stored (times 30): the
+// halved speeds, and the stencil's largest density and energy.
+struct FluxScale {
+  float am, s0, sE;
+};
 template <int NDIM>
-__device__ __forceinline__ bool beyond_flux_scale(const double (&out)[NDIM + 2], const double (&alpha)[NDIM + 2],
-                                                  float rho_max, float e_max) {
+__device__ __forceinline__ FluxScale flux_scale(const double (&alpha)[NDIM + 2], float rho_max, float e_max) {
+  const float am = 2.0f * fmaxf(hi_float(alpha[0]), hi_float(alpha[NDIM + 1]));
+  return {am, 2.0f * float(kFluxScale) * am * rho_max, 2.0f * float(kFluxScale) * am * e_max};
+}
+// Whether a flux exceeds it.
+template <int NDIM>
+__device__ __forceinline__ bool beyond_flux_scale(const double (&out)[NDIM + 2], const FluxScale& F) {
   constexpr int NVAR = NDIM + 2;
-  const float am = 2.0f * fmaxf(hi_float(alpha[0]), hi_float(alpha[NVAR - 1]));
-  const float s0 = 2.0f * float(kFluxScale) * am * rho_max, sE = 2.0f * float(kFluxScale) * am * e_max;
-  bool big = !(fabsf(hi_float(out[0])) <= s0) || !(fabsf(hi_float(out[NVAR - 1])) <= sE);
+  bool big = !(fabsf(hi_float(out[0])) <= F.s0) || !(fabsf(hi_float(out[NVAR - 1])) <= F.sE);
 #pragma unroll
-  for (int k = 0; k < NDIM; ++k) big = big || !(fabsf(hi_float(out[1 + k])) <= s0 * am);
+  for (int k = 0; k < NDIM; ++k) big = big || !(fabsf(hi_float(out[1 + k])) <= F.s0 * F.am);
   return big;
+}
+// Whether the fields' differences do (m: |f| of both sides added, times 30), one by
+// one: in a cold region beside a fast one the two acoustic ones go with alpha / c
+// and cancel in their sum.
+template <int NDIM, int DIR>
+__device__ __forceinline__ bool fields_beyond_flux_scale(const float (&m)[NDIM + 2], const double (&u)[NDIM], double H,
+                                                         double q2, const FluxScale& F) {
+  constexpr int NVAR = NDIM + 2;
+  const float fa = m[0] + m[NVAR - 1];
+  float en = fmaf(fabsf(hi_float(H)), fa, 0.5f * hi_float(q2) * m[1]);
+  bool big = !(fa + m[1] <= F.s0);
+  int g = 2;
+#pragma unroll
+  for (int k = 0; k < NDIM; ++k) {
+    if (k == DIR) continue;
+    const float ft = m[g++];
+    big = big || !(ft <= F.s0 * F.am);
+    en = fmaf(fabsf(hi_float(u[k])), ft, en);
+  }
+  return big || !(en <= F.sE);
 }
 
 template <int NDIM>
@@ -528,6 +555,7 @@ __device__ __forceinline__ uint32_t warp_correct(const double* __restrict__ U, c
   const unsigned lane = threadIdx.x & 31u;
   bool whole = false;
   double q2 = 0.0;
+  FluxScale scale{};
   __syncwarp();
   if (open) {
     I cells[6];
@@ -553,7 +581,8 @@ __device__ __forceinline__ uint32_t warp_correct(const double* __restrict__ U, c
         rm = fmaxf(rm, fabsf(hi_float(ldc<GH>(U, gc.U, ncell, 0, cells[j]))));
         em = fmaxf(em, fabsf(hi_float(ldc<GH>(U, gc.U, ncell, NVAR - 1, cells[j]))));
       }
-      whole = (open & kRough) || beyond_flux_scale<NDIM>(out, alpha, rm, em);
+      scale = flux_scale<NDIM>(alpha, rm, em);
+      whole = (open & kRough) || beyond_flux_scale<NDIM>(out, scale);
     }
 #pragma unroll
     for (int k = 0; k < NDIM; ++k) W.u[k][lane] = R.u[k];
@@ -567,126 +596,141 @@ __device__ __forceinline__ uint32_t warp_correct(const double* __restrict__ U, c
     W.q[lane] = q;
     q2 = R.q2;
   }
-  const unsigned mask = whole ? kAllOpen<NDIM> : open & kAllOpen<NDIM>;
-  unsigned n = 0;
+  unsigned mask = whole ? kAllOpen<NDIM> : open & kAllOpen<NDIM>;
+  for (;;) {
+    unsigned n = 0;
 #pragma unroll
-  for (int b = 0; b < NREC; ++b) {
-    const unsigned m = __ballot_sync(0xffffffffu, (mask >> b) & 1u);
-    if ((mask >> b) & 1u) {
-      W.item[n + __popc(m & ((1u << lane) - 1u))] =
-          static_cast<uint16_t>(lane | unsigned(b) << 5 | (whole ? 1u << 9 : 0u));
-    } else {
-      W.d[b][lane] = SELECT ? 7.0 : 0.0;
+    for (int b = 0; b < NREC; ++b) {
+      const unsigned m = __ballot_sync(0xffffffffu, (mask >> b) & 1u);
+      if ((mask >> b) & 1u) {
+        W.item[n + __popc(m & ((1u << lane) - 1u))] =
+            static_cast<uint16_t>(lane | unsigned(b) << 5 | (whole ? 1u << 9 : 0u));
+      } else {
+        W.d[b][lane] = SELECT ? 7.0 : 0.0;
+      }
+      n += __popc(m);
     }
-    n += __popc(m);
-  }
-  __syncwarp();
-  for (unsigned i = lane; i < n; i += 32u) {
-    const unsigned it = W.item[i];
-    const unsigned o = it & 31u, b = (it >> 5) & 15u, s = b >> 1;
-    const bool minus = b & 1u;
-    I cells[6];
-    unsigned flips;
-    cells_of(W.q[o], cells, flips);
-    double v[5];
-    auto point = [&](int j, double (&Uj)[NVAR], double& un) {
-      const int p = minus ? 5 - j : j;
-      const bool fj = (flips >> p) & 1u;
-      const I c = minus ? cells[5 - j] : cells[j];
-#pragma unroll
-      for (int k = 0; k < NVAR; ++k) Uj[k] = ldc<GH>(U, gc.U, ncell, k, c);
-      Uj[1 + DIR] = flip_sign(Uj[1 + DIR], fj);
-      un = flip_sign(ldc<GH>(aux, gc.aux, ncell, DIR, c), fj);
-      return ldc<GH>(aux, gc.aux, ncell, NDIM, c);
-    };
-    // the split values of the characteristic path (interface_flux)
-    if (s >= 2 && s < NVAR - 1) {   // shear field of the direction t
-      const int t = (int(s) - 2 < DIR) ? int(s) - 2 : int(s) - 1;
-      const double ut = W.u[t][o];
-#pragma unroll
-      for (int j = 0; j < 5; ++j) {
+    __syncwarp();
+    for (unsigned i = lane; i < n; i += 32u) {
+      const unsigned it = W.item[i];
+      const unsigned o = it & 31u, b = (it >> 5) & 15u, s = b >> 1;
+      const bool minus = b & 1u;
+      I cells[6];
+      unsigned flips;
+      cells_of(W.q[o], cells, flips);
+      double v[5];
+      auto point = [&](int j, double (&Uj)[NVAR], double& un) {
         const int p = minus ? 5 - j : j;
         const bool fj = (flips >> p) & 1u;
         const I c = minus ? cells[5 - j] : cells[j];
-        const double w = fma(-ut, ldc<GH>(U, gc.U, ncell, 0, c), ldc<GH>(U, gc.U, ncell, 1 + t, c));
-        v[j] = (flip_sign(ldc<GH>(aux, gc.aux, ncell, DIR, c), fj) + (minus ? -alpha[1] : alpha[1])) * w;
-      }
-    } else {
-      // acoustic (+-) and entropy fields: the row l_s = wA (hb2, -hb1 u, hb1) +
-      // (u_d, -e_d, 0) (+-hic) (+ e_0 for the entropy field) of project's
-      // combinations, z_s = wA b1 (u_d - u~_d)/2 -+ hic
-      const double hic = s == 0 ? W.hic[o] : (s == 1 ? 0.0 : -W.hic[o]);
-      const double wA = s == 1 ? -2.0 : 1.0;
-      const double mh = wA * W.hb1[o], ud = W.u[DIR][o];
-      double l[NVAR];
-      l[0] = fma(ud, hic, fma(wA, W.hb2[o], s == 1 ? 1.0 : 0.0));
 #pragma unroll
-      for (int k = 0; k < NDIM; ++k) l[1 + k] = k == DIR ? fma(-ud, mh, -hic) : -W.u[k][o] * mh;
-      l[NVAR - 1] = mh;
-      const double za = wA * W.b1[o], z0 = fma(-za, W.hud[o], -hic);
-      const double al = s == 0 ? alpha[0] : (s == 1 ? alpha[1] : alpha[NVAR - 1]);
-      const double as = minus ? -al : al;
+        for (int k = 0; k < NVAR; ++k) Uj[k] = ldc<GH>(U, gc.U, ncell, k, c);
+        Uj[1 + DIR] = flip_sign(Uj[1 + DIR], fj);
+        un = flip_sign(ldc<GH>(aux, gc.aux, ncell, DIR, c), fj);
+        return ldc<GH>(aux, gc.aux, ncell, NDIM, c);
+      };
+      // the split values of the characteristic path (interface_flux)
+      if (s >= 2 && s < NVAR - 1) {   // shear field of the direction t
+        const int t = (int(s) - 2 < DIR) ? int(s) - 2 : int(s) - 1;
+        const double ut = W.u[t][o];
 #pragma unroll
-      for (int j = 0; j < 5; ++j) {
-        double Uj[NVAR], un;
-        const double pn = point(j, Uj, un);
-        double w = l[0] * Uj[0];
-#pragma unroll
-        for (int k = 1; k < NVAR; ++k) w = fma(l[k], Uj[k], w);
-        v[j] = fma(un + as, w, pn * fma(za, un, z0));
-      }
-    }
-    const double e[4] = {v[1] - v[0], v[2] - v[1], v[3] - v[2], v[4] - v[3]};
-    const unsigned sel = teno_select(v, e, S);
-    if constexpr (SELECT) {
-      W.d[b][o] = double(sel);
-      continue;
-    }
-    double dl = 0.0;
-    if ((it >> 9) || sel == 0u) {   // the whole value; for no stencil at all, less the all-kept one
-      const unsigned r = it >> 9 ? sel : 7u;
-      dl = fma(c_lin[r][0], v[0], fma(c_lin[r][1], v[1], fma(c_lin[r][2], v[2], fma(c_lin[r][3], v[3], c_lin[r][4] * v[4]))));
-      if (!(it >> 9)) dl = -dl;
-    } else if (sel != 7u) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) dl = fma(c_cut[sel][j], e[j], dl);
-    }
-    W.d[b][o] = dl;
-  }
-  __syncwarp();
-  if constexpr (SELECT) {
-    uint32_t w = 0;
-#pragma unroll
-    for (int b = 0; b < NREC; ++b) w |= static_cast<uint32_t>(W.d[b][lane]) << (3 * b);
-    return w;
-  }
-  if (open) {
-    // back-projection of the differences (the whole values), as interface_flux's
-    double f[NVAR];
-#pragma unroll
-    for (int s = 0; s < NVAR; ++s) f[s] = (W.d[2 * s][lane] + W.d[2 * s + 1][lane]) * kFluxScale;
-    double u[NDIM];
-#pragma unroll
-    for (int k = 0; k < NDIM; ++k) u[k] = W.u[k][lane];
-    if (whole)
-#pragma unroll
-      for (int k = 0; k < NVAR; ++k) out[k] = 0.0;
-    const double sa = f[0] + f[NVAR - 1], da = (f[NVAR - 1] - f[0]) * W.cs[lane];
-    const double rho_f = sa + f[1];
-    out[0] += rho_f;
-    double eng = fma(W.H[lane], sa, fma(u[DIR], da, 0.5 * q2 * f[1]));
-    int g = 2;
-#pragma unroll
-    for (int k = 0; k < NDIM; ++k) {
-      if (k == DIR) {
-        out[1 + k] += fma(u[k], rho_f, da);
+        for (int j = 0; j < 5; ++j) {
+          const int p = minus ? 5 - j : j;
+          const bool fj = (flips >> p) & 1u;
+          const I c = minus ? cells[5 - j] : cells[j];
+          const double w = fma(-ut, ldc<GH>(U, gc.U, ncell, 0, c), ldc<GH>(U, gc.U, ncell, 1 + t, c));
+          v[j] = (flip_sign(ldc<GH>(aux, gc.aux, ncell, DIR, c), fj) + (minus ? -alpha[1] : alpha[1])) * w;
+        }
       } else {
-        out[1 + k] += fma(u[k], rho_f, f[g]);
-        eng = fma(u[k], f[g], eng);
-        ++g;
+        // acoustic (+-) and entropy fields: the row l_s = wA (hb2, -hb1 u, hb1) +
+        // (u_d, -e_d, 0) (+-hic) (+ e_0 for the entropy field) of project's
+        // combinations, z_s = wA b1 (u_d - u~_d)/2 -+ hic
+        const double hic = s == 0 ? W.hic[o] : (s == 1 ? 0.0 : -W.hic[o]);
+        const double wA = s == 1 ? -2.0 : 1.0;
+        const double mh = wA * W.hb1[o], ud = W.u[DIR][o];
+        double l[NVAR];
+        l[0] = fma(ud, hic, fma(wA, W.hb2[o], s == 1 ? 1.0 : 0.0));
+#pragma unroll
+        for (int k = 0; k < NDIM; ++k) l[1 + k] = k == DIR ? fma(-ud, mh, -hic) : -W.u[k][o] * mh;
+        l[NVAR - 1] = mh;
+        const double za = wA * W.b1[o], z0 = fma(-za, W.hud[o], -hic);
+        const double al = s == 0 ? alpha[0] : (s == 1 ? alpha[1] : alpha[NVAR - 1]);
+        const double as = minus ? -al : al;
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+          double Uj[NVAR], un;
+          const double pn = point(j, Uj, un);
+          double w = l[0] * Uj[0];
+#pragma unroll
+          for (int k = 1; k < NVAR; ++k) w = fma(l[k], Uj[k], w);
+          v[j] = fma(un + as, w, pn * fma(za, un, z0));
+        }
+      }
+      const double e[4] = {v[1] - v[0], v[2] - v[1], v[3] - v[2], v[4] - v[3]};
+      const unsigned sel = teno_select(v, e, S);
+      if constexpr (SELECT) {
+        W.d[b][o] = double(sel);
+        continue;
+      }
+      double dl = 0.0;
+      if ((it >> 9) || sel == 0u) {   // the whole value; for no stencil at all, less the all-kept one
+        const unsigned r = it >> 9 ? sel : 7u;
+        dl = fma(c_lin[r][0], v[0], fma(c_lin[r][1], v[1], fma(c_lin[r][2], v[2], fma(c_lin[r][3], v[3], c_lin[r][4] * v[4]))));
+        if (!(it >> 9)) dl = -dl;
+      } else if (sel != 7u) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) dl = fma(c_cut[sel][j], e[j], dl);
+      }
+      W.d[b][o] = dl;
+    }
+    __syncwarp();
+    if constexpr (SELECT) {
+      uint32_t w = 0;
+#pragma unroll
+      for (int b = 0; b < NREC; ++b) w |= static_cast<uint32_t>(W.d[b][lane]) << (3 * b);
+      return w;
+    }
+    bool again = false;
+    if (mask) {
+      // back-projection of the differences (the whole values), as interface_flux's
+      double f[NVAR];
+#pragma unroll
+      for (int s = 0; s < NVAR; ++s) f[s] = (W.d[2 * s][lane] + W.d[2 * s + 1][lane]) * kFluxScale;
+      double u[NDIM];
+#pragma unroll
+      for (int k = 0; k < NDIM; ++k) u[k] = W.u[k][lane];
+      float mag[NVAR];
+#pragma unroll
+      for (int s = 0; s < NVAR; ++s)
+        mag[s] = float(kFluxScale) * (fabsf(hi_float(W.d[2 * s][lane])) + fabsf(hi_float(W.d[2 * s + 1][lane])));
+      again = !whole && fields_beyond_flux_scale<NDIM, DIR>(mag, u, W.H[lane], q2, scale);
+      if (!again) {
+        if (whole)
+#pragma unroll
+          for (int k = 0; k < NVAR; ++k) out[k] = 0.0;
+        const double sa = f[0] + f[NVAR - 1], da = (f[NVAR - 1] - f[0]) * W.cs[lane];
+        const double rho_f = sa + f[1];
+        out[0] += rho_f;
+        double eng = fma(W.H[lane], sa, fma(u[DIR], da, 0.5 * q2 * f[1]));
+        int g = 2;
+#pragma unroll
+        for (int k = 0; k < NDIM; ++k) {
+          if (k == DIR) {
+            out[1 + k] += fma(u[k], rho_f, da);
+          } else {
+            out[1 + k] += fma(u[k], rho_f, f[g]);
+            eng = fma(u[k], f[g], eng);
+            ++g;
+          }
+        }
+        out[NVAR - 1] += eng;
       }
     }
-    out[NVAR - 1] += eng;
+    // (the lanes that are done hold nothing open in the second round)
+    mask = again ? kAllOpen<NDIM> : 0u;
+    whole = again;
+    if (!__any_sync(0xffffffffu, again)) break;
+    __syncwarp();
   }
   return 0u;
 }
@@ -702,9 +746,17 @@ __device__ __forceinline__ uint32_t warp_correct(const double* __restrict__ U, c
 // `fl` receives the flag bytes when WITH_FLAGS
 // (without flags, bits 0..2 still hold the selections used).
 // MODE kFluxFull computes the flux; kFluxChar skips the certified test and takes
-// the characteristic path (WENO-Z, which has no such test).
+// the characteristic path (WENO-Z, which has no such test); kFluxWhole does too, and
+// sums the whole characteristic values.
 // ---------------------------------------------------------------------------
-constexpr int kFluxFull = 0, kFluxChar = 1;
+constexpr int kFluxFull = 0, kFluxChar = 1, kFluxWhole = 2;
+
+template <int NDIM, int DIR, bool GH, class I>
+__device__ __noinline__ void interface_flux_whole(const double* __restrict__ U, const double* __restrict__ aux,
+                                                  int64_t ncell, const I (&cells)[6], unsigned flips,
+                                                  const double (&alpha)[NDIM + 2], const Scheme& S,
+                                                  double (&out)[NDIM + 2], int* __restrict__ status,
+                                                  const GhostCells& gc);
 
 template <int NDIM, int DIR, bool WITH_FLAGS, int MODE = kFluxFull, bool GH = false, class I = int64_t>
 __device__ __forceinline__ void interface_flux(const double* __restrict__ U,
@@ -762,7 +814,7 @@ __device__ __forceinline__ void interface_flux(const double* __restrict__ U,
       }
     };
 
-    if (!WITH_FLAGS && MODE != kFluxChar && S.keep_idx >= 0) {
+    if (!WITH_FLAGS && MODE == kFluxFull && S.keep_idx >= 0) {
       CertIfc<NDIM> C;
       cert_begin<NDIM, DIR>(R, alpha, C);
 #pragma unroll
@@ -779,7 +831,8 @@ __device__ __forceinline__ void interface_flux(const double* __restrict__ U,
     // As in warp_correct: the flux with every stencil kept plus the fields'
     // differences against it, unless that flux is far beyond the flux scale
     // (WENO-Z keeps no stencil exactly linear: always the whole values).
-    bool cut = S.variant != kSchemeWenoZ;
+    bool cut = MODE != kFluxWhole && S.variant != kSchemeWenoZ;
+    FluxScale scale{};
     if (cut) {
       float rm = 0.0f, em = 0.0f;
 #pragma unroll
@@ -788,7 +841,8 @@ __device__ __forceinline__ void interface_flux(const double* __restrict__ U,
         em = fmaxf(em, fabsf(hi_float(Ux[j][NVAR - 1])));
       }
       closed_in_registers<NDIM, DIR>(Ux, half, R, nal, out);
-      cut = !beyond_flux_scale<NDIM>(out, alpha, rm, em);
+      scale = flux_scale<NDIM>(alpha, rm, em);
+      cut = !beyond_flux_scale<NDIM>(out, scale);
     }
     if (!cut)
 #pragma unroll
@@ -825,16 +879,30 @@ __device__ __forceinline__ void interface_flux(const double* __restrict__ U,
         vm[j][f] = fma(nal[1], w[f], vp[j][f]);
       }
     }
+    float mag[NVAR];   // |difference+| + |difference-| at most
 #pragma unroll
     for (int s = 0; s < NVAR; ++s) {
       const double hp = teno5_lad<WITH_FLAGS>(vp[0][s], vp[1][s], vp[2][s], vp[3][s], vp[4][s], 0.0, S, fl[s][0], cut);
       fchar[s] = teno5_lad<WITH_FLAGS>(vm[5][s], vm[4][s], vm[3][s], vm[2][s], vm[1][s], hp, S, fl[s][1], cut);
+      mag[s] = float(kFluxScale) * fmaf(2.0f, fabsf(hi_float(hp)), fabsf(hi_float(fchar[s])));
     }
     if (cut) {   // every stencil kept: the differences are zeros
       bool none = true;
 #pragma unroll
       for (int s = 0; s < NVAR; ++s) none = none && (dbits(fchar[s]) << 1) == 0ull;
       if (none) return;
+      if (fields_beyond_flux_scale<NDIM, DIR>(mag, u, H, q2, scale)) {
+        I cc[6];
+        double aa[NVAR], oo[NVAR];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) cc[j] = cells[j];
+#pragma unroll
+        for (int v = 0; v < NVAR; ++v) aa[v] = alpha[v];
+        interface_flux_whole<NDIM, DIR, GH>(U, aux, ncell, cc, flips, aa, S, oo, status, gc);
+#pragma unroll
+        for (int v = 0; v < NVAR; ++v) out[v] = oo[v];
+        return;
+      }
     }
     // back-projection F^ = R f^char, columns r_0 = (1, u - c e_n, H - u_n c),
     // r_1 = (1, u, q2/2), r_t = (0, e_t, u_t), r_{nvar-1} = (1, u + c e_n, H + u_n c),
@@ -861,6 +929,21 @@ __device__ __forceinline__ void interface_flux(const double* __restrict__ U,
     }
     out[NVAR - 1] += eng;
   }
+}
+
+// the whole characteristic values of an interface whose fields' differences are far
+// beyond the flux scale (out of line: rare)
+template <int NDIM, int DIR, bool GH, class I>
+__device__ __noinline__ void interface_flux_whole(const double* __restrict__ U, const double* __restrict__ aux,
+                                                  int64_t ncell, const I (&cells)[6], unsigned flips,
+                                                  const double (&alpha)[NDIM + 2], const Scheme& S,
+                                                  double (&out)[NDIM + 2], int* __restrict__ status,
+                                                  const GhostCells& gc) {
+  double nal[NDIM + 2];
+#pragma unroll
+  for (int f = 0; f < NDIM + 2; ++f) nal[f] = -2.0 * alpha[f];
+  unsigned fl[NDIM + 2][2];
+  interface_flux<NDIM, DIR, false, kFluxWhole, GH>(U, aux, ncell, cells, flips, alpha, nal, S, out, fl, status, gc);
 }
 
 // ---------------------------------------------------------------------------
